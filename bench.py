@@ -393,7 +393,7 @@ def run_sweep(args):
                          "kernel_ms": round(kernel_ms, 4),
                          "algorithmic_bytes_per_launch": alg_bytes, "bytes_per_node": bpn},
             "e2e": e2e,
-            "gpu_launches": args.steps * 2,
+            "gpu_launches": args.steps + 1,  # one per step, the totals once per call
             "clocks": clocks,
         }
         if world == 1 and not args.no_cpu_baseline:
@@ -548,7 +548,7 @@ def main():
                          "algorithmic_bytes_per_launch": alg_bytes,
                          "bytes_per_node": bpn},
             "e2e": e2e,
-            "gpu_launches": args.steps * launches,
+            "gpu_launches": launches,
             "clocks": clocks,
             "mass_totals": [float(v) for v in m_after],
         }
@@ -627,7 +627,10 @@ def measure(args, cfg, fields, solid, precision, tile, kernel, world, local, dis
            "job": f"upload rho/phi/psi (fp64, pinned) + equilibrium init, {args.steps} steps, "
                   "download C1..C3 (fp64) + mass totals"}
     out = {"value": value, "ms": ms, "clocks": clocks, "mass": m_after, "kernel_ms": kernel_ms,
-           "kind": eng.kernel, "e2e": e2e, "launches": eng.launches_per_step}
+           "kind": eng.kernel, "e2e": e2e,
+           # the fused step reduces its totals once per call, the split step in every step
+           "launches": (args.steps * (eng.launches_per_step - 1) + 1 if eng.kernel == "fused"
+                        else args.steps * eng.launches_per_step)}
     eng.close()
     if keep_fields:
         out["C"] = [t.numpy() for t in outs]

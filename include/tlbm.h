@@ -213,7 +213,8 @@ size_t tlbm_state_bytes(const tlbm *t);
 tlbm_status tlbm_get_state(tlbm *t, void *host, size_t bytes);
 tlbm_status tlbm_set_state(tlbm *t, const void *host, size_t bytes);
 
-/* Kernel launches per tlbm_step(1) of the current configuration. */
+/* Kernel launches per tlbm_step(1) of the current configuration.  The fused
+ * kinds reduce the totals once per call: tlbm_step(n) is n + 1 launches. */
 int tlbm_launches_per_step(const tlbm *t);
 
 /*
@@ -313,7 +314,7 @@ tlbm_status tlbm_wetting_from_angles(const double kappa[3], double alpha, double
  * sweeps such as the contact-angle runs of Sec. Contact Angles.
  * Many independent lattices of one lattice type and storage format (for example
  * a contact-angle or kappa sweep over lattices of uneven size) advanced by ONE
- * kernel launch per step plus one launch for all their FP64 totals.  A batch
+ * kernel launch per step, and one launch per call for all their FP64 totals.  A batch
  * groups existing engines; each keeps its own state, parameters, solid mask and
  * accessors (tlbm_fields, tlbm_mass, ...), and a batched step gives bit for bit
  * the same populations as stepping each member alone with the same tile.

@@ -425,6 +425,7 @@ tlbm_status tlbm_step(tlbm* t, int64_t nsteps) {
         }
         ++t->steps;
     }
+    if (nsteps > 0) CK(t->ops->totals(t->d, kind, t->st));
     return TLBM_OK;
 }
 
@@ -708,6 +709,12 @@ tlbm_status batch_plain_steps(tlbm_batch* b, int64_t n) {
     return TLBM_OK;
 }
 
+// every member's totals of the step before, once per call
+tlbm_status batch_totals(tlbm_batch* b) {
+    const cudaError_t e = b->ops->batch_totals(b->bs, b->st);
+    return e == cudaSuccess ? TLBM_OK : bfail(b, TLBM_ERR_CUDA, "batched totals: %s", cudaGetErrorString(e));
+}
+
 }  // namespace
 
 extern "C" {
@@ -819,7 +826,11 @@ tlbm_status tlbm_batch_step(tlbm_batch* b, int64_t nsteps) {
     if (nsteps < 0) return bfail(b, TLBM_ERR_ARG, "nsteps must be >= 0");
     tlbm_status s = batch_aligned(b);
     if (s != TLBM_OK) return s;
-    if (!b->use_graph || b->timing || nsteps < 2) return batch_plain_steps(b, nsteps);
+    if (nsteps == 0) return TLBM_OK;
+    if (!b->use_graph || b->timing || nsteps < 2) {
+        s = batch_plain_steps(b, nsteps);
+        return s == TLBM_OK ? batch_totals(b) : s;
+    }
     // graph of two batched steps, captured once on a private stream and replayed
     // on the members' stream; it starts and ends at buffer parity graph_par
     if (b->exec && b->sims[0]->cur != b->graph_par) {
@@ -853,7 +864,8 @@ tlbm_status tlbm_batch_step(tlbm_batch* b, int64_t nsteps) {
         if (e != cudaSuccess) return bfail(b, TLBM_ERR_CUDA, "graph launch: %s", cudaGetErrorString(e));
         for (tlbm* m : b->members) m->steps += 2;
     }
-    return batch_plain_steps(b, nsteps & 1);
+    s = batch_plain_steps(b, nsteps & 1);
+    return s == TLBM_OK ? batch_totals(b) : s;
 }
 
 tlbm_status tlbm_batch_autotune(tlbm_batch* b, int trial_steps, int* variant, int* chunk) {
@@ -881,6 +893,7 @@ tlbm_status tlbm_batch_autotune(tlbm_batch* b, int trial_steps, int* variant, in
             cudaEventRecord(e0, b->st);
             if (batch_plain_steps(b, trial_steps) != TLBM_OK) continue;
             cudaEventRecord(e1, b->st);
+            if (batch_totals(b) != TLBM_OK) continue;
             float ms = 0.0f;
             if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) continue;
             if (ms < best) {

@@ -47,7 +47,17 @@ struct MGeom {
     long long rowstride;  // bytes between consecutive (b, m) rows: ncx * chunk bytes
     long long bytes;      // bytes of one population buffer (bounds-checked kernels)
     unsigned long long* check;  // first bounds violation (bounds-checked kernels)
+    int* flag;            // raised by a block whose sums are not finite
 };
+
+// a block's FP64 sums of rho, phi, psi: its partial sums and the non-finite flag
+__device__ __forceinline__ void put_block_sums(const MGeom& g, double* __restrict__ partials, int bid, double r,
+                                               double p, double s) {
+    partials[3 * bid + 0] = r;
+    partials[3 * bid + 1] = p;
+    partials[3 * bid + 2] = s;
+    if (!(isfinite(r) && isfinite(p) && isfinite(s))) *g.flag = 1;
+}
 
 // Bounds checks of the checked kernel variants (CHK).  A violation is recorded
 // as (code << 56 | offset) in *g.check -- the first one wins -- and the access
@@ -535,11 +545,7 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
     double mr, mp, ms;
     msum.get(mr, mp, ms);
     block_sum3(mr, mp, ms);
-    if (tid == 0) {
-        partials[3 * bid + 0] = mr;
-        partials[3 * bid + 1] = mp;
-        partials[3 * bid + 2] = ms;
-    }
+    if (tid == 0) put_block_sums(g, partials, bid, mr, mp, ms);
 }
 
 template <int Q, typename S, int TX, int TY, bool ILP, bool EARLY, bool PF = false, int HINT = 0, bool CHK = false>
@@ -898,11 +904,7 @@ __device__ __forceinline__ void solid_body(const MGeom& g, const S* __restrict__
     double mr, mp, ms;
     msum.get(mr, mp, ms);
     block_sum3(mr, mp, ms);
-    if (tid == 0) {
-        partials[3 * bid + 0] = mr;
-        partials[3 * bid + 1] = mp;
-        partials[3 * bid + 2] = ms;
-    }
+    if (tid == 0) put_block_sums(g, partials, bid, mr, mp, ms);
 }
 
 template <int Q, typename S, int TX, int TY, bool CHK = false>
@@ -1085,6 +1087,7 @@ inline MGeom mgeom(const tlbm_host::DevState& d, const FusedCfg<Q>& c) {
     g.NC = (g.NM + c.MC - 1) / c.MC;  // chunks of MC planes or one fewer (balanced)
     g.bytes = d.pop_bytes;
     g.check = d.check;
+    g.flag = d.flag;
     g.tilesA = (g.NA + c.TX - 1) / c.TX;
     g.tilesB = (g.NB + c.TY - 1) / c.TY;
     return g;
@@ -1095,12 +1098,6 @@ inline long long fused_blocks(const tlbm_host::DevState& d) {
     const FusedCfg<Q> c = fused_cfg<Q>(d);
     const MGeom g = mgeom<Q, S>(d, c);
     return (long long)g.tilesA * g.tilesB * g.NC;
-}
-
-// number of partial sums the last step wrote (for k_mass_final)
-template <int Q, typename S>
-inline int fused_partials(const tlbm_host::DevState& d, int kind) {
-    return kind == tlbm_host::KIND_FUSED ? (int)fused_blocks<Q, S>(d) : kMassBlocks;
 }
 
 // Launch of a kernel with STG staged values per thread of 128 (dynamic shared
@@ -1348,8 +1345,15 @@ inline cudaError_t batch_step(tlbm_host::BatchState& b, cudaStream_t st, cudaEve
         }
     }
     if (ev1) cudaEventRecord(ev1, st);
-    k_mass_final_batch<T><<<n, kThreads, 0, st>>>(d);
     for (int k = 0; k < n; ++k) b.sims[k]->cur ^= 1;
+    return cudaGetLastError();
+}
+
+// totals of every member's last batched step (the same sums under both parities)
+template <int Q, typename S>
+inline cudaError_t batch_totals(tlbm_host::BatchState& b, cudaStream_t st) {
+    using T = typename Store<S>::T;
+    k_mass_final_batch<T><<<b.count, kThreads, 0, st>>>(static_cast<const SimDesc<T>*>(b.desc));
     return cudaGetLastError();
 }
 

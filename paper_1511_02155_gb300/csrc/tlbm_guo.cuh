@@ -559,11 +559,7 @@ __device__ __forceinline__ void guo_body(const MGeom& g, const S* __restrict__ s
     double mr, mp, ms;
     msum.get(mr, mp, ms);
     block_sum3(mr, mp, ms);
-    if (tid == 0) {
-        partials[3 * bid + 0] = mr;
-        partials[3 * bid + 1] = mp;
-        partials[3 * bid + 2] = ms;
-    }
+    if (tid == 0) put_block_sums(g, partials, bid, mr, mp, ms);
 }
 
 template <int Q, typename S, int TX, int TY>

@@ -87,8 +87,13 @@ struct AdjJob {
 
 struct Ops {
     // one time step; flips cur.  When ev0/ev1 are not null they are recorded on
-    // the stream just before and just after the step's main kernel(s).
+    // the stream just before and just after the step's main kernel(s).  The fused
+    // kinds leave their FP64 sums per block (and raise the non-finite flag
+    // themselves); totals() reduces them.
     cudaError_t (*step)(DevState& d, int kind, cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1);
+    // totals of the last step from its block sums (nothing to do after a split
+    // step, which reduces its own)
+    cudaError_t (*totals)(DevState& d, int kind, cudaStream_t st);
     // populations at equilibrium of device double fields (u may be nullptr)
     cudaError_t (*init)(DevState& d, const double* rho, const double* phi, const double* psi,
                         const double* u, cudaStream_t st);
@@ -107,6 +112,8 @@ struct Ops {
     cudaError_t (*batch_build)(BatchState& b, cudaStream_t st);
     // one batched step of every member; ev0/ev1 (if not null) bracket the main kernel
     cudaError_t (*batch_step)(BatchState& b, cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1);
+    // every member's totals of the last batched step
+    cudaError_t (*batch_totals)(BatchState& b, cudaStream_t st);
     // forward run with checkpoints, then the adjoint back to the initial fields
     // (FP64 and FP32 storage; cudaErrorNotSupported for the 16-bit formats)
     cudaError_t (*adjoint)(DevState& d, int kind, const AdjJob& job, cudaStream_t st);
