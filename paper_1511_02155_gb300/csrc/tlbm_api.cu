@@ -899,7 +899,7 @@ tlbm_status tlbm_batch_autotune(tlbm_batch* b, int trial_steps, int* variant, in
             if (ms < best) {
                 best = ms;
                 bv = sh;
-                bc = ch;
+                bc = b->bs.auto_tile >> 8;  // the chunk that the automatic choice came to (0: each member its own)
             }
         }
     }

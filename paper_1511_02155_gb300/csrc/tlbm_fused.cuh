@@ -90,6 +90,13 @@ __device__ __forceinline__ long long chk_index(const MGeom& g, long long i, long
     return i;
 }
 
+// blocks per SM asked of the compiler: 16 warps; one-warp blocks in double keep up
+// to 255 registers
+template <typename S>
+constexpr int blocks_per_sm(int threads) {
+    return sizeof(S) == 8 && threads == 32 ? 8 : 512 / threads;
+}
+
 __device__ __forceinline__ int modp(int v, int n) {
     v %= n;
     return v < 0 ? v + n : v;
@@ -549,7 +556,7 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
 }
 
 template <int Q, typename S, int TX, int TY, bool ILP, bool EARLY, bool PF = false, int HINT = 0, bool CHK = false>
-__global__ void __launch_bounds__(TX * TY, 512 / (TX * TY))  // 16 warps per SM
+__global__ void __launch_bounds__(TX * TY, blocks_per_sm<S>(TX * TY))
 k_fused(MGeom g, const S* __restrict__ src, S* __restrict__ dst, Phys<typename Store<S>::T> P,
         double* __restrict__ partials) {
     fused_body<Q, S, TX, TY, ILP, EARLY, PF, HINT, 0, 1, CHK>(g, src, dst, P, partials, blockIdx.x);
@@ -908,7 +915,7 @@ __device__ __forceinline__ void solid_body(const MGeom& g, const S* __restrict__
 }
 
 template <int Q, typename S, int TX, int TY, bool CHK = false>
-__global__ void __launch_bounds__(TX * TY, 512 / (TX * TY))
+__global__ void __launch_bounds__(TX * TY, blocks_per_sm<S>(TX * TY))
 k_fused_solid(MGeom g, const S* __restrict__ src, S* __restrict__ dst, const uint32_t* __restrict__ nbm,
               Phys<typename Store<S>::T> P, double* __restrict__ partials) {
     solid_body<Q, S, TX, TY, CHK>(g, src, dst, nbm, P, partials, blockIdx.x);
@@ -951,7 +958,7 @@ __device__ __forceinline__ const SimDesc<T>& batch_member(const SimDesc<T>* __re
 }
 
 template <int Q, typename S, int TX, int TY, bool PF, int HINT>
-__global__ void __launch_bounds__(TX * TY, 512 / (TX * TY))
+__global__ void __launch_bounds__(TX * TY, blocks_per_sm<S>(TX * TY))
 k_fused_batch(const SimDesc<typename Store<S>::T>* __restrict__ d, int nsims) {
     __shared__ SimDesc<typename Store<S>::T> sh;
     const SimDesc<typename Store<S>::T>& m = batch_member(d, nsims, sh);
@@ -960,7 +967,7 @@ k_fused_batch(const SimDesc<typename Store<S>::T>* __restrict__ d, int nsims) {
 }
 
 template <int Q, typename S, int TX, int TY>
-__global__ void __launch_bounds__(TX * TY, 512 / (TX * TY))
+__global__ void __launch_bounds__(TX * TY, blocks_per_sm<S>(TX * TY))
 k_fused_solid_batch(const SimDesc<typename Store<S>::T>* __restrict__ d, int nsims) {
     __shared__ SimDesc<typename Store<S>::T> sh;
     const SimDesc<typename Store<S>::T>& m = batch_member(d, nsims, sh);
@@ -996,11 +1003,72 @@ inline int grid_of(long long n, int sms) {
     return (int)(b < 1 ? 1 : (b > cap ? cap : b));
 }
 
+// Cost of marching nb blocks of mc planes each, up to a factor.  A block pays for
+// its planes plus halo prologue planes; a plane of one of b blocks that share an
+// SM (res fit) takes 0.25 + 0.19 b' times a full SM's plane, b' = 4 b / res: alone
+// a block waits out the latency of its loads, together they fill each other's
+// waits.  Blocks beyond what fits wait for whole rounds; over many rounds the
+// blocks drift apart and only the sum counts.  FP64 is bound by its few FP64
+// units: there every node's operations count, about 400 for a collision and 72
+// for the moments of a (node, halo) pair, and two blocks hide each other.
+// Against the measured times of 14 lattices (64^2 .. 1000x701, 40^3 .. 160^2x96)
+// over chunks of 1 .. 64 planes the cheapest chunk of this model is within 8 % of
+// the fastest measured; halving 64 or 16 until 4 blocks per SM are reached, the
+// earlier rule, lost up to 27 % (FP32, one step: 64x64 15.4 us against 11.3,
+// 96^3 117.4 against 102.9, walled 144x128x80 299 against 267).
+inline double march_cost(double nb, int mc, int halo, int res, int sms, bool dbl) {
+    const double full = (double)res * sms;
+    if (dbl) {
+        const double per = nb / sms, b = per > 8.0 ? per : (double)(long long)(per + 0.9999);
+        return (mc * 400.0 + (mc + halo) * 72.0) * (b < 2.0 ? 1.3 : b);
+    }
+    auto plane = [&](double b) { return 0.25 + 0.19 * 4.0 * b / res; };
+    const double rounds = nb / full;
+    if (rounds >= 4.0) return (mc + halo) * plane(res) * rounds;
+    const double whole = (double)(long long)rounds;
+    const double rest = nb - whole * full;
+    const double b = (double)(long long)((rest + sms - 1) / sms);
+    return (mc + halo) * (whole * plane(res) + (rest > 0 ? plane(b) : 0.0));
+}
+
+// Planes per block (chunk) of one marching launch over n lattices with cols[k]
+// tile columns of nm[k] planes: the cheapest by march_cost whose block sums fit
+// (caps[k]).  At most 64 planes in 2-D; in 3-D 16 once the grid fills the device
+// eight times over (256^3 FP32: 16 planes 0.692 of HBM, 24..128 planes 0.66..0.69:
+// blocks that start together share their halo rows in L2).
+inline int pick_chunk(const long long* cols, const int* nm, const long long* caps, int n, int halo, int res, int sms,
+                      bool three_d, bool dbl) {
+    double best = 0.0;
+    int bmc = 0;
+    for (int mc = three_d ? 2 : 1; mc <= 64; ++mc) {
+        double nb = 0.0;
+        int used = 0;
+        bool fits = true;
+        for (int k = 0; k < n; ++k) {
+            const int nc = (nm[k] + mc - 1) / mc, per = (nm[k] + nc - 1) / nc;
+            nb += (double)cols[k] * nc;
+            used = per > used ? per : used;
+            fits = fits && cols[k] * nc <= caps[k];
+        }
+        if (!fits) continue;
+        const double c = march_cost(nb, used, halo, res, sms, dbl);
+        if (three_d && used > 16 && nb >= 8.0 * res * sms) continue;
+        if (bmc == 0 || c < best) {
+            best = c;
+            bmc = mc;
+        }
+    }
+    return bmc == 0 ? 64 : bmc;
+}
+
 template <int Q>
 struct FusedCfg {
     int TX, TY, MC;
     int mode;
     int shape;  // resolved D3Q19 shape (4..7: 32x4 kernels with staging)
+    // prologue planes a block recomputes, and blocks per SM (blocks_per_sm)
+    int halo(const tlbm_host::DevState& d) const { return d.solid || d.coupling ? 4 : 2; }
+    int res(const tlbm_host::DevState& d) const { return d.prec == 0 && TX == 32 ? 8 : 512 / (TX * TY); }
 };
 
 // d.tile = shape | mode << 4 | chunk << 8: shape 0 = default (D3Q19 shape 7,
@@ -1017,6 +1085,12 @@ struct FusedCfg {
 // the prefetch).  mode 0 is the default for the shape and format (D3Q19 32x4:
 // 8 for FP32, 12 for 16-bit storage; other D3Q19: 1; D2Q9: 13); 6 selects the
 // plain loop.  chunk = planes per block (0 = chosen from the lattice size).
+// D2Q9 in double: rows of 32 nodes (one warp) where rows of 128 in chunks of four
+// planes leave SMs idle; wider rows recompute fewer halo moments.
+// A batch launches one tile for all members: narrow only if every member is.
+inline bool narrow_rows(const tlbm_host::DevState& d) { return !d.rows128 && d.N < 512LL * d.sms; }
+
+
 template <int Q>
 inline FusedCfg<Q> fused_cfg(const tlbm_host::DevState& d) {
     const bool dbl = d.prec == 0;  // double storage: one default shape only
@@ -1031,7 +1105,8 @@ inline FusedCfg<Q> fused_cfg(const tlbm_host::DevState& d) {
     } else if (d.solid) {
         // solid-aware kernel: a fixed tile per lattice (D3Q19 in double: 16x4 keeps
         // its five-plane rings under the 48 KB static shared-memory limit)
-        c.TX = Q == 19 ? (dbl ? 16 : 32) : (dbl ? 128 : (variant == 2 ? 256 : (variant == 3 ? 64 : 128)));
+        c.TX = Q == 19 ? (dbl ? 16 : 32)
+                       : (dbl ? (narrow_rows(d) ? 32 : 128) : (variant == 2 ? 256 : (variant == 3 ? 64 : 128)));
         c.TY = Q == 19 ? 4 : 1;
     } else if (Q == 19 && dbl) {
         c.TX = 16;  // double storage: a smaller tile keeps the static shared ring small
@@ -1043,7 +1118,7 @@ inline FusedCfg<Q> fused_cfg(const tlbm_host::DevState& d) {
         c.shape = v;
     } else {
         const int v = variant == 0 ? 5 : variant;  // 128-node rows with staging measured fastest
-        c.TX = v == 2 ? 256 : (v == 3 ? 64 : 128);
+        c.TX = dbl ? (narrow_rows(d) ? 32 : 128) : (v == 2 ? 256 : (v == 3 ? 64 : 128));
         c.TY = 1;
         c.shape = v;
     }
@@ -1058,10 +1133,8 @@ inline FusedCfg<Q> fused_cfg(const tlbm_host::DevState& d) {
     const int NB = (Q == 19) ? d.ny : 1;
     const int NM = (Q == 19) ? d.nz : d.ny;
     if (mc <= 0) {
-        // enough blocks to fill every SM of the device a few times over
         const long long cols = (long long)((NA + c.TX - 1) / c.TX) * ((NB + c.TY - 1) / c.TY);
-        mc = (Q == 19) ? 16 : 64;
-        while (mc > 4 && cols * ((NM + mc - 1) / mc) < 4LL * d.sms) mc >>= 1;
+        mc = pick_chunk(&cols, &NM, &d.partials_cap, 1, c.halo(d), c.res(d), d.sms, Q == 19, dbl);
     }
     c.MC = mc < 1 ? 1 : (mc > NM ? NM : mc);
     return c;
@@ -1170,14 +1243,17 @@ inline cudaError_t fused_step(tlbm_host::DevState& d, const Phys<typename Store<
         } else {
             if (c.TX == 256) gos(k_fused_solid<Q, S, 256, 1>, 256);
             else if (c.TX == 64) gos(k_fused_solid<Q, S, 64, 1>, 64);
-            else gos(k_fused_solid<Q, S, 128, 1>, 128);
+            else if (c.TX == 32) {
+                if constexpr (sizeof(S) == 8) gos(k_fused_solid<Q, S, 32, 1>, 32);
+            } else gos(k_fused_solid<Q, S, 128, 1>, 128);
         }
         return cudaGetLastError();
     }
     auto go = [&](auto kern, int threads) { kern<<<(int)nb, threads, 0, st>>>(g, src, dst, P, d.partials); };
     if constexpr (sizeof(S) == 8) {
-        // double storage is the parity path: one tile shape per lattice
+        // double storage is the parity path: one tile shape per lattice and size
         if constexpr (Q == 19) go(k_fused<Q, S, 16, 8, false, false>, 128);
+        else if (c.TX == 32) go(k_fused<Q, S, 32, 1, false, false>, 32);
         else go(k_fused<Q, S, 128, 1, false, false>, 128);
     } else if constexpr (Q == 19) {
         if constexpr (sizeof(S) <= 4) {
@@ -1270,6 +1346,35 @@ inline cudaError_t batch_build(tlbm_host::BatchState& b, cudaStream_t st) {
     const bool solid = b.sims[0]->solid != nullptr;
     std::vector<SimDesc<T>> h(2 * (size_t)n);
     long long block0 = 0;
+    b.auto_tile = b.tile;
+    b.narrow = 1;
+    for (int k = 0; k < n; ++k) b.narrow = b.narrow && narrow_rows(*b.sims[k]);
+    if ((b.tile >> 8) == 0) {
+        // members whose own chunks do not fill the device twice keep them; beyond
+        // that the halo planes of short chunks are what costs, and one chunk is
+        // chosen for the whole grid (24 wells of 128x64 .. 768x384, FP32: 343 us a
+        // step with chunks of 4 to 8 planes, see k_fused_solid_batch)
+        std::vector<long long> cols, caps;
+        long long own = 0;
+        std::vector<int> nm;
+        FusedCfg<Q> c{};
+        tlbm_host::DevState d0 = *b.sims[0];
+        for (int k = 0; k < n; ++k) {
+            tlbm_host::DevState dd = *b.sims[k];
+            dd.tile = b.tile;
+            dd.rows128 = !b.narrow;
+            own += fused_blocks<Q, S>(dd);
+            c = fused_cfg<Q>(dd);
+            cols.push_back((long long)((dd.nx + c.TX - 1) / c.TX) * (Q == 19 ? (dd.ny + c.TY - 1) / c.TY : 1));
+            nm.push_back(Q == 19 ? dd.nz : dd.ny);
+            caps.push_back(dd.partials_cap);
+        }
+        if (own >= 2LL * c.res(d0) * d0.sms) {
+            const int mc = pick_chunk(cols.data(), nm.data(), caps.data(), n, c.halo(d0), c.res(d0), d0.sms, Q == 19,
+                                      d0.prec == 0);
+            b.auto_tile = (b.tile & 255) | mc << 8;
+        }
+    }
     for (int k = 0; k < n; ++k) {
         tlbm_host::DevState& d = *b.sims[k];
         if ((d.solid != nullptr) != solid || d.cur != b.sims[0]->cur) return cudaErrorInvalidValue;
@@ -1279,12 +1384,13 @@ inline cudaError_t batch_build(tlbm_host::BatchState& b, cudaStream_t st) {
             d.nbm_ready = 1;
         }
         tlbm_host::DevState dd = d;
-        dd.tile = b.tile;
+        dd.tile = b.auto_tile;
+        dd.rows128 = !b.narrow;
         const FusedCfg<Q> c = fused_cfg<Q>(dd);
         // shapes with a batched kernel (batch_step): every solid shape; periodic
         // D3Q19 32x4 (16x8 in double), periodic D2Q9 128
         const bool shape_ok = solid || (Q == 19 ? (sizeof(S) == 8 ? (c.TX == 16 && c.TY == 8) : (c.TX == 32 && c.TY == 4))
-                                                : c.TX == 128);
+                                                : (c.TX == 128 || sizeof(S) == 8));
         if (!shape_ok) return cudaErrorInvalidConfiguration;
         const MGeom g = mgeom<Q, S>(dd, c);
         const long long nb = (long long)g.tilesA * g.tilesB * g.NC;
@@ -1322,7 +1428,8 @@ inline cudaError_t batch_step(tlbm_host::BatchState& b, cudaStream_t st, cudaEve
     const int par = b.sims[0]->cur;
     const SimDesc<T>* d = static_cast<const SimDesc<T>*>(b.desc) + (size_t)par * n;
     tlbm_host::DevState probe = *b.sims[0];
-    probe.tile = b.tile;
+    probe.tile = b.auto_tile;
+    probe.rows128 = !b.narrow;
     const FusedCfg<Q> c = fused_cfg<Q>(probe);
     const int nb = (int)b.blocks;
     if (ev0) cudaEventRecord(ev0, st);
@@ -1333,13 +1440,17 @@ inline cudaError_t batch_step(tlbm_host::BatchState& b, cudaStream_t st, cudaEve
         } else {
             if (c.TX == 256) k_fused_solid_batch<Q, S, 256, 1><<<nb, 256, 0, st>>>(d, n);
             else if (c.TX == 64) k_fused_solid_batch<Q, S, 64, 1><<<nb, 64, 0, st>>>(d, n);
-            else k_fused_solid_batch<Q, S, 128, 1><<<nb, 128, 0, st>>>(d, n);
+            else if (c.TX == 32) {
+                if constexpr (sizeof(S) == 8) k_fused_solid_batch<Q, S, 32, 1><<<nb, 32, 0, st>>>(d, n);
+            } else k_fused_solid_batch<Q, S, 128, 1><<<nb, 128, 0, st>>>(d, n);
         }
     } else {
         if constexpr (Q == 19) {
             if constexpr (sizeof(S) == 8) k_fused_batch<Q, S, 16, 8, false, 0><<<nb, 128, 0, st>>>(d, n);
             else if constexpr (sizeof(S) == 2) k_fused_batch<Q, S, 32, 4, true, 1><<<nb, 128, 0, st>>>(d, n);
             else k_fused_batch<Q, S, 32, 4, false, 1><<<nb, 128, 0, st>>>(d, n);
+        } else if (sizeof(S) == 8 && c.TX == 32) {
+            if constexpr (sizeof(S) == 8) k_fused_batch<Q, S, 32, 1, false, 0><<<nb, 32, 0, st>>>(d, n);
         } else {
             k_fused_batch<Q, S, 128, 1, true, 2><<<nb, 128, 0, st>>>(d, n);
         }

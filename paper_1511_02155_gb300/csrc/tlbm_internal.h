@@ -50,6 +50,7 @@ struct DevState {
     int* flag;           // non-finite flag (int)
     PhysD phys;
     int tile;            // fused-kernel tile choice (0 = default)
+    int rows128;         // D2Q9 in double: no one-warp rows (a batch that keeps 128)
     int sms;             // multiprocessors of the device (sizes the fused grid's chunks)
     unsigned long long* check;  // device word: first bounds violation of a checked step
     int checked;         // 1: the fused step runs its bounds-checked kernels
@@ -65,6 +66,8 @@ struct BatchState {
     DevState** sims;     // member engines' device states
     void* desc;          // device descriptor array: [2][count], one set per buffer parity
     int tile;            // tile choice for every member (DevState::tile encoding)
+    int auto_tile;       // the same with the chunk resolved for the whole grid
+    int narrow;          // every member takes one-warp rows (D2Q9 in double)
     long long blocks;    // blocks of one batched step
     int built;           // descriptors are current
 };
