@@ -28,6 +28,7 @@
 #include <vector>
 
 #include "tlbm_kernels.cuh"
+#include "tlbm_node.cuh"
 
 namespace tlbm_dev {
 
@@ -373,6 +374,28 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
     moments_plane(M0 - 1, (M0 + 3) & 3, jn, rdn);
     moments_plane(M0, M0 & 3, jc, rdc);
 
+    // derivatives: on D2Q9 the ring's planes go through the node's rolling sums in
+    // order; on D3Q19 the 24 values they keep do not fit beside the collision in
+    // 128 registers, and all three planes are read again (the same bits)
+    constexpr bool KEEP = Q == 9;
+    Roll<Q, T> roll;
+    roll.clear();
+    T X0[3], g12[3][3], l6[3];
+    auto push_plane = [&](int m, T (&X)[3], T (&gr)[3][3], T (&la)[3]) {
+        const int slot = m & 3;
+        const T c1[3] = {sm[slot][0][h[0]], sm[slot][1][h[0]], sm[slot][2][h[0]]};
+        roll.push(
+            [&](int k, int i, int jj) -> T {
+                return sm[slot][k][(int)chk_index<CHK>(g, h[0] + jj * HW + i, HN, 4)];
+            },
+            c1, X, gr, la);
+    };
+    if (KEEP) {
+        __syncthreads();
+        push_plane(M0 + 3, X0, g12, l6);  // plane M0 - 1, in the slot of M0 + 3
+        push_plane(M0, X0, g12, l6);
+    }
+
     for (int m = M0; m < M1; ++m) {
         // Pulled populations of this thread's node at plane m, loaded before the
         // phase-M loads of plane m+1 so that both sets of requests are in flight
@@ -420,129 +443,21 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
         }
         moments_plane(m + 1, (m + 1) & 3, jn, rdn);
         __syncthreads();
+        if (!KEEP) {
+            roll.clear();
+            push_plane(m + 3, X0, g12, l6);  // plane m - 1
+            push_plane(m, X0, g12, l6);
+        }
+        push_plane(m + 1, X0, g12, l6);
         if (active) {
             if (!EARLY) load_node();
-            // ---- derivatives from the ring (pairs of opposite links)
-            const int c0 = h[0];
-            T X0[3], gA[3], gB[3], gM[3], lp[3];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                X0[c] = sm[m & 3][c][c0];
-                gA[c] = gB[c] = gM[c] = lp[c] = T(0);
-            }
-#pragma unroll
-            for (int i = 1; i < Q; ++i) {
-                if (opp<Q>(i) < i) continue;
-                const int sp = (m + A::cm(i)) & 3, sn = (m - A::cm(i)) & 3;
-                const int cp = (int)chk_index<CHK>(g, c0 + A::cb(i) * HW + A::ca(i), HN, 4);
-                const int cn = (int)chk_index<CHK>(g, c0 - A::cb(i) * HW - A::ca(i), HN, 4);
-                const T w = T(Lat<Q>::w(i));
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const T xpv = sm[sp][c][cp], xnv = sm[sn][c][cn];
-                    const T d = w * (xpv - xnv);
-                    if (A::ca(i)) gA[c] += T(A::ca(i)) * d;
-                    if (A::cb(i)) gB[c] += T(A::cb(i)) * d;
-                    if (A::cm(i)) gM[c] += T(A::cm(i)) * d;
-                    lp[c] += w * (xpv + xnv);
-                }
-            }
-            T grad[3][3], lap[3];
-            constexpr T wrest = T(1.0 - Lat<Q>::w(0));
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                lap[c] = T(6) * (lp[c] - wrest * X0[c]);
-                grad[c][0] = T(3) * gA[c];
-                if (D == 3) {
-                    grad[c][1] = T(3) * gB[c];
-                    grad[c][2] = T(3) * gM[c];
-                } else {
-                    grad[c][1] = T(3) * gM[c];
-                    grad[c][2] = T(0);
-                }
-            }
-            NodeEq<Q, T> E;
-            if (D == 3) E.setup(P, X0[0], jc[0], jc[1], jc[2], X0[1], X0[2], grad, lap, rdc);
-            else E.setup(P, X0[0], jc[0], jc[2], T(0), X0[1], X0[2], grad, lap, rdc);
+            const T jl[3] = {jc[0], D == 3 ? jc[1] : jc[2], D == 3 ? jc[2] : T(0)};  // lattice axes
             if constexpr (PAIR) msum.add(rdc, X0[1], X0[2]);
             else msum.add(rho_total<Q, S>(rdc), X0[1], X0[2]);
-
-            // ---- collide + store, direction pairs
             unsigned char* out = chk_node<Q, S, CHK>(
                 g, reinterpret_cast<unsigned char*>(dst),
                 reinterpret_cast<unsigned char*>(dst) + ((long long)m * g.NB + yb[0][1]) * g.rowstride + xc[0][1], 3);
-
-            auto st_ = [&](unsigned char* o, int ss, int ii, T d) {
-                if (HINT >= 1) Fmt<Q, S>::st_stream_delta(o, ss, ii, d);
-                else Fmt<Q, S>::st_delta(o, ss, ii, d);
-            };
-            // BGK with omega folded into the equilibria: x* = (1 - omega) x + omega x_eq,
-            // and omega x_eq = EV +- OD for a pair of opposite links, where
-            // EV = w (B + R (e.u)^2) [+ gradient terms for f] and OD = w O (e.u).
-            // On deviations d = x - w b (b = 1 for f in the offset formats, else 0):
-            // d* = (1 - omega) d + EV - omega w b +- OD, i.e. B is lowered by omega b:
-            // B = omega (bf - 1), with bf - 1 formed from rho - 1 (no cancellation).
-            constexpr bool OF = Fmt<Q, S>::OFFSET;
-            const T cf = T(1) - P.omega[0], cg = T(1) - P.omega[1], ck = T(1) - P.omega[2];
-            const T Bf = P.omega[0] * (OF ? E.bf1 : E.bf), Rf = T(4.5) * P.omega[0] * E.rho,
-                    Of = T(3) * P.omega[0] * E.rho;
-            const T Bg = P.omega[1] * E.bg, Rg = T(4.5) * P.omega[1] * E.phi, Og = T(3) * P.omega[1] * E.phi;
-            const T Bk = P.omega[2] * E.bk, Rk = T(4.5) * P.omega[2] * E.psi, Ok = T(3) * P.omega[2] * E.psi;
-#pragma unroll
-            for (int c = 0; c < 6; ++c) E.Gs[c] *= P.omega[0];
-            T sf = T(0), sg = T(0), sk = T(0);  // sums of omega x_eq over moving links
-            T qf = T(0), qg = T(0), qk = T(0);  // sums of the moving populations as stored
-#pragma unroll
-            for (int i = 1; i < Q; ++i) {
-                const int o = opp<Q>(i);
-                if (o < i) continue;
-                const T w = T(Lat<Q>::w(i));
-                const T e = E.eu(i);
-                const T e2 = e * e;
-                const T evf = w * (Bf + Rf * e2) + E.grad_term(i), odf = (w * Of) * e;
-                const T evg = w * (Bg + Rg * e2), odg = (w * Og) * e;
-                const T evk = w * (Bk + Rk * e2), odk = (w * Ok) * e;
-                sf += T(2) * evf;
-                sg += T(2) * evg;
-                sk += T(2) * evk;
-                const T v[6] = {cf * fv[i] + (evf + odf), cf * fv[o] + (evf - odf),
-                                cg * gv[i] + (evg + odg), cg * gv[o] + (evg - odg),
-                                ck * kv[i] + (evk + odk), ck * kv[o] + (evk - odk)};
-                if constexpr (Fmt<Q, S>::PAIRED) {  // three lane words (all offset formats)
-                    T q[6];  // the deviations as stored
-                    Fmt<Q, S>::template st_fg_q<(HINT >= 1)>(out, i, v[0], v[2], q[0], q[2]);
-                    Fmt<Q, S>::template st_fg_q<(HINT >= 1)>(out, o, v[1], v[3], q[1], q[3]);
-                    Fmt<Q, S>::template st_kk_q<(HINT >= 1)>(out, i, v[4], v[5], q[4], q[5]);
-                    qf += q[0] + q[1];
-                    qg += q[2] + q[3];
-                    qk += q[4] + q[5];
-                } else {
-                    st_(out, 0, i, v[0]);
-                    st_(out, 0, o, v[1]);
-                    st_(out, 1, i, v[2]);
-                    st_(out, 1, o, v[3]);
-                    st_(out, 2, i, v[4]);
-                    st_(out, 2, o, v[5]);
-                    if (OF) {
-                        qf += Fmt<Q, S>::qdelta_d(i, v[0]) + Fmt<Q, S>::qdelta_d(o, v[1]);
-                        qg += Fmt<Q, S>::qdelta_d(i, v[2]) + Fmt<Q, S>::qdelta_d(o, v[3]);
-                        qk += Fmt<Q, S>::qdelta_d(i, v[4]) + Fmt<Q, S>::qdelta_d(o, v[5]);
-                    }
-                }
-            }
-            if (OF) {
-                // rest = moment - moving populations as stored (deviations for f):
-                // every node keeps its rho, phi, psi through the rounding of the
-                // stored values (a rounding of the rest population alone)
-                st_(out, 0, 0, rdc - qf);
-                st_(out, 1, 0, E.phi - qg);
-                st_(out, 2, 0, E.psi - qk);
-            } else {
-                // omega x_eq_0 = omega X - sum of omega x_eq over the moving links
-                st_(out, 0, 0, cf * fv[0] + (P.omega[0] * E.rho - sf));
-                st_(out, 1, 0, cg * gv[0] + (P.omega[1] * E.phi - sg));
-                st_(out, 2, 0, ck * kv[0] + (P.omega[2] * E.psi - sk));
-            }
+            collide_node<Q, S, (HINT >= 1)>(out, fv, gv, kv, rdc, X0, jl, g12, l6, P);
         }
         jc[0] = jn[0];
         jc[1] = jn[1];
@@ -777,58 +692,42 @@ __device__ __forceinline__ void solid_body(const MGeom& g, const S* __restrict__
     __syncthreads();
 
     const int c0 = (ty + HB) * HW + tx + H;  // this thread's tile node in the region
+    constexpr bool KEEP = Q == 9;  // as in fused_body
+    Roll<Q, T> roll;
+    roll.clear();
+    auto push_plane = [&](int m, T (&X)[3], T (&gr)[3][3], T (&la)[3]) {
+        const int slot = modp(m, R);
+        const T c1[3] = {sm[slot][0][c0], sm[slot][1][c0], sm[slot][2][c0]};
+        roll.push(
+            [&](int k, int i, int jj) -> T {
+                return sm[slot][k][(int)chk_index<CHK>(g, c0 + jj * HW + i, HN, 4)];
+            },
+            c1, X, gr, la);
+    };
+    if (KEEP) {
+        T X0[3], g12[3][3], l6[3];
+        push_plane(M0 - 1, X0, g12, l6);
+        push_plane(M0, X0, g12, l6);
+    }
     for (int m = M0; m < M1; ++m) {
         moments_plane(m + 2);
         __syncthreads();
         ghosts_plane(m + 1);
         __syncthreads();
-        const int s0 = modp(m, R);
-        const uint32_t mk = sk[s0][c0];
-        if (!active || (mk & 1u)) continue;
+        const uint32_t mk = sk[modp(m, R)][c0];
+        T X0[3], g12[3][3], l6[3];
+        if (!KEEP) {
+            if (!active || (mk & 1u)) continue;
+            roll.clear();
+            push_plane(m - 1, X0, g12, l6);
+            push_plane(m, X0, g12, l6);
+        }
+        push_plane(m + 1, X0, g12, l6);  // ghost values on solid neighbours
+        if (KEEP && (!active || (mk & 1u))) continue;
 
-        // ---- derivatives from the ring (ghost values on solid neighbours)
-        T X0[3], gA[3], gB[3], gM[3], lp[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            X0[c] = sm[s0][c][c0];
-            gA[c] = gB[c] = gM[c] = lp[c] = T(0);
-        }
-#pragma unroll
-        for (int i = 1; i < Q; ++i) {
-            if (opp<Q>(i) < i) continue;
-            const int sp = modp(m + A::cm(i), R), sn = modp(m - A::cm(i), R);
-            const int cp = (int)chk_index<CHK>(g, c0 + A::cb(i) * HW + A::ca(i), HN, 4);
-            const int cn = (int)chk_index<CHK>(g, c0 - A::cb(i) * HW - A::ca(i), HN, 4);
-            const T w = T(Lat<Q>::w(i));
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const T xpv = sm[sp][c][cp], xnv = sm[sn][c][cn];
-                const T d = w * (xpv - xnv);
-                if (A::ca(i)) gA[c] += T(A::ca(i)) * d;
-                if (A::cb(i)) gB[c] += T(A::cb(i)) * d;
-                if (A::cm(i)) gM[c] += T(A::cm(i)) * d;
-                lp[c] += w * (xpv + xnv);
-            }
-        }
-        T grad[3][3], lap[3];
-        constexpr T wrest = T(1.0 - Lat<Q>::w(0));
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            lap[c] = T(6) * (lp[c] - wrest * X0[c]);
-            grad[c][0] = T(3) * gA[c];
-            if (D == 3) {
-                grad[c][1] = T(3) * gB[c];
-                grad[c][2] = T(3) * gM[c];
-            } else {
-                grad[c][1] = T(3) * gM[c];
-                grad[c][2] = T(0);
-            }
-        }
         const int t = ty * TX + tx, js = modp(m, 4);
         const T jA = sj[js][0][t], jB = sj[js][1][t], jM = sj[js][2][t], rdc = sj[js][3][t];
-        NodeEq<Q, T> E;
-        if (D == 3) E.setup(P, X0[0], jA, jB, jM, X0[1], X0[2], grad, lap);
-        else E.setup(P, X0[0], jA, jM, T(0), X0[1], X0[2], grad, lap);
+        const T jl[3] = {jA, D == 3 ? jB : jM, D == 3 ? jM : T(0)};  // lattice axes
         if constexpr (PAIR) msum.add(rdc, X0[1], X0[2]);
         else msum.add(rho_total<Q, S>(rdc), X0[1], X0[2]);
 
@@ -845,67 +744,20 @@ __device__ __forceinline__ void solid_body(const MGeom& g, const S* __restrict__
             // the collision is the last reader of these lines: evict-first loads
             // (FP32 storage; measured slower for the 16-bit formats)
             if (i > 0) {
-                T df, dg;
-                Fmt<Q, S>::template ld_fg<HL>(pfg, i, df, dg);
-                fv[i] = Fmt<Q, S>::unbias(0, i, df);
-                gv[i] = dg;
+                Fmt<Q, S>::template ld_fg<HL>(pfg, i, fv[i], gv[i]);
             } else {
-                fv[i] = HL ? Fmt<Q, S>::ld_last(p, 0, 0) : Fmt<Q, S>::ld(p, 0, 0);
-                gv[i] = HL ? Fmt<Q, S>::ld_last(p, 1, 0) : Fmt<Q, S>::ld(p, 1, 0);
+                fv[i] = HL ? Fmt<Q, S>::ld_last_delta(p, 0, 0) : Fmt<Q, S>::ld_delta(p, 0, 0);
+                gv[i] = HL ? Fmt<Q, S>::ld_last_delta(p, 1, 0) : Fmt<Q, S>::ld_delta(p, 1, 0);
             }
-            kv[i] = HL ? Fmt<Q, S>::ld_last(pk, 2, i) : Fmt<Q, S>::ld(pk, 2, i);
+            kv[i] = HL ? Fmt<Q, S>::ld_last_delta(pk, 2, i) : Fmt<Q, S>::ld_delta(pk, 2, i);
         }
 
-        // ---- collide + store (same arithmetic as k_fused)
+        // ---- collide + store
         unsigned char* out = chk_node<Q, S, CHK>(
             g, reinterpret_cast<unsigned char*>(dst),
             reinterpret_cast<unsigned char*>(dst) + ((long long)m * g.NB + yo[1]) * g.rowstride + xo[1], 3);
-        const T cf = T(1) - P.omega[0], cg = T(1) - P.omega[1], ck = T(1) - P.omega[2];
-        const T Bf = P.omega[0] * E.bf, Rf = T(4.5) * P.omega[0] * E.rho, Of = T(3) * P.omega[0] * E.rho;
-        const T Bg = P.omega[1] * E.bg, Rg = T(4.5) * P.omega[1] * E.phi, Og = T(3) * P.omega[1] * E.phi;
-        const T Bk = P.omega[2] * E.bk, Rk = T(4.5) * P.omega[2] * E.psi, Ok = T(3) * P.omega[2] * E.psi;
-#pragma unroll
-        for (int c = 0; c < 6; ++c) E.Gs[c] *= P.omega[0];
-        T sf = T(0), sg = T(0), sk2 = T(0), qf = T(0), qg = T(0), qk = T(0);
-#pragma unroll
-        for (int i = 1; i < Q; ++i) {
-            const int o = opp<Q>(i);
-            if (o < i) continue;
-            const T w = T(Lat<Q>::w(i));
-            const T e = E.eu(i);
-            const T e2 = e * e;
-            const T evf = w * (Bf + Rf * e2) + E.grad_term(i), odf = (w * Of) * e;
-            const T evg = w * (Bg + Rg * e2), odg = (w * Og) * e;
-            const T evk = w * (Bk + Rk * e2), odk = (w * Ok) * e;
-            sf += T(2) * evf;
-            sg += T(2) * evg;
-            sk2 += T(2) * evk;
-            const T v[6] = {cf * fv[i] + (evf + odf), cf * fv[o] + (evf - odf),
-                            cg * gv[i] + (evg + odg), cg * gv[o] + (evg - odg),
-                            ck * kv[i] + (evk + odk), ck * kv[o] + (evk - odk)};
-            // streamed out (evict-first, FP32): read only by the next step
-            Fmt<Q, S>::template st_fg<HL>(out, i, Fmt<Q, S>::dev(0, i, v[0]), v[2]);
-            Fmt<Q, S>::template st_fg<HL>(out, o, Fmt<Q, S>::dev(0, o, v[1]), v[3]);
-            Fmt<Q, S>::template st_kk<HL>(out, i, v[4], v[5]);
-            if (Fmt<Q, S>::OFFSET) {
-                qf += Fmt<Q, S>::qdelta(0, i, v[0]) + Fmt<Q, S>::qdelta(0, o, v[1]);
-                qg += Fmt<Q, S>::qdelta(1, i, v[2]) + Fmt<Q, S>::qdelta(1, o, v[3]);
-                qk += Fmt<Q, S>::qdelta(2, i, v[4]) + Fmt<Q, S>::qdelta(2, o, v[5]);
-            }
-        }
-        auto st_rest = [&](int s_, T d) {
-            if (HL) Fmt<Q, S>::st_stream_delta(out, s_, 0, d);
-            else Fmt<Q, S>::st_delta(out, s_, 0, d);
-        };
-        if (Fmt<Q, S>::OFFSET) {
-            st_rest(0, rdc - qf);
-            st_rest(1, E.phi - qg);
-            st_rest(2, E.psi - qk);
-        } else {
-            st_rest(0, Fmt<Q, S>::dev(0, 0, cf * fv[0] + (P.omega[0] * E.rho - sf)));
-            st_rest(1, cg * gv[0] + (P.omega[1] * E.phi - sg));
-            st_rest(2, ck * kv[0] + (P.omega[2] * E.psi - sk2));
-        }
+        // streamed out (evict-first, FP32): read only by the next step
+        collide_node<Q, S, HL>(out, fv, gv, kv, rdc, X0, jl, g12, l6, P);
     }
 
     double mr, mp, ms;
