@@ -233,14 +233,11 @@ tlbm_status tlbm_create(tlbm** out, tlbm_lattice lattice, int nx, int ny, int nz
     d.nx = nx; d.ny = ny; d.nz = nz; d.N = N;
     d.Np = (N + 63) / 64 * 64;
     d.ncx = (nx + 31) / 32;
-    // bytes of one 32-node chunk (see the layout notes in tlbm_lattice.cuh): FP64
-    // and D2Q9 FP32 all 3Q populations; D3Q19 FP32 3(Q-1)/2 runs of two-value
-    // lane words for the moving populations and two for the rest populations
-    // (one value unused); 16-bit formats 3(Q-1)/2 runs of 16-bit pairs and three
-    // FP32 rest runs
-    const long long chunk = esize == 2   ? (long long)((d.Q - 1) + (d.Q - 1) / 2 + 3) * 128
-                            : esize == 4 && d.Q == 19 ? (long long)((d.Q - 1) + (d.Q - 1) / 2 + 2) * 256
-                                         : 3LL * d.Q * 32 * (long long)esize;
+    // bytes of one 32-node chunk (see the layout notes in tlbm_lattice.cuh): all 3Q
+    // populations; 16-bit formats 3(Q-1)/2 runs of 16-bit pairs and three FP32 rest
+    // runs
+    const long long chunk = esize == 2 ? (long long)((d.Q - 1) + (d.Q - 1) / 2 + 3) * 128
+                                       : 3LL * d.Q * 32 * (long long)esize;
     d.pop_bytes = (long long)ny * nz * d.ncx * chunk;
     d.cur = 0;
     d.tile = 0;
@@ -488,6 +485,7 @@ tlbm_status tlbm_step_mass(tlbm* t, double out[3]) {
     CK(cudaMemcpyAsync(out, t->d.step_mass, 3 * sizeof(double), cudaMemcpyDeviceToHost, t->st));
     CK(cudaMemcpyAsync(&flag, t->d.flag, sizeof(int), cudaMemcpyDeviceToHost, t->st));
     CK(cudaStreamSynchronize(t->st));
+    if (flag & 2) return fail(t, TLBM_ERR_TIMEOUT, "a step's copies into shared memory did not arrive");
     if (flag) return fail(t, TLBM_ERR_NONFINITE, "a step produced a non-finite mass total");
     return TLBM_OK;
 }

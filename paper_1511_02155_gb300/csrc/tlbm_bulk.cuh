@@ -1,0 +1,491 @@
+// tlbm_bulk.cuh -- the periodic D3Q19 step with its populations brought into shared
+// memory by bulk copies (FP32 and 16-bit storage; Semprebon, Krueger,
+// Kusumaatmaja, arXiv:1511.02155).
+//
+// The marching scheme is that of tlbm_fused.cuh: a block owns one 32-node chunk of
+// x by TY rows and marches along z; the moments of a plane over the tile and its
+// one-node halo go to a shared ring, and the plane before it is collided with the
+// derivatives they complete.  What bounds that scheme with ordinary loads is the
+// latency of some 80 loads a node at 16 warps per SM (registers) and the L1 that
+// holds them in flight.  Here no thread waits for a load: while a plane is worked
+// on, the next one is copied by the TMA unit.  The layout makes that cheap: all
+// populations that a row of nodes pulls from one source row (y - e_y, z - e_z) are
+// one contiguous piece of a chunk, so nine copies of 384 or 1152 bytes (FP32) bring
+// a row's 57 populations, already in the place where the pull wants them but for
+// the x shift, which is a lane offset in shared memory.  The x neighbours beyond
+// the chunk are 114 single words per row, copied by 4- and 8-byte cp.async.
+//
+// Per plane p of a block's M1 - M0 + 2:
+//   wait for the copies of p
+//   populations of p into registers, moments of p: own node and at most one border
+//   node per thread -> ring
+//   barrier: nothing of the slot is needed any more
+//   start the copies of p + 1 into it
+//   derivatives of p - 1 (Roll), collision of p - 1 from registers, store
+// One slot: the copies run while the plane before is collided, the larger part of
+// the work, and the other blocks of the SM fill what wait is left.  A second slot
+// measured slower (FP32 1.96 against 1.55 ms at 256^3, FP16 1.38 against 1.00): it
+// takes the L1 that the words of x neighbours need on their way, a 128-byte line
+// for each.  One barrier a plane, since the ring holds two planes or more.
+#pragma once
+
+#include "tlbm_fused.cuh"
+
+namespace tlbm_dev {
+
+// What a row of nodes pulls, as runs of 32 lane words in shared memory.  FP32: the
+// chunk's own order.  16-bit formats: the chunk's first 26 runs, then the k words
+// whose two directions come from different rows, once for each direction.
+template <typename S>
+struct RowImage {
+    using F = Fmt<19, S>;
+    static constexpr bool PACKED = F::PACKED;
+    static constexpr int RUNS = PACKED ? 34 : 57;
+    static constexpr int BYTES = RUNS * 128;
+    static constexpr int COPIES = PACKED ? 17 : 9;
+    // byte offset of (s, i)
+    __host__ __device__ static constexpr int off(int s, int i) {
+        if (PACKED && s == 2 && i > 0 && F::krun(i) >= 26) return krun2(i) * 128 + F::khalf(i) * 2;
+        return F::off(s, i);
+    }
+    __host__ __device__ static constexpr int krun2(int i) {  // 3 4 5 6 11 14 12 13
+        return i <= 6 ? 23 + i : (i == 11 ? 30 : (i == 14 ? 31 : (i == 12 ? 32 : 33)));
+    }
+    // copy n: (e_y, e_z) of its source row, offset in the chunk and in the image, bytes
+    struct Copy {
+        int ey, ez, src, dst, bytes;
+    };
+    __host__ __device__ static constexpr Copy copy(int n) {
+        constexpr int ey[9] = {0, 1, -1, 0, 0, 1, 1, -1, -1}, ez[9] = {0, 0, 0, 1, -1, 1, -1, 1, -1};
+        if (n >= 9) {  // 16-bit: a k word for one of its two directions
+            constexpr int d[8] = {3, 4, 5, 6, 11, 14, 12, 13};
+            const int i = d[n < 17 ? n - 9 : 0];
+            return Copy{Lat<19>::cy(i), Lat<19>::cz(i), F::krun(i) * 128, krun2(i) * 128, 128};
+        }
+        // runs before group n and in it
+        const int len0 = PACKED ? 6 : 9, len = PACKED ? 4 : 9, one = PACKED ? 1 : 3;
+        const int at = n == 0 ? 0 : (n <= 4 ? len0 + (n - 1) * len : len0 + 4 * len + (n - 5) * one);
+        const int runs = n == 0 ? len0 : (n <= 4 ? len : one);
+        return Copy{ey[n], ez[n], at * 128, at * 128, runs * 128};
+    }
+    static __device__ __forceinline__ float value(const unsigned char* n, int s, int i) {
+        if constexpr (PACKED) {
+            if (i > 0) return Store<S>::get(*reinterpret_cast<const S*>(n + off(s, i)));
+        }
+        return *reinterpret_cast<const float*>(n + off(s, i));
+    }
+    // populations of direction i
+    static __device__ __forceinline__ void load(const unsigned char* n, int i, float& f, float& g, float& k) {
+        if constexpr (PACKED) {
+            if (i > 0) {
+                Store<S>::get2(*reinterpret_cast<const unsigned*>(n + off(0, i)), f, g);
+                k = value(n, 2, i);
+                return;
+            }
+        }
+        f = value(n, 0, i);
+        g = value(n, 1, i);
+        k = value(n, 2, i);
+    }
+};
+
+// A node's populations in registers: FP32 as they are, 16-bit formats in their
+// stored form (39 registers; converted where they are used).
+template <typename S>
+struct NodePops {
+    using I = RowImage<S>;
+    static constexpr int Q = 19;
+    float f[Q], g[Q], k[Q];  // FP32; 16-bit: the rest populations
+    unsigned fg[Q];          // 16-bit: (f, g) words, k
+    unsigned short kh[Q];
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            f[i] = g[i] = k[i] = 0.0f;
+            fg[i] = 0u;
+            kh[i] = 0;
+        }
+    }
+    // take direction i from the slot, and return its values
+    __device__ __forceinline__ void take(const unsigned char* n, int i, float& f_, float& g_, float& k_) {
+        if (I::PACKED && i > 0) {
+            fg[i] = *reinterpret_cast<const unsigned*>(n + I::off(0, i));
+            kh[i] = *reinterpret_cast<const unsigned short*>(n + I::off(2, i));
+        } else {
+            I::load(n, i, f[i], g[i], k[i]);
+        }
+        get(i, f_, g_, k_);
+    }
+    __device__ __forceinline__ void get(int i, float& f_, float& g_, float& k_) const {
+        if constexpr (I::PACKED) {
+            if (i > 0) {
+                Store<S>::get2(fg[i], f_, g_);
+                k_ = Store<S>::get(*reinterpret_cast<const S*>(&kh[i]));
+                return;
+            }
+        }
+        f_ = f[i];
+        g_ = g[i];
+        k_ = k[i];
+    }
+};
+
+// ------------------------------------------------------------- PTX wrappers
+
+__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void mbar_init(unsigned bar, unsigned count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(unsigned bar, unsigned bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ bool mbar_try(unsigned bar, unsigned parity) {
+    unsigned ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+// Waits for the phase with this parity, for at most about a second (a millisecond
+// once a wait of the block has run out): false then.
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, bool late) {
+    if (mbar_try(bar, parity)) return true;
+    unsigned long long t0, t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+    do {
+#pragma unroll 1
+        for (int n = 0; n < 64; ++n)
+            if (mbar_try(bar, parity)) return true;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    } while (t - t0 < (late ? 1000000ull : 1000000000ull));
+    return false;
+}
+__device__ __forceinline__ void bulk_load(unsigned dst, const void* src, unsigned bytes, unsigned bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void copy4(unsigned dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy8(unsigned dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
+// this thread's cp.async so far arrive at the barrier when they are done
+__device__ __forceinline__ void copy_arrive(unsigned bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+// ------------------------------------------------------------------ kernel
+
+template <typename S>
+struct BulkShape {
+    static constexpr int TY = 4;                                 // rows of a tile
+    static constexpr bool FRESH = RowImage<S>::PACKED;           // derivatives from three ring planes
+    static constexpr int ROWS = TY + 2;                          // tile and halo rows
+    static constexpr int SIDE = ROWS * RowImage<S>::BYTES;       // x neighbours, in the lanes of one more row
+    static constexpr int SLOT = SIDE + RowImage<S>::BYTES;
+    static constexpr int THREADS = 32 * TY;
+    static constexpr int RN = ROWS * 34;                         // a ring plane: tile and halo
+    static constexpr int NRING = FRESH ? 4 : 2;                  // planes of the ring
+    static constexpr int RING = SLOT, BAR = RING + NRING * 3 * RN * 4;
+    static constexpr int SMEM = BAR + 16;
+    static constexpr int BPS = RowImage<S>::PACKED ? 3 : 2;      // blocks per SM, by shared memory and registers
+    static_assert(ROWS * 4 <= 32 && BAR % 8 == 0, "side lanes; barrier alignment");
+    static_assert(ROWS * RowImage<S>::COPIES <= THREADS, "one bulk copy per thread");
+};
+
+template <typename S, bool CHK>
+__device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ src, S* __restrict__ dst,
+                                          const Phys<float>& P, double* __restrict__ partials, const int bid) {
+    constexpr int Q = 19;
+    using F = Fmt<Q, S>;
+    using I = RowImage<S>;
+    using B = BulkShape<S>;
+    using L = Lat<Q>;
+    constexpr int TY = B::TY;
+    extern __shared__ __align__(128) unsigned char tlbm_bulk_smem[];
+    float* const ring = reinterpret_cast<float*>(tlbm_bulk_smem + B::RING);
+    const unsigned char* const sl = tlbm_bulk_smem;
+    const unsigned smem0 = smem_u32(tlbm_bulk_smem), bar = smem0 + B::BAR;
+
+    const int tid = threadIdx.x, lane = tid & 31, ty = tid >> 5;
+    const int chunk = bid % g.tilesA;
+    const int rest = bid / g.tilesA;
+    const int B0 = (rest % g.tilesB) * TY;
+    const int mc = rest / g.tilesB;
+    const int M0 = (int)((long long)mc * g.NM / g.NC);
+    const int M1 = (int)((long long)(mc + 1) * g.NM / g.NC);
+    const int W = min(32, g.NA - 32 * chunk);  // nodes of this chunk
+    const int H = min(TY, g.NB - B0);          // rows of this tile
+    const int rows = H + 2;
+    const bool active = lane < W && ty < H;
+    const unsigned char* const srcb = reinterpret_cast<const unsigned char*>(src);
+    const long long pstride = (long long)g.NB * g.rowstride;
+    const int last = M1 - M0 + 1;  // planes 0 .. last of the march: M0 - 1 .. M1
+
+    // ---- this thread's bulk copy: row, group and source row are fixed
+    const unsigned char* bsrc = srcb;
+    unsigned bdst = 0, bbytes = 0;
+    int bez = 0;
+    if (tid < rows * I::COPIES) {
+        const int r = tid / I::COPIES, n = tid % I::COPIES;
+        typename I::Copy c = I::copy(0);
+#pragma unroll
+        for (int k = 1; k < I::COPIES; ++k) {
+            const typename I::Copy ck = I::copy(k);
+            if (n == k) c = ck;
+        }
+        const int y = modp(B0 + r - 1 - c.ey, g.NB);
+        bsrc = chk_node<Q, S, CHK>(g, srcb, srcb + y * g.rowstride + chunk * F::CHUNK, 1) + c.src;
+        bdst = r * I::BYTES + c.dst;
+        bbytes = c.bytes;
+        bez = c.ez;
+    }
+    // ---- this thread's x neighbours: (row, direction) items, two to three lane words
+    // each of one position (e_x = 0, either side) or of two adjacent ones (e_x != 0).
+    // Lane 4 r + {0, 1, 2, 3} of the side row holds x0 - 2, x0 - 1, x0 + W, x0 + W + 1
+    // of row r.
+    constexpr int NPOS = 28;  // 9 directions with e_x = 0, twice; 10 others
+    constexpr int NI = (B::ROWS * NPOS + B::THREADS - 1) / B::THREADS;
+    const unsigned char* isrc[NI];
+    unsigned idst[NI], idel[NI];  // image offset; deltas of the second word: chunk << 16 | image
+    int iez[NI];                  // e_z, + 8 where a third word follows, + 16 for two positions
+    int idx2[NI];                 // bytes to the second position's word: 4 where one 8-byte copy serves
+#pragma unroll
+    for (int k = 0; k < NI; ++k) {
+        const int it = tid + k * B::THREADS;
+        isrc[k] = nullptr;
+        idst[k] = idel[k] = 0;
+        iez[k] = idx2[k] = 0;
+        if (it < rows * NPOS) {
+            const int r = it / NPOS, p = it % NPOS;
+            const int slot = p < 18 ? 1 + (p & 1) : (p < 23 ? 0 : 2);
+            const int mu = slot < 2 ? slot - 2 : W + slot - 2;
+            const int which = p < 18 ? p / 2 : (p < 23 ? p - 18 : p - 23);
+            int o0 = 0, o1 = 0, d0 = 0, d1 = 0, ey = 0, ez = 0;
+            int n0 = 0, np = 0, nm = 0;
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                const bool mine = L::cx(i) == 0 ? (p < 18 && which == n0)
+                                                : (L::cx(i) > 0 ? (p >= 18 && p < 23 && which == np) : (p >= 23 && which == nm));
+                if (mine) {
+                    o0 = F::off(0, i);
+                    d0 = I::off(0, i);
+                    // second word: 16-bit the k word, else (and for the rest) g, and then k
+                    o1 = (I::PACKED && i > 0) ? F::krun(i) * 128 : F::off(1, i);
+                    d1 = (I::PACKED && i > 0) ? I::off(2, i) - F::khalf(i) * 2 : I::off(1, i);
+                    ey = L::cy(i);
+                    ez = L::cz(i) + ((I::PACKED && i > 0) ? 0 : 8);
+                }
+                n0 += L::cx(i) == 0;
+                np += L::cx(i) > 0;
+                nm += L::cx(i) < 0;
+            }
+            const int x = modp(32 * chunk + mu, g.NA), x2 = modp(x + 1, g.NA), y = modp(B0 + r - 1 - ey, g.NB);
+            const int at = (x >> 5) * (int)F::CHUNK + (x & 31) * 4, at2 = (x2 >> 5) * (int)F::CHUNK + (x2 & 31) * 4;
+            isrc[k] = chk_node<Q, S, CHK>(g, srcb, srcb + y * g.rowstride + at, 2) + o0;
+            idst[k] = B::SIDE + d0 + (4 * r + slot) * 4;
+            idel[k] = (unsigned)(o1 - o0) << 16 | (unsigned)(d1 - d0);
+            // two positions: one 8-byte copy where both lanes are one aligned pair
+            idx2[k] = (at2 - at == 4 && (x & 1) == 0) ? 4 : at2 - at + 1;
+            iez[k] = ez + (p < 18 ? 0 : 16);
+        }
+    }
+    // byte offsets of the planes z - 1, z, z + 1 of the march plane whose copies start next
+    long long zm = (long long)modp(M0 - 2, g.NM) * pstride, zc = (long long)modp(M0 - 1, g.NM) * pstride,
+              zp = (long long)modp(M0, g.NM) * pstride;
+    const long long zend = (long long)g.NM * pstride;
+    auto start = [&]() {
+        if (tid == 0) mbar_expect(bar, rows * I::BYTES);
+        if (bbytes) bulk_load(smem0 + bdst, bsrc + (bez == 0 ? zc : (bez > 0 ? zm : zp)), bbytes, bar);
+#pragma unroll
+        for (int k = 0; k < NI; ++k) {
+            if (isrc[k]) {
+                const bool two = iez[k] >= 15, third = ((iez[k] + 1) & 8) != 0;  // e_z + 8 third + 16 two
+                const int ez = ((iez[k] + 1) & 7) - 1;
+                const unsigned char* s = isrc[k] + (ez == 0 ? zc : (ez > 0 ? zm : zp));
+                const unsigned d = smem0 + idst[k], dd = idel[k] & 0xffffu, ds = idel[k] >> 16;
+                if (two && idx2[k] == 4) {
+                    copy8(d, s);
+                    copy8(d + dd, s + ds);
+                    if (third) copy8(d + 2 * dd, s + 2 * ds);
+                } else {
+                    copy4(d, s);
+                    copy4(d + dd, s + ds);
+                    if (third) copy4(d + 2 * dd, s + 2 * ds);
+                    if (two) {
+                        const unsigned char* s2 = s + (idx2[k] - 1);
+                        copy4(d + 4, s2);
+                        copy4(d + 4 + dd, s2 + ds);
+                        if (third) copy4(d + 4 + 2 * dd, s2 + 2 * ds);
+                    }
+                }
+            }
+        }
+        copy_arrive(bar);
+        zm = zc;
+        zc = zp;
+        zp = zp + pstride == zend ? 0 : zp + pstride;
+    };
+
+    if (tid == 0) {
+        mbar_init(bar, B::THREADS + 1);  // every thread's cp.async, and the bulk copies' bytes
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __syncthreads();
+    start();
+
+    // ---- offsets in a slot of the words that a node at lane mu of row r pulls, for
+    // e_x = 0, +1 (from mu - 1), -1 (from mu + 1)
+    auto word = [&](int r, int mu) -> int {
+        if (mu >= 0 && mu < W) return r * I::BYTES + mu * 4;
+        return B::SIDE + (4 * r + (mu < 0 ? mu + 2 : min(mu - W, 1) + 2)) * 4;
+    };
+    const int r0 = ty + 1;
+    const int own[3] = {r0 * I::BYTES + lane * 4, word(r0, lane - 1), word(r0, lane + 1)};
+    const int c0 = r0 * 34 + lane + 1;  // own node in the ring
+    // border node: rows 0 and H + 1 over W + 2 columns, then the two side columns
+    int bord[3] = {0, 0, 0}, cb = -1;
+    if (tid < 2 * (W + 2) + 2 * H) {
+        int r, q;
+        if (tid < 2 * (W + 2)) {
+            r = tid < W + 2 ? 0 : H + 1;
+            q = tid < W + 2 ? tid : tid - (W + 2);
+        } else {
+            const int k = tid - 2 * (W + 2);
+            r = 1 + (k >> 1);
+            q = (k & 1) ? W + 1 : 0;
+        }
+        bord[0] = word(r, q - 1);
+        bord[1] = word(r, q - 2);
+        bord[2] = word(r, q);
+        cb = (int)chk_index<CHK>(g, r * 34 + q, B::RN, 4);
+    }
+    unsigned char* const outb =
+        reinterpret_cast<unsigned char*>(dst) + (active ? (long long)(B0 + ty) * g.rowstride : 0) +
+        (long long)chunk * F::CHUNK + lane * F::ESZ;
+
+    MassSum<float, true> msum;
+    Roll<Q, float> roll;
+    roll.clear();
+    NodePops<S> cur, nxt;
+    cur.clear();
+    float jc[3] = {0.0f, 0.0f, 0.0f}, rdc = 0.0f;
+    bool late = false;
+
+#pragma unroll 1
+    for (int p = 0; p <= last; ++p) {
+        if (!mbar_wait(bar, p & 1, late)) late = true;
+
+        // ---- populations and moments of plane p
+        float* const rg = ring + (p & (B::NRING - 1)) * 3 * B::RN;
+        float jn[3] = {0.0f, 0.0f, 0.0f}, rdn = 0.0f, c1[3] = {0.0f, 0.0f, 0.0f};
+        {
+            const unsigned char* const b0 = sl + own[0];
+            const unsigned char* const bp = sl + own[1];
+            const unsigned char* const bm = sl + own[2];
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                const unsigned char* n = L::cx(i) == 0 ? b0 : (L::cx(i) > 0 ? bp : bm);
+                float f, gg, kk;
+                nxt.take(n, i, f, gg, kk);
+                rdn += f;
+                if (L::cx(i)) jn[0] += (float)L::cx(i) * f;
+                if (L::cy(i)) jn[1] += (float)L::cy(i) * f;
+                if (L::cz(i)) jn[2] += (float)L::cz(i) * f;
+                c1[1] += gg;
+                c1[2] += kk;
+            }
+            c1[0] = rdn + 1.0f;
+            if (active) {
+                rg[c0] = c1[0];
+                rg[B::RN + c0] = c1[1];
+                rg[2 * B::RN + c0] = c1[2];
+            }
+        }
+        if (cb >= 0) {
+            const unsigned char* const b0 = sl + bord[0];
+            const unsigned char* const bp = sl + bord[1];
+            const unsigned char* const bm = sl + bord[2];
+            float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                const unsigned char* n = L::cx(i) == 0 ? b0 : (L::cx(i) > 0 ? bp : bm);
+                float f, gg, kk;
+                I::load(n, i, f, gg, kk);
+                s0 += f;
+                s1 += gg;
+                s2 += kk;
+            }
+            rg[cb] = s0 + 1.0f;
+            rg[B::RN + cb] = s1;
+            rg[2 * B::RN + cb] = s2;
+        }
+        __syncthreads();  // the slot is read, the ring written
+        if (p < last) start();
+
+        // ---- derivatives and collision of plane p - 1
+        if (active) {
+            float X[3], g12[3][3], l6[3];
+            auto push = [&](const float* const rq, const float (&c)[3]) {
+                roll.push(
+                    [&](int k, int i, int jj) -> float {
+                        return rq[k * B::RN + (int)chk_index<CHK>(g, c0 + jj * 34 + i, B::RN, 4)];
+                    },
+                    c, X, g12, l6);
+            };
+            if (B::FRESH) {
+                roll.clear();
+#pragma unroll
+                for (int k = 2; k >= 1; --k) {
+                    const float* const rq = ring + ((p - k) & (B::NRING - 1)) * 3 * B::RN;
+                    const float c[3] = {rq[c0], rq[B::RN + c0], rq[2 * B::RN + c0]};
+                    push(rq, c);
+                }
+            }
+            push(rg, c1);
+            if (p >= 2) {
+                msum.add(rdc, X[1], X[2]);
+                unsigned char* const out = chk_node<Q, S, CHK>(g, reinterpret_cast<unsigned char*>(dst),
+                                                               outb + (long long)(M0 + p - 2) * pstride, 3);
+                float fv[Q], gv[Q], kv[Q];
+#pragma unroll
+                for (int i = 0; i < Q; ++i) cur.get(i, fv[i], gv[i], kv[i]);
+                collide_node<Q, S, true>(out, fv, gv, kv, rdc, X, jc, g12, l6, P);
+            }
+        }
+        cur = nxt;
+        jc[0] = jn[0];
+        jc[1] = jn[1];
+        jc[2] = jn[2];
+        rdc = rdn;
+    }
+    if (late) atomicOr(g.flag, 2);  // a copy did not arrive: the step's results are void
+    double mr, mp, ms;
+    msum.get(mr, mp, ms);
+    block_sum3(mr, mp, ms);
+    if (tid == 0) put_block_sums(g, partials, bid, mr, mp, ms);
+}
+
+template <typename S, bool CHK>
+__global__ void __launch_bounds__(BulkShape<S>::THREADS, BulkShape<S>::BPS)
+k_bulk(MGeom g, const S* __restrict__ src, S* __restrict__ dst, Phys<float> P, double* __restrict__ partials) {
+    bulk_body<S, CHK>(g, src, dst, P, partials, blockIdx.x);
+}
+
+template <typename S>
+__global__ void __launch_bounds__(BulkShape<S>::THREADS, BulkShape<S>::BPS)
+k_bulk_batch(const SimDesc<float>* __restrict__ d, int nsims) {
+    __shared__ SimDesc<float> sh;
+    const SimDesc<float>& m = batch_member(d, nsims, sh);
+    bulk_body<S, false>(m.g, static_cast<const S*>(m.src), static_cast<S*>(m.dst), m.P, m.partials,
+                        (int)blockIdx.x - m.block0);
+}
+
+}  // namespace tlbm_dev

@@ -25,8 +25,6 @@
 // write of the 3Q populations plus the halo's share (about 2/MC extra planes).
 #pragma once
 
-#include <vector>
-
 #include "tlbm_kernels.cuh"
 #include "tlbm_node.cuh"
 
@@ -57,7 +55,7 @@ __device__ __forceinline__ void put_block_sums(const MGeom& g, double* __restric
     partials[3 * bid + 0] = r;
     partials[3 * bid + 1] = p;
     partials[3 * bid + 2] = s;
-    if (!(isfinite(r) && isfinite(p) && isfinite(s))) *g.flag = 1;
+    if (!(isfinite(r) && isfinite(p) && isfinite(s))) atomicOr(g.flag, 1);
 }
 
 // Bounds checks of the checked kernel variants (CHK).  A violation is recorded
@@ -121,27 +119,11 @@ __device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
 // STG: STG of the 3Q pulled populations of a thread's own node, loaded in
 //      phase M, are kept in shared memory (2 plane slots x STG x NT values) and
 //      the collision reads them from there instead of pulling them again from
-//      L2; stage_rank orders the candidates (STGO 0: the lane-shifted
-//      directions first, whose warp loads span two chunks; 1: set by set).
-// position of population (s, i) in the staging order: STGO 1 set by set; STGO 0
-// the lane-shifted directions (e_x != 0) of all three sets first
-template <int Q, int STGO>
+//      L2; stage_rank orders the candidates.  D2Q9.
+// position of population (s, i) in the staging order: the lane-shifted directions
+// (e_x != 0) of all three sets first, whose warp loads span two chunks
+template <int Q>
 __host__ __device__ constexpr int stage_rank(int s, int i) {
-    if (STGO == 1) return s * Q + i;
-    if (Q == 19) {
-        const bool sh = (i == 1 || i == 2) || (i >= 7 && i <= 10) || (i >= 15);
-        const int is = i <= 2 ? i - 1 : (i <= 10 ? i - 5 : i - 9);
-        const int iu = i == 0 ? 0 : (i <= 6 ? i - 2 : i - 6);
-        if (STGO == 2) {
-            // paired lane words: the k values first (each a lone value of its
-            // word), lane-shifted first; then the lane-shifted (f, g) pairs; then
-            // the other pairs and the rest populations
-            if (i == 0) return 54 + s;
-            if (s == 2) return sh ? is : 10 + iu - 1;
-            return 18 + (sh ? 2 * is + s : 20 + 2 * (iu - 1) + s);
-        }
-        return sh ? s * 10 + is : 30 + s * 9 + iu;
-    }
     const bool sh = i == 1 || i == 2 || i >= 5;
     const int is = i <= 2 ? i - 1 : i - 3;
     const int iu = i == 0 ? 0 : i - 2;
@@ -194,16 +176,8 @@ struct MassSum<float, true> {
     }
 };
 
-// FP32 load through the non-coherent path with an L2 fetch size of 256 bytes:
-// a miss brings the neighbouring 128-byte run of the chunk into L2 as well.
-__device__ __forceinline__ float ld_l2x256(const unsigned char* p) {
-    float v;
-    asm("ld.global.nc.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
-    return v;
-}
-
 template <int Q, typename S, int TX, int TY, bool ILP, bool EARLY, bool PF = false, int HINT = 0, int STG = 0,
-          int STGO = 1, bool CHK = false, int LDH = 0>
+          bool CHK = false>
 __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__ src, S* __restrict__ dst,
                                            const Phys<typename Store<S>::T>& P, double* __restrict__ partials,
                                            const int bid) {
@@ -277,12 +251,8 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
     const int nnodes = tid < NBORDER ? 2 : 1;
 
     const unsigned char* srcb = reinterpret_cast<const unsigned char*>(src);
-    // stored value (x - bias) of (s, i) at node pointer p (LDH 1, FP32: with the
-    // 256-byte L2 fetch hint)
-    auto ldp = [&](const unsigned char* p, int s, int i) -> T {
-        if constexpr (LDH == 1 && sizeof(S) == 4) return ld_l2x256(p + Fmt<Q, S>::off(s, i));
-        else return Fmt<Q, S>::ld_delta(p, s, i);
-    };
+    // stored value (x - bias) of (s, i) at node pointer p
+    auto ldp = [&](const unsigned char* p, int s, int i) -> T { return Fmt<Q, S>::ld_delta(p, s, i); };
     // pull source of direction (ca, cb, cm) for node n at plane rows zr
     auto src_of = [&](int n, const int (&zr)[3], int ca, int cb, int cm) -> const unsigned char* {
         const long long row = (long long)zr[1 - cm] * g.NB + yb[n][1 - cb];
@@ -313,8 +283,8 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
             psi0 += kk;
             if constexpr (STG > 0) {
                 T* sp = stg + (size_t)((m & 1) * STG) * NT + tid;
-                const int r0 = stage_rank<Q, STGO>(0, i), r1 = stage_rank<Q, STGO>(1, i),
-                              r2 = stage_rank<Q, STGO>(2, i);
+                const int r0 = stage_rank<Q>(0, i), r1 = stage_rank<Q>(1, i),
+                              r2 = stage_rank<Q>(2, i);
                 if (r0 < STG) sp[(size_t)r0 * NT] = f;
                 if (r1 < STG) sp[(size_t)r1 * NT] = gg;
                 if (r2 < STG) sp[(size_t)r2 * NT] = kk;
@@ -367,7 +337,7 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
         j[2] = jm;
     };
 
-    constexpr bool PAIR = Fmt<Q, S>::OFFSET && !(Q == 19 && sizeof(S) == 4);
+    constexpr bool PAIR = Fmt<Q, S>::OFFSET;
     MassSum<T, PAIR> msum;
     T jc[3], jn[3], rdc, rdn;
 
@@ -414,8 +384,8 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
                 };
                 if constexpr (STG > 0) {
                     const T* sp = stg + (size_t)((m & 1) * STG) * NT + tid;
-                    const int r0 = stage_rank<Q, STGO>(0, i), r1 = stage_rank<Q, STGO>(1, i),
-                              r2 = stage_rank<Q, STGO>(2, i);
+                    const int r0 = stage_rank<Q>(0, i), r1 = stage_rank<Q>(1, i),
+                              r2 = stage_rank<Q>(2, i);
                     if (Fmt<Q, S>::PAIRED && i > 0 && r0 >= STG && r1 >= STG) {
                         Fmt<Q, S>::template ld_fg<(HINT >= 2)>(pi, i, fv[i], gv[i]);  // one lane word
                     } else {
@@ -474,17 +444,16 @@ template <int Q, typename S, int TX, int TY, bool ILP, bool EARLY, bool PF = fal
 __global__ void __launch_bounds__(TX * TY, blocks_per_sm<S>(TX * TY))
 k_fused(MGeom g, const S* __restrict__ src, S* __restrict__ dst, Phys<typename Store<S>::T> P,
         double* __restrict__ partials) {
-    fused_body<Q, S, TX, TY, ILP, EARLY, PF, HINT, 0, 1, CHK>(g, src, dst, P, partials, blockIdx.x);
+    fused_body<Q, S, TX, TY, ILP, EARLY, PF, HINT, 0, CHK>(g, src, dst, P, partials, blockIdx.x);
 }
 
-// Variants of the periodic step with shared-memory staging of the pulled
-// populations (STG values in the order STGO), at BPS blocks per SM.
-template <int Q, typename S, int TX, int TY, int STG, int STGO, int BPS, bool ILP, bool PF, int HINT,
-          bool CHK = false, int LDH = 0>
-__global__ void __launch_bounds__(TX * TY, BPS)
+// Variants of the periodic D2Q9 step with shared-memory staging of STG of the
+// pulled populations, at four blocks per SM.
+template <int Q, typename S, int TX, int TY, int STG, bool CHK = false>
+__global__ void __launch_bounds__(TX * TY, 4)
 k_fused_x(MGeom g, const S* __restrict__ src, S* __restrict__ dst, Phys<typename Store<S>::T> P,
           double* __restrict__ partials) {
-    fused_body<Q, S, TX, TY, ILP, false, PF, HINT, STG, STGO, CHK, LDH>(g, src, dst, P, partials, blockIdx.x);
+    fused_body<Q, S, TX, TY, false, false, true, 2, STG, CHK>(g, src, dst, P, partials, blockIdx.x);
 }
 
 // ------------------------------------------------------ solid-aware variant
@@ -842,482 +811,8 @@ __global__ void k_mass_final_batch(const SimDesc<T>* __restrict__ d) {
         m.step_mass[0] = a;
         m.step_mass[1] = b;
         m.step_mass[2] = c;
-        if (!(isfinite(a) && isfinite(b) && isfinite(c))) *m.flag = 1;
+        if (!(isfinite(a) && isfinite(b) && isfinite(c))) atomicOr(m.flag, 1);
     }
-}
-
-// ------------------------------------------------------------ host side
-
-// grid of a grid-stride kernel of 256 threads over n items: at most 8 blocks
-// per SM (results do not depend on it)
-inline int grid_of(long long n, int sms) {
-    const long long b = (n + 255) / 256, cap = 8LL * (sms < 1 ? 1 : sms);
-    return (int)(b < 1 ? 1 : (b > cap ? cap : b));
-}
-
-// Cost of marching nb blocks of mc planes each, up to a factor.  A block pays for
-// its planes plus halo prologue planes; a plane of one of b blocks that share an
-// SM (res fit) takes 0.25 + 0.19 b' times a full SM's plane, b' = 4 b / res: alone
-// a block waits out the latency of its loads, together they fill each other's
-// waits.  Blocks beyond what fits wait for whole rounds; over many rounds the
-// blocks drift apart and only the sum counts.  FP64 is bound by its few FP64
-// units: there every node's operations count, about 400 for a collision and 72
-// for the moments of a (node, halo) pair, and two blocks hide each other.
-// Against the measured times of 14 lattices (64^2 .. 1000x701, 40^3 .. 160^2x96)
-// over chunks of 1 .. 64 planes the cheapest chunk of this model is within 8 % of
-// the fastest measured; halving 64 or 16 until 4 blocks per SM are reached, the
-// earlier rule, lost up to 27 % (FP32, one step: 64x64 15.4 us against 11.3,
-// 96^3 117.4 against 102.9, walled 144x128x80 299 against 267).
-inline double march_cost(double nb, int mc, int halo, int res, int sms, bool dbl) {
-    const double full = (double)res * sms;
-    if (dbl) {
-        const double per = nb / sms, b = per > 8.0 ? per : (double)(long long)(per + 0.9999);
-        return (mc * 400.0 + (mc + halo) * 72.0) * (b < 2.0 ? 1.3 : b);
-    }
-    auto plane = [&](double b) { return 0.25 + 0.19 * 4.0 * b / res; };
-    const double rounds = nb / full;
-    if (rounds >= 4.0) return (mc + halo) * plane(res) * rounds;
-    const double whole = (double)(long long)rounds;
-    const double rest = nb - whole * full;
-    const double b = (double)(long long)((rest + sms - 1) / sms);
-    return (mc + halo) * (whole * plane(res) + (rest > 0 ? plane(b) : 0.0));
-}
-
-// Planes per block (chunk) of one marching launch over n lattices with cols[k]
-// tile columns of nm[k] planes: the cheapest by march_cost whose block sums fit
-// (caps[k]).  At most 64 planes in 2-D; in 3-D 16 once the grid fills the device
-// eight times over (256^3 FP32: 16 planes 0.692 of HBM, 24..128 planes 0.66..0.69:
-// blocks that start together share their halo rows in L2).
-inline int pick_chunk(const long long* cols, const int* nm, const long long* caps, int n, int halo, int res, int sms,
-                      bool three_d, bool dbl) {
-    double best = 0.0;
-    int bmc = 0;
-    for (int mc = three_d ? 2 : 1; mc <= 64; ++mc) {
-        double nb = 0.0;
-        int used = 0;
-        bool fits = true;
-        for (int k = 0; k < n; ++k) {
-            const int nc = (nm[k] + mc - 1) / mc, per = (nm[k] + nc - 1) / nc;
-            nb += (double)cols[k] * nc;
-            used = per > used ? per : used;
-            fits = fits && cols[k] * nc <= caps[k];
-        }
-        if (!fits) continue;
-        const double c = march_cost(nb, used, halo, res, sms, dbl);
-        if (three_d && used > 16 && nb >= 8.0 * res * sms) continue;
-        if (bmc == 0 || c < best) {
-            best = c;
-            bmc = mc;
-        }
-    }
-    return bmc == 0 ? 64 : bmc;
-}
-
-template <int Q>
-struct FusedCfg {
-    int TX, TY, MC;
-    int mode;
-    int shape;  // resolved D3Q19 shape (4..7: 32x4 kernels with staging)
-    // prologue planes a block recomputes, and blocks per SM (blocks_per_sm)
-    int halo(const tlbm_host::DevState& d) const { return d.solid || d.coupling ? 4 : 2; }
-    int res(const tlbm_host::DevState& d) const { return d.prec == 0 && TX == 32 ? 8 : 512 / (TX * TY); }
-};
-
-// d.tile = shape | mode << 4 | chunk << 8: shape 0 = default (D3Q19 shape 7,
-// D2Q9 shape 5); D3Q19 1 = 32x8, 2 = 64x4, 3 = 32x4, 4..7 = 32x4 with the pulled
-// populations of a thread's node staged in shared memory for the collision
-// (4: the 19 f values; 5: lane-shifted values first, 28 for FP32, 19 with the
-// per-warp prefetch for 16-bit storage; 6: 19 lane-shifted values; 7: as 5 in
-// the order of the paired lane words, the k values first, then the
-// lane-shifted (f, g) pairs, so that the collision reloads whole words); D2Q9
-// shape 0 = 5: 128-node rows with all 27 values staged, 1 = 128, 2 = 256, 3 =
-// 64, 4 = 128 with the 18 lane-shifted values staged.  mode (shapes 1..3) bit 0: interleaved border
-// loads; bit 1: early phase-C loads; bit 2: per-warp L2 prefetch three planes
-// ahead; 8 / 9: evict-first stores / stores and collision loads (12, 13 with
-// the prefetch).  mode 0 is the default for the shape and format (D3Q19 32x4:
-// 8 for FP32, 12 for 16-bit storage; other D3Q19: 1; D2Q9: 13); 6 selects the
-// plain loop.  chunk = planes per block (0 = chosen from the lattice size).
-// D2Q9 in double: rows of 32 nodes (one warp) where rows of 128 in chunks of four
-// planes leave SMs idle; wider rows recompute fewer halo moments.
-// A batch launches one tile for all members: narrow only if every member is.
-inline bool narrow_rows(const tlbm_host::DevState& d) { return !d.rows128 && d.N < 512LL * d.sms; }
-
-
-template <int Q>
-inline FusedCfg<Q> fused_cfg(const tlbm_host::DevState& d) {
-    const bool dbl = d.prec == 0;  // double storage: one default shape only
-    const int tile = d.checked ? 0 : d.tile;  // the checked kernels use the default tile
-    const int variant = dbl ? 0 : (tile & 15);
-    int mc = tile >> 8;
-    FusedCfg<Q> c{};
-    if (d.coupling) {
-        // forcing coupling (k_guo_fused): the solid-aware kernel's tiles (two-node halo)
-        c.TX = Q == 19 ? (dbl ? 16 : 32) : 128;
-        c.TY = Q == 19 ? 4 : 1;
-    } else if (d.solid) {
-        // solid-aware kernel: a fixed tile per lattice (D3Q19 in double: 16x4 keeps
-        // its five-plane rings under the 48 KB static shared-memory limit)
-        c.TX = Q == 19 ? (dbl ? 16 : 32)
-                       : (dbl ? (narrow_rows(d) ? 32 : 128) : (variant == 2 ? 256 : (variant == 3 ? 64 : 128)));
-        c.TY = Q == 19 ? 4 : 1;
-    } else if (Q == 19 && dbl) {
-        c.TX = 16;  // double storage: a smaller tile keeps the static shared ring small
-        c.TY = 8;
-    } else if (Q == 19) {
-        const int v = variant == 0 ? 7 : variant;  // 32x4 with pair-aware staging measured fastest on 256^3
-        c.TX = v == 2 ? 64 : 32;
-        c.TY = v == 1 ? 8 : 4;
-        c.shape = v;
-    } else {
-        const int v = variant == 0 ? 5 : variant;  // 128-node rows with staging measured fastest
-        c.TX = dbl ? (narrow_rows(d) ? 32 : 128) : (v == 2 ? 256 : (v == 3 ? 64 : 128));
-        c.TY = 1;
-        c.shape = v;
-    }
-    c.mode = dbl ? 0 : ((tile >> 4) & 15);
-    // defaults measured on GB300: D3Q19 32x4 with evict-first stores, plus a
-    // per-warp L2 prefetch for the 16-bit formats (a plane of FP32 populations
-    // is too large for the prefetch to stay in L2); 64x4 and 32x8 interleaved
-    // border loads; D2Q9 prefetch, evict-first stores and collision loads
-    if (c.mode == 0)
-        c.mode = (Q == 19) ? (c.TX == 32 && c.TY == 4 ? (d.prec >= 2 ? 12 : 8) : 1) : 13;
-    const int NA = d.nx;
-    const int NB = (Q == 19) ? d.ny : 1;
-    const int NM = (Q == 19) ? d.nz : d.ny;
-    if (mc <= 0) {
-        const long long cols = (long long)((NA + c.TX - 1) / c.TX) * ((NB + c.TY - 1) / c.TY);
-        mc = pick_chunk(&cols, &NM, &d.partials_cap, 1, c.halo(d), c.res(d), d.sms, Q == 19, dbl);
-    }
-    c.MC = mc < 1 ? 1 : (mc > NM ? NM : mc);
-    return c;
-}
-
-template <int Q, typename S>
-inline bool fused_supported(const tlbm_host::DevState& d) {
-    return d.solid == nullptr || d.nbm != nullptr;
-}
-
-template <int Q, typename S>
-inline int fused_launches(const tlbm_host::DevState&) {
-    return 1;
-}
-
-template <int Q, typename S>
-inline MGeom mgeom(const tlbm_host::DevState& d, const FusedCfg<Q>& c) {
-    MGeom g;
-    g.NA = d.nx;
-    g.NB = (Q == 19) ? d.ny : 1;
-    g.NM = (Q == 19) ? d.nz : d.ny;
-    g.rowstride = (long long)d.ncx * Fmt<Q, S>::CHUNK;
-    g.NC = (g.NM + c.MC - 1) / c.MC;  // chunks of MC planes or one fewer (balanced)
-    g.bytes = d.pop_bytes;
-    g.check = d.check;
-    g.flag = d.flag;
-    g.tilesA = (g.NA + c.TX - 1) / c.TX;
-    g.tilesB = (g.NB + c.TY - 1) / c.TY;
-    return g;
-}
-
-template <int Q, typename S>
-inline long long fused_blocks(const tlbm_host::DevState& d) {
-    const FusedCfg<Q> c = fused_cfg<Q>(d);
-    const MGeom g = mgeom<Q, S>(d, c);
-    return (long long)g.tilesA * g.tilesB * g.NC;
-}
-
-// Launch of a kernel with STG staged values per thread of 128 (dynamic shared
-// memory), with the smallest shared-memory carveout that still holds four
-// blocks per SM, so that the rest of the SM's 256 KB stays L1 (which holds the
-// kernel's loads in flight).
-template <typename K, typename... Args>
-inline cudaError_t launch_staged_t(K kern, int stg, int threads, int bps, long long nb, cudaStream_t st,
-                                   Args... args) {
-    const int dyn = stg * 2 * threads * (int)sizeof(float);
-    cudaFuncAttributes fa{};
-    cudaError_t e = cudaFuncGetAttributes(&fa, kern);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-    if (e != cudaSuccess) return e;
-    const long long need = (long long)bps * ((long long)fa.sharedSizeBytes + dyn + 1024);
-    const int pct = (int)((need * 100 + 233471) / 233472);
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, pct > 100 ? 100 : pct);
-    if (e != cudaSuccess) return e;
-    kern<<<(int)nb, threads, dyn, st>>>(args...);
-    return cudaSuccess;
-}
-template <typename K, typename... Args>
-inline cudaError_t launch_staged(K kern, int stg, long long nb, cudaStream_t st, Args... args) {
-    return launch_staged_t(kern, stg, 128, 4, nb, st, args...);
-}
-
-template <int Q, typename S>
-inline cudaError_t fused_step(tlbm_host::DevState& d, const Phys<typename Store<S>::T>& P, cudaStream_t st) {
-    const FusedCfg<Q> c = fused_cfg<Q>(d);
-    const MGeom g = mgeom<Q, S>(d, c);
-    const long long nb = (long long)g.tilesA * g.tilesB * g.NC;
-    if (nb > 0x7fffffffLL || nb > d.partials_cap) return cudaErrorInvalidConfiguration;
-    const S* src = static_cast<const S*>(d.pop[d.cur]);
-    S* dst = static_cast<S*>(d.pop[1 - d.cur]);
-    if (d.solid && !d.nbm_ready) {
-        const Geom gg{d.nx, d.ny, d.nz, d.N, d.Np, d.ncx};
-        k_nbmask<Q><<<grid_of(d.N, d.sms), 256, 0, st>>>(gg, d.solid, d.nbm);
-        d.nbm_ready = 1;
-    }
-    if (d.checked) {
-        // bounds-checked kernels of the default FP32 tiles (recording, never trapping)
-        if constexpr (sizeof(S) == 4) {
-            if (!d.check) return cudaErrorInvalidValue;
-            if (d.solid) {
-                if constexpr (Q == 19) k_fused_solid<Q, S, 32, 4, true><<<(int)nb, 128, 0, st>>>(g, src, dst, d.nbm, P, d.partials);
-                else k_fused_solid<Q, S, 128, 1, true><<<(int)nb, 128, 0, st>>>(g, src, dst, d.nbm, P, d.partials);
-            } else {
-                if constexpr (Q == 19) {
-                    const cudaError_t e = launch_staged(k_fused_x<Q, S, 32, 4, 28, 2, 4, false, false, 1, true>, 28, nb,
-                                                        st, g, src, dst, P, d.partials);
-                    if (e != cudaSuccess) return e;
-                } else {
-                    const cudaError_t e = launch_staged(k_fused_x<Q, S, 128, 1, 27, 0, 4, false, true, 2, true>, 27, nb,
-                                                        st, g, src, dst, P, d.partials);
-                    if (e != cudaSuccess) return e;
-                }
-            }
-            return cudaGetLastError();
-        } else {
-            return cudaErrorNotSupported;
-        }
-    }
-    if (d.solid) {
-        auto gos = [&](auto kern, int threads) {
-            kern<<<(int)nb, threads, 0, st>>>(g, src, dst, d.nbm, P, d.partials);
-        };
-        if constexpr (Q == 19) {
-            if constexpr (sizeof(S) == 8) gos(k_fused_solid<Q, S, 16, 4>, 64);
-            else gos(k_fused_solid<Q, S, 32, 4>, 128);
-        } else {
-            if (c.TX == 256) gos(k_fused_solid<Q, S, 256, 1>, 256);
-            else if (c.TX == 64) gos(k_fused_solid<Q, S, 64, 1>, 64);
-            else if (c.TX == 32) {
-                if constexpr (sizeof(S) == 8) gos(k_fused_solid<Q, S, 32, 1>, 32);
-            } else gos(k_fused_solid<Q, S, 128, 1>, 128);
-        }
-        return cudaGetLastError();
-    }
-    auto go = [&](auto kern, int threads) { kern<<<(int)nb, threads, 0, st>>>(g, src, dst, P, d.partials); };
-    if constexpr (sizeof(S) == 8) {
-        // double storage is the parity path: one tile shape per lattice and size
-        if constexpr (Q == 19) go(k_fused<Q, S, 16, 8, false, false>, 128);
-        else if (c.TX == 32) go(k_fused<Q, S, 32, 1, false, false>, 32);
-        else go(k_fused<Q, S, 128, 1, false, false>, 128);
-    } else if constexpr (Q == 19) {
-        if constexpr (sizeof(S) <= 4) {
-            if (c.shape >= 4) {
-                // 32x4 kernels with shared-memory staging of the pulled populations:
-                // 4 the 19 f values; 5 the lane-shifted values first, 28 of them for
-                // FP32, 19 with the per-warp L2 prefetch for the 16-bit formats; 6
-                // 19 lane-shifted values (no prefetch); 7 (default) as 5 in the
-                // paired-word order (k values, then lane-shifted (f, g) pairs)
-                cudaError_t e;
-                if constexpr (sizeof(S) == 2) {
-                    switch (c.shape) {
-                        case 4: e = launch_staged(k_fused_x<Q, S, 32, 4, 19, 1, 4, false, true, 1>, 19, nb, st, g, src, dst, P, d.partials); break;
-                        case 6: e = launch_staged(k_fused_x<Q, S, 32, 4, 19, 0, 4, false, false, 1>, 19, nb, st, g, src, dst, P, d.partials); break;
-                        case 5: e = launch_staged(k_fused_x<Q, S, 32, 4, 19, 0, 4, false, true, 1>, 19, nb, st, g, src, dst, P, d.partials); break;
-                        default: e = launch_staged(k_fused_x<Q, S, 32, 4, 19, 2, 4, false, true, 1>, 19, nb, st, g, src, dst, P, d.partials);
-                    }
-                } else {
-                    switch (c.shape) {
-                        case 4: e = launch_staged(k_fused_x<Q, S, 32, 4, 19, 1, 4, false, false, 1>, 19, nb, st, g, src, dst, P, d.partials); break;
-                        case 6: e = launch_staged(k_fused_x<Q, S, 32, 4, 19, 0, 4, false, false, 1>, 19, nb, st, g, src, dst, P, d.partials); break;
-                        case 5: e = launch_staged(k_fused_x<Q, S, 32, 4, 28, 0, 4, false, false, 1>, 28, nb, st, g, src, dst, P, d.partials); break;
-                        default: e = launch_staged(k_fused_x<Q, S, 32, 4, 28, 2, 4, false, false, 1>, 28, nb, st, g, src, dst, P, d.partials);
-                    }
-                }
-                return e != cudaSuccess ? e : cudaGetLastError();
-            }
-        }
-        if (c.TX == 64) {
-            switch (c.mode) {
-                case 2: go(k_fused<Q, S, 64, 4, false, true>, 256); break;
-                case 4: go(k_fused<Q, S, 64, 4, false, false, true>, 256); break;
-                case 5: go(k_fused<Q, S, 64, 4, true, false, true>, 256); break;
-                case 6: go(k_fused<Q, S, 64, 4, false, false>, 256); break;
-                default: go(k_fused<Q, S, 64, 4, true, false>, 256);
-            }
-        } else if (c.TY == 4) {
-            switch (c.mode) {
-                case 1: go(k_fused<Q, S, 32, 4, true, false>, 128); break;
-                case 4: go(k_fused<Q, S, 32, 4, false, false, true>, 128); break;
-                case 8: go(k_fused<Q, S, 32, 4, false, false, false, 1>, 128); break;
-                case 9: go(k_fused<Q, S, 32, 4, false, false, false, 2>, 128); break;
-                case 12: go(k_fused<Q, S, 32, 4, false, false, true, 1>, 128); break;
-                case 13: go(k_fused<Q, S, 32, 4, false, false, true, 2>, 128); break;
-                default: go(k_fused<Q, S, 32, 4, false, false>, 128);
-            }
-        } else {
-            if (c.mode == 6) go(k_fused<Q, S, 32, 8, false, false>, 256);
-            else go(k_fused<Q, S, 32, 8, true, false>, 256);
-        }
-    } else {
-        if (c.shape >= 4 && !d.solid) {
-            // 128-node rows with staging: 4 the 18 lane-shifted values, 5 (default)
-            // all 27, with the per-warp prefetch and evict-first stores and
-            // collision loads
-            const cudaError_t e =
-                c.shape == 4 ? launch_staged(k_fused_x<Q, S, 128, 1, 18, 0, 4, false, true, 2>, 18, nb, st, g, src, dst, P, d.partials)
-                             : launch_staged(k_fused_x<Q, S, 128, 1, 27, 0, 4, false, true, 2>, 27, nb, st, g, src, dst, P, d.partials);
-            return e != cudaSuccess ? e : cudaGetLastError();
-        }
-        if (c.TX == 256) {
-            switch (c.mode) {
-                case 1: go(k_fused<Q, S, 256, 1, true, false>, 256); break;
-                case 2: go(k_fused<Q, S, 256, 1, false, true>, 256); break;
-                case 3: go(k_fused<Q, S, 256, 1, true, true>, 256); break;
-                default: go(k_fused<Q, S, 256, 1, false, false>, 256);
-            }
-        } else if (c.TX == 64) {
-            go(k_fused<Q, S, 64, 1, false, false>, 64);
-        } else if (c.mode == 4) {
-            go(k_fused<Q, S, 128, 1, false, false, true>, 128);
-        } else if (c.mode == 12) {
-            go(k_fused<Q, S, 128, 1, false, false, true, 1>, 128);
-        } else if (c.mode == 13) {
-            go(k_fused<Q, S, 128, 1, false, false, true, 2>, 128);
-        } else {
-            go(k_fused<Q, S, 128, 1, false, false>, 128);  // plain loop
-        }
-    }
-    return cudaGetLastError();
-}
-
-// ---- batches: every member uses the batch's tile; descriptors for both parities
-
-template <int Q, typename S>
-inline cudaError_t batch_build(tlbm_host::BatchState& b, cudaStream_t st) {
-    using T = typename Store<S>::T;
-    const int n = b.count;
-    if (n < 1) return cudaErrorInvalidValue;
-    const bool solid = b.sims[0]->solid != nullptr;
-    std::vector<SimDesc<T>> h(2 * (size_t)n);
-    long long block0 = 0;
-    b.auto_tile = b.tile;
-    b.narrow = 1;
-    for (int k = 0; k < n; ++k) b.narrow = b.narrow && narrow_rows(*b.sims[k]);
-    if ((b.tile >> 8) == 0) {
-        // members whose own chunks do not fill the device twice keep them; beyond
-        // that the halo planes of short chunks are what costs, and one chunk is
-        // chosen for the whole grid (24 wells of 128x64 .. 768x384, FP32: 343 us a
-        // step with chunks of 4 to 8 planes, see k_fused_solid_batch)
-        std::vector<long long> cols, caps;
-        long long own = 0;
-        std::vector<int> nm;
-        FusedCfg<Q> c{};
-        tlbm_host::DevState d0 = *b.sims[0];
-        for (int k = 0; k < n; ++k) {
-            tlbm_host::DevState dd = *b.sims[k];
-            dd.tile = b.tile;
-            dd.rows128 = !b.narrow;
-            own += fused_blocks<Q, S>(dd);
-            c = fused_cfg<Q>(dd);
-            cols.push_back((long long)((dd.nx + c.TX - 1) / c.TX) * (Q == 19 ? (dd.ny + c.TY - 1) / c.TY : 1));
-            nm.push_back(Q == 19 ? dd.nz : dd.ny);
-            caps.push_back(dd.partials_cap);
-        }
-        if (own >= 2LL * c.res(d0) * d0.sms) {
-            const int mc = pick_chunk(cols.data(), nm.data(), caps.data(), n, c.halo(d0), c.res(d0), d0.sms, Q == 19,
-                                      d0.prec == 0);
-            b.auto_tile = (b.tile & 255) | mc << 8;
-        }
-    }
-    for (int k = 0; k < n; ++k) {
-        tlbm_host::DevState& d = *b.sims[k];
-        if ((d.solid != nullptr) != solid || d.cur != b.sims[0]->cur) return cudaErrorInvalidValue;
-        if (solid && !d.nbm_ready) {
-            const Geom gg{d.nx, d.ny, d.nz, d.N, d.Np, d.ncx};
-            k_nbmask<Q><<<grid_of(d.N, d.sms), 256, 0, st>>>(gg, d.solid, d.nbm);
-            d.nbm_ready = 1;
-        }
-        tlbm_host::DevState dd = d;
-        dd.tile = b.auto_tile;
-        dd.rows128 = !b.narrow;
-        const FusedCfg<Q> c = fused_cfg<Q>(dd);
-        // shapes with a batched kernel (batch_step): every solid shape; periodic
-        // D3Q19 32x4 (16x8 in double), periodic D2Q9 128
-        const bool shape_ok = solid || (Q == 19 ? (sizeof(S) == 8 ? (c.TX == 16 && c.TY == 8) : (c.TX == 32 && c.TY == 4))
-                                                : (c.TX == 128 || sizeof(S) == 8));
-        if (!shape_ok) return cudaErrorInvalidConfiguration;
-        const MGeom g = mgeom<Q, S>(dd, c);
-        const long long nb = (long long)g.tilesA * g.tilesB * g.NC;
-        if (nb > d.partials_cap) return cudaErrorInvalidConfiguration;
-        for (int par = 0; par < 2; ++par) {
-            SimDesc<T>& e = h[(size_t)par * n + k];
-            e.g = g;
-            e.src = d.pop[par];
-            e.dst = d.pop[1 - par];
-            e.nbm = d.nbm;
-            e.P = to_phys<T>(d.phys);
-            e.partials = d.partials;
-            e.step_mass = d.step_mass;
-            e.flag = d.flag;
-            e.block0 = (int)block0;
-            e.nblocks = (int)nb;
-        }
-        block0 += nb;
-    }
-    if (block0 > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    b.blocks = block0;
-    cudaError_t e = cudaSuccess;
-    if (!b.desc) e = cudaMalloc(&b.desc, sizeof(SimDesc<T>) * 2 * (size_t)n);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(b.desc, h.data(), sizeof(SimDesc<T>) * 2 * (size_t)n, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e == cudaSuccess) b.built = 1;
-    return e;
-}
-
-template <int Q, typename S>
-inline cudaError_t batch_step(tlbm_host::BatchState& b, cudaStream_t st, cudaEvent_t ev0 = nullptr,
-                              cudaEvent_t ev1 = nullptr) {
-    using T = typename Store<S>::T;
-    const int n = b.count;
-    const int par = b.sims[0]->cur;
-    const SimDesc<T>* d = static_cast<const SimDesc<T>*>(b.desc) + (size_t)par * n;
-    tlbm_host::DevState probe = *b.sims[0];
-    probe.tile = b.auto_tile;
-    probe.rows128 = !b.narrow;
-    const FusedCfg<Q> c = fused_cfg<Q>(probe);
-    const int nb = (int)b.blocks;
-    if (ev0) cudaEventRecord(ev0, st);
-    if (probe.solid) {
-        if constexpr (Q == 19) {
-            if constexpr (sizeof(S) == 8) k_fused_solid_batch<Q, S, 16, 4><<<nb, 64, 0, st>>>(d, n);
-            else k_fused_solid_batch<Q, S, 32, 4><<<nb, 128, 0, st>>>(d, n);
-        } else {
-            if (c.TX == 256) k_fused_solid_batch<Q, S, 256, 1><<<nb, 256, 0, st>>>(d, n);
-            else if (c.TX == 64) k_fused_solid_batch<Q, S, 64, 1><<<nb, 64, 0, st>>>(d, n);
-            else if (c.TX == 32) {
-                if constexpr (sizeof(S) == 8) k_fused_solid_batch<Q, S, 32, 1><<<nb, 32, 0, st>>>(d, n);
-            } else k_fused_solid_batch<Q, S, 128, 1><<<nb, 128, 0, st>>>(d, n);
-        }
-    } else {
-        if constexpr (Q == 19) {
-            if constexpr (sizeof(S) == 8) k_fused_batch<Q, S, 16, 8, false, 0><<<nb, 128, 0, st>>>(d, n);
-            else if constexpr (sizeof(S) == 2) k_fused_batch<Q, S, 32, 4, true, 1><<<nb, 128, 0, st>>>(d, n);
-            else k_fused_batch<Q, S, 32, 4, false, 1><<<nb, 128, 0, st>>>(d, n);
-        } else if (sizeof(S) == 8 && c.TX == 32) {
-            if constexpr (sizeof(S) == 8) k_fused_batch<Q, S, 32, 1, false, 0><<<nb, 32, 0, st>>>(d, n);
-        } else {
-            k_fused_batch<Q, S, 128, 1, true, 2><<<nb, 128, 0, st>>>(d, n);
-        }
-    }
-    if (ev1) cudaEventRecord(ev1, st);
-    for (int k = 0; k < n; ++k) b.sims[k]->cur ^= 1;
-    return cudaGetLastError();
-}
-
-// totals of every member's last batched step (the same sums under both parities)
-template <int Q, typename S>
-inline cudaError_t batch_totals(tlbm_host::BatchState& b, cudaStream_t st) {
-    using T = typename Store<S>::T;
-    k_mass_final_batch<T><<<b.count, kThreads, 0, st>>>(static_cast<const SimDesc<T>*>(b.desc));
-    return cudaGetLastError();
 }
 
 }  // namespace tlbm_dev

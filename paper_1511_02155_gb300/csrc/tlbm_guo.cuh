@@ -23,8 +23,8 @@
 //                   source, store x*(r) in the other buffer
 #pragma once
 
-#include "tlbm_fused.cuh"
 #include "tlbm_kernels.cuh"
+#include "tlbm_launch.cuh"
 
 namespace tlbm_dev {
 

@@ -153,7 +153,7 @@ static __global__ void k_mass_final(const double* __restrict__ partials, int nbl
     block_sum3(a, b, c);
     if (threadIdx.x == 0) {
         out[0] = a; out[1] = b; out[2] = c;
-        if (!(isfinite(a) && isfinite(b) && isfinite(c))) *flag = 1;
+        if (!(isfinite(a) && isfinite(b) && isfinite(c))) atomicOr(flag, 1);
     }
 }
 

@@ -171,18 +171,23 @@ struct Store<__nv_bfloat16> {
 // so a node is one byte offset, chunk + lane * ESZ, and every population of it
 // is that offset plus a constant.
 //   FP64, and FP32 on D2Q9: 3Q runs of S, run s*Q + i for set s, direction i.
-//   FP32 on D3Q19: 64-bit lane words of two values, paired as in the 16-bit
-//     formats below ((f_i, g_i), (k_i, k_opp(i))), and the rest populations as
-//     (f_0, g_0) and (k_0, unused).  FP32 keeps f as its deviation f_i - w_i
-//     from the rest state at rho = 1 (g and k as they are): deviations are
-//     small, so FP32 rounding of the stored values, and with it the drift of
-//     the total momentum, is ~100x smaller.
+//   FP32 on D3Q19: 3Q runs of S ordered by (e_y, e_z), the row that a pull reads
+//     them from: the runs of one such group are one contiguous piece of the
+//     chunk, so the nine pieces that a row of nodes pulls from nine source rows
+//     are nine bulk copies (tlbm_bulk.cuh).  Within a group direction by
+//     direction: f_i, g_i, k_i.
+//   FP32 keeps f as its deviation f_i - w_i from the rest state at rho = 1 (g and
+//     k as they are): deviations are small, so FP32 rounding of the stored
+//     values, and with it the drift of the total momentum, is ~100x smaller.
 //   16-bit formats (packed): f is kept as its deviation f_i - w_i from the
 //     rest state at rho = 1, g and k as they are.  Every lane word is 32 bits:
 //     for each moving direction i one run of (f_i, g_i) pairs (the two share a
-//     pull source: one load), for each pair of opposite directions i < opp(i)
-//     one run of (k_i, k_opp(i)) pairs (the collision writes both at once: one
-//     store), and three FP32 runs of the rest populations f_0 - w_0, g_0, k_0.
+//     pull source: one load), one run for each pair (k_i, k_kmate(i)), and three
+//     FP32 runs of the rest populations f_0 - w_0, g_0, k_0.  kmate(i) is opp(i),
+//     which one collision step writes together, except for the x edges of D3Q19,
+//     whose k pairs (7, 9), (8, 10), (15, 17), (16, 18) share a source row: on
+//     D3Q19 these runs too are ordered by (e_y, e_z), with the four pairs of
+//     directions from different rows at the end.
 //     That is 3(Q-1) 16-bit values and three FP32 values per node, as dense as
 //     16 bits allow.  The rest populations carry nearly all of phi and psi,
 //     which 16 bits would round by up to 2.4e-4 per step; the moving
@@ -208,46 +213,51 @@ struct Fmt {
     // f kept as its deviation f_i - w_i from the rest state at rho = 1 (FP32 and
     // the 16-bit formats; FP64 stores f as it is)
     static constexpr bool OFFSET = sizeof(S) <= 4;
-    // lane words of two values: the 16-bit formats, and FP32 on D3Q19 (measured:
-    // 0.5 % faster there; on D2Q9, whose kernels run near the HBM limit, the
-    // unused fourth word of the FP32 rest populations costs 5 %); FP64 one value
-    static constexpr bool PAIRED = sizeof(S) == 2 || (sizeof(S) == 4 && Q == 19);
+    // lane words of two values: the 16-bit formats
+    static constexpr bool PAIRED = sizeof(S) == 2;
     static constexpr int VSZ = (int)sizeof(S);              // bytes of one value
     static constexpr int ESZ = PAIRED ? 2 * VSZ : VSZ;       // bytes between lanes of a run
     static constexpr int RUN = 32 * ESZ;                     // bytes of a run
     static constexpr int NKP = (Q - 1) / 2;                  // runs of k pairs
-    // runs of the rest populations: 16-bit formats one FP32 word each; FP32 the
-    // words (f_0, g_0) and (k_0, unused)
-    static constexpr int NREST = PACKED ? 3 : 2;
-    static constexpr long long CHUNK = PAIRED ? (long long)((Q - 1) + NKP + NREST) * RUN : 3LL * Q * 32 * ESZ;
-    // packed: run of the k pair of direction i (the pairs of opposite directions
-    // numbered by their lower direction), and the half of its lane word (0: i is
-    // the lower direction of its pair).  Tables, so that they fold to immediates.
-    __host__ __device__ static constexpr int kpair(int i) {
+    static constexpr long long CHUNK = PAIRED ? (long long)((Q - 1) + NKP + 3) * RUN : 3LL * Q * 32 * ESZ;
+    // packed: the direction that shares i's k lane word, and the half of the word
+    // that i is in (0: the lower).  Tables, so that they fold to immediates.
+    __host__ __device__ static constexpr int kmate(int i) {
         if (Q == 19) {
-            // pairs (1,2) (3,4) (5,6) (7,10) (8,9) (11,14) (12,13) (15,18) (16,17)
-            constexpr int v[19] = {0, 0, 0, 1, 1, 2, 2, 3, 4, 4, 3, 5, 6, 6, 5, 7, 8, 8, 7};
+            constexpr int v[19] = {0, 2, 1, 4, 3, 6, 5, 9, 10, 7, 8, 14, 13, 12, 11, 17, 18, 15, 16};
             return v[i];
         }
-        // D2Q9: opposites adjacent, pairs (1,2) (3,4) (5,6) (7,8)
-        return (i - 1) / 2;
+        return i == 0 ? 0 : ((i - 1) ^ 1) + 1;  // D2Q9: opposites adjacent
     }
-    __host__ __device__ static constexpr int khalf(int i) {
+    __host__ __device__ static constexpr int khalf(int i) { return i < kmate(i) ? 0 : 1; }
+    // D3Q19: position of direction i in the order by (e_y, e_z): (0,0) 1 2 and rest,
+    // (1,0) 3 7 9, (-1,0) 4 8 10, (0,1) 5 15 17, (0,-1) 6 16 18, (1,1), (1,-1),
+    // (-1,1), (-1,-1)
+    __host__ __device__ static constexpr int gpos(int i) {
+        constexpr int v[19] = {0, 1, 2, 3, 6, 9, 12, 4, 7, 5, 8, 15, 16, 17, 18, 10, 13, 11, 14};
+        return Q == 19 ? v[i] : i;
+    }
+    // packed: run of the pair (f_i, g_i) and of the k word of direction i
+    __host__ __device__ static constexpr int fgrun(int i) {
         if (Q == 19) {
-            constexpr int v[19] = {0, 0, 1, 0, 1, 0, 1, 0, 0, 1, 1, 0, 0, 1, 1, 0, 0, 1, 1};
+            constexpr int v[19] = {3, 0, 1, 6, 10, 14, 18, 7, 11, 8, 12, 22, 23, 24, 25, 15, 19, 16, 20};
             return v[i];
         }
-        return (i - 1) & 1;
+        return i - 1;
+    }
+    __host__ __device__ static constexpr int krun(int i) {
+        if (Q == 19) {
+            constexpr int v[19] = {5, 2, 2, 26, 26, 27, 27, 9, 13, 9, 13, 28, 29, 29, 28, 17, 21, 17, 21};
+            return v[i];
+        }
+        return (Q - 1) + (i - 1) / 2;
     }
     // byte offset of (s, i) in the lane word of lane 0
     __host__ __device__ static constexpr int off(int s, int i) {
-        if (!PAIRED) return (s * Q + i) * 32 * ESZ;
-        if (i == 0) {
-            if (PACKED) return ((Q - 1) + NKP + s) * RUN;
-            return ((Q - 1) + NKP + (s == 2 ? 1 : 0)) * RUN + (s == 1 ? 4 : 0);
-        }
-        if (s < 2) return (i - 1) * RUN + s * VSZ;
-        return ((Q - 1) + kpair(i)) * RUN + khalf(i) * VSZ;
+        if (!PAIRED) return (Q == 19 && sizeof(S) == 4 ? 3 * gpos(i) + s : s * Q + i) * 32 * ESZ;
+        if (i == 0) return ((Q == 19 ? 3 : (Q - 1) + NKP) + s) * RUN;
+        if (s < 2) return fgrun(i) * RUN + s * VSZ;
+        return krun(i) * RUN + khalf(i) * VSZ;
     }
     // rest-state value subtracted before storage (set f, offset formats)
     __host__ __device__ static constexpr double bias(int s, int i) {
@@ -298,11 +308,6 @@ struct Fmt {
         if constexpr (PACKED) {
             const unsigned* p = reinterpret_cast<const unsigned*>(n + off(0, i));
             Store<S>::get2(LAST ? __ldcs(p) : *p, f, g);
-        } else if constexpr (PAIRED) {
-            const float2* p = reinterpret_cast<const float2*>(n + off(0, i));
-            const float2 v = LAST ? __ldcs(p) : *p;
-            f = v.x;
-            g = v.y;
         } else {
             f = LAST ? ld_last_delta(n, 0, i) : ld_delta(n, 0, i);
             g = LAST ? ld_last_delta(n, 1, i) : ld_delta(n, 1, i);
@@ -343,17 +348,13 @@ struct Fmt {
         st_delta(n, s, i, b == 0.0 ? v : v - T(b));
     }
     // store the deviations of f_i, g_i (i >= 1) and, in a second call, of k_i and
-    // k_o for o = opp(i) (packed: one 32-bit store each; STREAM: evict-first)
+    // k_o for o = opp(i) (packed: one 32-bit store where they share a word; STREAM:
+    // evict-first)
     template <bool STREAM>
     static __device__ __forceinline__ void st_fg(unsigned char* n, int i, T df, T dg) {
         if constexpr (PACKED) {
             unsigned* p = reinterpret_cast<unsigned*>(n + off(0, i));
             const unsigned w = Store<S>::put2(df, dg);
-            if (STREAM) __stcs(p, w);
-            else *p = w;
-        } else if constexpr (PAIRED) {
-            float2* p = reinterpret_cast<float2*>(n + off(0, i));
-            const float2 w = make_float2(df, dg);
             if (STREAM) __stcs(p, w);
             else *p = w;
         } else if (STREAM) {
@@ -366,18 +367,9 @@ struct Fmt {
     }
     template <bool STREAM>
     static __device__ __forceinline__ void st_kk(unsigned char* n, int i, T dki, T dko) {
-        if constexpr (PACKED) {
-            const bool lo = khalf(i) == 0;  // the lower direction sits in the low half
-            unsigned* p = reinterpret_cast<unsigned*>(n + off(2, lo ? i : opp<Q>(i)));
-            const unsigned w = lo ? Store<S>::put2(dki, dko) : Store<S>::put2(dko, dki);
-            if (STREAM) __stcs(p, w);
-            else *p = w;
-        } else if constexpr (PAIRED) {
-            const bool lo = khalf(i) == 0;
-            float2* p = reinterpret_cast<float2*>(n + off(2, lo ? i : opp<Q>(i)));
-            const float2 w = lo ? make_float2(dki, dko) : make_float2(dko, dki);
-            if (STREAM) __stcs(p, w);
-            else *p = w;
+        if (PACKED && kmate(i) == opp<Q>(i)) {
+            T qi, qo;
+            st_kword_q<STREAM>(n, khalf(i) == 0 ? i : opp<Q>(i), khalf(i) == 0 ? dki : dko, khalf(i) == 0 ? dko : dki, qi, qo);
         } else if (STREAM) {
             st_stream_delta(n, 2, i, dki);
             st_stream_delta(n, 2, opp<Q>(i), dko);
@@ -386,8 +378,20 @@ struct Fmt {
             st_delta(n, 2, opp<Q>(i), dko);
         }
     }
-    // st_fg / st_kk that also return the deviations as stored (read back from
-    // the lane word itself: no second conversion of each value)
+    // packed: the whole k word of directions lo and kmate(lo), khalf(lo) = 0, and
+    // the deviations as stored
+    template <bool STREAM>
+    static __device__ __forceinline__ void st_kword_q(unsigned char* n, int lo, T dlo, T dhi, T& qlo, T& qhi) {
+        if constexpr (PACKED) {
+            unsigned* p = reinterpret_cast<unsigned*>(n + off(2, lo));
+            const unsigned w = Store<S>::put2(dlo, dhi);
+            if (STREAM) __stcs(p, w);
+            else *p = w;
+            Store<S>::get2(w, qlo, qhi);
+        }
+    }
+    // st_fg that also returns the deviations as stored (read back from the lane
+    // word itself: no second conversion of each value)
     template <bool STREAM>
     static __device__ __forceinline__ void st_fg_q(unsigned char* n, int i, T df, T dg, T& qf, T& qg) {
         if constexpr (PACKED) {
@@ -400,22 +404,6 @@ struct Fmt {
             st_fg<STREAM>(n, i, df, dg);
             qf = df;
             qg = dg;
-        }
-    }
-    template <bool STREAM>
-    static __device__ __forceinline__ void st_kk_q(unsigned char* n, int i, T dki, T dko, T& qi, T& qo) {
-        if constexpr (PACKED) {
-            const bool lo = khalf(i) == 0;
-            unsigned* p = reinterpret_cast<unsigned*>(n + off(2, lo ? i : opp<Q>(i)));
-            const unsigned w = lo ? Store<S>::put2(dki, dko) : Store<S>::put2(dko, dki);
-            if (STREAM) __stcs(p, w);
-            else *p = w;
-            if (lo) Store<S>::get2(w, qi, qo);
-            else Store<S>::get2(w, qo, qi);
-        } else {
-            st_kk<STREAM>(n, i, dki, dko);
-            qi = dki;
-            qo = dko;
         }
     }
     // the deviation a store of population value v leaves in memory, as read back

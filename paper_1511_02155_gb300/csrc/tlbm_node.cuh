@@ -15,6 +15,9 @@ namespace tlbm_dev {
 
 __device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+// products that are added later: rounded here, never contracted into the sum
+__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
 
 // Derivatives of the three fields along one node's march, one plane at a time.
 // The weights of the isotropic stencils (axis links twice, on D2Q9 four times,
@@ -128,7 +131,7 @@ __device__ __forceinline__ void collide_node(unsigned char* out, const typename 
     constexpr bool OF = F::OFFSET;
     const T rho = X[0], phi = X[1], psi = X[2];
     const T inv = T(1) / rho;
-    const T u[3] = {j[0] * inv, j[1] * inv, D == 3 ? j[2] * inv : T(0)};
+    const T u[3] = {mul_(j[0], inv), mul_(j[1], inv), D == 3 ? mul_(j[2], inv) : T(0)};
     T uu = fma_(u[1], u[1], u[0] * u[0]);
     if constexpr (D == 3) uu = fma_(u[2], u[2], uu);
     const T huu = T(-1.5) * uu;
@@ -204,6 +207,11 @@ __device__ __forceinline__ void collide_node(unsigned char* out, const typename 
     const T Of = T(3) * of_r, Og = T(3) * og_p, Ok = T(3) * ok_p;
     T sf = T(0), sg = T(0), sk = T(0);  // half sums of omega x_eq over the moving links (FP64)
     T qf = T(0), qg = T(0), qk = T(0);  // sums of the moving populations as stored
+    T kn[Q];                            // packed: new k of directions whose word is not out yet
+    auto put = [&](int s, int i, T d) {
+        if (STREAM) F::st_stream_delta(out, s, i, d);
+        else F::st_delta(out, s, i, d);
+    };
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
         const int o = opp<Q>(i);
@@ -234,31 +242,42 @@ __device__ __forceinline__ void collide_node(unsigned char* out, const typename 
         const T v[6] = {fma_(cf, fv[i], fma_(of_w, e, evf)), fma_(cf, fv[o], fma_(-of_w, e, evf)),
                         fma_(cg, gv[i], fma_(og_w, e, evg)), fma_(cg, gv[o], fma_(-og_w, e, evg)),
                         fma_(ck, kv[i], fma_(ok_w, e, evk)), fma_(ck, kv[o], fma_(-ok_w, e, evk))};
-        T q[6];  // the deviations as stored
+        T q[4];  // the deviations as stored
         F::template st_fg_q<STREAM>(out, i, v[0], v[2], q[0], q[2]);
         F::template st_fg_q<STREAM>(out, o, v[1], v[3], q[1], q[3]);
-        F::template st_kk_q<STREAM>(out, i, v[4], v[5], q[4], q[5]);
         if (OF) {
             qf += q[0] + q[1];
             qg += q[2] + q[3];
-            qk += q[4] + q[5];
+        }
+        if constexpr (F::PACKED) {
+            // a k word goes out once both of its directions are collided
+            kn[i] = v[4];
+            kn[o] = v[5];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int d = h ? o : i, m = F::kmate(d), ml = m < opp<Q>(m) ? m : opp<Q>(m);
+                if (ml > i || (ml == i && F::khalf(d) != 0)) continue;
+                const int lo = F::khalf(d) == 0 ? d : m;
+                T ql, qh;
+                F::template st_kword_q<STREAM>(out, lo, kn[lo], kn[F::kmate(lo)], ql, qh);
+                qk += ql + qh;
+            }
+        } else {
+            F::template st_kk<STREAM>(out, i, v[4], v[5]);
+            if (OF) qk += v[4] + v[5];
         }
     }
-    auto rest = [&](int s, T d) {
-        if (STREAM) F::st_stream_delta(out, s, 0, d);
-        else F::st_delta(out, s, 0, d);
-    };
     if (OF) {
         // rest = moment - moving populations as stored (deviations for f): every
         // node keeps its rho, phi, psi through the rounding of the stored values
-        rest(0, rd - qf);
-        rest(1, phi - qg);
-        rest(2, psi - qk);
+        put(0, 0, rd - qf);
+        put(1, 0, phi - qg);
+        put(2, 0, psi - qk);
     } else {
         // omega x_eq_0 = omega X - sum of omega x_eq over the moving links
-        rest(0, fma_(cf, fv[0], fma_(T(-2), sf, of_r)));
-        rest(1, fma_(cg, gv[0], fma_(T(-2), sg, og_p)));
-        rest(2, fma_(ck, kv[0], fma_(T(-2), sk, ok_p)));
+        put(0, 0, fma_(cf, fv[0], fma_(T(-2), sf, of_r)));
+        put(1, 0, fma_(cg, gv[0], fma_(T(-2), sg, og_p)));
+        put(2, 0, fma_(ck, kv[0], fma_(T(-2), sk, ok_p)));
     }
 }
 

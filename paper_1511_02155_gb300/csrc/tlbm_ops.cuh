@@ -3,9 +3,9 @@
 #pragma once
 
 #include "tlbm_adjoint.cuh"
-#include "tlbm_fused.cuh"
 #include "tlbm_guo.cuh"
 #include "tlbm_kernels.cuh"
+#include "tlbm_launch.cuh"
 
 namespace tlbm_dev {
 
