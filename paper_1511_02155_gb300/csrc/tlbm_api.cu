@@ -31,6 +31,7 @@ struct tlbm {
     int timing;            // 1: time the main kernel(s) of every step
     double kernel_ms;      // accumulated main-kernel time in timing mode
     int64_t kernel_steps;  // steps accumulated in kernel_ms
+    std::vector<uint8_t> units;  // solid nodes per 32-node unit (DevState::units)
     std::string err;
 };
 
@@ -65,6 +66,53 @@ int resolve_kind(const tlbm* t) {
     if (t->kind_req == TLBM_KERNEL_SPLIT) return tlbm_host::KIND_SPLIT;
     if (t->kind_req == TLBM_KERNEL_FUSED) return tlbm_host::KIND_FUSED;
     return t->ops->has_fused(t->d) ? tlbm_host::KIND_FUSED : tlbm_host::KIND_SPLIT;
+}
+
+// solid nodes per 32-node unit of every row: bit 0 one between two nodes before and
+// two behind the unit (periodic), bit 1 every node of the unit
+void mark_units(tlbm* t, const uint8_t* mask) {
+    const DevState& d = t->d;
+    const long long rows = (long long)d.ny * d.nz;
+    t->units.assign((size_t)(rows * d.ncx), 0);
+    for (long long r = 0; r < rows; ++r) {
+        const uint8_t* m = mask + r * d.nx;
+        uint8_t* u = t->units.data() + r * d.ncx;
+        for (int c = 0; c < d.ncx; ++c) {
+            const int x0 = 32 * c, x1 = x0 + 32 < d.nx ? x0 + 32 : d.nx;
+            uint64_t w[4] = {0, 0, 0, 0};
+            memcpy(w, m + x0, (size_t)(x1 - x0));
+            bool any = (w[0] | w[1] | w[2] | w[3]) != 0;
+            int n = 0;
+            for (int x = x0; any && x < x1; ++x) n += m[x] != 0;
+            for (int k = 1; k <= 2 && !any; ++k)
+                any = m[(((x0 - k) % d.nx) + d.nx) % d.nx] != 0 || m[(x1 - 1 + k) % d.nx] != 0;
+            u[c] = (uint8_t)((any ? 1 : 0) | (n == x1 - x0 ? 2 : 0));
+        }
+    }
+    t->d.units = t->units.data();
+}
+
+// work items of the fused step at the current tile (lattices with solid nodes)
+cudaError_t set_items(tlbm* t) {
+    DevState& d = t->d;
+    if (!d.solid) return cudaSuccess;
+    std::vector<int4> items;
+    const int dirty = t->ops->solid_items(d, items);
+    cudaError_t e = cudaStreamSynchronize(t->st);  // no step in flight reads what is replaced
+    if (e != cudaSuccess) return e;
+    cudaFree(const_cast<void*>(d.items));
+    d.items = nullptr;
+    d.nitems = d.ndirty = 0;
+    if (items.empty()) return cudaSuccess;
+    void* p = nullptr;
+    e = cudaMalloc(&p, sizeof(int4) * items.size());
+    if (e != cudaSuccess) return e;
+    d.items = p;
+    e = cudaMemcpy(p, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return e;
+    d.nitems = (int)items.size();
+    d.ndirty = dirty;
+    return cudaSuccess;
 }
 
 tlbm_status ensure_staging(tlbm* t) {
@@ -156,6 +204,7 @@ void tlbm_destroy(tlbm* t) {
     cudaFree(t->d.pop[1]);
     cudaFree((void*)t->d.solid);
     cudaFree(t->d.nbm);
+    cudaFree(const_cast<void*>(t->d.items));
     cudaFree(t->d.mom);
     cudaFree(t->d.aux);
     cudaFree(t->d.partials);
@@ -281,7 +330,9 @@ tlbm_status tlbm_create(tlbm** out, tlbm_lattice lattice, int nx, int ny, int nz
     }
     t->partials_len = 3 * (size_t)(nblk + tlbm_host::mass_blocks());
     d.partials_cap = nblk;
-    cudaError_t e = cudaMalloc(&d.partials, sizeof(double) * t->partials_len);
+    if (any_solid) mark_units(t, solid_mask);
+    cudaError_t e = set_items(t);
+    if (e == cudaSuccess) e = cudaMalloc(&d.partials, sizeof(double) * t->partials_len);
     if (e == cudaSuccess) e = cudaMalloc(&d.step_mass, sizeof(double) * 3);
     if (e == cudaSuccess) e = cudaMalloc(&d.mass_tmp, sizeof(double) * 3);
     if (e == cudaSuccess) e = cudaMalloc(&d.flag, sizeof(int));
@@ -327,7 +378,8 @@ tlbm_status tlbm_set_tile(tlbm* t, int variant, int chunk) {
     if (variant < 0 || variant > 255 || (variant & 15) > 7 || chunk < 0 || chunk > 4096)
         return fail(t, TLBM_ERR_ARG, "bad tile");
     t->d.tile = variant + 256 * chunk;
-    // partial sums must fit: blocks grow as chunks shrink
+    // partial sums must fit: blocks grow as chunks shrink (checked by the step)
+    CK(set_items(t));
     return TLBM_OK;
 }
 
@@ -772,6 +824,7 @@ void tlbm_batch_destroy(tlbm_batch* b) {
     for (cudaEvent_t e : b->ev)
         if (e) cudaEventDestroy(e);
     cudaFree(b->bs.desc);
+    cudaFree(b->bs.items);
     delete b;
 }
 

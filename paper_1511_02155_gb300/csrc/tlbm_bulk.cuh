@@ -214,12 +214,8 @@ __device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ 
     const unsigned smem0 = smem_u32(tlbm_bulk_smem), bar = smem0 + B::BAR;
 
     const int tid = threadIdx.x, lane = tid & 31, ty = tid >> 5;
-    const int chunk = bid % g.tilesA;
-    const int rest = bid / g.tilesA;
-    const int B0 = (rest % g.tilesB) * TY;
-    const int mc = rest / g.tilesB;
-    const int M0 = (int)((long long)mc * g.NM / g.NC);
-    const int M1 = (int)((long long)(mc + 1) * g.NM / g.NC);
+    const Work wk = work_of<32, TY>(g, bid);
+    const int chunk = wk.A0 >> 5, B0 = wk.B0, M0 = wk.M0, M1 = wk.M1;
     const int W = min(32, g.NA - 32 * chunk);  // nodes of this chunk
     const int H = min(TY, g.NB - B0);          // rows of this tile
     const int rows = H + 2;
@@ -484,8 +480,8 @@ __global__ void __launch_bounds__(BulkShape<S>::THREADS, BulkShape<S>::BPS)
 k_bulk_batch(const SimDesc<float>* __restrict__ d, int nsims) {
     __shared__ SimDesc<float> sh;
     const SimDesc<float>& m = batch_member(d, nsims, sh);
-    bulk_body<S, false>(m.g, static_cast<const S*>(m.src), static_cast<S*>(m.dst), m.P, m.partials,
-                        (int)blockIdx.x - m.block0);
+    bulk_body<S, false>(member_geom(m.g), as_global(static_cast<const S*>(m.src)), as_global(static_cast<S*>(m.dst)),
+                        m.P, as_global(m.partials), (int)blockIdx.x - m.block0);
 }
 
 }  // namespace tlbm_dev

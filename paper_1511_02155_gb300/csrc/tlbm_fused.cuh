@@ -47,7 +47,24 @@ struct MGeom {
     long long bytes;      // bytes of one population buffer (bounds-checked kernels)
     unsigned long long* check;  // first bounds violation (bounds-checked kernels)
     int* flag;            // raised by a block whose sums are not finite
+    const int4* items;    // lattices with solid nodes: the blocks' work (Work), else null
 };
+
+// One block's share of a march: the tile at (A0, B0), planes M0 .. M1 - 1.
+struct Work {
+    int A0, B0, M0, M1;
+    bool dirty;  // solid nodes within two nodes of the tile: the solid-aware body
+};
+template <int TX, int TY>
+__device__ __forceinline__ Work work_of(const MGeom& g, int bid) {
+    if (g.items) {
+        const int4 it = g.items[bid];
+        return Work{it.x, it.y, it.z, it.w >> 1, (it.w & 1) != 0};
+    }
+    const int rest = bid / g.tilesA, chunk = rest / g.tilesB;
+    return Work{(bid % g.tilesA) * TX, (rest % g.tilesB) * TY, (int)((long long)chunk * g.NM / g.NC),
+                (int)((long long)(chunk + 1) * g.NM / g.NC), true};
+}
 
 // a block's FP64 sums of rho, phi, psi: its partial sums and the non-finite flag
 __device__ __forceinline__ void put_block_sums(const MGeom& g, double* __restrict__ partials, int bid, double r,
@@ -176,17 +193,30 @@ struct MassSum<float, true> {
     }
 };
 
+// bytes of fused_body's moment ring (four planes, tile and one-node halo) and of
+// its dynamic shared memory with STG staged values per thread
+template <int Q, typename S>
+__host__ __device__ constexpr int ring_bytes(int TX, int TY) {
+    const int n = 4 * 3 * (TX + 2) * (TY + (Q == 19 ? 2 : 0)) * (int)sizeof(typename Store<S>::T);
+    return (n + 15) / 16 * 16;
+}
+template <int Q, typename S>
+__host__ __device__ constexpr int fused_smem(int TX, int TY, int STG) {
+    return ring_bytes<Q, S>(TX, TY) + 2 * STG * TX * TY * (int)sizeof(typename Store<S>::T);
+}
+
 template <int Q, typename S, int TX, int TY, bool ILP, bool EARLY, bool PF = false, int HINT = 0, int STG = 0,
           bool CHK = false>
 __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__ src, S* __restrict__ dst,
                                            const Phys<typename Store<S>::T>& P, double* __restrict__ partials,
-                                           const int bid) {
+                                           const int bid, const Work w) {
     using T = typename Store<S>::T;
     using A = Axes<Q>;
-    // staging ring in dynamic shared memory (declared here so that the compiler
-    // knows the stores are shared-memory stores that cannot alias the loads)
-    extern __shared__ __align__(16) unsigned char tlbm_stage_smem[];
-    T* const stg = reinterpret_cast<T*>(tlbm_stage_smem);
+    // dynamic shared memory: the moment ring, then the staging ring (declared here
+    // so that the compiler knows the stores are shared-memory stores that cannot
+    // alias the loads)
+    extern __shared__ __align__(16) unsigned char tlbm_smem[];
+    T* const stg = reinterpret_cast<T*>(tlbm_smem + ring_bytes<Q, S>(TX, TY));
     constexpr int D = Lat<Q>::D;
     constexpr int HY = (D == 3) ? 1 : 0;  // halo rows along b
     constexpr int HW = TX + 2;
@@ -197,17 +227,11 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
     static_assert(D == 3 || TY == 1, "2-D tiles are one row");
     static_assert(NBORDER <= NT, "one border node per thread at most");
 
-    __shared__ T sm[4][3][HN];  // moment ring: rho, phi, psi over tile + halo
+    T (*const sm)[3][HN] = reinterpret_cast<T(*)[3][HN]>(tlbm_smem);  // moment ring: rho, phi, psi over tile + halo
 
     const int tid = threadIdx.x;
     const int tx = tid % TX, ty = tid / TX;
-    const int tileA = bid % g.tilesA;
-    const int rest = bid / g.tilesA;
-    const int tileB = rest % g.tilesB;
-    const int chunk = rest / g.tilesB;
-    const int A0 = tileA * TX, B0 = tileB * TY;
-    const int M0 = (int)((long long)chunk * g.NM / g.NC);
-    const int M1 = (int)((long long)(chunk + 1) * g.NM / g.NC);
+    const int A0 = w.A0, B0 = w.B0, M0 = w.M0, M1 = w.M1;
     const bool active = (A0 + tx < g.NA) && (B0 + ty < g.NB);
 
     // Node 0 of every thread: its own tile slot (coordinates wrap for threads past
@@ -444,7 +468,8 @@ template <int Q, typename S, int TX, int TY, bool ILP, bool EARLY, bool PF = fal
 __global__ void __launch_bounds__(TX * TY, blocks_per_sm<S>(TX * TY))
 k_fused(MGeom g, const S* __restrict__ src, S* __restrict__ dst, Phys<typename Store<S>::T> P,
         double* __restrict__ partials) {
-    fused_body<Q, S, TX, TY, ILP, EARLY, PF, HINT, 0, CHK>(g, src, dst, P, partials, blockIdx.x);
+    fused_body<Q, S, TX, TY, ILP, EARLY, PF, HINT, 0, CHK>(g, src, dst, P, partials, blockIdx.x,
+                                                           work_of<TX, TY>(g, blockIdx.x));
 }
 
 // Variants of the periodic D2Q9 step with shared-memory staging of STG of the
@@ -453,7 +478,8 @@ template <int Q, typename S, int TX, int TY, int STG, bool CHK = false>
 __global__ void __launch_bounds__(TX * TY, 4)
 k_fused_x(MGeom g, const S* __restrict__ src, S* __restrict__ dst, Phys<typename Store<S>::T> P,
           double* __restrict__ partials) {
-    fused_body<Q, S, TX, TY, false, false, true, 2, STG, CHK>(g, src, dst, P, partials, blockIdx.x);
+    fused_body<Q, S, TX, TY, false, false, true, 2, STG, CHK>(g, src, dst, P, partials, blockIdx.x,
+                                                              work_of<TX, TY>(g, blockIdx.x));
 }
 
 // ------------------------------------------------------ solid-aware variant
@@ -488,13 +514,20 @@ __global__ void k_nbmask(Geom g, const uint8_t* __restrict__ solid, uint32_t* __
 //   C(m):   derivatives, equilibria, BGK and store for the fluid tile nodes.
 // The moment and mask rings have five plane slots and the momentum ring four, so
 // a fast warp writing plane m+2 never touches data a slow warp still reads.
+template <int Q, typename S>
+__host__ __device__ constexpr int solid_smem(int TX, int TY) {
+    const int hn = (TX + 4) * (TY + (Q == 19 ? 4 : 0)), t = (int)sizeof(typename Store<S>::T);
+    return t * (15 * hn + 16 * TX * TY) + 4 * 5 * hn;
+}
+
 template <int Q, typename S, int TX, int TY, bool CHK = false>
 __device__ __forceinline__ void solid_body(const MGeom& g, const S* __restrict__ src, S* __restrict__ dst,
                                            const uint32_t* __restrict__ nbm,
                                            const Phys<typename Store<S>::T>& P, double* __restrict__ partials,
-                                           const int bid) {
+                                           const int bid, const Work w) {
     using T = typename Store<S>::T;
     using A = Axes<Q>;
+    extern __shared__ __align__(16) unsigned char tlbm_smem[];
     constexpr int D = Lat<Q>::D;
     constexpr int H = 2;                  // halo width along a
     constexpr int HB = (D == 3) ? 2 : 0;  // halo width along b
@@ -507,19 +540,15 @@ __device__ __forceinline__ void solid_body(const MGeom& g, const S* __restrict__
     static_assert(D == 3 || TY == 1, "2-D tiles are one row");
     static_assert(KS <= 3, "at most three region nodes per thread");
 
-    __shared__ T sm[R][3][HN];       // effective rho, phi, psi (ghosts on solid nodes)
-    __shared__ uint32_t sk[R][HN];   // neighbour masks
-    __shared__ T sj[4][4][NT];       // j and summed f deviations of the tile
+    // dynamic shared memory (solid_smem): effective rho, phi, psi (ghosts on solid
+    // nodes), j and summed f deviations of the tile, neighbour masks
+    T (*const sm)[3][HN] = reinterpret_cast<T(*)[3][HN]>(tlbm_smem);
+    T (*const sj)[4][NT] = reinterpret_cast<T(*)[4][NT]>(tlbm_smem + sizeof(T) * R * 3 * HN);
+    uint32_t (*const sk)[HN] = reinterpret_cast<uint32_t(*)[HN]>(tlbm_smem + sizeof(T) * (R * 3 * HN + 16 * NT));
 
     const int tid = threadIdx.x;
     const int tx = tid % TX, ty = tid / TX;
-    const int tileA = bid % g.tilesA;
-    const int rest = bid / g.tilesA;
-    const int tileB = rest % g.tilesB;
-    const int chunk = rest / g.tilesB;
-    const int A0 = tileA * TX, B0 = tileB * TY;
-    const int M0 = (int)((long long)chunk * g.NM / g.NC);
-    const int M1 = (int)((long long)(chunk + 1) * g.NM / g.NC);
+    const int A0 = w.A0, B0 = w.B0, M0 = w.M0, M1 = w.M1;
     const bool active = (A0 + tx < g.NA) && (B0 + ty < g.NB);
     const long long plane = (long long)g.NA * g.NB;
 
@@ -739,7 +768,37 @@ template <int Q, typename S, int TX, int TY, bool CHK = false>
 __global__ void __launch_bounds__(TX * TY, blocks_per_sm<S>(TX * TY))
 k_fused_solid(MGeom g, const S* __restrict__ src, S* __restrict__ dst, const uint32_t* __restrict__ nbm,
               Phys<typename Store<S>::T> P, double* __restrict__ partials) {
-    solid_body<Q, S, TX, TY, CHK>(g, src, dst, nbm, P, partials, blockIdx.x);
+    solid_body<Q, S, TX, TY, CHK>(g, src, dst, nbm, P, partials, blockIdx.x, work_of<TX, TY>(g, blockIdx.x));
+}
+
+// D2Q9 with solid nodes: a block whose planes keep two nodes away from every solid
+// node runs the periodic body, the others the solid-aware one (which blocks is
+// decided per lattice, Work).  The solid-aware body costs twice as much: two
+// barriers a plane, four halo planes, two loads of every mask.  FP32 4096x2048 with 32 wells
+// (2.6 % of its planes near solids): see DESIGN for both sides.
+template <int Q, typename S>
+struct Mix {
+    static constexpr bool DBL = sizeof(S) == 8;
+    static constexpr int STG = DBL ? 0 : 27;
+    static constexpr int smem(int TX) {
+        const int a = fused_smem<Q, S>(TX, 1, STG), b = solid_smem<Q, S>(TX, 1);
+        return a > b ? a : b;
+    }
+};
+template <int Q, typename S, int TX>
+__device__ __forceinline__ void mix_body(const MGeom& g, const S* __restrict__ src, S* __restrict__ dst,
+                                         const uint32_t* __restrict__ nbm, const Phys<typename Store<S>::T>& P,
+                                         double* __restrict__ partials, const int bid) {
+    const Work w = work_of<TX, 1>(g, bid);
+    if (w.dirty) solid_body<Q, S, TX, 1>(g, src, dst, nbm, P, partials, bid, w);
+    else fused_body<Q, S, TX, 1, false, false, !Mix<Q, S>::DBL, Mix<Q, S>::DBL ? 0 : 2, Mix<Q, S>::STG>(g, src, dst, P, partials,
+                                                                                                  bid, w);
+}
+template <int Q, typename S, int TX>
+__global__ void __launch_bounds__(TX, blocks_per_sm<S>(TX))
+k_mix(MGeom g, const S* __restrict__ src, S* __restrict__ dst, const uint32_t* __restrict__ nbm,
+      Phys<typename Store<S>::T> P, double* __restrict__ partials) {
+    mix_body<Q, S, TX>(g, src, dst, nbm, P, partials, blockIdx.x);
 }
 
 // ------------------------------------------------------------- batches
@@ -778,13 +837,34 @@ __device__ __forceinline__ const SimDesc<T>& batch_member(const SimDesc<T>* __re
     return sh;
 }
 
-template <int Q, typename S, int TX, int TY, bool PF, int HINT>
+// p, known to point to global memory: pointers read from a descriptor are generic to
+// the compiler, whose generic loads and stores may alias the shared rings and run
+// one after another (16 lattices of 768x384, FP32: 330 us a step against 176 of one
+// lattice of their size)
+template <typename P>
+__device__ __forceinline__ P* as_global(P* p) {
+    __builtin_assume(__isGlobal(p));
+    return p;
+}
+// a member's geometry in registers: the descriptor in shared memory could alias the
+// rings as well
+__device__ __forceinline__ MGeom member_geom(const MGeom& m) {
+    MGeom g = m;
+    if (g.items) g.items = as_global(g.items);
+    g.flag = as_global(g.flag);
+    return g;
+}
+
+template <int Q, typename S, int TX, int TY, bool PF, int HINT, int STG>
 __global__ void __launch_bounds__(TX * TY, blocks_per_sm<S>(TX * TY))
 k_fused_batch(const SimDesc<typename Store<S>::T>* __restrict__ d, int nsims) {
     __shared__ SimDesc<typename Store<S>::T> sh;
     const SimDesc<typename Store<S>::T>& m = batch_member(d, nsims, sh);
-    fused_body<Q, S, TX, TY, false, false, PF, HINT>(m.g, static_cast<const S*>(m.src), static_cast<S*>(m.dst),
-                                                     m.P, m.partials, (int)blockIdx.x - m.block0);
+    const int bid = (int)blockIdx.x - m.block0;
+    const MGeom g = member_geom(m.g);
+    fused_body<Q, S, TX, TY, false, false, PF, HINT, STG>(g, as_global(static_cast<const S*>(m.src)),
+                                                          as_global(static_cast<S*>(m.dst)), m.P, as_global(m.partials),
+                                                          bid, work_of<TX, TY>(g, bid));
 }
 
 template <int Q, typename S, int TX, int TY>
@@ -792,8 +872,14 @@ __global__ void __launch_bounds__(TX * TY, blocks_per_sm<S>(TX * TY))
 k_fused_solid_batch(const SimDesc<typename Store<S>::T>* __restrict__ d, int nsims) {
     __shared__ SimDesc<typename Store<S>::T> sh;
     const SimDesc<typename Store<S>::T>& m = batch_member(d, nsims, sh);
-    solid_body<Q, S, TX, TY>(m.g, static_cast<const S*>(m.src), static_cast<S*>(m.dst), m.nbm, m.P,
-                             m.partials, (int)blockIdx.x - m.block0);
+    const int bid = (int)blockIdx.x - m.block0;
+    const S* src = as_global(static_cast<const S*>(m.src));
+    S* dst = as_global(static_cast<S*>(m.dst));
+    const uint32_t* nbm = as_global(m.nbm);
+    double* partials = as_global(m.partials);
+    const MGeom g = member_geom(m.g);
+    if constexpr (Q == 9) mix_body<Q, S, TX>(g, src, dst, nbm, m.P, partials, bid);
+    else solid_body<Q, S, TX, TY>(g, src, dst, nbm, m.P, partials, bid, work_of<TX, TY>(g, bid));
 }
 
 // FP64 totals of every member: block i sums member i's partials in a fixed order

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 namespace tlbm_host {
 
 // Physical parameters in double; each translation unit converts to its compute type.
@@ -43,6 +45,9 @@ struct DevState {
     const uint8_t* solid;  // device mask (nullptr when there are no solid nodes)
     uint32_t* nbm;       // per-node neighbour-solid bits for the fused step (with solids)
     int nbm_ready;       // nbm has been built
+    const uint8_t* units;  // host: solid nodes per 32-node unit (column_runs), with solids
+    const void* items;   // device work items of the fused step (Work), dirty ones first; or null
+    int nitems, ndirty;
     void* mom;           // split-step moment arrays [3][Np] (compute type); scratch
     double* partials;    // mass partial sums, 3 per block
     double* step_mass;   // [3] totals accumulated inside the last step
@@ -64,6 +69,7 @@ struct DevState {
 struct BatchState {
     int count;
     DevState** sims;     // member engines' device states
+    void* items;         // device work items of all members (lattices with solid nodes)
     void* desc;          // device descriptor array: [2][count], one set per buffer parity
     int tile;            // tile choice for every member (DevState::tile encoding)
     int auto_tile;       // the same with the chunk resolved for the whole grid
@@ -110,6 +116,9 @@ struct Ops {
     // compute-type values per node of the forcing coupling's node arrays
     int (*aux_per_node)();
     bool (*has_fused)(const DevState& d);
+    // work items (int4) of the fused step on a lattice with solid nodes, dirty ones
+    // first; returns the number of dirty ones (empty: one grid over the lattice)
+    int (*solid_items)(const DevState& d, std::vector<int4>& out);
     // batches: build the descriptors of both parities (and neighbour masks);
     // one step of every member (flips every member's cur)
     cudaError_t (*batch_build)(BatchState& b, cudaStream_t st);

@@ -2,6 +2,7 @@
 // batches.
 #pragma once
 
+#include <algorithm>
 #include <vector>
 
 #include "tlbm_bulk.cuh"
@@ -46,25 +47,43 @@ inline double march_cost(double nb, int mc, int halo, int res, int sms, bool dbl
     return (mc + halo) * (whole * plane(res) + (rest > 0 ? plane(b) : 0.0));
 }
 
-// Planes per block (chunk) of one marching launch over n lattices with cols[k]
-// tile columns of nm[k] planes: the cheapest by march_cost whose block sums fit
-// (caps[k]).  At most 64 planes in 2-D; in 3-D 16 once the grid fills the device
-// eight times over (256^3 FP32: 16 planes 0.692 of HBM, 24..128 planes 0.66..0.69:
-// blocks that start together share their halo rows in L2).
-inline int pick_chunk(const long long* cols, const int* nm, const long long* caps, int n, int halo, int res, int sms,
+// cols columns of tiles, each with nm planes to march, of lattice `member`
+struct Run {
+    long long cols;
+    int nm, member;
+    bool dirty;
+};
+
+// Planes per block of the solid-aware body where clean blocks march mc: a plane of it
+// takes about 1.6 times as long and it has four halo planes, and a block that
+// outlasts the others is the step's time (sweep of 24 wells: one 60-plane block
+// was 260 of 310 us).
+inline int dirty_chunk(int mc) { return mc <= 4 ? mc : (mc / 2 - 2 > 4 ? mc / 2 - 2 : 4); }
+
+// Planes per block (chunk) of one marching launch over these runs: the cheapest by
+// march_cost whose blocks' sums fit every member (caps).  At most 64 planes in
+// 2-D; in 3-D 16 once the grid fills the device eight times over (256^3 FP32: 16
+// planes 0.692 of HBM, 24..128 planes 0.66..0.69: blocks that start together share
+// their halo rows in L2).
+inline int pick_chunk(const std::vector<Run>& runs, const std::vector<long long>& caps, int halo, int res, int sms,
                       bool three_d, bool dbl) {
     double best = 0.0;
     int bmc = 0;
+    std::vector<long long> nbs(caps.size());
     for (int mc = three_d ? 2 : 1; mc <= 64; ++mc) {
         double nb = 0.0;
         int used = 0;
-        bool fits = true;
-        for (int k = 0; k < n; ++k) {
-            const int nc = (nm[k] + mc - 1) / mc, per = (nm[k] + nc - 1) / nc;
-            nb += (double)cols[k] * nc;
+        for (long long& v : nbs) v = 0;
+        for (const Run& r : runs) {
+            const int ch = r.dirty ? dirty_chunk(mc) : mc;
+            const int nc = (r.nm + ch - 1) / ch, per = r.dirty ? 0 : (r.nm + nc - 1) / nc;
+            nb += (double)r.cols * nc;
+            nbs[(size_t)r.member] += r.cols * nc;
             used = per > used ? per : used;
-            fits = fits && cols[k] * nc <= caps[k];
         }
+        bool fits = true;
+        if (used == 0) used = mc;
+        for (size_t k = 0; k < caps.size(); ++k) fits = fits && nbs[k] <= caps[k];
         if (!fits) continue;
         const double c = march_cost(nb, used, halo, res, sms, dbl);
         if (three_d && used > 16 && nb >= 8.0 * res * sms) continue;
@@ -140,10 +159,130 @@ inline FusedCfg<Q> fused_cfg(const tlbm_host::DevState& d) {
     const int NM = (Q == 19) ? d.nz : d.ny;
     if (mc <= 0) {
         const long long cols = (long long)((NA + c.TX - 1) / c.TX) * ((NB + c.TY - 1) / c.TY);
-        mc = pick_chunk(&cols, &NM, &d.partials_cap, 1, c.halo(d), c.res(d), d.sms, Q == 19, dbl);
+        mc = pick_chunk({Run{cols, NM, 0, false}}, {d.partials_cap}, c.halo(d), c.res(d), d.sms, Q == 19, dbl);
     }
     c.MC = mc < 1 ? 1 : (mc > NM ? NM : mc);
     return c;
+}
+
+// ---- lattices with solid nodes: the blocks' work
+
+// A column's planes as runs of one kind: dirty planes have a solid node within two
+// nodes of the tile (ghosts of the one-node halo need moments of the second, whose
+// pulls a solid node turns back); planes whose tile nodes are all solid are left
+// out.  Clean gaps shorter than four planes join their dirty neighbours (each
+// block has 2 (clean) or 4 (dirty) halo planes to recompute).
+struct ColumnRun {
+    int A0, B0, m0, nm;
+    bool dirty;
+};
+
+// d.units[(m NB + b) ncx + u], for 32 nodes u of row b, plane m: bit 0 a solid node
+// in x from two before to two behind, bit 1 all of them solid.
+template <int Q>
+inline std::vector<ColumnRun> column_runs(const tlbm_host::DevState& d, const FusedCfg<Q>& c) {
+    const int NB = Q == 19 ? d.ny : 1, NM = Q == 19 ? d.nz : d.ny, HB = Q == 19 ? 2 : 0;
+    std::vector<ColumnRun> out;
+    std::vector<unsigned char> near((size_t)NM), full((size_t)NM), kind((size_t)NM);
+    for (int B0 = 0; B0 < NB; B0 += c.TY)
+        for (int A0 = 0; A0 < d.nx; A0 += c.TX) {
+            const int u0 = A0 / 32, u1 = (A0 + c.TX + 31) / 32 < d.ncx ? (A0 + c.TX + 31) / 32 : d.ncx;
+            for (int m = 0; m < NM; ++m) {
+                unsigned char any = 0, all = 1;
+                for (int b = B0 - HB; b < B0 + c.TY + HB; ++b) {
+                    const bool tile = b >= B0 && b < B0 + c.TY && b < NB;
+                    const unsigned char* row = d.units + ((size_t)m * NB + (size_t)(((b % NB) + NB) % NB)) * d.ncx;
+                    for (int u = u0; u < u1; ++u) {
+                        any |= row[u] & 1;
+                        if (tile && !(row[u] & 2)) all = 0;
+                    }
+                }
+                near[(size_t)m] = any;
+                full[(size_t)m] = all;
+            }
+            for (int m = 0; m < NM; ++m) {
+                unsigned char any = 0;
+                for (int k = -2; k <= 2; ++k) any |= near[(size_t)((((m + k) % NM) + NM) % NM)];
+                kind[(size_t)m] = full[(size_t)m] ? 2 : any;
+            }
+            for (int m = 0; m < NM;) {  // short clean gaps
+                int e = m;
+                while (e < NM && kind[(size_t)e] == 0) ++e;
+                if (e > m && e - m < 4 && e - m < NM)
+                    for (int k = m; k < e; ++k) kind[(size_t)k] = 1;
+                m = e > m ? e : m + 1;
+            }
+            for (int m = 0; m < NM;) {
+                int e = m + 1;
+                while (e < NM && kind[(size_t)e] == kind[(size_t)m]) ++e;
+                if (kind[(size_t)m] != 2) out.push_back(ColumnRun{A0, B0, m, e - m, kind[(size_t)m] == 1});
+                m = e;
+            }
+        }
+    return out;
+}
+
+// Whether an engine's solid lattice is stepped by work items: D2Q9 always (k_mix);
+// D3Q19 (FP32, 16-bit: dirty blocks by k_fused_solid, clean ones by k_bulk, two
+// launches) where the clean blocks alone fill the device.
+template <int Q>
+inline bool wants_items(const tlbm_host::DevState& d) {
+    return d.solid && d.units && (Q == 9 || d.prec != 0);
+}
+
+// The work items (A0, B0, M0, 2 M1 + dirty) of chunk mc, dirty ones first: they take
+// longest.  Returns the number of dirty ones.
+inline int make_items(const std::vector<ColumnRun>& runs, int mc, std::vector<int4>& out) {
+    int dirty = 0;
+    for (int pass = 1; pass >= 0; --pass) {
+        const size_t first = out.size();
+        for (const ColumnRun& r : runs) {
+            if (r.dirty != (pass == 1)) continue;
+            const int ch = r.dirty ? dirty_chunk(mc) : mc, nc = (r.nm + ch - 1) / ch;
+            for (int c = 0; c < nc; ++c)
+                out.push_back(make_int4(r.A0, r.B0, r.m0 + (int)((long long)c * r.nm / nc),
+                                        2 * (r.m0 + (int)((long long)(c + 1) * r.nm / nc)) + pass));
+        }
+        // blocks that start together work on neighbouring planes and share rows in L2
+        std::stable_sort(out.begin() + (long)first, out.end(), [](const int4& a, const int4& b) { return a.z < b.z; });
+        if (pass == 1) dirty = (int)out.size();
+    }
+    return dirty;
+}
+
+inline int runs_halo(const std::vector<ColumnRun>& runs) {
+    long long d = 0, c = 0;
+    for (const ColumnRun& r : runs) (r.dirty ? d : c) += r.nm;
+    return c > d ? 2 : 4;
+}
+
+inline void add_runs(const std::vector<ColumnRun>& runs, int member, std::vector<Run>& out) {
+    for (const ColumnRun& r : runs) out.push_back(Run{1, r.nm, member, r.dirty});
+}
+
+// Work items of an engine's lattice at its tile and chunk; none where one grid over
+// the whole lattice serves (ndirty = 0, out empty).
+template <int Q, typename S>
+inline int solid_items(const tlbm_host::DevState& d, std::vector<int4>& out) {
+    out.clear();
+    if (!wants_items<Q>(d)) return 0;
+    tlbm_host::DevState dd = d;
+    dd.tile = d.tile | ((d.tile >> 8) ? 0 : 1 << 8);  // any chunk: only the tile is wanted
+    const FusedCfg<Q> c = fused_cfg<Q>(dd);
+    const std::vector<ColumnRun> runs = column_runs<Q>(d, c);
+    int mc = d.tile >> 8;
+    if (mc == 0) {
+        std::vector<Run> all;
+        add_runs(runs, 0, all);
+        mc = pick_chunk(all, {d.partials_cap}, runs_halo(runs), c.res(d), d.sms, Q == 19, d.prec == 0);
+    }
+    int dirty = make_items(runs, mc, out);
+    const long long clean = (long long)out.size() - dirty;
+    if ((long long)out.size() > d.partials_cap || (Q == 19 && clean < 2LL * d.sms)) {
+        out.clear();
+        dirty = 0;
+    }
+    return dirty;
 }
 
 template <int Q, typename S>
@@ -152,8 +291,8 @@ inline bool fused_supported(const tlbm_host::DevState& d) {
 }
 
 template <int Q, typename S>
-inline int fused_launches(const tlbm_host::DevState&) {
-    return 1;
+inline int fused_launches(const tlbm_host::DevState& d) {
+    return Q == 19 && d.nitems > 0 && d.ndirty > 0 && !d.checked ? 2 : 1;
 }
 
 template <int Q, typename S>
@@ -167,6 +306,7 @@ inline MGeom mgeom(const tlbm_host::DevState& d, const FusedCfg<Q>& c) {
     g.bytes = d.pop_bytes;
     g.check = d.check;
     g.flag = d.flag;
+    g.items = d.checked ? nullptr : static_cast<const int4*>(d.items);
     g.tilesA = (g.NA + c.TX - 1) / c.TX;
     g.tilesB = (g.NB + c.TY - 1) / c.TY;
     return g;
@@ -174,6 +314,7 @@ inline MGeom mgeom(const tlbm_host::DevState& d, const FusedCfg<Q>& c) {
 
 template <int Q, typename S>
 inline long long fused_blocks(const tlbm_host::DevState& d) {
+    if (d.nitems > 0 && !d.checked) return d.nitems;
     const FusedCfg<Q> c = fused_cfg<Q>(d);
     const MGeom g = mgeom<Q, S>(d, c);
     return (long long)g.tilesA * g.tilesB * g.NC;
@@ -196,9 +337,9 @@ inline cudaError_t launch_smem(K kern, int dyn, int threads, int bps, long long 
     return cudaSuccess;
 }
 // ... of a D2Q9 kernel with stg staged values per thread of 128
-template <typename K, typename... Args>
+template <typename S, typename K, typename... Args>
 inline cudaError_t launch_staged(K kern, int stg, long long nb, cudaStream_t st, Args... args) {
-    return launch_smem(kern, stg * 2 * 128 * (int)sizeof(float), 128, 4, nb, st, args...);
+    return launch_smem(kern, fused_smem<9, S>(128, 1, stg), 128, 4, nb, st, args...);
 }
 // ... of k_bulk
 template <typename S, typename K, typename... Args>
@@ -211,7 +352,7 @@ template <int Q, typename S>
 inline cudaError_t fused_step(tlbm_host::DevState& d, const Phys<typename Store<S>::T>& P, cudaStream_t st) {
     const FusedCfg<Q> c = fused_cfg<Q>(d);
     const MGeom g = mgeom<Q, S>(d, c);
-    const long long nb = (long long)g.tilesA * g.tilesB * g.NC;
+    const long long nb = fused_blocks<Q, S>(d);
     if (nb > 0x7fffffffLL || nb > d.partials_cap) return cudaErrorInvalidConfiguration;
     const S* src = static_cast<const S*>(d.pop[d.cur]);
     S* dst = static_cast<S*>(d.pop[1 - d.cur]);
@@ -225,12 +366,14 @@ inline cudaError_t fused_step(tlbm_host::DevState& d, const Phys<typename Store<
         if constexpr (sizeof(S) == 4) {
             if (!d.check) return cudaErrorInvalidValue;
             if (d.solid) {
-                if constexpr (Q == 19) k_fused_solid<Q, S, 32, 4, true><<<(int)nb, 128, 0, st>>>(g, src, dst, d.nbm, P, d.partials);
-                else k_fused_solid<Q, S, 128, 1, true><<<(int)nb, 128, 0, st>>>(g, src, dst, d.nbm, P, d.partials);
+                cudaError_t e;
+                if constexpr (Q == 19) e = launch_smem(k_fused_solid<Q, S, 32, 4, true>, solid_smem<Q, S>(32, 4), 128, 4, nb, st, g, src, dst, d.nbm, P, d.partials);
+                else e = launch_smem(k_fused_solid<Q, S, 128, 1, true>, solid_smem<Q, S>(128, 1), 128, 4, nb, st, g, src, dst, d.nbm, P, d.partials);
+                if (e != cudaSuccess) return e;
             } else {
                 cudaError_t e;
                 if constexpr (Q == 19) e = launch_bulk<S>(k_bulk<S, true>, nb, st, g, src, dst, P, d.partials);
-                else e = launch_staged(k_fused_x<Q, S, 128, 1, 27, true>, 27, nb, st, g, src, dst, P, d.partials);
+                else e = launch_staged<S>(k_fused_x<Q, S, 128, 1, 27, true>, 27, nb, st, g, src, dst, P, d.partials);
                 if (e != cudaSuccess) return e;
             }
             return cudaGetLastError();
@@ -239,22 +382,39 @@ inline cudaError_t fused_step(tlbm_host::DevState& d, const Phys<typename Store<
         }
     }
     if (d.solid) {
-        auto gos = [&](auto kern, int threads) {
-            kern<<<(int)nb, threads, 0, st>>>(g, src, dst, d.nbm, P, d.partials);
-        };
+        if (nb == 0) return cudaSuccess;  // no fluid node
+        cudaError_t e = cudaSuccess;
         if constexpr (Q == 19) {
-            if constexpr (sizeof(S) == 8) gos(k_fused_solid<Q, S, 16, 4>, 64);
-            else gos(k_fused_solid<Q, S, 32, 4>, 128);
+            constexpr int TX = sizeof(S) == 8 ? 16 : 32;
+            const long long nd = d.nitems > 0 ? d.ndirty : nb;
+            if (nd > 0)
+                e = launch_smem(k_fused_solid<Q, S, TX, 4>, solid_smem<Q, S>(TX, 4), TX * 4, 512 / (TX * 4), nd, st, g, src,
+                                dst, d.nbm, P, d.partials);
+            if constexpr (sizeof(S) < 8) {
+                if (e == cudaSuccess && nb > nd) {
+                    MGeom gc = g;
+                    gc.items = g.items + nd;
+                    e = launch_bulk<S>(k_bulk<S, false>, nb - nd, st, gc, src, dst, P, d.partials + 3 * nd);
+                }
+            }
         } else {
-            if (c.TX == 256) gos(k_fused_solid<Q, S, 256, 1>, 256);
-            else if (c.TX == 64) gos(k_fused_solid<Q, S, 64, 1>, 64);
-            else if (c.TX == 32) {
-                if constexpr (sizeof(S) == 8) gos(k_fused_solid<Q, S, 32, 1>, 32);
-            } else gos(k_fused_solid<Q, S, 128, 1>, 128);
+            auto mix = [&](auto kern, int TX) {
+                e = launch_smem(kern, Mix<Q, S>::smem(TX), TX, blocks_per_sm<S>(TX), nb, st, g, src, dst, d.nbm, P, d.partials);
+            };
+            if constexpr (sizeof(S) == 8) {
+                if (c.TX == 32) mix(k_mix<Q, S, 32>, 32);
+                else mix(k_mix<Q, S, 128>, 128);
+            } else {
+                if (c.TX == 256) mix(k_mix<Q, S, 256>, 256);
+                else if (c.TX == 64) mix(k_mix<Q, S, 64>, 64);
+                else mix(k_mix<Q, S, 128>, 128);
+            }
         }
-        return cudaGetLastError();
+        return e != cudaSuccess ? e : cudaGetLastError();
     }
-    auto go = [&](auto kern, int threads) { kern<<<(int)nb, threads, 0, st>>>(g, src, dst, P, d.partials); };
+    auto go = [&](auto kern, int threads) {
+        kern<<<(int)nb, threads, fused_smem<Q, S>(c.TX, c.TY, 0), st>>>(g, src, dst, P, d.partials);
+    };
     if constexpr (sizeof(S) == 8) {
         // double storage is the parity path: one tile shape per lattice and size
         if constexpr (Q == 19) go(k_fused<Q, S, 16, 8, false, false>, 128);
@@ -269,8 +429,8 @@ inline cudaError_t fused_step(tlbm_host::DevState& d, const Phys<typename Store<
             // all 27, with the per-warp prefetch and evict-first stores and
             // collision loads
             const cudaError_t e =
-                c.shape == 4 ? launch_staged(k_fused_x<Q, S, 128, 1, 18>, 18, nb, st, g, src, dst, P, d.partials)
-                             : launch_staged(k_fused_x<Q, S, 128, 1, 27>, 27, nb, st, g, src, dst, P, d.partials);
+                c.shape == 4 ? launch_staged<S>(k_fused_x<Q, S, 128, 1, 18>, 18, nb, st, g, src, dst, P, d.partials)
+                             : launch_staged<S>(k_fused_x<Q, S, 128, 1, 27>, 27, nb, st, g, src, dst, P, d.partials);
             return e != cudaSuccess ? e : cudaGetLastError();
         }
         if (c.TX == 256) {
@@ -308,32 +468,70 @@ inline cudaError_t batch_build(tlbm_host::BatchState& b, cudaStream_t st) {
     b.auto_tile = b.tile;
     b.narrow = 1;
     for (int k = 0; k < n; ++k) b.narrow = b.narrow && narrow_rows(*b.sims[k]);
+    // tile of member k (chunk 1 stands for any), its runs and its blocks with chunk 0
+    // (its own choice) or mc
+    auto member = [&](int k, int mc) {
+        tlbm_host::DevState dd = *b.sims[k];
+        dd.tile = (b.tile & 255) | mc << 8;
+        dd.rows128 = !b.narrow;
+        dd.items = nullptr;
+        dd.nitems = 0;
+        return dd;
+    };
+    std::vector<std::vector<int4>> items((size_t)n);
+    auto blocks = [&](int k, const tlbm_host::DevState& dd) -> long long {
+        if (Q == 9 && solid) {
+            solid_items<Q, S>(dd, items[(size_t)k]);
+            if (!items[(size_t)k].empty()) return (long long)items[(size_t)k].size();
+        }
+        return fused_blocks<Q, S>(dd);
+    };
     if ((b.tile >> 8) == 0) {
         // members whose own chunks do not fill the device twice keep them; beyond
         // that the halo planes of short chunks are what costs, and one chunk is
         // chosen for the whole grid (24 wells of 128x64 .. 768x384, FP32: 343 us a
-        // step with chunks of 4 to 8 planes, see k_fused_solid_batch)
-        std::vector<long long> cols, caps;
+        // step with chunks of 4 to 8 planes)
+        std::vector<Run> runs;
+        std::vector<long long> caps;
         long long own = 0;
-        std::vector<int> nm;
+        const tlbm_host::DevState d0 = member(0, 1);
         FusedCfg<Q> c{};
-        tlbm_host::DevState d0 = *b.sims[0];
+        int halo = 0;
         for (int k = 0; k < n; ++k) {
-            tlbm_host::DevState dd = *b.sims[k];
-            dd.tile = b.tile;
-            dd.rows128 = !b.narrow;
-            own += fused_blocks<Q, S>(dd);
+            own += blocks(k, member(k, 0));
+            const tlbm_host::DevState dd = member(k, 1);
             c = fused_cfg<Q>(dd);
-            cols.push_back((long long)((dd.nx + c.TX - 1) / c.TX) * (Q == 19 ? (dd.ny + c.TY - 1) / c.TY : 1));
-            nm.push_back(Q == 19 ? dd.nz : dd.ny);
+            if (Q == 9 && solid) {
+                const std::vector<ColumnRun> cr = column_runs<Q>(dd, c);
+                add_runs(cr, k, runs);
+                halo += runs_halo(cr);
+            } else {
+                runs.push_back(Run{(long long)((dd.nx + c.TX - 1) / c.TX) * (Q == 19 ? (dd.ny + c.TY - 1) / c.TY : 1),
+                                   Q == 19 ? dd.nz : dd.ny, k, false});
+                halo += c.halo(dd);
+            }
             caps.push_back(dd.partials_cap);
         }
         if (own >= 2LL * c.res(d0) * d0.sms) {
-            const int mc = pick_chunk(cols.data(), nm.data(), caps.data(), n, c.halo(d0), c.res(d0), d0.sms, Q == 19,
-                                      d0.prec == 0);
+            const int mc = pick_chunk(runs, caps, (halo + n / 2) / n, c.res(d0), d0.sms, Q == 19, d0.prec == 0);
             b.auto_tile = (b.tile & 255) | mc << 8;
         }
     }
+    size_t nit = 0;
+    std::vector<long long> nbs((size_t)n);
+    for (int k = 0; k < n; ++k) {
+        nbs[(size_t)k] = blocks(k, member(k, b.auto_tile >> 8));
+        nit += items[(size_t)k].size();
+    }
+    cudaError_t e = cudaSuccess;
+    if (nit > 0) {
+        e = cudaStreamSynchronize(st);  // no step in flight reads the items that are replaced
+        if (e == cudaSuccess && b.items) e = cudaFree(b.items);
+        b.items = nullptr;
+        if (e == cudaSuccess) e = cudaMalloc(&b.items, sizeof(int4) * nit);
+        if (e != cudaSuccess) return e;
+    }
+    size_t it0 = 0;
     for (int k = 0; k < n; ++k) {
         tlbm_host::DevState& d = *b.sims[k];
         if ((d.solid != nullptr) != solid || d.cur != b.sims[0]->cur) return cudaErrorInvalidValue;
@@ -342,18 +540,23 @@ inline cudaError_t batch_build(tlbm_host::BatchState& b, cudaStream_t st) {
             k_nbmask<Q><<<grid_of(d.N, d.sms), 256, 0, st>>>(gg, d.solid, d.nbm);
             d.nbm_ready = 1;
         }
-        tlbm_host::DevState dd = d;
-        dd.tile = b.auto_tile;
-        dd.rows128 = !b.narrow;
+        const tlbm_host::DevState dd = member(k, b.auto_tile >> 8);
         const FusedCfg<Q> c = fused_cfg<Q>(dd);
         // shapes with a batched kernel (batch_step): every solid shape; periodic
         // D3Q19 all but 1 and 2; periodic D2Q9 rows of 128 and the one-warp rows
         const int variant = sizeof(S) == 8 ? 0 : (b.tile & 15);
         const bool shape_ok = solid || (Q == 19 ? variant != 1 && variant != 2 : c.TX == 128 || sizeof(S) == 8);
         if (!shape_ok) return cudaErrorInvalidConfiguration;
-        const MGeom g = mgeom<Q, S>(dd, c);
-        const long long nb = (long long)g.tilesA * g.tilesB * g.NC;
-        if (nb > d.partials_cap) return cudaErrorInvalidConfiguration;
+        MGeom g = mgeom<Q, S>(dd, c);
+        const long long nb = nbs[(size_t)k];
+        if (nb > d.partials_cap || nb < 1) return cudaErrorInvalidConfiguration;
+        if (!items[(size_t)k].empty()) {
+            int4* to = static_cast<int4*>(b.items) + it0;
+            e = cudaMemcpyAsync(to, items[(size_t)k].data(), sizeof(int4) * items[(size_t)k].size(), cudaMemcpyHostToDevice, st);
+            if (e != cudaSuccess) return e;
+            g.items = to;
+            it0 += items[(size_t)k].size();
+        }
         for (int par = 0; par < 2; ++par) {
             SimDesc<T>& e = h[(size_t)par * n + k];
             e.g = g;
@@ -371,7 +574,6 @@ inline cudaError_t batch_build(tlbm_host::BatchState& b, cudaStream_t st) {
     }
     if (block0 > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     b.blocks = block0;
-    cudaError_t e = cudaSuccess;
     if (!b.desc) e = cudaMalloc(&b.desc, sizeof(SimDesc<T>) * 2 * (size_t)n);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b.desc, h.data(), sizeof(SimDesc<T>) * 2 * (size_t)n, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -392,30 +594,38 @@ inline cudaError_t batch_step(tlbm_host::BatchState& b, cudaStream_t st, cudaEve
     const FusedCfg<Q> c = fused_cfg<Q>(probe);
     const int nb = (int)b.blocks;
     if (ev0) cudaEventRecord(ev0, st);
+    cudaError_t e = cudaSuccess;
     if (probe.solid) {
         if constexpr (Q == 19) {
-            if constexpr (sizeof(S) == 8) k_fused_solid_batch<Q, S, 16, 4><<<nb, 64, 0, st>>>(d, n);
-            else k_fused_solid_batch<Q, S, 32, 4><<<nb, 128, 0, st>>>(d, n);
+            constexpr int TX = sizeof(S) == 8 ? 16 : 32;
+            e = launch_smem(k_fused_solid_batch<Q, S, TX, 4>, solid_smem<Q, S>(TX, 4), TX * 4, 512 / (TX * 4), nb, st, d, n);
         } else {
-            if (c.TX == 256) k_fused_solid_batch<Q, S, 256, 1><<<nb, 256, 0, st>>>(d, n);
-            else if (c.TX == 64) k_fused_solid_batch<Q, S, 64, 1><<<nb, 64, 0, st>>>(d, n);
-            else if (c.TX == 32) {
-                if constexpr (sizeof(S) == 8) k_fused_solid_batch<Q, S, 32, 1><<<nb, 32, 0, st>>>(d, n);
-            } else k_fused_solid_batch<Q, S, 128, 1><<<nb, 128, 0, st>>>(d, n);
+            auto mix = [&](auto kern, int TX) {
+                e = launch_smem(kern, Mix<Q, S>::smem(TX), TX, blocks_per_sm<S>(TX), nb, st, d, n);
+            };
+            if constexpr (sizeof(S) == 8) {
+                if (c.TX == 32) mix(k_fused_solid_batch<Q, S, 32, 1>, 32);
+                else mix(k_fused_solid_batch<Q, S, 128, 1>, 128);
+            } else {
+                if (c.TX == 256) mix(k_fused_solid_batch<Q, S, 256, 1>, 256);
+                else if (c.TX == 64) mix(k_fused_solid_batch<Q, S, 64, 1>, 64);
+                else mix(k_fused_solid_batch<Q, S, 128, 1>, 128);
+            }
         }
     } else {
+        auto go = [&](auto kern, int threads, int stg) {
+            e = launch_smem(kern, fused_smem<Q, S>(c.TX, c.TY, stg), threads, blocks_per_sm<S>(threads), nb, st, d, n);
+        };
         if constexpr (Q == 19) {
-            if constexpr (sizeof(S) == 8) k_fused_batch<Q, S, 16, 8, false, 0><<<nb, 128, 0, st>>>(d, n);
-            else {
-                const cudaError_t e = launch_bulk<S>(k_bulk_batch<S>, nb, st, d, n);
-                if (e != cudaSuccess) return e;
-            }
+            if constexpr (sizeof(S) == 8) go(k_fused_batch<Q, S, 16, 8, false, 0, 0>, 128, 0);
+            else e = launch_bulk<S>(k_bulk_batch<S>, nb, st, d, n);
         } else if (sizeof(S) == 8 && c.TX == 32) {
-            if constexpr (sizeof(S) == 8) k_fused_batch<Q, S, 32, 1, false, 0><<<nb, 32, 0, st>>>(d, n);
+            if constexpr (sizeof(S) == 8) go(k_fused_batch<Q, S, 32, 1, false, 0, 0>, 32, 0);
         } else {
-            k_fused_batch<Q, S, 128, 1, true, 2><<<nb, 128, 0, st>>>(d, n);
+            go(k_fused_batch<Q, S, 128, 1, true, 2, sizeof(S) == 8 ? 0 : 27>, 128, sizeof(S) == 8 ? 0 : 27);
         }
     }
+    if (e != cudaSuccess) return e;
     if (ev1) cudaEventRecord(ev1, st);
     for (int k = 0; k < n; ++k) b.sims[k]->cur ^= 1;
     return cudaGetLastError();

@@ -165,6 +165,7 @@ struct Impl {
         return (d.solid ? 3 : 2) + 1;
     }
 
+    static int solid_work(const DevState& d, std::vector<int4>& out) { return solid_items<Q, S>(d, out); }
     static bool has_fused(const DevState& d) { return fused_supported<Q, S>(d); }
 
     template <bool SOLID>
@@ -264,7 +265,7 @@ struct Impl {
 
     static const tlbm_host::Ops* table() {
         static const tlbm_host::Ops o = {&step,     &totals,       &init,      &fields, &mass,    &get_box,
-                                         &set_pops, &launches,     &aux_per_node, &has_fused, &bbuild,
+                                         &set_pops, &launches,     &aux_per_node, &has_fused, &solid_work, &bbuild,
                                          &bstep,    &btotals,      &adjoint};
         return &o;
     }
