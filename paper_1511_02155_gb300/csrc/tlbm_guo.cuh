@@ -479,6 +479,7 @@ __device__ __forceinline__ void guo_body(const MGeom& g, const S* __restrict__ s
     constexpr bool PAIR = Fmt<Q, S>::OFFSET && !(Q == 19 && sizeof(S) == 4);
     MassSum<T, PAIR> msum;
 
+    grid_ready();
     moments_plane(M0 - 2);
     moments_plane(M0 - 1);
     moments_plane(M0);
@@ -578,13 +579,14 @@ inline cudaError_t guo_fused_step(tlbm_host::DevState& d, const Phys<typename St
     if (nb > 0x7fffffffLL || nb > d.partials_cap) return cudaErrorInvalidConfiguration;
     const S* src = static_cast<const S*>(d.pop[d.cur]);
     S* dst = static_cast<S*>(d.pop[1 - d.cur]);
+    cudaError_t e;
     if constexpr (Q == 19) {
-        if constexpr (sizeof(S) == 8) k_guo_fused<Q, S, 16, 4><<<(int)nb, 64, 0, st>>>(g, src, dst, P, d.partials);
-        else k_guo_fused<Q, S, 32, 4><<<(int)nb, 128, 0, st>>>(g, src, dst, P, d.partials);
+        constexpr int TX = sizeof(S) == 8 ? 16 : 32;
+        e = launch_step(k_guo_fused<Q, S, TX, 4>, 0, TX * 4, nb, st, g, src, dst, P, d.partials);
     } else {
-        k_guo_fused<Q, S, 128, 1><<<(int)nb, 128, 0, st>>>(g, src, dst, P, d.partials);
+        e = launch_step(k_guo_fused<Q, S, 128, 1>, 0, 128, nb, st, g, src, dst, P, d.partials);
     }
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace tlbm_dev

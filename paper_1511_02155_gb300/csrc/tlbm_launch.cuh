@@ -306,6 +306,7 @@ inline MGeom mgeom(const tlbm_host::DevState& d, const FusedCfg<Q>& c) {
     g.bytes = d.pop_bytes;
     g.check = d.check;
     g.flag = d.flag;
+    g.beside = 0;
     g.items = d.checked ? nullptr : static_cast<const int4*>(d.items);
     g.tilesA = (g.NA + c.TX - 1) / c.TX;
     g.tilesB = (g.NB + c.TY - 1) / c.TY;
@@ -320,7 +321,22 @@ inline long long fused_blocks(const tlbm_host::DevState& d) {
     return (long long)g.tilesA * g.tilesB * g.NC;
 }
 
-// Launch with dyn bytes of dynamic shared memory and the smallest shared-memory
+// Launch of a step kernel (grid_ready) with dyn bytes of dynamic shared memory.
+template <typename K, typename... Args>
+inline cudaError_t launch_step(K kern, int dyn, int threads, long long nb, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3((unsigned)nb);
+    c.blockDim = dim3((unsigned)threads);
+    c.dynamicSmemBytes = (size_t)dyn;
+    c.stream = st;
+    cudaLaunchAttribute a{};
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &a;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kern, args...);
+}
+// The same with the smallest shared-memory
 // carveout that holds bps blocks per SM, so that the rest of the SM's 256 KB stays
 // L1 (which holds the kernel's loads in flight).
 template <typename K, typename... Args>
@@ -333,8 +349,7 @@ inline cudaError_t launch_smem(K kern, int dyn, int threads, int bps, long long 
     const int pct = (int)((need * 100 + 233471) / 233472);
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, pct > 100 ? 100 : pct);
     if (e != cudaSuccess) return e;
-    kern<<<(int)nb, threads, dyn, st>>>(args...);
-    return cudaSuccess;
+    return launch_step(kern, dyn, threads, nb, st, args...);
 }
 // ... of a D2Q9 kernel with stg staged values per thread of 128
 template <typename S, typename K, typename... Args>
@@ -394,6 +409,7 @@ inline cudaError_t fused_step(tlbm_host::DevState& d, const Phys<typename Store<
                 if (e == cudaSuccess && nb > nd) {
                     MGeom gc = g;
                     gc.items = g.items + nd;
+                    gc.beside = nd > 0;
                     e = launch_bulk<S>(k_bulk<S, false>, nb - nd, st, gc, src, dst, P, d.partials + 3 * nd);
                 }
             }
@@ -412,8 +428,9 @@ inline cudaError_t fused_step(tlbm_host::DevState& d, const Phys<typename Store<
         }
         return e != cudaSuccess ? e : cudaGetLastError();
     }
+    cudaError_t e = cudaSuccess;
     auto go = [&](auto kern, int threads) {
-        kern<<<(int)nb, threads, fused_smem<Q, S>(c.TX, c.TY, 0), st>>>(g, src, dst, P, d.partials);
+        e = launch_step(kern, fused_smem<Q, S>(c.TX, c.TY, 0), threads, nb, st, g, src, dst, P, d.partials);
     };
     if constexpr (sizeof(S) == 8) {
         // double storage is the parity path: one tile shape per lattice and size
@@ -421,15 +438,13 @@ inline cudaError_t fused_step(tlbm_host::DevState& d, const Phys<typename Store<
         else if (c.TX == 32) go(k_fused<Q, S, 32, 1, false, false>, 32);
         else go(k_fused<Q, S, 128, 1, false, false>, 128);
     } else if constexpr (Q == 19) {
-        const cudaError_t e = launch_bulk<S>(k_bulk<S, false>, nb, st, g, src, dst, P, d.partials);
-        if (e != cudaSuccess) return e;
+        e = launch_bulk<S>(k_bulk<S, false>, nb, st, g, src, dst, P, d.partials);
     } else {
         if (c.shape >= 4 && !d.solid) {
             // 128-node rows with staging: 4 the 18 lane-shifted values, 5 (default)
             // all 27, with the per-warp prefetch and evict-first stores and
             // collision loads
-            const cudaError_t e =
-                c.shape == 4 ? launch_staged<S>(k_fused_x<Q, S, 128, 1, 18>, 18, nb, st, g, src, dst, P, d.partials)
+            e = c.shape == 4 ? launch_staged<S>(k_fused_x<Q, S, 128, 1, 18>, 18, nb, st, g, src, dst, P, d.partials)
                              : launch_staged<S>(k_fused_x<Q, S, 128, 1, 27>, 27, nb, st, g, src, dst, P, d.partials);
             return e != cudaSuccess ? e : cudaGetLastError();
         }
@@ -452,7 +467,7 @@ inline cudaError_t fused_step(tlbm_host::DevState& d, const Phys<typename Store<
             go(k_fused<Q, S, 128, 1, false, false>, 128);  // plain loop
         }
     }
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // ---- batches: every member uses the batch's tile; descriptors for both parities
