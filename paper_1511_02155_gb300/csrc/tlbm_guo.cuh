@@ -90,6 +90,43 @@ __device__ __forceinline__ void guo_node(const Phys<T>& P, const T (&X)[3], cons
     mu_psi = mu[2] - (mu[0] + mu[1]) * T(0.5);
 }
 
+// The same from Roll's scaled derivatives (12 grad, 6 lap), in the concentrations:
+// G_ab = sum_m kappa_m d_a C_m d_b C_m and L = sum_m kappa_m C_m lap C_m.
+template <int Q, typename T>
+__device__ __forceinline__ void guo_node12(const Phys<T>& P, const T (&X)[3], const T (&g12)[3][3], const T (&l6)[3],
+                                           T (&pi)[GuoAux<Q>::NPI], T& mu_phi, T& mu_psi) {
+    using A = GuoAux<Q>;
+    const T C[3] = {T(0.5) * ((X[0] - X[2]) + X[1]), T(0.5) * ((X[0] - X[2]) - X[1]), X[2]};
+    const T lC[3] = {T(0.5) * ((l6[0] - l6[2]) + l6[1]), T(0.5) * ((l6[0] - l6[2]) - l6[1]), l6[2]};
+    T mu[3], pL = T(0), G[A::NPI];
+    const T a6 = P.a2 * T(1.0 / 6.0), sc = P.a2 * T(1.0 / 144.0);
+#pragma unroll
+    for (int c = 0; c < A::NPI; ++c) G[c] = T(0);
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+        const T c = C[m], b = fma_(-c, c, c), al = a6 * lC[m];
+        mu[m] = P.kappa[m] * fma_(b, fma_(T(-2), c, T(1)), -al);
+        pL = fma_(P.kappa[m] * c, fma_(T(0.5) * b, fma_(T(-3), c, T(1)), -al), pL);
+        T gc[3];
+#pragma unroll
+        for (int a = 0; a < A::D; ++a) {
+            const T rp = g12[0][a] - g12[2][a];
+            gc[a] = m == 0 ? T(0.5) * (rp + g12[1][a]) : (m == 1 ? T(0.5) * (rp - g12[1][a]) : g12[2][a]);
+        }
+        const T km = sc * P.kappa[m];
+#pragma unroll
+        for (int q = 0; q < A::NPI; ++q) G[q] = fma_(km * gc[A::ca(q)], gc[A::cb(q)], G[q]);
+    }
+    T tr = T(0);
+#pragma unroll
+    for (int a = 0; a < A::D; ++a) tr += G[a];
+    const T iso = fma_(T(-0.5), tr, pL);
+#pragma unroll
+    for (int q = 0; q < A::NPI; ++q) pi[q] = G[q] + (A::ca(q) == A::cb(q) ? iso : T(0));
+    mu_phi = T(0.5) * (mu[0] - mu[1]);
+    mu_psi = fma_(T(-0.5), mu[0] + mu[1], mu[2]);
+}
+
 // Pi and mu_phi, mu_psi of every node from the moment arrays (periodic).
 template <int Q, typename T>
 __global__ void __launch_bounds__(kThreads)
@@ -154,8 +191,11 @@ struct GuoEq {
 // Guo source (f only), stored at node pointer cb.  f, gg, k: the pulled
 // populations as stored (f as deviations where Fmt::OFFSET); rd their summed f
 // (rho - 1 where OFFSET, else rho); j the momentum, F the force (lattice axes);
-// bg, bk = 3 Gamma mu_phi, 3 Gamma mu_psi.
-template <int Q, typename S>
+// bg, bk = 3 Gamma mu_phi, 3 Gamma mu_psi.  STREAM marks the stores evict-first.
+// As in collide_node, omega is folded in and a pair of opposite links shares
+//   EV = omega w (b + 9/2 rho e^2 - 3/2 rho u.u) + s w (9 e e.F - 3 u.F),
+//   OD = w (3 omega rho e + 3 s e.F),  s = 1 - omega / 2, e = e_i.u (g, k: no F).
+template <int Q, typename S, bool STREAM>
 __device__ __forceinline__ void guo_collide_node(unsigned char* cb, const typename Store<S>::T (&f)[Q],
                                                  const typename Store<S>::T (&gg)[Q],
                                                  const typename Store<S>::T (&k)[Q], typename Store<S>::T rd,
@@ -167,59 +207,67 @@ __device__ __forceinline__ void guo_collide_node(unsigned char* cb, const typena
     constexpr bool OF = Fmt<Q, S>::OFFSET;
     const T rho = OF ? T(1) + rd : rd;
     const T inv = T(1) / rho;
-    const T u[3] = {(j[0] + T(0.5) * F[0]) * inv, (j[1] + T(0.5) * F[1]) * inv, (j[2] + T(0.5) * F[2]) * inv};
-    GuoEq<T> E;
-    E.rho = rho; E.phi = phi; E.psi = psi;
-    E.fb = OF ? rd : rho;
-    E.uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    E.bg = bg;
-    E.bk = bk;
-    const T uF = u[0] * F[0] + u[1] * F[1] + u[2] * F[2];
-    const T src_c = T(1) - T(0.5) * P.omega[0];
-    T sf = T(0), sg = T(0), sk = T(0);  // sums of the moving equilibria (deviations)
+    const T u[3] = {mul_(fma_(T(0.5), F[0], j[0]), inv), mul_(fma_(T(0.5), F[1], j[1]), inv),
+                    mul_(fma_(T(0.5), F[2], j[2]), inv)};
+    const T uu = fma_(u[2], u[2], fma_(u[1], u[1], u[0] * u[0]));
+    const T uF = fma_(u[2], F[2], fma_(u[1], F[1], u[0] * F[0]));
+    const T of = P.omega[0], og = P.omega[1], ok = P.omega[2];
+    const T cf = T(1) - of, cg = T(1) - og, ck = T(1) - ok, sc = fma_(T(-0.5), of, T(1));
+    const T huu = T(-1.5) * uu;
+    const T Bf = of * fma_(rho, huu, OF ? rd : rho), Bg = og * fma_(phi, huu, bg), Bk = ok * fma_(psi, huu, bk);
+    const T Rf = of * rho, Rg = og * phi, Rk = ok * psi;
+    const T Of = T(3) * Rf, Og = T(3) * Rg, Ok = T(3) * Rk;
+    const T s3 = T(3) * sc, s9 = T(9) * sc, S0 = T(-3) * sc * uF;
+    T sf = T(0), sg = T(0), sk = T(0);  // half sums of omega x_eq over the moving links (FP64)
     T qf = T(0), qg = T(0), qk = T(0);  // sums of the moving populations as stored
-    // opposite directions in pairs, so that the paired lane words are stored whole
+    auto put = [&](int s, T d) {
+        if (STREAM) Fmt<Q, S>::st_stream_delta(cb, s, 0, d);
+        else Fmt<Q, S>::st_delta(cb, s, 0, d);
+    };
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
         const int o = opp<Q>(i);
         if (o < i) continue;
-        T vf[2], vg[2], vk[2];
+        const T w = T(Lat<Q>::w(i)), rw = T(4.5) * w;
+        T e = T(0), eF = T(0);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int d = h ? o : i;
-            T e = T(0), eF = T(0);
-            if (Lat<Q>::cx(d)) { e += T(Lat<Q>::cx(d)) * u[0]; eF += T(Lat<Q>::cx(d)) * F[0]; }
-            if (Lat<Q>::cy(d)) { e += T(Lat<Q>::cy(d)) * u[1]; eF += T(Lat<Q>::cy(d)) * F[1]; }
-            if (Lat<Q>::cz(d)) { e += T(Lat<Q>::cz(d)) * u[2]; eF += T(Lat<Q>::cz(d)) * F[2]; }
-            const T w = T(Lat<Q>::w(d));
-            T fe, ge, ke;
-            E.eq(w, e, fe, ge, ke);
-            sf += fe; sg += ge; sk += ke;
-            const T Si = src_c * w * (T(3) * (eF - uF) + T(9) * e * eF);
-            vf[h] = f[d] + P.omega[0] * (fe - f[d]) + Si;
-            vg[h] = gg[d] + P.omega[1] * (ge - gg[d]);
-            vk[h] = k[d] + P.omega[2] * (ke - k[d]);
-            if (OF) {
-                qf += Fmt<Q, S>::qdelta_d(d, vf[h]);
-                qg += Fmt<Q, S>::qdelta_d(d, vg[h]);
-                qk += Fmt<Q, S>::qdelta_d(d, vk[h]);
-            }
+        for (int a = 0; a < 3; ++a) {
+            const int c = comp<Q>(i, a);
+            if (c > 0) e += u[a], eF += F[a];
+            if (c < 0) e -= u[a], eF -= F[a];
         }
-        Fmt<Q, S>::template st_fg<false>(cb, i, vf[0], vg[0]);
-        Fmt<Q, S>::template st_fg<false>(cb, o, vf[1], vg[1]);
-        Fmt<Q, S>::template st_kk<false>(cb, i, vk[0], vk[1]);
+        const T e2 = e * e;
+        const T qvf = fma_(rw * Rf, e2, w * Bf);
+        const T evf = fma_(w, fma_(s9 * e, eF, S0), qvf), odf = mul_(w, fma_(Of, e, s3 * eF));
+        const T evg = fma_(rw * Rg, e2, w * Bg), odg = w * Og;
+        const T evk = fma_(rw * Rk, e2, w * Bk), odk = w * Ok;
+        if (!OF) {
+            sf += qvf;
+            sg += evg;
+            sk += evk;
+        }
+        const T v[6] = {fma_(cf, f[i], evf + odf), fma_(cf, f[o], evf - odf),
+                        fma_(cg, gg[i], fma_(odg, e, evg)), fma_(cg, gg[o], fma_(-odg, e, evg)),
+                        fma_(ck, k[i], fma_(odk, e, evk)), fma_(ck, k[o], fma_(-odk, e, evk))};
+        if (OF) {
+            qf += Fmt<Q, S>::qdelta_d(i, v[0]) + Fmt<Q, S>::qdelta_d(o, v[1]);
+            qg += Fmt<Q, S>::qdelta_d(i, v[2]) + Fmt<Q, S>::qdelta_d(o, v[3]);
+            qk += Fmt<Q, S>::qdelta_d(i, v[4]) + Fmt<Q, S>::qdelta_d(o, v[5]);
+        }
+        Fmt<Q, S>::template st_fg<STREAM>(cb, i, v[0], v[2]);
+        Fmt<Q, S>::template st_fg<STREAM>(cb, o, v[1], v[3]);
+        Fmt<Q, S>::template st_kk<STREAM>(cb, i, v[4], v[5]);
     }
     if (OF) {
         // the source sums to zero over i: the rest population is what keeps
         // the node's rho, phi, psi through the storage rounding
-        Fmt<Q, S>::st_delta(cb, 0, 0, rd - qf);
-        Fmt<Q, S>::st_delta(cb, 1, 0, phi - qg);
-        Fmt<Q, S>::st_delta(cb, 2, 0, psi - qk);
+        put(0, rd - qf);
+        put(1, phi - qg);
+        put(2, psi - qk);
     } else {
-        const T S0 = src_c * T(Lat<Q>::w(0)) * (T(-3) * uF);
-        Fmt<Q, S>::st_delta(cb, 0, 0, f[0] + P.omega[0] * ((rho - sf) - f[0]) + S0);
-        Fmt<Q, S>::st_delta(cb, 1, 0, gg[0] + P.omega[1] * ((phi - sg) - gg[0]));
-        Fmt<Q, S>::st_delta(cb, 2, 0, k[0] + P.omega[2] * ((psi - sk) - k[0]));
+        put(0, fma_(T(Lat<Q>::w(0)), S0, fma_(cf, f[0], fma_(T(-2), sf, Rf))));
+        put(1, fma_(cg, gg[0], fma_(T(-2), sg, Rg)));
+        put(2, fma_(ck, k[0], fma_(T(-2), sk, Rk)));
     }
 }
 
@@ -252,7 +300,7 @@ k_guo_collide(Geom g, const S* __restrict__ src, S* __restrict__ dst,
         }
         T F[3];
         guo_force<Q, T>(g, aux, x, y, z, F);
-        guo_collide_node<Q, S>(cb, f, gg, k, rd, j, phi, psi, F, T(3) * P.gamma[0] * aux[A::MU * g.Np + r],
+        guo_collide_node<Q, S, false>(cb, f, gg, k, rd, j, phi, psi, F, T(3) * P.gamma[0] * aux[A::MU * g.Np + r],
                                T(3) * P.gamma[1] * aux[(A::MU + 1) * g.Np + r], P);
     }
 }
@@ -326,18 +374,29 @@ k_guo_velocity(Geom g, const T* __restrict__ mom, const T* __restrict__ aux, dou
 // halo of Pi and works two planes ahead:
 //   M(m+2): moments of plane m+2 over tile + two-node halo   -> moment ring
 //   barrier
-//   P(m+1): Pi of plane m+1 over tile + one-node halo          -> Pi ring
+//   P(m+1): Pi of plane m+1 over tile + one-node halo          -> Pi ring,
+//           mu_phi, mu_psi of the tile                         -> mu ring
 //   barrier
-//   C(m):   mu_phi, mu_psi from the moment ring's Laplacians, F from the Pi
-//           ring, pull, guo_collide_node, store x*(r).
+//   C(m):   F from the Pi ring, pull, guo_collide_node, store x*(r).
 // Ring slots: moments five (a fast warp writes plane m+2 while a slow one still
 // reads planes m-2..m in C(m-1)); Pi three (P(m+1) starts after the barrier
 // that every warp reaches only once its C(m-1), the last reader of plane
-// m-2, is done); momentum four.
+// m-2, is done); momentum and mu four.
+// What it costs is the halo: with 32x4 tiles on D3Q19 the moments of 288 nodes and Pi
+// of 204 for 128 of the tile.  Tiles of 32x8 (432 and 340 for 256), mu kept from P
+// instead of a second set of derivatives in C, and link pairs in the collision:
+// 128^3 FP32 351 us a step before.
+template <int Q, typename S>
+constexpr int guo_smem(int TX, int TY) {
+    const int b = Q == 19 ? 1 : 0, hn = (TX + 4) * (TY + 4 * b), pn = (TX + 2) * (TY + 2 * b);
+    return (int)sizeof(typename Store<S>::T) * (15 * hn + 3 * GuoAux<Q>::NPI * pn + 24 * TX * TY);
+}
+
 template <int Q, typename S, int TX, int TY>
 __device__ __forceinline__ void guo_body(const MGeom& g, const S* __restrict__ src, S* __restrict__ dst,
                                          const Phys<typename Store<S>::T>& P, double* __restrict__ partials,
                                          const int bid) {
+    extern __shared__ __align__(16) unsigned char tlbm_smem[];
     using T = typename Store<S>::T;
     using A = Axes<Q>;
     using GA = GuoAux<Q>;
@@ -357,9 +416,11 @@ __device__ __forceinline__ void guo_body(const MGeom& g, const S* __restrict__ s
     static_assert(D == 3 || TY == 1, "2-D tiles are one row");
     static_assert(KS <= 3 && KP <= 2, "region nodes per thread");
 
-    __shared__ T sm[5][3][HN];    // rho, phi, psi over tile + two-node halo
-    __shared__ T sp[3][NPI][PN];  // Pi over tile + one-node halo
-    __shared__ T sj[4][4][NT];    // j (marching axes) and summed f of the tile
+    // dynamic shared memory (guo_smem)
+    T (*const sm)[3][HN] = reinterpret_cast<T(*)[3][HN]>(tlbm_smem);  // rho, phi, psi over tile + two-node halo
+    T (*const sp)[NPI][PN] = reinterpret_cast<T(*)[NPI][PN]>(tlbm_smem + sizeof(T) * 15 * HN);  // Pi, tile + one node
+    // j (marching axes), summed f, mu_phi, mu_psi of the tile
+    T (*const sj)[6][NT] = reinterpret_cast<T(*)[6][NT]>(tlbm_smem + sizeof(T) * (15 * HN + 3 * NPI * PN));
 
     const int tid = threadIdx.x;
     const int tx = tid % TX, ty = tid / TX;
@@ -425,58 +486,38 @@ __device__ __forceinline__ void guo_body(const MGeom& g, const S* __restrict__ s
         }
     };
 
-    // derivatives (lattice axes) of the three fields at moment-region node h of plane m
-    auto derivs_ring = [&](int m, int h, T (&X0)[3], T (&grad)[3][3], T (&lap)[3]) {
-        const int s0 = modp(m, 5);
-        T gA[3], gB[3], gM[3], lp[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            X0[c] = sm[s0][c][h];
-            gA[c] = gB[c] = gM[c] = lp[c] = T(0);
-        }
-#pragma unroll
-        for (int i = 1; i < Q; ++i) {
-            if (opp<Q>(i) < i) continue;
-            const int sp_ = modp(m + A::cm(i), 5), sn = modp(m - A::cm(i), 5);
-            const int cp = h + A::cb(i) * HW + A::ca(i), cn = h - A::cb(i) * HW - A::ca(i);
-            const T w = T(Lat<Q>::w(i));
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const T xpv = sm[sp_][c][cp], xnv = sm[sn][c][cn];
-                const T d = w * (xpv - xnv);
-                if (A::ca(i)) gA[c] += T(A::ca(i)) * d;
-                if (A::cb(i)) gB[c] += T(A::cb(i)) * d;
-                if (A::cm(i)) gM[c] += T(A::cm(i)) * d;
-                lp[c] += w * (xpv + xnv);
-            }
-        }
-        constexpr T wrest = T(1.0 - Lat<Q>::w(0));
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            lap[c] = T(6) * (lp[c] - wrest * X0[c]);
-            grad[c][0] = T(3) * gA[c];
-            grad[c][1] = T(3) * (D == 3 ? gB[c] : gM[c]);
-            grad[c][2] = D == 3 ? T(3) * gM[c] : T(0);
-        }
-    };
-
-    // P: Pi of plane q over the one-node halo region
+    // P: Pi of plane q over the one-node halo region, mu of the tile
     auto pi_plane = [&](int q) {
-        const int slot = modp(q, 3);
+        const int slot = modp(q, 3), js = modp(q, 4);
+        const int s0 = modp(q - 1, 5), s1 = modp(q, 5), s2 = modp(q + 1, 5);
 #pragma unroll
         for (int k = 0; k < KP; ++k) {
             const int pn = tid + k * NT;
             if (pn >= PN) break;
-            const int h = (pn / PW + HB - PB) * HW + pn % PW + H - 1;  // the same node in the moment region
-            T X[3], grad[3][3], lap[3], pi[NPI], mp, ms;
-            derivs_ring(q, h, X, grad, lap);
-            guo_node<Q, T>(P, X, grad, lap, pi, mp, ms);
+            const int py = pn / PW, px = pn % PW;
+            const int h = (py + HB - PB) * HW + px + H - 1;  // the same node in the moment region
+            T X[3], g12[3][3], l6[3], pi[NPI], mp, ms;
+            Roll<Q, T> roll;
+            roll.clear();
+            auto push = [&](int sl) {
+                const T c1[3] = {sm[sl][0][h], sm[sl][1][h], sm[sl][2][h]};
+                roll.push([&](int c, int i, int jj) -> T { return sm[sl][c][h + jj * HW + i]; }, c1, X, g12, l6);
+            };
+            push(s0);
+            push(s1);
+            push(s2);
+            guo_node12<Q, T>(P, X, g12, l6, pi, mp, ms);
 #pragma unroll
             for (int c = 0; c < NPI; ++c) sp[slot][c][pn] = pi[c];
+            if (px >= 1 && px <= TX && py >= PB && py < PB + TY) {
+                const int t = (py - PB) * TX + px - 1;
+                sj[js][4][t] = mp;
+                sj[js][5][t] = ms;
+            }
         }
     };
 
-    constexpr bool PAIR = Fmt<Q, S>::OFFSET && !(Q == 19 && sizeof(S) == 4);
+    constexpr bool PAIR = Fmt<Q, S>::OFFSET;
     MassSum<T, PAIR> msum;
 
     grid_ready();
@@ -509,10 +550,8 @@ __device__ __forceinline__ void guo_body(const MGeom& g, const S* __restrict__ s
         __syncthreads();
         if (!active) continue;
 
-        // mu_phi, mu_psi from the node's fields and Laplacians
-        T X0[3], grad[3][3], lap[3], pi0[NPI], mu_phi, mu_psi;
-        derivs_ring(m, c0, X0, grad, lap);
-        guo_node<Q, T>(P, X0, grad, lap, pi0, mu_phi, mu_psi);
+        const int s0 = modp(m, 5);
+        const T X0[3] = {sm[s0][0][c0], sm[s0][1][c0], sm[s0][2][c0]};
         // F_a = -3 sum_i w_i sum_b e_ib Pi_ab(r + e_i) (lattice axes)
         T F[3] = {T(0), T(0), T(0)};
 #pragma unroll
@@ -537,7 +576,9 @@ __device__ __forceinline__ void guo_body(const MGeom& g, const S* __restrict__ s
         if constexpr (PAIR) msum.add(rdc, X0[1], X0[2]);
         else msum.add(rho_total<Q, S>(rdc), X0[1], X0[2]);
 
-        // pulled populations of the node at plane m (deviations where OFFSET)
+        // pulled populations of the node at plane m (deviations where OFFSET), their
+        // last use: evict-first for FP32, as in the solid-aware kernel
+        constexpr bool HL = sizeof(S) == 4;
         const int zr[3] = {wrap1(m - 1, g.NM), m, wrap1(m + 1, g.NM)};
         T fv[Q], gv[Q], kv[Q];
 #pragma unroll
@@ -545,17 +586,17 @@ __device__ __forceinline__ void guo_body(const MGeom& g, const S* __restrict__ s
             const unsigned char* p =
                 srcb + ((long long)zr[1 - A::cm(i)] * g.NB + yo[1 - A::cb(i)]) * g.rowstride + xo[1 - A::ca(i)];
             if (Fmt<Q, S>::PAIRED && i > 0) {
-                Fmt<Q, S>::ld_fg(p, i, fv[i], gv[i]);
+                Fmt<Q, S>::template ld_fg<HL>(p, i, fv[i], gv[i]);
             } else {
-                fv[i] = Fmt<Q, S>::ld_delta(p, 0, i);
-                gv[i] = Fmt<Q, S>::ld_delta(p, 1, i);
+                fv[i] = HL ? Fmt<Q, S>::ld_last_delta(p, 0, i) : Fmt<Q, S>::ld_delta(p, 0, i);
+                gv[i] = HL ? Fmt<Q, S>::ld_last_delta(p, 1, i) : Fmt<Q, S>::ld_delta(p, 1, i);
             }
-            kv[i] = Fmt<Q, S>::ld_delta(p, 2, i);
+            kv[i] = HL ? Fmt<Q, S>::ld_last_delta(p, 2, i) : Fmt<Q, S>::ld_delta(p, 2, i);
         }
         unsigned char* out =
             reinterpret_cast<unsigned char*>(dst) + ((long long)m * g.NB + yo[1]) * g.rowstride + xo[1];
-        guo_collide_node<Q, S>(out, fv, gv, kv, rdc, jl, X0[1], X0[2], F, T(3) * P.gamma[0] * mu_phi,
-                               T(3) * P.gamma[1] * mu_psi, P);
+        guo_collide_node<Q, S, HL>(out, fv, gv, kv, rdc, jl, X0[1], X0[2], F, T(3) * P.gamma[0] * sj[js][4][t],
+                                   T(3) * P.gamma[1] * sj[js][5][t], P);
     }
     double mr, mp, ms;
     msum.get(mr, mp, ms);
@@ -581,10 +622,11 @@ inline cudaError_t guo_fused_step(tlbm_host::DevState& d, const Phys<typename St
     S* dst = static_cast<S*>(d.pop[1 - d.cur]);
     cudaError_t e;
     if constexpr (Q == 19) {
-        constexpr int TX = sizeof(S) == 8 ? 16 : 32;
-        e = launch_step(k_guo_fused<Q, S, TX, 4>, 0, TX * 4, nb, st, g, src, dst, P, d.partials);
+        constexpr int TX = sizeof(S) == 8 ? 16 : 32, TY = sizeof(S) == 8 ? 4 : 8;
+        e = launch_smem(k_guo_fused<Q, S, TX, TY>, guo_smem<Q, S>(TX, TY), TX * TY, 512 / (TX * TY), nb, st, g, src, dst, P,
+                        d.partials);
     } else {
-        e = launch_step(k_guo_fused<Q, S, 128, 1>, 0, 128, nb, st, g, src, dst, P, d.partials);
+        e = launch_smem(k_guo_fused<Q, S, 128, 1>, guo_smem<Q, S>(128, 1), 128, 4, nb, st, g, src, dst, P, d.partials);
     }
     return e != cudaSuccess ? e : cudaGetLastError();
 }
