@@ -250,7 +250,8 @@ k_adj_seed(Geom g, const S* __restrict__ x, const uint8_t* __restrict__ solid, c
 // read at the node itself (x' of r is stored at r).  INIT: fields from mom,
 // j = 0, omega = 1, lambda pulled (eq of r was pushed to the pull slots).
 // Outputs node arrays dX[3][Np], dJ[3][Np], dG[9][Np] (dG[3X+a]), dLap[3][Np];
-// kappa partials per block (fixed grid).
+// adds to the kappa partials of its block (fixed grid), which are reduced once at
+// the end of the run.
 template <int Q, typename S, bool SOLID, bool INIT>
 __global__ void __launch_bounds__(kThreads)
 k_adj_node(Geom g, const S* __restrict__ x, const uint8_t* __restrict__ solid,
@@ -328,16 +329,16 @@ k_adj_node(Geom g, const S* __restrict__ x, const uint8_t* __restrict__ solid,
     }
     block_sum3(k0, k1, k2);
     if (threadIdx.x == 0) {
-        partials[3 * blockIdx.x + 0] = k0;
-        partials[3 * blockIdx.x + 1] = k1;
-        partials[3 * blockIdx.x + 2] = k2;
+        partials[3 * blockIdx.x + 0] += k0;
+        partials[3 * blockIdx.x + 1] += k1;
+        partials[3 * blockIdx.x + 2] += k2;
     }
 }
 
 // Transpose of the derivative stencils, at every node (in place on dX):
 // dX(r) += sum_i [3 w_i e_i . dG(r - e_i) + 6 w_i dLap(r - e_i)] - 6 (1 - w_0) dLap(r).
 // On solid nodes the total is the ghost's adjoint; its share of dL/dG_X
-// (-1, or -sqrt 2 for diagonal-only ghosts) goes to per-block partials.
+// (-1, or -sqrt 2 for diagonal-only ghosts) is added to per-block partials.
 template <int Q, typename T, bool SOLID>
 __global__ void __launch_bounds__(kThreads)
 k_adj_gather(Geom g, const uint8_t* __restrict__ solid, T* __restrict__ dX, const T* __restrict__ dG,
@@ -378,9 +379,9 @@ k_adj_gather(Geom g, const uint8_t* __restrict__ solid, T* __restrict__ dX, cons
     }
     block_sum3(p0, p1, p2);
     if (threadIdx.x == 0) {
-        partials[3 * blockIdx.x + 0] = p0;
-        partials[3 * blockIdx.x + 1] = p1;
-        partials[3 * blockIdx.x + 2] = p2;
+        partials[3 * blockIdx.x + 0] += p0;
+        partials[3 * blockIdx.x + 1] += p1;
+        partials[3 * blockIdx.x + 2] += p2;
     }
 }
 

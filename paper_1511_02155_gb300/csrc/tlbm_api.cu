@@ -84,8 +84,12 @@ void mark_units(tlbm* t, const uint8_t* mask) {
             bool any = (w[0] | w[1] | w[2] | w[3]) != 0;
             int n = 0;
             for (int x = x0; any && x < x1; ++x) n += m[x] != 0;
-            for (int k = 1; k <= 2 && !any; ++k)
-                any = m[(((x0 - k) % d.nx) + d.nx) % d.nx] != 0 || m[(x1 - 1 + k) % d.nx] != 0;
+            if (!any) {
+                if (x0 >= 2 && x1 + 2 <= d.nx) any = (m[x0 - 2] | m[x0 - 1] | m[x1] | m[x1 + 1]) != 0;
+                else
+                    for (int k = 1; k <= 2; ++k)
+                        any = any || m[(((x0 - k) % d.nx) + d.nx) % d.nx] != 0 || m[(x1 - 1 + k) % d.nx] != 0;
+            }
             u[c] = (uint8_t)((any ? 1 : 0) | (n == x1 - x0 ? 2 : 0));
         }
     }
@@ -628,7 +632,7 @@ tlbm_status tlbm_adjoint_c3_misfit(tlbm* t, int64_t nsteps, int checkpoint_every
     J.state_bytes = sb;
     void* blocks[9] = {};
     const size_t sizes[9] = {sb * (size_t)nseg, sb * (size_t)K, sb, sb, sb, sizeof(double) * 18 * Np,
-                             sizeof(double) * 3 * (size_t)nblk, sizeof(double) * 8, sizeof(double) * 4 * N};
+                             sizeof(double) * 9 * (size_t)nblk, sizeof(double) * 8, sizeof(double) * 4 * N};
     cudaError_t e = cudaSuccess;
     for (int k = 0; k < 9 && e == cudaSuccess; ++k) e = cudaMalloc(&blocks[k], sizes[k]);
     auto release = [&]() {

@@ -89,7 +89,7 @@ struct AdjJob {
     void* fin;            // x(nsteps), restored at the end
     void* lam[2];         // adjoint states (population layout)
     double* work;         // dX[3], dJ[3], dG[9], dLap[3] node arrays (18 Np values of the compute type)
-    double* partials;     // 3 doubles per block of the fixed grid
+    double* partials;     // 9 doubles per block of the fixed grid
     double* acc;          // [0] loss, [1..3] dL/dkappa (local part), [4..6] dL/dG_X
     double* dfields;      // [3][N] dL/d(rho, phi, psi) of the initial fields
 };

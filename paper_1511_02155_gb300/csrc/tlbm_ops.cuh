@@ -185,6 +185,13 @@ struct Impl {
         auto chk = [&](cudaError_t r) {
             if (e == cudaSuccess && r != cudaSuccess) e = r;
         };
+        // kappa and G_X sums per block, over all steps; one reduction at the end (two
+        // one-block reductions a step were 16 of 234 us on 256x128 in FP64)
+        double *node_sums = J.partials + 3 * kMassBlocks, *gather_sums = J.partials + 6 * kMassBlocks;
+        // blocks of one warp spread a small lattice over all SMs, whose two FP64 lanes
+        // bound these kernels (256x128: 7 warps on the fullest SM instead of 8); the
+        // fixed grid keeps the order of the sums a function of the lattice alone
+        const int adj_threads = g.N <= 2LL * 32 * kMassBlocks ? 32 : kThreads;
         // moments (with wetting ghosts) of state x into mom
         auto moments_of = [&](const S* x) {
             k_moments<Q, S, SOLID, true><<<kMassBlocks, kThreads, 0, st>>>(g, x, d.solid, mom, d.partials);
@@ -194,15 +201,14 @@ struct Impl {
         auto adjoint_core = [&](const S* x, const S* lam, auto init_tag) {
             constexpr bool INIT = decltype(init_tag)::value;
             moments_of(x);
-            k_adj_node<Q, S, SOLID, INIT><<<kMassBlocks, kThreads, 0, st>>>(g, x, d.solid, mom, lam, P, dX, dJ,
-                                                                             dG, dL, J.partials);
-            k_adj_acc<<<1, kThreads, 0, st>>>(J.partials, kMassBlocks, 3, J.acc + 1);
-            k_adj_gather<Q, T, SOLID><<<kMassBlocks, kThreads, 0, st>>>(g, d.solid, dX, dG, dL, J.partials);
-            k_adj_acc<<<1, kThreads, 0, st>>>(J.partials, kMassBlocks, 3, J.acc + 4);
+            k_adj_node<Q, S, SOLID, INIT><<<kMassBlocks, adj_threads, 0, st>>>(g, x, d.solid, mom, lam, P, dX, dJ,
+                                                                                dG, dL, node_sums);
+            k_adj_gather<Q, T, SOLID><<<kMassBlocks, adj_threads, 0, st>>>(g, d.solid, dX, dG, dL, gather_sums);
         };
         const long long T = J.nsteps;
         const int K = J.K;
         const long long nseg = (T + K - 1) / K;
+        chk(cudaMemsetAsync(node_sums, 0, sizeof(double) * 6 * kMassBlocks, st));
         // forward, checkpoints at multiples of K
         chk(cp(state(J.ckpt, 0), d.pop[d.cur]));
         for (long long t = 1; t <= T && e == cudaSuccess; ++t) {
@@ -241,6 +247,8 @@ struct Impl {
         const S* x0 = reinterpret_cast<const S*>(state(J.ckpt, 0));
         adjoint_core(x0, static_cast<const S*>(J.lam[li]), std::true_type{});
         k_adj_pull<Q, S, SOLID, true><<<grid, kThreads, 0, st>>>(g, d.solid, dX, dJ, nullptr, P, nullptr, J.dfields);
+        k_adj_acc<<<1, kThreads, 0, st>>>(node_sums, kMassBlocks, 3, J.acc + 1);
+        k_adj_acc<<<1, kThreads, 0, st>>>(gather_sums, kMassBlocks, 3, J.acc + 4);
         // leave the engine at x(T)
         d.cur = curT;
         chk(cp(d.pop[d.cur], J.fin));
