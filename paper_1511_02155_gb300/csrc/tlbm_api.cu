@@ -25,6 +25,7 @@ struct tlbm {
     double kappa[3], alpha, tau_f, M_phi, M_psi, gamma[2], h[3];
     size_t esize;          // bytes per stored population
     size_t tsize;          // bytes per compute value
+    void* block;           // the one device allocation of tlbm_create (DevState points into it)
     double* staging;       // device doubles for init/fields (8 N), allocated on demand
     size_t partials_len;   // doubles in d.partials
     cudaEvent_t ev[2];     // kernel timing events (timing mode)
@@ -204,18 +205,10 @@ void tlbm_destroy(tlbm* t) {
     cudaSetDevice(t->device);
     if (t->st) cudaStreamSynchronize(t->st);
     else cudaDeviceSynchronize();
-    cudaFree(t->d.pop[0]);
-    cudaFree(t->d.pop[1]);
-    cudaFree((void*)t->d.solid);
-    cudaFree(t->d.nbm);
+    cudaFree(t->block);  // populations, masks, reductions
     cudaFree(const_cast<void*>(t->d.items));
     cudaFree(t->d.mom);
     cudaFree(t->d.aux);
-    cudaFree(t->d.partials);
-    cudaFree(t->d.step_mass);
-    cudaFree(t->d.mass_tmp);
-    cudaFree(t->d.flag);
-    cudaFree(t->d.check);
     cudaFree(t->staging);
     if (t->ev[0]) cudaEventDestroy(t->ev[0]);
     if (t->ev[1]) cudaEventDestroy(t->ev[1]);
@@ -272,6 +265,7 @@ tlbm_status tlbm_create(tlbm** out, tlbm_lattice lattice, int nx, int ny, int nz
     t->gamma[0] = t->gamma[1] = 1.0;
     t->esize = esize; t->tsize = tsize;
     t->staging = nullptr;
+    t->block = nullptr;
     t->ev[0] = t->ev[1] = nullptr;
     t->timing = 0;
     t->kernel_ms = 0.0;
@@ -302,29 +296,9 @@ tlbm_status tlbm_create(tlbm** out, tlbm_lattice lattice, int nx, int ny, int nz
         return s;
     };
     const size_t popbytes = (size_t)d.pop_bytes;
-    for (int b = 0; b < 2; ++b) {
-        cudaError_t e = cudaMalloc(&d.pop[b], popbytes);
-        if (e != cudaSuccess)
-            return bail(fail(t, TLBM_ERR_OOM, "cudaMalloc(%zu bytes) for populations: %s", popbytes,
-                             cudaGetErrorString(e)));
-        e = cudaMemsetAsync(d.pop[b], 0, popbytes, t->st);
-        if (e != cudaSuccess) return bail(fail(t, TLBM_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e)));
-    }
     bool any_solid = false;
     if (solid_mask)
         for (long long r = 0; r < N && !any_solid; ++r) any_solid = solid_mask[r] != 0;
-    if (any_solid) {
-        uint8_t* ds = nullptr;
-        cudaError_t e = cudaMalloc(&ds, (size_t)N);
-        if (e != cudaSuccess) return bail(fail(t, TLBM_ERR_OOM, "cudaMalloc(mask): %s", cudaGetErrorString(e)));
-        d.solid = ds;
-        e = cudaMemcpy(ds, solid_mask, (size_t)N, cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) return bail(fail(t, TLBM_ERR_CUDA, "cudaMemcpy(mask): %s", cudaGetErrorString(e)));
-        // neighbour-solid bits of the fused step, built by its first launch
-        e = cudaMalloc(&d.nbm, sizeof(uint32_t) * (size_t)N);
-        if (e != cudaSuccess) return bail(fail(t, TLBM_ERR_OOM, "cudaMalloc(neighbour mask): %s", cudaGetErrorString(e)));
-        d.nbm_ready = 0;
-    }
     // mass partials: step partials (up to one per fused block) + tlbm_mass partials
     long long nblk = 0;
     {
@@ -334,18 +308,48 @@ tlbm_status tlbm_create(tlbm** out, tlbm_lattice lattice, int nx, int ny, int nz
     }
     t->partials_len = 3 * (size_t)(nblk + tlbm_host::mass_blocks());
     d.partials_cap = nblk;
-    if (any_solid) mark_units(t, solid_mask);
-    cudaError_t e = set_items(t);
-    if (e == cudaSuccess) e = cudaMalloc(&d.partials, sizeof(double) * t->partials_len);
-    if (e == cudaSuccess) e = cudaMalloc(&d.step_mass, sizeof(double) * 3);
-    if (e == cudaSuccess) e = cudaMalloc(&d.mass_tmp, sizeof(double) * 3);
-    if (e == cudaSuccess) e = cudaMalloc(&d.flag, sizeof(int));
-    if (e == cudaSuccess) e = cudaMalloc(&d.check, sizeof(unsigned long long));
-    if (e != cudaSuccess) return bail(fail(t, TLBM_ERR_OOM, "cudaMalloc(reductions): %s", cudaGetErrorString(e)));
+    // one allocation for everything whose size is known here: an engine that lives
+    // for one gradient (inverse.c3_misfit) pays for each cudaMalloc and cudaFree
+    size_t at = 0;
+    auto part = [&](size_t bytes) {
+        const size_t p = at;
+        at += (bytes + 511) / 512 * 512;
+        return p;
+    };
+    const size_t p0 = part(popbytes), p1 = part(popbytes), ps = any_solid ? part((size_t)N) : 0,
+                 pn = any_solid ? part(sizeof(uint32_t) * (size_t)N) : 0, pp = part(sizeof(double) * t->partials_len),
+                 pr = part(sizeof(double) * 8);
+    cudaError_t e = cudaMalloc(&t->block, at);
+    if (e != cudaSuccess)
+        return bail(fail(t, TLBM_ERR_OOM, "cudaMalloc(%zu bytes, populations %zu): %s", at, 2 * popbytes,
+                         cudaGetErrorString(e)));
+    char* const base = static_cast<char*>(t->block);
+    d.pop[0] = base + p0;
+    d.pop[1] = base + p1;
+    d.partials = reinterpret_cast<double*>(base + pp);
+    d.step_mass = reinterpret_cast<double*>(base + pr);  // 3 doubles, 3 of mass_tmp, the check word, the flag
+    d.mass_tmp = d.step_mass + 3;
+    d.check = reinterpret_cast<unsigned long long*>(d.step_mass + 6);
+    d.flag = reinterpret_cast<int*>(d.step_mass + 7);
+    for (int b = 0; b < 2; ++b) {
+        e = cudaMemsetAsync(d.pop[b], 0, popbytes, t->st);
+        if (e != cudaSuccess) return bail(fail(t, TLBM_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e)));
+    }
+    if (any_solid) {
+        d.solid = reinterpret_cast<uint8_t*>(base + ps);
+        // neighbour-solid bits of the fused step, built by its first launch
+        d.nbm = reinterpret_cast<uint32_t*>(base + pn);
+        d.nbm_ready = 0;
+        e = cudaMemcpy(base + ps, solid_mask, (size_t)N, cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) return bail(fail(t, TLBM_ERR_CUDA, "cudaMemcpy(mask): %s", cudaGetErrorString(e)));
+        mark_units(t, solid_mask);
+        e = set_items(t);
+        if (e != cudaSuccess) return bail(fail(t, e == cudaErrorMemoryAllocation ? TLBM_ERR_OOM : TLBM_ERR_CUDA,
+                                               "work items: %s", cudaGetErrorString(e)));
+    }
     const double nan3[3] = {NAN, NAN, NAN};
     e = cudaMemcpy(d.step_mass, nan3, sizeof nan3, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(d.flag, 0, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(d.check, 0, sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaMemset(d.check, 0, 2 * sizeof(unsigned long long));  // and the flag
     if (e == cudaSuccess) e = cudaStreamSynchronize(t->st);
     if (e != cudaSuccess) return bail(fail(t, TLBM_ERR_CUDA, "initialisation: %s", cudaGetErrorString(e)));
     *out = t;
@@ -630,28 +634,31 @@ tlbm_status tlbm_adjoint_c3_misfit(tlbm* t, int64_t nsteps, int checkpoint_every
     J.nsteps = T;
     J.K = K;
     J.state_bytes = sb;
-    void* blocks[9] = {};
     const size_t sizes[9] = {sb * (size_t)nseg, sb * (size_t)K, sb, sb, sb, sizeof(double) * 18 * Np,
                              sizeof(double) * 9 * (size_t)nblk, sizeof(double) * 8, sizeof(double) * 4 * N};
-    cudaError_t e = cudaSuccess;
-    for (int k = 0; k < 9 && e == cudaSuccess; ++k) e = cudaMalloc(&blocks[k], sizes[k]);
-    auto release = [&]() {
-        for (void* b : blocks) cudaFree(b);
-    };
+    size_t at[9], total = 0;
+    for (int k = 0; k < 9; ++k) {
+        at[k] = total;
+        total += (sizes[k] + 511) / 512 * 512;
+    }
+    void* block = nullptr;  // one allocation for the run
+    cudaError_t e = cudaMalloc(&block, total);
+    auto release = [&]() { cudaFree(block); };
     if (e != cudaSuccess) {
         release();
         return fail(t, TLBM_ERR_OOM, "adjoint buffers (%zu MB of checkpoints and segment states): %s",
                     (sizes[0] + sizes[1]) >> 20, cudaGetErrorString(e));
     }
-    J.ckpt = blocks[0];
-    J.seg = blocks[1];
-    J.fin = blocks[2];
-    J.lam[0] = blocks[3];
-    J.lam[1] = blocks[4];
-    J.work = static_cast<double*>(blocks[5]);
-    J.partials = static_cast<double*>(blocks[6]);
-    J.acc = static_cast<double*>(blocks[7]);
-    double* tgt = static_cast<double*>(blocks[8]);
+    char* const base = static_cast<char*>(block);
+    J.ckpt = base + at[0];
+    J.seg = base + at[1];
+    J.fin = base + at[2];
+    J.lam[0] = base + at[3];
+    J.lam[1] = base + at[4];
+    J.work = reinterpret_cast<double*>(base + at[5]);
+    J.partials = reinterpret_cast<double*>(base + at[6]);
+    J.acc = reinterpret_cast<double*>(base + at[7]);
+    double* tgt = reinterpret_cast<double*>(base + at[8]);
     J.target = tgt;
     J.dfields = tgt + N;
     double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};

@@ -1,0 +1,174 @@
+"""GPU parity of the marching kernels at the edges of their tiles and rules.
+
+Every case takes one step from populations that the engine itself holds (rounded
+to its storage) and compares with the FP64 oracle's step from the same numbers.
+Bounds, per population:
+- FP64 storage: 1e-13 (a few hundred operations on values below 1);
+- FP32 storage: 2e-6, the rounding of one step used by the full-size tests;
+- 16-bit storage: 2e-6 plus half a unit in the last place of the stored value,
+  |x| 2^-11 (FP16) or |x| 2^-8 (BF16), at the largest moving deviation.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import paper_1511_02155_gb300 as tl
+from paper_1511_02155_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover - CPU-only machines
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+KAPPA = (0.012, 0.02, 0.016)
+H = (0.0005, -0.0004, 0.0003)
+HALF_ULP = {"fp16": 2.0 ** -11, "bf16": 2.0 ** -8}
+
+
+def _weights(Q):
+    if Q == 9:
+        return np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4)
+    return np.array([1 / 3] + [1 / 18] * 6 + [1 / 36] * 12)
+
+
+def _one_step(Q, shape, precision, solid=None, tile=(0, 0), forcing=False, steps=1):
+    """Largest error of `steps` steps against the oracle, and the bound for one."""
+    nx, ny, nz = shape
+    sh = (ny, nx) if Q == 9 else (nz, ny, nx)
+    C = W.spinodal(sh, seed=nx + ny + nz, amp=0.2)
+    fields = W.to_aux(*C)
+    if solid is not None:
+        for a in fields:
+            a[solid != 0] = 0.0
+    h = H if solid is not None else (0.0, 0.0, 0.0)
+    eng = tl.TernaryLB(Q, nx, ny, nz, KAPPA, 1.0, 0.8, 0.1, 0.1, h, None if solid is None else solid.reshape(-1), precision)
+    if forcing:
+        eng.set_coupling("forcing")
+    eng.set_tile(*tile)
+    rng = np.random.default_rng(5)
+    u = [rng.uniform(-0.02, 0.02, sh) for _ in range(3)]
+    if Q == 9:
+        u[2][:] = 0.0
+    eng.init_fields(*fields, u=u)
+    eng.step(2)  # away from equilibrium
+    P = eng.get_populations()
+    p = oracle.make_params(Q, nx, ny, nz, KAPPA, 1.0, 0.8, 0.1, 0.1, h)
+    f, g, k = (np.ascontiguousarray(P[s]) for s in range(3))
+    before = eng.mass()
+    eng.step(steps)
+    if forcing:
+        oracle.step_guo(p, f, g, k, steps)
+    else:
+        oracle.step(p, f, g, k, steps, *(() if solid is None else (solid.reshape(-1),)))
+    got = eng.get_populations()
+    want = np.stack([a.reshape(Q, -1) for a in (f, g, k)])
+    if solid is not None:
+        got, want = got[:, :, solid.reshape(-1) == 0], want[:, :, solid.reshape(-1) == 0]
+    err = np.abs(got - want).max()
+    if steps == 1:
+        assert np.allclose(eng.step_mass(), before, rtol=0, atol=1e-9 * max(1.0, np.prod(sh)))
+    eng.close()
+    bound = {"fp64": 1e-13, "fp32": 2e-6}.get(precision, 2e-6)
+    if precision in HALF_ULP:
+        moving = want[:, 1:].copy()
+        moving[0] -= _weights(Q)[1:, None]
+        bound += HALF_ULP[precision] * np.abs(moving).max()
+        # the rest population closes the node's moment over Q - 1 rounded values
+        bound *= Q - 1
+    return err, bound
+
+
+# D3Q19 chunks of 32 nodes: one partial, one whole, a tail of one, of two, an odd
+# tail; rows fewer than, equal to and one more than a tile; one plane
+@pytest.mark.parametrize("precision", ["fp32", "fp16", "bf16"])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (2, 3, 2), (31, 4, 3), (32, 5, 1), (33, 8, 4), (34, 9, 5), (65, 2, 7),
+                                   (96, 13, 6)])
+def test_periodic_d3q19_at_tile_edges(shape, precision):
+    err, bound = _one_step(19, shape, precision)
+    assert err <= bound, (err, bound)
+
+
+@pytest.mark.parametrize("chunk", [1, 3, 7])
+def test_periodic_d3q19_chunks(chunk):
+    err, bound = _one_step(19, (40, 7, 11), "fp32", tile=(0, chunk))
+    assert err <= bound, (err, bound)
+
+
+# rows narrower and wider than one-warp rows and than 128, few and many planes
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp16"])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (31, 5, 1), (32, 64, 1), (33, 9, 1), (129, 40, 1)])
+def test_periodic_d2q9_small_lattices(shape, precision):
+    err, bound = _one_step(9, shape, precision)
+    assert err <= bound, (err, bound)
+
+
+def _mask(Q, shape, kind):
+    """Solid nodes that leave clean, dirty and all-solid blocks in many places."""
+    nx, ny, nz = shape
+    s = np.zeros((ny, nx) if Q == 9 else (nz, ny, nx), np.uint8)
+    up = s  # march axis first
+    if kind == "walls":
+        up[:2] = 1
+        up[-1] = 1
+    elif kind == "block":
+        up[:9] = 1
+        up[4:9, ..., nx // 4:nx // 2] = 0
+        up[-1] = 1
+    elif kind == "speck":  # one node at a tile's corner, and one at the periodic edge
+        up[s.shape[0] // 2, ..., 31] = 1
+        up[0, ..., 0] = 1
+    elif kind == "porous":
+        up[np.random.default_rng(3).random(s.shape) < 0.03] = 1
+    return s
+
+
+@pytest.mark.parametrize("precision,tile", [("fp32", (0, 0)), ("fp32", (2, 5)), ("fp32", (3, 16)), ("fp16", (0, 0)),
+                                            ("fp64", (0, 0))])
+@pytest.mark.parametrize("kind", ["walls", "block", "speck", "porous"])
+@pytest.mark.parametrize("shape", [(40, 30, 1), (161, 90, 1), (300, 48, 1)])
+def test_solid_d2q9_clean_and_dirty_blocks(shape, kind, precision, tile):
+    err, bound = _one_step(9, shape, precision, _mask(9, shape, kind), tile)
+    assert err <= bound, (err, bound)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "bf16"])
+@pytest.mark.parametrize("kind", ["walls", "speck"])
+def test_solid_d3q19_with_a_launch_for_clean_blocks(kind, precision):
+    shape = (98, 165, 40)  # columns enough for clean blocks to fill the device
+    solid = _mask(19, shape, kind)
+    err, bound = _one_step(19, shape, precision, solid)
+    assert err <= bound, (err, bound)
+    eng = tl.TernaryLB(19, *shape, KAPPA, solid=solid.reshape(-1), precision=precision)
+    assert eng.launches_per_step == 3
+    eng.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("Q,shape", [(19, (33, 9, 5)), (19, (31, 7, 2)), (19, (2, 1, 1)), (9, (129, 6, 1)), (9, (5, 3, 1))])
+def test_forcing_at_tile_edges(Q, shape, precision):
+    err, bound = _one_step(Q, shape, precision, forcing=True)
+    assert err <= bound, (err, bound)
+
+
+def test_many_steps_in_one_call_equal_single_steps():
+    """Steps overlap their launches; a call of n steps gives the bits of n calls."""
+    for Q, shape, solid in ((9, (70, 50, 1), None), (9, (70, 50, 1), "walls"), (19, (40, 9, 8), None)):
+        s = None if solid is None else _mask(Q, shape, solid)
+        states = []
+        for split in (False, True):
+            eng = tl.TernaryLB(Q, *shape, KAPPA, h=H if s is not None else (0, 0, 0),
+                               solid=None if s is None else s.reshape(-1), precision="fp32")
+            C = W.spinodal((shape[1], shape[0]) if Q == 9 else shape[::-1], seed=4, amp=0.1)
+            f = W.to_aux(*C)
+            if s is not None:
+                for a in f:
+                    a[s != 0] = 0.0
+            eng.init_fields(*f)
+            for _ in range(9 if split else 1):
+                eng.step(1 if split else 9)
+                if split:
+                    eng.step_mass()
+            states.append((eng.get_populations(), eng.step_mass()))
+            eng.close()
+        assert np.array_equal(states[0][0], states[1][0]) and np.array_equal(states[0][1], states[1][1])
