@@ -24,19 +24,23 @@ inline int grid_of(long long n, int sms) {
 // SM (res fit) takes 0.25 + 0.19 b' times a full SM's plane, b' = 4 b / res: alone
 // a block waits out the latency of its loads, together they fill each other's
 // waits.  Blocks beyond what fits wait for whole rounds; over many rounds the
-// blocks drift apart and only the sum counts.  FP64 is bound by its few FP64
-// units: there every node's operations count, about 400 for a collision and 72
-// for the moments of a (node, halo) pair, and two blocks hide each other.
+// blocks drift apart and only the sum counts.  FP64 is bound by its few FP64 units
+// once some five warps share an SM (2.8 us for a warp's collision, 0.75 for its
+// moments with the halo), and below that by the latency of a warp's own chain (3.5
+// us for either): 64x64 takes one plane a block, walled 256x128 two (seven, the
+// choice by operations alone, left 1.7 warps on an SM).
 // Against the measured times of 14 lattices (64^2 .. 1000x701, 40^3 .. 160^2x96)
 // over chunks of 1 .. 64 planes the cheapest chunk of this model is within 8 % of
 // the fastest measured; halving 64 or 16 until 4 blocks per SM are reached, the
 // earlier rule, lost up to 27 % (FP32, one step: 64x64 15.4 us against 11.3,
 // 96^3 117.4 against 102.9, walled 144x128x80 299 against 267).
-inline double march_cost(double nb, int mc, int halo, int res, int sms, bool dbl) {
+inline double march_cost(double nb, int mc, int halo, int res, int threads, int sms, bool dbl) {
     const double full = (double)res * sms;
     if (dbl) {
         const double per = nb / sms, b = per > 8.0 ? per : (double)(long long)(per + 0.9999);
-        return (mc * 400.0 + (mc + halo) * 72.0) * (b < 2.0 ? 1.3 : b);
+        const double warps = threads / 32.0;
+        const double chain = 3.5 * (2 * mc + halo), units = b * warps * (2.8 * mc + 0.75 * (mc + halo));
+        return chain > units ? chain : units;
     }
     auto plane = [&](double b) { return 0.25 + 0.19 * 4.0 * b / res; };
     const double rounds = nb / full;
@@ -65,8 +69,8 @@ inline int dirty_chunk(int mc) { return mc <= 4 ? mc : (mc / 2 - 2 > 4 ? mc / 2 
 // 2-D; in 3-D 16 once the grid fills the device eight times over (256^3 FP32: 16
 // planes 0.692 of HBM, 24..128 planes 0.66..0.69: blocks that start together share
 // their halo rows in L2).
-inline int pick_chunk(const std::vector<Run>& runs, const std::vector<long long>& caps, int halo, int res, int sms,
-                      bool three_d, bool dbl) {
+inline int pick_chunk(const std::vector<Run>& runs, const std::vector<long long>& caps, int halo, int res, int threads,
+                      int sms, bool three_d, bool dbl) {
     double best = 0.0;
     int bmc = 0;
     std::vector<long long> nbs(caps.size());
@@ -85,7 +89,7 @@ inline int pick_chunk(const std::vector<Run>& runs, const std::vector<long long>
         if (used == 0) used = mc;
         for (size_t k = 0; k < caps.size(); ++k) fits = fits && nbs[k] <= caps[k];
         if (!fits) continue;
-        const double c = march_cost(nb, used, halo, res, sms, dbl);
+        const double c = march_cost(nb, used, halo, res, threads, sms, dbl);
         if (three_d && used > 16 && nb >= 8.0 * res * sms) continue;
         if (bmc == 0 || c < best) {
             best = c;
@@ -158,7 +162,7 @@ inline FusedCfg<Q> fused_cfg(const tlbm_host::DevState& d) {
     const int NM = (Q == 19) ? d.nz : d.ny;
     if (mc <= 0) {
         const long long cols = (long long)((NA + c.TX - 1) / c.TX) * ((NB + c.TY - 1) / c.TY);
-        mc = pick_chunk({Run{cols, NM, 0, false}}, {d.partials_cap}, c.halo(d), c.res(d), d.sms, Q == 19, dbl);
+        mc = pick_chunk({Run{cols, NM, 0, false}}, {d.partials_cap}, c.halo(d), c.res(d), c.TX * c.TY, d.sms, Q == 19, dbl);
     }
     c.MC = mc < 1 ? 1 : (mc > NM ? NM : mc);
     return c;
@@ -273,7 +277,7 @@ inline int solid_items(const tlbm_host::DevState& d, std::vector<int4>& out) {
     if (mc == 0) {
         std::vector<Run> all;
         add_runs(runs, 0, all);
-        mc = pick_chunk(all, {d.partials_cap}, runs_halo(runs), c.res(d), d.sms, Q == 19, d.prec == 0);
+        mc = pick_chunk(all, {d.partials_cap}, runs_halo(runs), c.res(d), c.TX * c.TY, d.sms, Q == 19, d.prec == 0);
     }
     int dirty = make_items(runs, mc, out);
     const long long clean = (long long)out.size() - dirty;
@@ -527,7 +531,8 @@ inline cudaError_t batch_build(tlbm_host::BatchState& b, cudaStream_t st) {
             caps.push_back(dd.partials_cap);
         }
         if (own >= 2LL * c.res(d0) * d0.sms) {
-            const int mc = pick_chunk(runs, caps, (halo + n / 2) / n, c.res(d0), d0.sms, Q == 19, d0.prec == 0);
+            const int mc = pick_chunk(runs, caps, (halo + n / 2) / n, c.res(d0), c.TX * c.TY, d0.sms, Q == 19,
+                                      d0.prec == 0);
             b.auto_tile = (b.tile & 255) | mc << 8;
         }
     }

@@ -14,11 +14,11 @@ using tlbm_host::PhysD;
 
 inline Geom geom(const DevState& d) { return Geom{d.nx, d.ny, d.nz, d.N, d.Np, d.ncx}; }
 
-// grid of a grid-stride kernel over n items: at most 8 blocks per SM (the
-// results do not depend on the grid)
-inline int grid_for(long long n, int sms) {
-    long long b = (n + kThreads - 1) / kThreads;
-    const long long cap = 8LL * (sms < 1 ? 1 : sms);
+// grid of a grid-stride kernel over n items in blocks of `threads`: at most 2048
+// threads per SM (the results do not depend on the grid)
+inline int grid_for(long long n, int sms, int threads = kThreads) {
+    long long b = (n + threads - 1) / threads;
+    const long long cap = 2048LL / threads * (sms < 1 ? 1 : sms);
     return (int)(b < 1 ? 1 : (b > cap ? cap : b));
 }
 
@@ -173,7 +173,7 @@ struct Impl {
         const Geom g = geom(d);
         const Phys<T> P = to_phys<T>(d.phys);
         T* mom = static_cast<T*>(d.mom);
-        const int grid = grid_for(g.N, d.sms);
+        const int grid = grid_for(g.N, d.sms, 64), threads = 64;
         const long long Np = g.Np;
         T* wk = reinterpret_cast<T*>(J.work);
         T *dX = wk, *dJ = wk + 3 * Np, *dG = wk + 6 * Np, *dL = wk + 15 * Np;
@@ -194,8 +194,8 @@ struct Impl {
         const int adj_threads = g.N <= 2LL * 32 * kMassBlocks ? 32 : kThreads;
         // moments (with wetting ghosts) of state x into mom
         auto moments_of = [&](const S* x) {
-            k_moments<Q, S, SOLID, true><<<kMassBlocks, kThreads, 0, st>>>(g, x, d.solid, mom, d.partials);
-            if (SOLID) k_ghosts<Q, T><<<grid, kThreads, 0, st>>>(g, d.solid, mom, P);
+            k_moments<Q, S, SOLID, true><<<kMassBlocks, adj_threads, 0, st>>>(g, x, d.solid, mom, d.partials);
+            if (SOLID) k_ghosts<Q, T><<<grid, threads, 0, st>>>(g, d.solid, mom, P);
         };
         // node adjoint and stencil transpose (the last stage follows at the call site)
         auto adjoint_core = [&](const S* x, const S* lam, auto init_tag) {
@@ -238,7 +238,7 @@ struct Impl {
                 const S* lin = static_cast<const S*>(J.lam[li]);
                 S* lout = static_cast<S*>(J.lam[1 - li]);
                 adjoint_core(x, lin, std::false_type{});
-                k_adj_pull<Q, S, SOLID, false><<<grid, kThreads, 0, st>>>(g, d.solid, dX, dJ, lin, P, lout, nullptr);
+                k_adj_pull<Q, S, SOLID, false><<<grid, threads, 0, st>>>(g, d.solid, dX, dJ, lin, P, lout, nullptr);
                 li ^= 1;
             }
             chk(cudaGetLastError());
@@ -246,7 +246,7 @@ struct Impl {
         // initialisation: x(0) = equilibrium of the fields
         const S* x0 = reinterpret_cast<const S*>(state(J.ckpt, 0));
         adjoint_core(x0, static_cast<const S*>(J.lam[li]), std::true_type{});
-        k_adj_pull<Q, S, SOLID, true><<<grid, kThreads, 0, st>>>(g, d.solid, dX, dJ, nullptr, P, nullptr, J.dfields);
+        k_adj_pull<Q, S, SOLID, true><<<grid, threads, 0, st>>>(g, d.solid, dX, dJ, nullptr, P, nullptr, J.dfields);
         k_adj_acc<<<1, kThreads, 0, st>>>(node_sums, kMassBlocks, 3, J.acc + 1);
         k_adj_acc<<<1, kThreads, 0, st>>>(gather_sums, kMassBlocks, 3, J.acc + 4);
         // leave the engine at x(T)
