@@ -121,23 +121,12 @@ tlbm_status tlbm_set_kernel(tlbm *t, tlbm_kernel kind);
 /* Which implementation tlbm_step uses now (resolves AUTO). */
 tlbm_kernel tlbm_get_kernel(const tlbm *t);
 
-/* Tile of the fused step.  variant = shape | mode << 4: shape 0 = default
- * (D3Q19 shape 7, D2Q9 shape 5), D3Q19 1 = 32x8, 2 = 64x4, 3 = 32x4 nodes
- * per block, 4..7 = 32x4 with part of each node's pulled populations kept in
- * shared memory from the moment pass to the collision (4: the 19 f values;
- * 5: the lane-shifted values first, 28 for FP32, 19 plus a per-warp L2
- * prefetch for the 16-bit formats; 6: 19 lane-shifted values; 7: as 5, the
- * k values first and then the lane-shifted (f, g) pairs); D2Q9 1 = 128,
- * 2 = 256, 3 = 64 nodes per row, 4 = 128 with the 18 lane-shifted values
- * staged, 5 = 128 with all 27 staged.  mode (shapes 1..3) selects the
- * load order and cache hints inside a plane (0 default for the lattice and
- * storage; 1 interleaved halo loads; 2 collision operands loaded first; 3 both;
- * 4 per-warp L2 prefetch three planes ahead; 5 = 1 + 4; 6 plain order;
- * 8 evict-first stores; 9 also evict-first collision loads; 12, 13 = 8, 9 with
- * the prefetch; a mode not built for a shape falls back to its default; the
- * variant must be below 256, its shape below 8).
- * chunk = planes marched per block (0 = chosen from the lattice size).  Double
- * storage ignores the choice.  Results do not depend on the tile. */
+/* Tile of the fused step.  variant = shape | mode << 4 (below 256, shape below 8).
+ * D2Q9 in FP32 and 16 bits: shape 2 = rows of 256 nodes per block, 3 = 64, all
+ * others 128 (with solid nodes as well).  D3Q19 and double storage have one tile;
+ * the other shapes, and every mode, are accepted and change nothing.
+ * chunk = planes marched per block (0 = chosen from the lattice size; blocks near
+ * solid nodes march fewer).  Results do not depend on the tile. */
 tlbm_status tlbm_set_tile(tlbm *t, int variant, int chunk);
 
 /*
@@ -183,7 +172,9 @@ tlbm_status tlbm_mass(tlbm *t, double out[3]);
 /*
  * Totals of the state at the start of the most recent step, as accumulated
  * inside that step (NaN before the first step), and the non-finite flag of all
- * steps since the last init.  Synchronises the stream.
+ * steps since the last init.  TLBM_ERR_TIMEOUT if a block of one of these steps
+ * gave up waiting for its copies into shared memory (after about a second): the
+ * state is void then.  Synchronises the stream.
  */
 tlbm_status tlbm_step_mass(tlbm *t, double out[3]);
 
@@ -371,8 +362,9 @@ void tlbm_batch_destroy(tlbm_batch *b);
  * device word as (code << 56 | offending offset or index), codes 1 pull
  * source, 2 bounce-back source, 3 store target, 4 moment-ring index, 5 mask
  * index; the access is redirected to a valid address and the kernel carries on
- * (no trap, no fault).  The checked kernels use the default tile and compute
- * the same results as the unchecked ones.  The checked kernels are those of
+ * (no trap, no fault).  The checked kernels use the default tile, the solid-aware
+ * one on every block of a lattice with solid nodes, and compute the same results
+ * as the unchecked ones.  The checked kernels are those of
  * the pressure-tensor coupling (an engine under TLBM_COUPLING_FORCING runs its
  * unchecked kernels).  TLBM_ERR_UNSUPPORTED for other storage formats.
  * tlbm_bounds_check_word waits for the engine's stream,

@@ -36,19 +36,21 @@ namespace tlbm_dev {
 // What a row of nodes pulls, as runs of 32 lane words in shared memory.  FP32: the
 // chunk's own order.  16-bit formats: the chunk's first 26 runs, then the k words
 // whose two directions come from different rows, once for each direction.
-template <typename S>
+template <typename S, int Q = 19>
 struct RowImage {
-    using F = Fmt<19, S>;
+    using F = Fmt<Q, S>;
     static constexpr bool PACKED = F::PACKED;
-    static constexpr int RUNS = PACKED ? 34 : 57;
+    static constexpr int KEPT = Q == 19 ? 26 : 14;  // 16-bit: runs of one source row each
+    static constexpr int RUNS = PACKED ? (Q == 19 ? 34 : 16) : 3 * Q;
     static constexpr int BYTES = RUNS * 128;
-    static constexpr int COPIES = PACKED ? 17 : 9;
+    static constexpr int COPIES = PACKED ? (Q == 19 ? 17 : 5) : (Q == 19 ? 9 : 3);
     // byte offset of (s, i)
     __host__ __device__ static constexpr int off(int s, int i) {
-        if (PACKED && s == 2 && i > 0 && F::krun(i) >= 26) return krun2(i) * 128 + F::khalf(i) * 2;
+        if (PACKED && s == 2 && i > 0 && F::krun(i) >= KEPT) return krun2(i) * 128 + F::khalf(i) * 2;
         return F::off(s, i);
     }
-    __host__ __device__ static constexpr int krun2(int i) {  // 3 4 5 6 11 14 12 13
+    __host__ __device__ static constexpr int krun2(int i) {  // D3Q19 3 4 5 6 11 14 12 13, D2Q9 3 4
+        if (Q == 9) return 11 + i;
         return i <= 6 ? 23 + i : (i == 11 ? 30 : (i == 14 ? 31 : (i == 12 ? 32 : 33)));
     }
     // copy n: (e_y, e_z) of its source row, offset in the chunk and in the image, bytes
@@ -56,11 +58,16 @@ struct RowImage {
         int ey, ez, src, dst, bytes;
     };
     __host__ __device__ static constexpr Copy copy(int n) {
+        if (Q == 9) {  // groups e_y = 0, 1, -1, then the k word of 3 and of 4
+            const int len0 = PACKED ? 6 : 9, len = PACKED ? 4 : 9, e = n == 0 ? 0 : (n == 1 || n == 3 ? 1 : -1);
+            const int at = n == 0 ? 0 : (n <= 2 ? len0 + (n - 1) * len : KEPT);
+            return Copy{e, 0, at * 128, (n <= 2 ? at : KEPT + n - 3) * 128, (n == 0 ? len0 : (n <= 2 ? len : 1)) * 128};
+        }
         constexpr int ey[9] = {0, 1, -1, 0, 0, 1, 1, -1, -1}, ez[9] = {0, 0, 0, 1, -1, 1, -1, 1, -1};
         if (n >= 9) {  // 16-bit: a k word for one of its two directions
             constexpr int d[8] = {3, 4, 5, 6, 11, 14, 12, 13};
             const int i = d[n < 17 ? n - 9 : 0];
-            return Copy{Lat<19>::cy(i), Lat<19>::cz(i), F::krun(i) * 128, krun2(i) * 128, 128};
+            return Copy{Lat<Q>::cy(i), Lat<Q>::cz(i), F::krun(i) * 128, krun2(i) * 128, 128};
         }
         // runs before group n and in it
         const int len0 = PACKED ? 6 : 9, len = PACKED ? 4 : 9, one = PACKED ? 1 : 3;
@@ -89,14 +96,15 @@ struct RowImage {
     }
 };
 
-// A node's populations in registers: FP32 as they are, 16-bit formats in their
-// stored form (39 registers; converted where they are used).
-template <typename S>
+// A node's populations in registers: as FP32 values, except for D3Q19 in 16 bits,
+// where they keep their stored form (39 registers instead of 57; converted where
+// they are used).
+template <typename S, int Q = 19>
 struct NodePops {
-    using I = RowImage<S>;
-    static constexpr int Q = 19;
-    float f[Q], g[Q], k[Q];  // FP32; 16-bit: the rest populations
-    unsigned fg[Q];          // 16-bit: (f, g) words, k
+    using I = RowImage<S, Q>;
+    static constexpr bool STORED = I::PACKED && Q == 19;
+    float f[Q], g[Q], k[Q];  // values (STORED: of the rest populations)
+    unsigned fg[Q];          // STORED: (f, g) words, k
     unsigned short kh[Q];
     __device__ __forceinline__ void clear() {
 #pragma unroll
@@ -108,7 +116,7 @@ struct NodePops {
     }
     // take direction i from the slot, and return its values
     __device__ __forceinline__ void take(const unsigned char* n, int i, float& f_, float& g_, float& k_) {
-        if (I::PACKED && i > 0) {
+        if (STORED && i > 0) {
             fg[i] = *reinterpret_cast<const unsigned*>(n + I::off(0, i));
             kh[i] = *reinterpret_cast<const unsigned short*>(n + I::off(2, i));
         } else {
@@ -117,7 +125,7 @@ struct NodePops {
         get(i, f_, g_, k_);
     }
     __device__ __forceinline__ void get(int i, float& f_, float& g_, float& k_) const {
-        if constexpr (I::PACKED) {
+        if constexpr (STORED) {
             if (i > 0) {
                 Store<S>::get2(fg[i], f_, g_);
                 k_ = Store<S>::get(*reinterpret_cast<const S*>(&kh[i]));
@@ -474,6 +482,230 @@ __device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ 
     if (tid == 0) put_block_sums(g, partials, bid, mr, mp, ms);
 }
 
+// ---------------------------------------------------------------- D2Q9
+
+// The same for D2Q9 (periodic body of FP32 and 16-bit storage): a block owns TX nodes of
+// a row, TX / 32 chunks with three copies each (five in 16 bits), and marches along y.
+// Only the two words beyond either end of the tile come by cp.async.  The kernel it
+// replaces loaded a plane's 27 populations a node, summed, waited at the barrier
+// and only then collided: at 16 warps an SM its waits filled 60 % of the time.
+template <typename S, int TX>
+struct Bulk2Shape {
+    using I = RowImage<S, 9>;
+    static constexpr int CH = TX / 32;
+    static constexpr int SIDE = CH * I::BYTES;       // x neighbours: lanes 0..3 of one more chunk image
+    static constexpr int SLOT = SIDE + I::BYTES;
+    static constexpr int RN = TX + 2;
+    static constexpr int RING = 2 * SLOT, BAR = (RING + 2 * 3 * RN * 4 + 7) / 8 * 8;
+    static constexpr int SMEM = BAR + 16;
+    static constexpr int ITEMS = 18;                 // (direction, x neighbour) pairs
+};
+
+template <typename S, int TX, bool CHK>
+__device__ __forceinline__ void bulk2_body(const MGeom& g, const S* __restrict__ src, S* __restrict__ dst,
+                                           const Phys<float>& P, double* __restrict__ partials, const int bid,
+                                           const Work wk) {
+    constexpr int Q = 9;
+    using F = Fmt<Q, S>;
+    using I = RowImage<S, Q>;
+    using B = Bulk2Shape<S, TX>;
+    using L = Lat<Q>;
+    extern __shared__ __align__(16) unsigned char tlbm_smem[];
+    float* const ring = reinterpret_cast<float*>(tlbm_smem + B::RING);
+    const unsigned smem0 = smem_u32(tlbm_smem), bar0 = smem0 + B::BAR;
+
+    const int tid = threadIdx.x;
+    const int A0 = wk.A0, M0 = wk.M0, M1 = wk.M1;
+    const int W = min(TX, g.NA - A0);  // nodes of this tile
+    const bool active = tid < W;
+    const unsigned char* const srcb = reinterpret_cast<const unsigned char*>(src);
+    const int last = M1 - M0 + 1;
+
+    // ---- this thread's bulk copy (threads of the second warp)
+    const unsigned char* bsrc = srcb;
+    unsigned bdst = 0, bbytes = 0;
+    int bey = 0;
+    const int nch = (W + 31) >> 5;
+    {
+        const int t = tid - 32;
+        if (t >= 0 && t < nch * I::COPIES) {
+            const int c = t / I::COPIES, n = t % I::COPIES;
+            typename I::Copy cp = I::copy(0);
+#pragma unroll
+            for (int k = 1; k < I::COPIES; ++k) {
+                const typename I::Copy ck = I::copy(k);
+                if (n == k) cp = ck;
+            }
+            bsrc = chk_node<Q, S, CHK>(g, srcb, srcb + (A0 / 32 + c) * F::CHUNK, 1) + cp.src;
+            bdst = c * I::BYTES + cp.dst;
+            bbytes = cp.bytes;
+            bey = cp.ey;
+        }
+    }
+    // ---- this thread's x neighbour (threads 0 .. 17): lanes {0, 1, 2, 3} of the side
+    // image hold A0 - 2, A0 - 1, A0 + W, A0 + W + 1; directions with e_x = 0 need the
+    // inner two, e_x = 1 the left two, e_x = -1 the right two
+    const unsigned char* isrc = srcb;
+    unsigned idst = 0, idel_s = 0, idel_d = 0;
+    int iey = 0;
+    bool ithird = false;
+    if (tid < B::ITEMS) {
+        const int p = tid, which = p < 6 ? p / 2 : (p - 6) % 6 / 2;
+        const int slot = p < 6 ? 1 + (p & 1) : (p < 12 ? (p & 1) : 2 + (p & 1));
+        const int mu = slot < 2 ? slot - 2 : W + slot - 2;
+        int o0 = 0, o1 = 0, d0 = 0, d1 = 0, n0 = 0, np = 0, nm = 0;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            const bool mine = L::cx(i) == 0 ? (p < 6 && which == n0)
+                                            : (L::cx(i) > 0 ? (p >= 6 && p < 12 && which == np) : (p >= 12 && which == nm));
+            if (mine) {
+                o0 = F::off(0, i);
+                d0 = I::off(0, i);
+                o1 = (I::PACKED && i > 0) ? F::krun(i) * 128 : F::off(1, i);
+                d1 = (I::PACKED && i > 0) ? I::off(2, i) - F::khalf(i) * 2 : I::off(1, i);
+                iey = L::cy(i);
+                ithird = !(I::PACKED && i > 0);
+            }
+            n0 += L::cx(i) == 0;
+            np += L::cx(i) > 0;
+            nm += L::cx(i) < 0;
+        }
+        const int x = modp(A0 + mu, g.NA);
+        isrc = chk_node<Q, S, CHK>(g, srcb, srcb + (x >> 5) * F::CHUNK + (x & 31) * F::ESZ, 2) + o0;
+        idst = B::SIDE + d0 + slot * 4;
+        idel_s = (unsigned)(o1 - o0);
+        idel_d = (unsigned)(d1 - d0);
+    }
+    // byte offsets of the rows y - 1, y, y + 1 of the plane whose copies start next
+    long long ym = (long long)modp(M0 - 2, g.NM) * g.rowstride, yc = (long long)modp(M0 - 1, g.NM) * g.rowstride,
+              yp = (long long)modp(M0, g.NM) * g.rowstride;
+    const long long yend = (long long)g.NM * g.rowstride;
+    auto start = [&](int p) {
+        const unsigned sl = smem0 + (p & 1) * B::SLOT, bar = bar0 + (p & 1) * 8;
+        if (tid == 32) mbar_expect(bar, nch * I::BYTES);
+        if (bbytes) bulk_load(sl + bdst, bsrc + (bey == 0 ? yc : (bey > 0 ? ym : yp)), bbytes, bar);
+        if (tid < B::ITEMS) {
+            const unsigned char* s = isrc + (iey == 0 ? yc : (iey > 0 ? ym : yp));
+            const unsigned d = sl + idst;
+            copy4(d, s);
+            copy4(d + idel_d, s + idel_s);
+            if (ithird) copy4(d + 2 * idel_d, s + 2 * idel_s);
+            copy_arrive(bar);
+        }
+        ym = yc;
+        yc = yp;
+        yp = yp + g.rowstride == yend ? 0 : yp + g.rowstride;
+    };
+    if (tid == 0) {
+        mbar_init(bar0, B::ITEMS + 1);
+        mbar_init(bar0 + 8, B::ITEMS + 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __syncthreads();
+    grid_ready();
+    start(0);
+    start(1);
+
+    // offset in a slot of the lane word of tile node x (-2 .. W + 1)
+    auto word = [&](int x) -> int {
+        if (x >= 0 && x < W) return (x >> 5) * I::BYTES + (x & 31) * 4;
+        return B::SIDE + (x < 0 ? x + 2 : min(x - W, 1) + 2) * 4;
+    };
+    const int own[3] = {(tid >> 5) * I::BYTES + (tid & 31) * 4, word(tid - 1), word(tid + 1)};
+    // the two border nodes: lanes 0, 1, 2 of the last two warps, one set each
+    const int bx = tid < TX - 32 ? -1 : W, bset = tid & 31;
+    const bool border = tid >= TX - 64 && bset < 3;
+    const int bord[3] = {word(bx), word(bx - 1), word(bx + 1)};
+    unsigned char* const outb = reinterpret_cast<unsigned char*>(dst) +
+                                (active ? (long long)((A0 + tid) >> 5) * F::CHUNK : 0) + (tid & 31) * F::ESZ;
+
+    MassSum<float, true> msum;
+    Roll<Q, float> roll;
+    roll.clear();
+    NodePops<S, Q> cur, nxt;
+    cur.clear();
+    float jc[3] = {0.0f, 0.0f, 0.0f}, rdc = 0.0f;
+    bool late = false;
+#pragma unroll 1
+    for (int p = 0; p <= last; ++p) {
+        if (!mbar_wait(bar0 + (p & 1) * 8, (p >> 1) & 1, late)) late = true;
+
+        // ---- populations and moments of plane p
+        const unsigned char* const sl = tlbm_smem + (p & 1) * B::SLOT;
+        float* const rg = ring + (p & 1) * 3 * B::RN + 1;  // rg[0]: tile node 0
+        float jn[3] = {0.0f, 0.0f, 0.0f}, rdn = 0.0f, c1[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            float f, gg, kk;
+            nxt.take(sl + own[L::cx(i) == 0 ? 0 : (L::cx(i) > 0 ? 1 : 2)], i, f, gg, kk);
+            rdn += f;
+            if (L::cx(i)) jn[0] += (float)L::cx(i) * f;
+            if (L::cy(i)) jn[1] += (float)L::cy(i) * f;
+            c1[1] += gg;
+            c1[2] += kk;
+        }
+        c1[0] = rdn + 1.0f;
+        if (active) {
+            rg[tid] = c1[0];
+            rg[B::RN + tid] = c1[1];
+            rg[2 * B::RN + tid] = c1[2];
+        }
+        if (border) {  // in the order of the sums above
+            float acc = 0.0f;
+            if (!I::PACKED || bset < 2) {
+                const int so = bset * 128, sh = I::PACKED ? bset * 2 : so;  // from f to g, k: runs; 16-bit: halves
+#pragma unroll
+                for (int i = 0; i < Q; ++i) {
+                    const unsigned char* n = sl + bord[L::cx(i) == 0 ? 0 : (L::cx(i) > 0 ? 1 : 2)] + I::off(0, i);
+                    if (I::PACKED && i > 0) acc += Store<S>::get(*reinterpret_cast<const S*>(n + sh));
+                    else acc += *reinterpret_cast<const float*>(n + so);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < Q; ++i) acc += I::value(sl + bord[L::cx(i) == 0 ? 0 : (L::cx(i) > 0 ? 1 : 2)], 2, i);
+            }
+            rg[bset * B::RN + bx] = bset == 0 ? acc + 1.0f : acc;
+        }
+        __syncthreads();  // the slot is read, the ring written
+        if (p + 2 <= last) start(p + 2);
+
+        // ---- derivatives and collision of plane p - 1
+        if (active) {
+            float X[3], g12[3][3], l6[3];
+            roll.push(
+                [&](int k, int i, int) -> float {
+                    return rg[k * B::RN + (int)chk_index<CHK>(g, tid + i + 1, B::RN, 4) - 1];
+                },
+                c1, X, g12, l6);
+            if (p >= 2) {
+                msum.add(rdc, X[1], X[2]);
+                unsigned char* const out = chk_node<Q, S, CHK>(g, reinterpret_cast<unsigned char*>(dst),
+                                                               outb + (long long)(M0 + p - 2) * g.rowstride, 3);
+                float fv[Q], gv[Q], kv[Q];
+#pragma unroll
+                for (int i = 0; i < Q; ++i) cur.get(i, fv[i], gv[i], kv[i]);
+                collide_node<Q, S, true>(out, fv, gv, kv, rdc, X, jc, g12, l6, P);
+            }
+        }
+        cur = nxt;
+        jc[0] = jn[0];
+        jc[1] = jn[1];
+        rdc = rdn;
+    }
+    if (late) atomicOr(g.flag, 2);  // a copy did not arrive: the step's results are void
+    double mr, mp, ms;
+    msum.get(mr, mp, ms);
+    block_sum3(mr, mp, ms);
+    if (tid == 0) put_block_sums(g, partials, bid, mr, mp, ms);
+}
+
+template <typename S, int TX, bool CHK>
+__global__ void __launch_bounds__(TX, 512 / TX)
+k_bulk2(MGeom g, const S* __restrict__ src, S* __restrict__ dst, Phys<float> P, double* __restrict__ partials) {
+    bulk2_body<S, TX, CHK>(g, src, dst, P, partials, blockIdx.x, work_of<TX, 1>(g, blockIdx.x));
+}
+
 template <typename S, bool CHK>
 __global__ void __launch_bounds__(BulkShape<S>::THREADS, BulkShape<S>::BPS)
 k_bulk(MGeom g, const S* __restrict__ src, S* __restrict__ dst, Phys<float> P, double* __restrict__ partials) {
@@ -487,6 +719,70 @@ k_bulk_batch(const SimDesc<float>* __restrict__ d, int nsims) {
     const SimDesc<float>& m = batch_member(d, nsims, sh);
     bulk_body<S, false>(member_geom(m.g), as_global(static_cast<const S*>(m.src)), as_global(static_cast<S*>(m.dst)),
                         m.P, as_global(m.partials), (int)blockIdx.x - m.block0);
+}
+
+// ------------------------------------------------- solid lattices, batches
+
+// D2Q9 with solid nodes: a block whose planes keep two nodes away from every solid
+// node runs the periodic body, the others the solid-aware one (which blocks is
+// decided per lattice, Work).  The solid-aware body costs twice as much: two
+// barriers a plane, four halo planes, two loads of every mask.  FP32 4096x2048 with 32 wells
+// (2.6 % of its planes near solids): see DESIGN for both sides.
+template <int Q, typename S>
+struct Mix {
+    static constexpr bool DBL = sizeof(S) == 8;
+    template <int TX>
+    static constexpr int smem() {
+        int a = 0;
+        if constexpr (DBL) a = fused_smem<Q, S>(TX, 1);
+        else a = Bulk2Shape<S, TX>::SMEM;
+        return a > solid_smem<Q, S>(TX, 1) ? a : solid_smem<Q, S>(TX, 1);
+    }
+};
+template <int Q, typename S, int TX>
+__device__ __forceinline__ void mix_body(const MGeom& g, const S* __restrict__ src, S* __restrict__ dst,
+                                         const uint32_t* __restrict__ nbm, const Phys<typename Store<S>::T>& P,
+                                         double* __restrict__ partials, const int bid) {
+    const Work w = work_of<TX, 1>(g, bid);
+    if (w.dirty) solid_body<Q, S, TX, 1>(g, src, dst, nbm, P, partials, bid, w);
+    else if constexpr (sizeof(S) == 8) fused_body<Q, S, TX, 1>(g, src, dst, P, partials, bid, w);
+    else bulk2_body<S, TX, false>(g, src, dst, P, partials, bid, w);
+}
+template <int Q, typename S, int TX>
+__global__ void __launch_bounds__(TX, blocks_per_sm<S>(TX))
+k_mix(MGeom g, const S* __restrict__ src, S* __restrict__ dst, const uint32_t* __restrict__ nbm,
+      Phys<typename Store<S>::T> P, double* __restrict__ partials) {
+    mix_body<Q, S, TX>(g, src, dst, nbm, P, partials, blockIdx.x);
+}
+
+template <int Q, typename S, int TX, int TY>
+__global__ void __launch_bounds__(TX * TY, blocks_per_sm<S>(TX * TY))
+k_fused_batch(const SimDesc<typename Store<S>::T>* __restrict__ d, int nsims) {
+    __shared__ SimDesc<typename Store<S>::T> sh;
+    const SimDesc<typename Store<S>::T>& m = batch_member(d, nsims, sh);
+    const int bid = (int)blockIdx.x - m.block0;
+    const MGeom g = member_geom(m.g);
+    const S* src = as_global(static_cast<const S*>(m.src));
+    S* dst = as_global(static_cast<S*>(m.dst));
+    double* partials = as_global(m.partials);
+    const Work w = work_of<TX, TY>(g, bid);
+    if constexpr (sizeof(S) == 8) fused_body<Q, S, TX, TY>(g, src, dst, m.P, partials, bid, w);
+    else bulk2_body<S, TX, false>(g, src, dst, m.P, partials, bid, w);
+}
+
+template <int Q, typename S, int TX, int TY>
+__global__ void __launch_bounds__(TX * TY, blocks_per_sm<S>(TX * TY))
+k_fused_solid_batch(const SimDesc<typename Store<S>::T>* __restrict__ d, int nsims) {
+    __shared__ SimDesc<typename Store<S>::T> sh;
+    const SimDesc<typename Store<S>::T>& m = batch_member(d, nsims, sh);
+    const int bid = (int)blockIdx.x - m.block0;
+    const S* src = as_global(static_cast<const S*>(m.src));
+    S* dst = as_global(static_cast<S*>(m.dst));
+    const uint32_t* nbm = as_global(m.nbm);
+    double* partials = as_global(m.partials);
+    const MGeom g = member_geom(m.g);
+    if constexpr (Q == 9) mix_body<Q, S, TX>(g, src, dst, nbm, m.P, partials, bid);
+    else solid_body<Q, S, TX, TY>(g, src, dst, nbm, m.P, partials, bid, work_of<TX, TY>(g, bid));
 }
 
 }  // namespace tlbm_dev

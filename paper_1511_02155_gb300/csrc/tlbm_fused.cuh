@@ -133,31 +133,6 @@ __device__ __forceinline__ int modp(int v, int n) {
 __device__ __forceinline__ int wrap1(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
 
 
-// L2 bulk prefetch (TMA unit) of [p, p + bytes); p 16-byte aligned, bytes a
-// multiple of 16.  A hint: it does not fault and does not wait.
-__device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
-// ILP: a thread's border node loads interleave with its own node's loads.
-// EARLY: phase C's loads are issued before phase M's (values held across M).
-// PF: each warp prefetches its own 32-node chunk three planes ahead into L2.
-// HINT: 1 streams the stores out (evict-first); 2 also marks phase C's loads,
-//       the last use of those lines, evict-first.
-// STG: STG of the 3Q pulled populations of a thread's own node, loaded in
-//      phase M, are kept in shared memory (2 plane slots x STG x NT values) and
-//      the collision reads them from there instead of pulling them again from
-//      L2; stage_rank orders the candidates.  D2Q9.
-// position of population (s, i) in the staging order: the lane-shifted directions
-// (e_x != 0) of all three sets first, whose warp loads span two chunks
-template <int Q>
-__host__ __device__ constexpr int stage_rank(int s, int i) {
-    const bool sh = i == 1 || i == 2 || i >= 5;
-    const int is = i <= 2 ? i - 1 : i - 3;
-    const int iu = i == 0 ? 0 : i - 2;
-    return sh ? s * 6 + is : 18 + s * 3 + iu;
-}
-
 // Mass totals (rho, phi, psi of the step's input state) of the nodes a thread
 // collides, given rd (rho, or rho - 1 where f is stored as f_i - w_i), phi, psi.
 // PAIR false sums in double, as the other kernels do.  PAIR true (float
@@ -205,29 +180,25 @@ struct MassSum<float, true> {
 };
 
 // bytes of fused_body's moment ring (four planes, tile and one-node halo) and of
-// its dynamic shared memory with STG staged values per thread
+// its dynamic shared memory
 template <int Q, typename S>
 __host__ __device__ constexpr int ring_bytes(int TX, int TY) {
     const int n = 4 * 3 * (TX + 2) * (TY + (Q == 19 ? 2 : 0)) * (int)sizeof(typename Store<S>::T);
     return (n + 15) / 16 * 16;
 }
 template <int Q, typename S>
-__host__ __device__ constexpr int fused_smem(int TX, int TY, int STG) {
-    return ring_bytes<Q, S>(TX, TY) + 2 * STG * TX * TY * (int)sizeof(typename Store<S>::T);
+__host__ __device__ constexpr int fused_smem(int TX, int TY) {
+    return ring_bytes<Q, S>(TX, TY);
 }
 
-template <int Q, typename S, int TX, int TY, bool ILP, bool EARLY, bool PF = false, int HINT = 0, int STG = 0,
-          bool CHK = false>
+template <int Q, typename S, int TX, int TY>
 __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__ src, S* __restrict__ dst,
                                            const Phys<typename Store<S>::T>& P, double* __restrict__ partials,
                                            const int bid, const Work w) {
     using T = typename Store<S>::T;
     using A = Axes<Q>;
-    // dynamic shared memory: the moment ring, then the staging ring (declared here
-    // so that the compiler knows the stores are shared-memory stores that cannot
-    // alias the loads)
     extern __shared__ __align__(16) unsigned char tlbm_smem[];
-    T* const stg = reinterpret_cast<T*>(tlbm_smem + ring_bytes<Q, S>(TX, TY));
+    constexpr bool CHK = false;  // the checked kernels are those of FP32 storage
     constexpr int D = Lat<Q>::D;
     constexpr int HY = (D == 3) ? 1 : 0;  // halo rows along b
     constexpr int HW = TX + 2;
@@ -255,8 +226,9 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
         hy[0] = ty + HY;
         hx[1] = 0;
         hy[1] = 0;
-        if (D == 2) {
-            hx[1] = tid == 0 ? 0 : HW - 1;
+        if (D == 2) {  // border nodes are summed by whole warps, below
+            hx[1] = hx[0];
+            hy[1] = hy[0];
         } else if (tid < HW) {
             hx[1] = tid;
         } else if (tid < 2 * HW) {
@@ -283,7 +255,37 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
             yb[n][2] = (D == 3) ? wrap1(bb + 1, g.NB) : 0;
         }
     }
-    const int nnodes = tid < NBORDER ? 2 : 1;
+    const int nnodes = D == 3 && tid < NBORDER ? 2 : 1;
+
+    // D2Q9: the tile's two border nodes belong to warp 0 and warp 1 (both to the one
+    // warp of a 32-node row).  Each of 27 lanes loads one of the node's populations
+    // beside the loads of its own node; summed by one thread after its own node they
+    // were a second load latency on every plane's path to the barrier.
+    constexpr int BN = NT >= 64 ? 1 : 2;
+    const int lane = tid & 31;
+    const bool bwarp = D == 2 && (NT < 64 || tid < 64);
+    int boff[BN], bslot[BN], bval_off = 0, bcm = 0, bdir = 0;  // byte offset in a row, ring slot; of the lane's population
+    if constexpr (D == 2) {
+        const int l = lane < 3 * Q ? lane : 3 * Q - 1, bs = l / Q;
+        int bca = 0;
+        bdir = l % Q;
+#pragma unroll
+        for (int i = 0; i < Q; ++i)
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                if (bdir == i && bs == c) {
+                    bca = A::ca(i);
+                    bcm = A::cm(i);
+                    bval_off = Fmt<Q, S>::off(c, i);
+                }
+#pragma unroll
+        for (int n = 0; n < BN; ++n) {
+            const bool left = BN == 2 ? n == 0 : tid < 32;
+            bslot[n] = left ? 0 : HW - 1;
+            const int x = wrap1(modp(A0 + bslot[n] - 1, g.NA) - bca, g.NA);
+            boff[n] = (x >> 5) * (int)Fmt<Q, S>::CHUNK + (x & 31) * Fmt<Q, S>::ESZ;
+        }
+    }
 
     const unsigned char* srcb = reinterpret_cast<const unsigned char*>(src);
     // stored value (x - bias) of (s, i) at node pointer p
@@ -303,6 +305,19 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
         const bool two = nnodes == 2;
         T rho0 = T(0), ja = T(0), jb = T(0), jm = T(0), phi0 = T(0), psi0 = T(0);
         T rho1 = T(0), phi1 = T(0), psi1 = T(0);
+        T bval[BN];
+        if constexpr (D == 2) {
+            if (bwarp) {
+                const int row = bcm == 0 ? zr[1] : (bcm > 0 ? zr[0] : zr[2]);
+#pragma unroll
+                for (int n = 0; n < BN; ++n) {
+                    const unsigned char* p =
+                        chk_node<Q, S, CHK>(g, srcb, srcb + (long long)row * g.rowstride + boff[n], 1) + bval_off;
+                    if (Fmt<Q, S>::PACKED && bdir == 0) bval[n] = *reinterpret_cast<const T*>(p);
+                    else bval[n] = Store<S>::get(*reinterpret_cast<const S*>(p));
+                }
+            }
+        }
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             const unsigned char* p0 = src_of(0, zr, A::ca(i), A::cb(i), A::cm(i));
@@ -316,29 +331,8 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
             if (A::cm(i)) jm += T(A::cm(i)) * f;
             phi0 += gg;
             psi0 += kk;
-            if constexpr (STG > 0) {
-                T* sp = stg + (size_t)((m & 1) * STG) * NT + tid;
-                const int r0 = stage_rank<Q>(0, i), r1 = stage_rank<Q>(1, i),
-                              r2 = stage_rank<Q>(2, i);
-                if (r0 < STG) sp[(size_t)r0 * NT] = f;
-                if (r1 < STG) sp[(size_t)r1 * NT] = gg;
-                if (r2 < STG) sp[(size_t)r2 * NT] = kk;
-            }
-            if (ILP && two) {  // border node of this thread, loads interleaved with node 0
-                const unsigned char* p1 = src_of(1, zr, A::ca(i), A::cb(i), A::cm(i));
-                if (Fmt<Q, S>::PAIRED && i > 0) {
-                    T a, b;
-                    Fmt<Q, S>::ld_fg(p1, i, a, b);
-                    rho1 += a;
-                    phi1 += b;
-                } else {
-                    rho1 += ldp(p1, 0, i);
-                    phi1 += ldp(p1, 1, i);
-                }
-                psi1 += ldp(p1, 2, i);
-            }
         }
-        if (!ILP && two) {
+        if (two) {
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
                 const unsigned char* p1 = src_of(1, zr, A::ca(i), A::cb(i), A::cm(i));
@@ -362,6 +356,19 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
         sm[slot][0][h[0]] = rho0;
         sm[slot][1][h[0]] = phi0;
         sm[slot][2][h[0]] = psi0;
+        if constexpr (D == 2) {
+            if (bwarp) {
+#pragma unroll
+                for (int n = 0; n < BN; ++n) {  // lanes 0, 1, 2: rho, phi, psi in the order of the sums above
+                    T acc = T(0);
+#pragma unroll
+                    for (int i = 0; i < Q; ++i) acc += __shfl_sync(0xffffffffu, bval[n], (lane % 3) * Q + i);
+                    if (lane < 3)
+                        sm[slot][lane][(int)chk_index<CHK>(g, bslot[n], HN, 4)] =
+                            Fmt<Q, S>::OFFSET && lane == 0 ? acc + T(1) : acc;
+                }
+            }
+        }
         if (two) {
             sm[slot][0][h[1]] = rho1;
             sm[slot][1][h[1]] = phi1;
@@ -403,50 +410,6 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
     }
 
     for (int m = M0; m < M1; ++m) {
-        // Pulled populations of this thread's node at plane m, loaded before the
-        // phase-M loads of plane m+1 so that both sets of requests are in flight
-        // together (these were read one iteration ago and hit in L2).
-        const int zr[3] = {wrap1(m - 1, g.NM), m, wrap1(m + 1, g.NM)};
-        // stored values (deviations x - bias: the 16-bit formats keep f as f_i - w_i;
-        // the collision below works on deviations, with the bias folded into its
-        // constants)
-        T fv[Q], gv[Q], kv[Q];
-        auto load_node = [&]() {
-#pragma unroll
-            for (int i = 0; i < Q; ++i) {
-                const unsigned char* pi = src_of(0, zr, A::ca(i), A::cb(i), A::cm(i));
-                auto lc = [&](int s_) -> T {
-                    return HINT >= 2 ? Fmt<Q, S>::ld_last_delta(pi, s_, i) : Fmt<Q, S>::ld_delta(pi, s_, i);
-                };
-                if constexpr (STG > 0) {
-                    const T* sp = stg + (size_t)((m & 1) * STG) * NT + tid;
-                    const int r0 = stage_rank<Q>(0, i), r1 = stage_rank<Q>(1, i),
-                              r2 = stage_rank<Q>(2, i);
-                    if (Fmt<Q, S>::PAIRED && i > 0 && r0 >= STG && r1 >= STG) {
-                        Fmt<Q, S>::template ld_fg<(HINT >= 2)>(pi, i, fv[i], gv[i]);  // one lane word
-                    } else {
-                        fv[i] = r0 < STG ? sp[(size_t)r0 * NT] : lc(0);
-                        gv[i] = r1 < STG ? sp[(size_t)r1 * NT] : lc(1);
-                    }
-                    kv[i] = r2 < STG ? sp[(size_t)r2 * NT] : lc(2);
-                } else {
-                    if (Fmt<Q, S>::PAIRED && i > 0) {
-                        Fmt<Q, S>::template ld_fg<(HINT >= 2)>(pi, i, fv[i], gv[i]);
-                    } else {
-                        fv[i] = lc(0);
-                        gv[i] = lc(1);
-                    }
-                    kv[i] = lc(2);
-                }
-            }
-        };
-        if (EARLY && active) load_node();
-        if (PF && (tid & 31) == 0 && active && m + 3 <= M1 + 1) {
-            // this warp's chunk of plane m+3 (all populations of its 32 nodes)
-            const long long row = (long long)wrap1(m + 3 >= g.NM ? m + 3 - g.NM : m + 3, g.NM) * g.NB + yb[0][1];
-            prefetch_l2(srcb + row * g.rowstride + xc[0][1] - ((A0 + tx) & 31) * Fmt<Q, S>::ESZ,
-                        (unsigned)Fmt<Q, S>::CHUNK);
-        }
         moments_plane(m + 1, (m + 1) & 3, jn, rdn);
         __syncthreads();
         if (!KEEP) {
@@ -456,14 +419,24 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
         }
         push_plane(m + 1, X0, g12, l6);
         if (active) {
-            if (!EARLY) load_node();
+            // stored values (deviations x - bias) of the node's pulled populations: phase M
+            // read them one iteration ago
+            const int zr[3] = {wrap1(m - 1, g.NM), m, wrap1(m + 1, g.NM)};
+            T fv[Q], gv[Q], kv[Q];
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                const unsigned char* pi = src_of(0, zr, A::ca(i), A::cb(i), A::cm(i));
+                fv[i] = ldp(pi, 0, i);
+                gv[i] = ldp(pi, 1, i);
+                kv[i] = ldp(pi, 2, i);
+            }
             const T jl[3] = {jc[0], D == 3 ? jc[1] : jc[2], D == 3 ? jc[2] : T(0)};  // lattice axes
             if constexpr (PAIR) msum.add(rdc, X0[1], X0[2]);
             else msum.add(rho_total<Q, S>(rdc), X0[1], X0[2]);
             unsigned char* out = chk_node<Q, S, CHK>(
                 g, reinterpret_cast<unsigned char*>(dst),
                 reinterpret_cast<unsigned char*>(dst) + ((long long)m * g.NB + yb[0][1]) * g.rowstride + xc[0][1], 3);
-            collide_node<Q, S, (HINT >= 1)>(out, fv, gv, kv, rdc, X0, jl, g12, l6, P);
+            collide_node<Q, S, false>(out, fv, gv, kv, rdc, X0, jl, g12, l6, P);
         }
         jc[0] = jn[0];
         jc[1] = jn[1];
@@ -476,22 +449,11 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
     if (tid == 0) put_block_sums(g, partials, bid, mr, mp, ms);
 }
 
-template <int Q, typename S, int TX, int TY, bool ILP, bool EARLY, bool PF = false, int HINT = 0, bool CHK = false>
+template <int Q, typename S, int TX, int TY>
 __global__ void __launch_bounds__(TX * TY, blocks_per_sm<S>(TX * TY))
 k_fused(MGeom g, const S* __restrict__ src, S* __restrict__ dst, Phys<typename Store<S>::T> P,
         double* __restrict__ partials) {
-    fused_body<Q, S, TX, TY, ILP, EARLY, PF, HINT, 0, CHK>(g, src, dst, P, partials, blockIdx.x,
-                                                           work_of<TX, TY>(g, blockIdx.x));
-}
-
-// Variants of the periodic D2Q9 step with shared-memory staging of STG of the
-// pulled populations, at four blocks per SM.
-template <int Q, typename S, int TX, int TY, int STG, bool CHK = false>
-__global__ void __launch_bounds__(TX * TY, 4)
-k_fused_x(MGeom g, const S* __restrict__ src, S* __restrict__ dst, Phys<typename Store<S>::T> P,
-          double* __restrict__ partials) {
-    fused_body<Q, S, TX, TY, false, false, true, 2, STG, CHK>(g, src, dst, P, partials, blockIdx.x,
-                                                              work_of<TX, TY>(g, blockIdx.x));
+    fused_body<Q, S, TX, TY>(g, src, dst, P, partials, blockIdx.x, work_of<TX, TY>(g, blockIdx.x));
 }
 
 // ------------------------------------------------------ solid-aware variant
@@ -784,36 +746,6 @@ k_fused_solid(MGeom g, const S* __restrict__ src, S* __restrict__ dst, const uin
     solid_body<Q, S, TX, TY, CHK>(g, src, dst, nbm, P, partials, blockIdx.x, work_of<TX, TY>(g, blockIdx.x));
 }
 
-// D2Q9 with solid nodes: a block whose planes keep two nodes away from every solid
-// node runs the periodic body, the others the solid-aware one (which blocks is
-// decided per lattice, Work).  The solid-aware body costs twice as much: two
-// barriers a plane, four halo planes, two loads of every mask.  FP32 4096x2048 with 32 wells
-// (2.6 % of its planes near solids): see DESIGN for both sides.
-template <int Q, typename S>
-struct Mix {
-    static constexpr bool DBL = sizeof(S) == 8;
-    static constexpr int STG = DBL ? 0 : 27;
-    static constexpr int smem(int TX) {
-        const int a = fused_smem<Q, S>(TX, 1, STG), b = solid_smem<Q, S>(TX, 1);
-        return a > b ? a : b;
-    }
-};
-template <int Q, typename S, int TX>
-__device__ __forceinline__ void mix_body(const MGeom& g, const S* __restrict__ src, S* __restrict__ dst,
-                                         const uint32_t* __restrict__ nbm, const Phys<typename Store<S>::T>& P,
-                                         double* __restrict__ partials, const int bid) {
-    const Work w = work_of<TX, 1>(g, bid);
-    if (w.dirty) solid_body<Q, S, TX, 1>(g, src, dst, nbm, P, partials, bid, w);
-    else fused_body<Q, S, TX, 1, false, false, !Mix<Q, S>::DBL, Mix<Q, S>::DBL ? 0 : 2, Mix<Q, S>::STG>(g, src, dst, P, partials,
-                                                                                                  bid, w);
-}
-template <int Q, typename S, int TX>
-__global__ void __launch_bounds__(TX, blocks_per_sm<S>(TX))
-k_mix(MGeom g, const S* __restrict__ src, S* __restrict__ dst, const uint32_t* __restrict__ nbm,
-      Phys<typename Store<S>::T> P, double* __restrict__ partials) {
-    mix_body<Q, S, TX>(g, src, dst, nbm, P, partials, blockIdx.x);
-}
-
 // ------------------------------------------------------------- batches
 
 // One member of a batched step: its geometry, buffers for this step's parity,
@@ -866,33 +798,6 @@ __device__ __forceinline__ MGeom member_geom(const MGeom& m) {
     if (g.items) g.items = as_global(g.items);
     g.flag = as_global(g.flag);
     return g;
-}
-
-template <int Q, typename S, int TX, int TY, bool PF, int HINT, int STG>
-__global__ void __launch_bounds__(TX * TY, blocks_per_sm<S>(TX * TY))
-k_fused_batch(const SimDesc<typename Store<S>::T>* __restrict__ d, int nsims) {
-    __shared__ SimDesc<typename Store<S>::T> sh;
-    const SimDesc<typename Store<S>::T>& m = batch_member(d, nsims, sh);
-    const int bid = (int)blockIdx.x - m.block0;
-    const MGeom g = member_geom(m.g);
-    fused_body<Q, S, TX, TY, false, false, PF, HINT, STG>(g, as_global(static_cast<const S*>(m.src)),
-                                                          as_global(static_cast<S*>(m.dst)), m.P, as_global(m.partials),
-                                                          bid, work_of<TX, TY>(g, bid));
-}
-
-template <int Q, typename S, int TX, int TY>
-__global__ void __launch_bounds__(TX * TY, blocks_per_sm<S>(TX * TY))
-k_fused_solid_batch(const SimDesc<typename Store<S>::T>* __restrict__ d, int nsims) {
-    __shared__ SimDesc<typename Store<S>::T> sh;
-    const SimDesc<typename Store<S>::T>& m = batch_member(d, nsims, sh);
-    const int bid = (int)blockIdx.x - m.block0;
-    const S* src = as_global(static_cast<const S*>(m.src));
-    S* dst = as_global(static_cast<S*>(m.dst));
-    const uint32_t* nbm = as_global(m.nbm);
-    double* partials = as_global(m.partials);
-    const MGeom g = member_geom(m.g);
-    if constexpr (Q == 9) mix_body<Q, S, TX>(g, src, dst, nbm, m.P, partials, bid);
-    else solid_body<Q, S, TX, TY>(g, src, dst, nbm, m.P, partials, bid, work_of<TX, TY>(g, bid));
 }
 
 // FP64 totals of every member: block i sums member i's partials in a fixed order

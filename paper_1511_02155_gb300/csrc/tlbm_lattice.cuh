@@ -170,11 +170,11 @@ struct Store<__nv_bfloat16> {
 // Inside a chunk, each run holds one lane word per node, Fmt::ESZ bytes apart,
 // so a node is one byte offset, chunk + lane * ESZ, and every population of it
 // is that offset plus a constant.
-//   FP64, and FP32 on D2Q9: 3Q runs of S, run s*Q + i for set s, direction i.
-//   FP32 on D3Q19: 3Q runs of S ordered by (e_y, e_z), the row that a pull reads
-//     them from: the runs of one such group are one contiguous piece of the
-//     chunk, so the nine pieces that a row of nodes pulls from nine source rows
-//     are nine bulk copies (tlbm_bulk.cuh).  Within a group direction by
+//   FP64: 3Q runs of S, run s*Q + i for set s, direction i.
+//   FP32: 3Q runs of S ordered by (e_y, e_z) (D2Q9: e_y), the row that a pull
+//     reads them from: the runs of one such group are one contiguous piece of the
+//     chunk, so the nine (three) pieces that a row of nodes pulls from as many
+//     source rows are bulk copies (tlbm_bulk.cuh).  Within a group direction by
 //     direction: f_i, g_i, k_i.
 //   FP32 keeps f as its deviation f_i - w_i from the rest state at rho = 1 (g and
 //     k as they are): deviations are small, so FP32 rounding of the stored
@@ -184,10 +184,10 @@ struct Store<__nv_bfloat16> {
 //     for each moving direction i one run of (f_i, g_i) pairs (the two share a
 //     pull source: one load), one run for each pair (k_i, k_kmate(i)), and three
 //     FP32 runs of the rest populations f_0 - w_0, g_0, k_0.  kmate(i) is opp(i),
-//     which one collision step writes together, except for the x edges of D3Q19,
-//     whose k pairs (7, 9), (8, 10), (15, 17), (16, 18) share a source row: on
-//     D3Q19 these runs too are ordered by (e_y, e_z), with the four pairs of
-//     directions from different rows at the end.
+//     which one collision step writes together, except for links oblique to x,
+//     whose k pairs (7, 9), (8, 10), (15, 17), (16, 18) (D2Q9: (5, 7), (6, 8))
+//     share a source row.  These runs too are ordered by source row, with the pairs
+//     of directions from different rows at the end.
 //     That is 3(Q-1) 16-bit values and three FP32 values per node, as dense as
 //     16 bits allow.  The rest populations carry nearly all of phi and psi,
 //     which 16 bits would round by up to 2.4e-4 per step; the moving
@@ -227,15 +227,17 @@ struct Fmt {
             constexpr int v[19] = {0, 2, 1, 4, 3, 6, 5, 9, 10, 7, 8, 14, 13, 12, 11, 17, 18, 15, 16};
             return v[i];
         }
-        return i == 0 ? 0 : ((i - 1) ^ 1) + 1;  // D2Q9: opposites adjacent
+        constexpr int u[9] = {0, 2, 1, 4, 3, 7, 8, 5, 6};
+        return u[i];
     }
     __host__ __device__ static constexpr int khalf(int i) { return i < kmate(i) ? 0 : 1; }
-    // D3Q19: position of direction i in the order by (e_y, e_z): (0,0) 1 2 and rest,
-    // (1,0) 3 7 9, (-1,0) 4 8 10, (0,1) 5 15 17, (0,-1) 6 16 18, (1,1), (1,-1),
-    // (-1,1), (-1,-1)
+    // position of direction i in the order by source row.  D3Q19, by (e_y, e_z): (0,0)
+    // 1 2 and rest, (1,0) 3 7 9, (-1,0) 4 8 10, (0,1) 5 15 17, (0,-1) 6 16 18, (1,1),
+    // (1,-1), (-1,1), (-1,-1).  D2Q9, by e_y: 0 rest 1 2, 1 3 5 7, -1 4 6 8
     __host__ __device__ static constexpr int gpos(int i) {
         constexpr int v[19] = {0, 1, 2, 3, 6, 9, 12, 4, 7, 5, 8, 15, 16, 17, 18, 10, 13, 11, 14};
-        return Q == 19 ? v[i] : i;
+        constexpr int u[9] = {0, 1, 2, 3, 6, 4, 7, 5, 8};
+        return Q == 19 ? v[i] : u[i];
     }
     // packed: run of the pair (f_i, g_i) and of the k word of direction i
     __host__ __device__ static constexpr int fgrun(int i) {
@@ -243,19 +245,21 @@ struct Fmt {
             constexpr int v[19] = {3, 0, 1, 6, 10, 14, 18, 7, 11, 8, 12, 22, 23, 24, 25, 15, 19, 16, 20};
             return v[i];
         }
-        return i - 1;
+        constexpr int u[9] = {3, 0, 1, 6, 10, 7, 11, 8, 12};
+        return u[i];
     }
     __host__ __device__ static constexpr int krun(int i) {
         if (Q == 19) {
             constexpr int v[19] = {5, 2, 2, 26, 26, 27, 27, 9, 13, 9, 13, 28, 29, 29, 28, 17, 21, 17, 21};
             return v[i];
         }
-        return (Q - 1) + (i - 1) / 2;
+        constexpr int u[9] = {5, 2, 2, 14, 14, 9, 13, 9, 13};
+        return u[i];
     }
     // byte offset of (s, i) in the lane word of lane 0
     __host__ __device__ static constexpr int off(int s, int i) {
-        if (!PAIRED) return (Q == 19 && sizeof(S) == 4 ? 3 * gpos(i) + s : s * Q + i) * 32 * ESZ;
-        if (i == 0) return ((Q == 19 ? 3 : (Q - 1) + NKP) + s) * RUN;
+        if (!PAIRED) return (sizeof(S) == 4 ? 3 * gpos(i) + s : s * Q + i) * 32 * ESZ;
+        if (i == 0) return (3 + s) * RUN;
         if (s < 2) return fgrun(i) * RUN + s * VSZ;
         return krun(i) * RUN + khalf(i) * VSZ;
     }

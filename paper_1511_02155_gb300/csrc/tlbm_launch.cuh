@@ -102,8 +102,6 @@ inline int pick_chunk(const std::vector<Run>& runs, const std::vector<long long>
 template <int Q>
 struct FusedCfg {
     int TX, TY, MC;
-    int mode;
-    int shape;  // D2Q9 shape
     // prologue planes a block recomputes, and blocks per SM (blocks_per_sm)
     int halo(const tlbm_host::DevState& d) const { return d.solid || d.coupling ? 4 : 2; }
     int res(const tlbm_host::DevState& d) const {
@@ -112,15 +110,11 @@ struct FusedCfg {
     }
 };
 
-// d.tile = shape | mode << 4 | chunk << 8: shape 0 = default.  D3Q19 has one
-// kernel per storage format (FP32 and 16-bit: k_bulk; double: k_fused, 16x8 nodes);
-// its shapes are accepted and change nothing.  D2Q9 shape 0 = 5: 128-node rows with
-// all 27 values staged, 1 = 128, 2 = 256, 3 = 64, 4 = 128 with the 18 lane-shifted
-// values staged.  mode (shapes 1..3) bit 0: interleaved border loads; bit 1: early
-// phase-C loads; bit 2: per-warp L2 prefetch three planes ahead; 8 / 9: evict-first
-// stores / stores and collision loads (12, 13 with the prefetch).  mode 0 is the
-// default for the shape (13); 6 selects the plain loop.  chunk = planes per block
-// (0 = pick_chunk).
+// d.tile = shape | mode << 4 | chunk << 8: shape 0 = default.  D3Q19 has one tile per
+// storage format (FP32 and 16-bit: k_bulk, 32x4 nodes; double: k_fused, 16x8), and
+// D2Q9 in FP32 and 16 bits one kernel on rows of 128 nodes (k_bulk2; shape 2: 256,
+// 3: 64).  The other shapes and the modes are accepted and change nothing.  chunk =
+// planes per block (0 = pick_chunk).
 // D2Q9 in double: rows of 32 nodes (one warp) where rows of 128 in chunks of four
 // planes leave SMs idle; wider rows recompute fewer halo moments.
 // A batch launches one tile for all members: narrow only if every member is.
@@ -150,13 +144,9 @@ inline FusedCfg<Q> fused_cfg(const tlbm_host::DevState& d) {
         c.TX = 32;  // k_bulk
         c.TY = 4;
     } else {
-        const int v = variant == 0 ? 5 : variant;  // 128-node rows with staging measured fastest
-        c.TX = dbl ? (narrow_rows(d) ? 32 : 128) : (v == 2 ? 256 : (v == 3 ? 64 : 128));
+        c.TX = dbl ? (narrow_rows(d) ? 32 : 128) : (variant == 2 ? 256 : (variant == 3 ? 64 : 128));  // k_bulk2
         c.TY = 1;
-        c.shape = v;
     }
-    c.mode = dbl ? 0 : ((tile >> 4) & 15);
-    if (c.mode == 0) c.mode = 13;  // D2Q9: prefetch, evict-first stores and collision loads
     const int NA = d.nx;
     const int NB = (Q == 19) ? d.ny : 1;
     const int NM = (Q == 19) ? d.nz : d.ny;
@@ -186,6 +176,11 @@ template <int Q>
 inline std::vector<ColumnRun> column_runs(const tlbm_host::DevState& d, const FusedCfg<Q>& c) {
     const int NB = Q == 19 ? d.ny : 1, NM = Q == 19 ? d.nz : d.ny, HB = Q == 19 ? 2 : 0;
     std::vector<ColumnRun> out;
+    auto around = [](int v, int n) {  // periodic; without a division for every node
+        while (v < 0) v += n;
+        while (v >= n) v -= n;
+        return v;
+    };
     std::vector<unsigned char> near((size_t)NM), full((size_t)NM), kind((size_t)NM);
     for (int B0 = 0; B0 < NB; B0 += c.TY)
         for (int A0 = 0; A0 < d.nx; A0 += c.TX) {
@@ -194,7 +189,7 @@ inline std::vector<ColumnRun> column_runs(const tlbm_host::DevState& d, const Fu
                 unsigned char any = 0, all = 1;
                 for (int b = B0 - HB; b < B0 + c.TY + HB; ++b) {
                     const bool tile = b >= B0 && b < B0 + c.TY && b < NB;
-                    const unsigned char* row = d.units + ((size_t)m * NB + (size_t)(((b % NB) + NB) % NB)) * d.ncx;
+                    const unsigned char* row = d.units + ((size_t)m * NB + (size_t)around(b, NB)) * d.ncx;
                     for (int u = u0; u < u1; ++u) {
                         any |= row[u] & 1;
                         if (tile && !(row[u] & 2)) all = 0;
@@ -205,7 +200,7 @@ inline std::vector<ColumnRun> column_runs(const tlbm_host::DevState& d, const Fu
             }
             for (int m = 0; m < NM; ++m) {
                 unsigned char any = 0;
-                for (int k = -2; k <= 2; ++k) any |= near[(size_t)((((m + k) % NM) + NM) % NM)];
+                for (int k = -2; k <= 2; ++k) any |= near[(size_t)around(m + k, NM)];
                 kind[(size_t)m] = full[(size_t)m] ? 2 : any;
             }
             for (int m = 0; m < NM;) {  // short clean gaps
@@ -354,10 +349,10 @@ inline cudaError_t launch_smem(K kern, int dyn, int threads, int bps, long long 
     if (e != cudaSuccess) return e;
     return launch_step(kern, dyn, threads, nb, st, args...);
 }
-// ... of a D2Q9 kernel with stg staged values per thread of 128
-template <typename S, typename K, typename... Args>
-inline cudaError_t launch_staged(K kern, int stg, long long nb, cudaStream_t st, Args... args) {
-    return launch_smem(kern, fused_smem<9, S>(128, 1, stg), 128, 4, nb, st, args...);
+// ... of k_bulk2
+template <typename S, int TX, typename K, typename... Args>
+inline cudaError_t launch_bulk2(K kern, long long nb, cudaStream_t st, Args... args) {
+    return launch_smem(kern, Bulk2Shape<S, TX>::SMEM, TX, 512 / TX, nb, st, args...);
 }
 // ... of k_bulk
 template <typename S, typename K, typename... Args>
@@ -391,7 +386,7 @@ inline cudaError_t fused_step(tlbm_host::DevState& d, const Phys<typename Store<
             } else {
                 cudaError_t e;
                 if constexpr (Q == 19) e = launch_bulk<S>(k_bulk<S, true>, nb, st, g, src, dst, P, d.partials);
-                else e = launch_staged<S>(k_fused_x<Q, S, 128, 1, 27, true>, 27, nb, st, g, src, dst, P, d.partials);
+                else e = launch_bulk2<S, 128>(k_bulk2<S, 128, true>, nb, st, g, src, dst, P, d.partials);
                 if (e != cudaSuccess) return e;
             }
             return cudaGetLastError();
@@ -417,58 +412,35 @@ inline cudaError_t fused_step(tlbm_host::DevState& d, const Phys<typename Store<
                 }
             }
         } else {
-            auto mix = [&](auto kern, int TX) {
-                e = launch_smem(kern, Mix<Q, S>::smem(TX), TX, blocks_per_sm<S>(TX), nb, st, g, src, dst, d.nbm, P, d.partials);
+            auto mix = [&](auto kern, int TX, int dyn) {
+                e = launch_smem(kern, dyn, TX, blocks_per_sm<S>(TX), nb, st, g, src, dst, d.nbm, P, d.partials);
             };
             if constexpr (sizeof(S) == 8) {
-                if (c.TX == 32) mix(k_mix<Q, S, 32>, 32);
-                else mix(k_mix<Q, S, 128>, 128);
+                if (c.TX == 32) mix(k_mix<Q, S, 32>, 32, Mix<Q, S>::template smem<32>());
+                else mix(k_mix<Q, S, 128>, 128, Mix<Q, S>::template smem<128>());
             } else {
-                if (c.TX == 256) mix(k_mix<Q, S, 256>, 256);
-                else if (c.TX == 64) mix(k_mix<Q, S, 64>, 64);
-                else mix(k_mix<Q, S, 128>, 128);
+                if (c.TX == 256) mix(k_mix<Q, S, 256>, 256, Mix<Q, S>::template smem<256>());
+                else if (c.TX == 64) mix(k_mix<Q, S, 64>, 64, Mix<Q, S>::template smem<64>());
+                else mix(k_mix<Q, S, 128>, 128, Mix<Q, S>::template smem<128>());
             }
         }
         return e != cudaSuccess ? e : cudaGetLastError();
     }
     cudaError_t e = cudaSuccess;
-    auto go = [&](auto kern, int threads) {
-        e = launch_step(kern, fused_smem<Q, S>(c.TX, c.TY, 0), threads, nb, st, g, src, dst, P, d.partials);
-    };
     if constexpr (sizeof(S) == 8) {
         // double storage is the parity path: one tile shape per lattice and size
-        if constexpr (Q == 19) go(k_fused<Q, S, 16, 8, false, false>, 128);
-        else if (c.TX == 32) go(k_fused<Q, S, 32, 1, false, false>, 32);
-        else go(k_fused<Q, S, 128, 1, false, false>, 128);
+        auto go = [&](auto kern, int threads) {
+            e = launch_step(kern, fused_smem<Q, S>(c.TX, c.TY), threads, nb, st, g, src, dst, P, d.partials);
+        };
+        if constexpr (Q == 19) go(k_fused<Q, S, 16, 8>, 128);
+        else if (c.TX == 32) go(k_fused<Q, S, 32, 1>, 32);
+        else go(k_fused<Q, S, 128, 1>, 128);
     } else if constexpr (Q == 19) {
         e = launch_bulk<S>(k_bulk<S, false>, nb, st, g, src, dst, P, d.partials);
     } else {
-        if (c.shape >= 4 && !d.solid) {
-            // 128-node rows with staging: 4 the 18 lane-shifted values, 5 (default)
-            // all 27, with the per-warp prefetch and evict-first stores and
-            // collision loads
-            e = c.shape == 4 ? launch_staged<S>(k_fused_x<Q, S, 128, 1, 18>, 18, nb, st, g, src, dst, P, d.partials)
-                             : launch_staged<S>(k_fused_x<Q, S, 128, 1, 27>, 27, nb, st, g, src, dst, P, d.partials);
-            return e != cudaSuccess ? e : cudaGetLastError();
-        }
-        if (c.TX == 256) {
-            switch (c.mode) {
-                case 1: go(k_fused<Q, S, 256, 1, true, false>, 256); break;
-                case 2: go(k_fused<Q, S, 256, 1, false, true>, 256); break;
-                case 3: go(k_fused<Q, S, 256, 1, true, true>, 256); break;
-                default: go(k_fused<Q, S, 256, 1, false, false>, 256);
-            }
-        } else if (c.TX == 64) {
-            go(k_fused<Q, S, 64, 1, false, false>, 64);
-        } else if (c.mode == 4) {
-            go(k_fused<Q, S, 128, 1, false, false, true>, 128);
-        } else if (c.mode == 12) {
-            go(k_fused<Q, S, 128, 1, false, false, true, 1>, 128);
-        } else if (c.mode == 13) {
-            go(k_fused<Q, S, 128, 1, false, false, true, 2>, 128);
-        } else {
-            go(k_fused<Q, S, 128, 1, false, false>, 128);  // plain loop
-        }
+        if (c.TX == 256) e = launch_bulk2<S, 256>(k_bulk2<S, 256, false>, nb, st, g, src, dst, P, d.partials);
+        else if (c.TX == 64) e = launch_bulk2<S, 64>(k_bulk2<S, 64, false>, nb, st, g, src, dst, P, d.partials);
+        else e = launch_bulk2<S, 128>(k_bulk2<S, 128, false>, nb, st, g, src, dst, P, d.partials);
     }
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -619,29 +591,30 @@ inline cudaError_t batch_step(tlbm_host::BatchState& b, cudaStream_t st, cudaEve
             constexpr int TX = sizeof(S) == 8 ? 16 : 32;
             e = launch_smem(k_fused_solid_batch<Q, S, TX, 4>, solid_smem<Q, S>(TX, 4), TX * 4, 512 / (TX * 4), nb, st, d, n);
         } else {
-            auto mix = [&](auto kern, int TX) {
-                e = launch_smem(kern, Mix<Q, S>::smem(TX), TX, blocks_per_sm<S>(TX), nb, st, d, n);
+            auto mix = [&](auto kern, int TX, int dyn) {
+                e = launch_smem(kern, dyn, TX, blocks_per_sm<S>(TX), nb, st, d, n);
             };
             if constexpr (sizeof(S) == 8) {
-                if (c.TX == 32) mix(k_fused_solid_batch<Q, S, 32, 1>, 32);
-                else mix(k_fused_solid_batch<Q, S, 128, 1>, 128);
+                if (c.TX == 32) mix(k_fused_solid_batch<Q, S, 32, 1>, 32, Mix<Q, S>::template smem<32>());
+                else mix(k_fused_solid_batch<Q, S, 128, 1>, 128, Mix<Q, S>::template smem<128>());
             } else {
-                if (c.TX == 256) mix(k_fused_solid_batch<Q, S, 256, 1>, 256);
-                else if (c.TX == 64) mix(k_fused_solid_batch<Q, S, 64, 1>, 64);
-                else mix(k_fused_solid_batch<Q, S, 128, 1>, 128);
+                if (c.TX == 256) mix(k_fused_solid_batch<Q, S, 256, 1>, 256, Mix<Q, S>::template smem<256>());
+                else if (c.TX == 64) mix(k_fused_solid_batch<Q, S, 64, 1>, 64, Mix<Q, S>::template smem<64>());
+                else mix(k_fused_solid_batch<Q, S, 128, 1>, 128, Mix<Q, S>::template smem<128>());
             }
         }
     } else {
-        auto go = [&](auto kern, int threads, int stg) {
-            e = launch_smem(kern, fused_smem<Q, S>(c.TX, c.TY, stg), threads, blocks_per_sm<S>(threads), nb, st, d, n);
+        auto go = [&](auto kern, int threads) {
+            e = launch_smem(kern, fused_smem<Q, S>(c.TX, c.TY), threads, blocks_per_sm<S>(threads), nb, st, d, n);
         };
         if constexpr (Q == 19) {
-            if constexpr (sizeof(S) == 8) go(k_fused_batch<Q, S, 16, 8, false, 0, 0>, 128, 0);
+            if constexpr (sizeof(S) == 8) go(k_fused_batch<Q, S, 16, 8>, 128);
             else e = launch_bulk<S>(k_bulk_batch<S>, nb, st, d, n);
-        } else if (sizeof(S) == 8 && c.TX == 32) {
-            if constexpr (sizeof(S) == 8) go(k_fused_batch<Q, S, 32, 1, false, 0, 0>, 32, 0);
+        } else if constexpr (sizeof(S) == 8) {
+            if (c.TX == 32) go(k_fused_batch<Q, S, 32, 1>, 32);
+            else go(k_fused_batch<Q, S, 128, 1>, 128);
         } else {
-            go(k_fused_batch<Q, S, 128, 1, true, 2, sizeof(S) == 8 ? 0 : 27>, 128, sizeof(S) == 8 ? 0 : 27);
+            e = launch_bulk2<S, 128>(k_fused_batch<Q, S, 128, 1>, nb, st, d, n);
         }
     }
     if (e != cudaSuccess) return e;
