@@ -1,6 +1,7 @@
 // tlbm_fused.cuh -- one-kernel time step of the ternary free-energy LB method
-// (Semprebon, Krueger, Kusumaatmaja, arXiv:1511.02155) for periodic lattices
-// without solid nodes.
+// (Semprebon, Krueger, Kusumaatmaja, arXiv:1511.02155): the periodic step in double
+// (the other storages bring the same march's populations by bulk copies,
+// tlbm_bulk.cuh) and the solid-aware step in every storage.
 //
 // The equilibria at r need gradients and Laplacians of rho, phi, psi at the
 // same time level, i.e. the moments of r's neighbours, which depend on the
@@ -139,9 +140,8 @@ __device__ __forceinline__ int wrap1(int v, int n) { return v < 0 ? v + n : (v >
 // formats) keeps per quantity an error-free pair (hi, lo) updated by Knuth's
 // TwoSum, and rho as the node count plus the summed deviations: no FP64
 // instruction runs per node, and the pairs become doubles once per block.
-// Measured on GB300: the pairs are 1-2 % faster for D2Q9 and for 16-bit D3Q19
-// storage; the FP32 D3Q19 kernel, at its register limit, spills with them and
-// keeps the double sums.
+// Measured on GB300: the pairs are 1-2 % faster.  The solid-aware FP32 D3Q19 body, at
+// its register limit, spills with them and keeps the double sums.
 template <typename T, bool PAIR>
 struct MassSum {
     double r = 0.0, p = 0.0, s = 0.0;

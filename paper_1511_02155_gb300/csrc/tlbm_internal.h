@@ -55,7 +55,7 @@ struct DevState {
     int* flag;           // non-finite flag (int)
     PhysD phys;
     int tile;            // fused-kernel tile choice (0 = default)
-    int rows128;         // D2Q9 in double: no one-warp rows (a batch that keeps 128)
+    int rows;            // D2Q9 in double: 32 or 128 nodes a row as told, 0 by the lattice (narrow_rows)
     int sms;             // multiprocessors of the device (sizes the fused grid's chunks)
     unsigned long long* check;  // device word: first bounds violation of a checked step
     int checked;         // 1: the fused step runs its bounds-checked kernels

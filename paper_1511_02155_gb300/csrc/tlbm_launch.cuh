@@ -117,9 +117,13 @@ struct FusedCfg {
 // planes per block (0 = pick_chunk).
 // D2Q9 in double: rows of 32 nodes (one warp) where rows of 128 in chunks of four
 // planes leave SMs idle; wider rows recompute fewer halo moments.
-// A batch launches one tile for all members: narrow only if every member is.
-inline bool narrow_rows(const tlbm_host::DevState& d) { return !d.rows128 && d.N < 512LL * d.sms; }
-
+// A given chunk whose blocks' sums do not fit the scratch on narrow rows takes rows of
+// 128.  A batch launches one tile for all members: narrow only if every member is.
+inline bool narrow_rows(const tlbm_host::DevState& d) {
+    if (d.rows != 0) return d.rows == 32;
+    const int mc = d.tile >> 8;
+    return d.N < 512LL * d.sms && (mc == 0 || (long long)((d.nx + 31) / 32) * ((d.ny + mc - 1) / mc) <= d.partials_cap);
+}
 
 template <int Q>
 inline FusedCfg<Q> fused_cfg(const tlbm_host::DevState& d) {
@@ -150,6 +154,15 @@ inline FusedCfg<Q> fused_cfg(const tlbm_host::DevState& d) {
     const int NA = d.nx;
     const int NB = (Q == 19) ? d.ny : 1;
     const int NM = (Q == 19) ? d.nz : d.ny;
+    if (Q == 19 && mc > 0 && !dbl && !d.solid && !d.coupling && (variant == 1 || variant == 2)) {
+        // shapes 1 and 2 name tiles of 32x8 and 64x4 nodes: a chunk whose sums fit the
+        // scratch on those is doubled until they fit on 32x4
+        auto nb = [&](int tx, int ty, int ch) {
+            return (long long)((NA + tx - 1) / tx) * ((NB + ty - 1) / ty) * ((NM + ch - 1) / ch);
+        };
+        if (nb(variant == 2 ? 64 : 32, variant == 1 ? 8 : 4, mc) <= d.partials_cap)
+            while (mc < NM && nb(32, 4, mc) > d.partials_cap) mc *= 2;
+    }
     if (mc <= 0) {
         const long long cols = (long long)((NA + c.TX - 1) / c.TX) * ((NB + c.TY - 1) / c.TY);
         mc = pick_chunk({Run{cols, NM, 0, false}}, {d.partials_cap}, c.halo(d), c.res(d), c.TX * c.TY, d.sms, Q == 19, dbl);
@@ -265,6 +278,7 @@ inline int solid_items(const tlbm_host::DevState& d, std::vector<int4>& out) {
     out.clear();
     if (!wants_items<Q>(d)) return 0;
     tlbm_host::DevState dd = d;
+    dd.rows = narrow_rows(d) ? 32 : 128;
     dd.tile = d.tile | ((d.tile >> 8) ? 0 : 1 << 8);  // any chunk: only the tile is wanted
     const FusedCfg<Q> c = fused_cfg<Q>(dd);
     const std::vector<ColumnRun> runs = column_runs<Q>(d, c);
@@ -457,13 +471,17 @@ inline cudaError_t batch_build(tlbm_host::BatchState& b, cudaStream_t st) {
     long long block0 = 0;
     b.auto_tile = b.tile;
     b.narrow = 1;
-    for (int k = 0; k < n; ++k) b.narrow = b.narrow && narrow_rows(*b.sims[k]);
+    for (int k = 0; k < n; ++k) {
+        tlbm_host::DevState dd = *b.sims[k];
+        dd.tile = b.tile;
+        b.narrow = b.narrow && narrow_rows(dd);
+    }
     // tile of member k (chunk 1 stands for any), its runs and its blocks with chunk 0
     // (its own choice) or mc
     auto member = [&](int k, int mc) {
         tlbm_host::DevState dd = *b.sims[k];
         dd.tile = (b.tile & 255) | mc << 8;
-        dd.rows128 = !b.narrow;
+        dd.rows = b.narrow ? 32 : 128;
         dd.items = nullptr;
         dd.nitems = 0;
         return dd;
@@ -581,7 +599,7 @@ inline cudaError_t batch_step(tlbm_host::BatchState& b, cudaStream_t st, cudaEve
     const SimDesc<T>* d = static_cast<const SimDesc<T>*>(b.desc) + (size_t)par * n;
     tlbm_host::DevState probe = *b.sims[0];
     probe.tile = b.auto_tile;
-    probe.rows128 = !b.narrow;
+    probe.rows = b.narrow ? 32 : 128;
     const FusedCfg<Q> c = fused_cfg<Q>(probe);
     const int nb = (int)b.blocks;
     if (ev0) cudaEventRecord(ev0, st);

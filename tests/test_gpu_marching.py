@@ -151,6 +151,38 @@ def test_forcing_at_tile_edges(Q, shape, precision):
     assert err <= bound, (err, bound)
 
 
+@pytest.mark.parametrize("Q,shape,precision,tile", [
+    # chunks of one plane whose sums fit the scratch (max(1216, N / 64 + 1) blocks) only on wider tiles
+    (9, (128, 600, 1), "fp64", (0, 1)), (9, (33, 1000, 1), "fp64", (0, 1)), (9, (64, 640, 1), "fp64", (0, 1)),
+    (19, (64, 1, 1800), "fp32", (2, 1)), (19, (5, 5, 1216), "fp16", (1, 1))])
+def test_given_chunks_of_one_plane_still_fit_the_scratch(Q, shape, precision, tile):
+    err, bound = _one_step(Q, shape, precision, tile=tile)
+    assert err <= bound
+
+
+def test_batch_of_double_members_with_chunks_of_one_plane():
+    """One member's sums fit only on rows of 128, the other's on either: three steps to rounding."""
+    def engines():
+        out = []
+        for nx, ny in ((128, 600), (64, 40)):
+            eng = tl.TernaryLB(9, nx, ny, 1, KAPPA, precision="fp64")
+            eng.init_fields(*W.to_aux(*W.spinodal((ny, nx), seed=nx, amp=0.1)))
+            out.append(eng)
+        return out
+
+    alone, members = engines(), engines()
+    batch = tl.TernaryBatch(members)
+    batch.set_tile(0, 1)
+    batch.step(3)
+    for x, y in zip(alone, members):
+        x.set_tile(0, 1)
+        x.step(3)
+        assert np.abs(x.get_populations() - y.get_populations()).max() <= 3e-13
+    batch.close()
+    for e in alone + members:
+        e.close()
+
+
 def test_many_steps_in_one_call_equal_single_steps():
     """Steps overlap their launches; a call of n steps gives the bits of n calls."""
     for Q, shape, solid in ((9, (70, 50, 1), None), (9, (70, 50, 1), "walls"), (19, (40, 9, 8), None)):
