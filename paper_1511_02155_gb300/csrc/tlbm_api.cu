@@ -104,17 +104,23 @@ cudaError_t set_items(tlbm* t) {
     std::vector<int4> items;
     const int dirty = t->ops->solid_items(d, items);
     cudaError_t e = cudaStreamSynchronize(t->st);  // no step in flight reads what is replaced
-    if (e != cudaSuccess) return e;
     cudaFree(const_cast<void*>(d.items));
-    d.items = nullptr;
+    d.items = nullptr;  // where what follows fails: one grid at the new tile
     d.nitems = d.ndirty = 0;
-    if (items.empty()) return cudaSuccess;
+    if (e != cudaSuccess || items.empty()) return e;
     void* p = nullptr;
     e = cudaMalloc(&p, sizeof(int4) * items.size());
     if (e != cudaSuccess) return e;
+    // on the engine's own stream: a copy on the default stream has no order with the
+    // steps of a non-blocking one, and a kernel that reads its items too early works
+    // on planes that do not exist
+    e = cudaMemcpyAsync(p, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice, t->st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(t->st);
+    if (e != cudaSuccess) {
+        cudaFree(p);
+        return e;
+    }
     d.items = p;
-    e = cudaMemcpy(p, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return e;
     d.nitems = (int)items.size();
     d.ndirty = dirty;
     return cudaSuccess;
@@ -340,16 +346,16 @@ tlbm_status tlbm_create(tlbm** out, tlbm_lattice lattice, int nx, int ny, int nz
         // neighbour-solid bits of the fused step, built by its first launch
         d.nbm = reinterpret_cast<uint32_t*>(base + pn);
         d.nbm_ready = 0;
-        e = cudaMemcpy(base + ps, solid_mask, (size_t)N, cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) return bail(fail(t, TLBM_ERR_CUDA, "cudaMemcpy(mask): %s", cudaGetErrorString(e)));
+        e = cudaMemcpyAsync(base + ps, solid_mask, (size_t)N, cudaMemcpyHostToDevice, t->st);
+        if (e != cudaSuccess) return bail(fail(t, TLBM_ERR_CUDA, "cudaMemcpyAsync(mask): %s", cudaGetErrorString(e)));
         mark_units(t, solid_mask);
         e = set_items(t);
         if (e != cudaSuccess) return bail(fail(t, e == cudaErrorMemoryAllocation ? TLBM_ERR_OOM : TLBM_ERR_CUDA,
                                                "work items: %s", cudaGetErrorString(e)));
     }
     const double nan3[3] = {NAN, NAN, NAN};
-    e = cudaMemcpy(d.step_mass, nan3, sizeof nan3, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(d.check, 0, 2 * sizeof(unsigned long long));  // and the flag
+    e = cudaMemcpyAsync(d.step_mass, nan3, sizeof nan3, cudaMemcpyHostToDevice, t->st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d.check, 0, 2 * sizeof(unsigned long long), t->st);  // and the flag
     if (e == cudaSuccess) e = cudaStreamSynchronize(t->st);
     if (e != cudaSuccess) return bail(fail(t, TLBM_ERR_CUDA, "initialisation: %s", cudaGetErrorString(e)));
     *out = t;
@@ -422,9 +428,9 @@ tlbm_status tlbm_set_bounds_check(tlbm* t, int on) {
 tlbm_status tlbm_bounds_check_word(tlbm* t, uint64_t* word) {
     if (!t || !word) return TLBM_ERR_ARG;
     unsigned long long w = 0;
+    CK(cudaMemcpyAsync(&w, t->d.check, sizeof w, cudaMemcpyDeviceToHost, t->st));
     CK(cudaStreamSynchronize(t->st));
-    CK(cudaMemcpy(&w, t->d.check, sizeof w, cudaMemcpyDeviceToHost));
-    if (w) CK(cudaMemset(t->d.check, 0, sizeof w));
+    if (w) CK(cudaMemsetAsync(t->d.check, 0, sizeof w, t->st));
     *word = (uint64_t)w;
     return TLBM_OK;
 }

@@ -319,7 +319,7 @@ inline MGeom mgeom(const tlbm_host::DevState& d, const FusedCfg<Q>& c) {
     g.check = d.check;
     g.flag = d.flag;
     g.beside = 0;
-    g.items = d.checked ? nullptr : static_cast<const int4*>(d.items);
+    g.items = d.checked || d.nitems == 0 ? nullptr : static_cast<const int4*>(d.items);
     g.tilesA = (g.NA + c.TX - 1) / c.TX;
     g.tilesB = (g.NB + c.TY - 1) / c.TY;
     return g;

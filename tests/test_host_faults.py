@@ -1,0 +1,93 @@
+"""What the C ABI's host code does with streams, failed calls and void states, seen on
+a CUDA runtime of host memory (fake_cuda.cpp): no GPU, and no GPU fault, is needed."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_1511_02155_gb300 import _build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+SIDE = ctypes.c_void_p(7)  # a stream that is not ordered with the default one
+N = (40, 30)
+dp = ctypes.POINTER(ctypes.c_double)
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    out = str(tmp_path_factory.mktemp("fake") / "libfake.so")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_build.nvcc()))), "include")
+    if not os.path.exists(os.path.join(cuda, "cuda_runtime.h")):
+        cuda = "/usr/local/cuda/include"
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", cuda, "-x", "c++",
+                    os.path.join(_build.CSRC, "tlbm_api.cu"), os.path.join(HERE, "fake_cuda.cpp"), "-o", out], check=True)
+    f = ctypes.CDLL(out)
+    f.fake_log.restype = f.tlbm_last_error.restype = f.tlbm_batch_last_error.restype = ctypes.c_char_p
+    d = ctypes.c_double
+    f.tlbm_create.argtypes = [ctypes.POINTER(ctypes.c_void_p)] + [ctypes.c_int] * 4 + [dp, d, d, d, d, dp, ctypes.c_void_p,
+                                                                                      ctypes.c_int, ctypes.c_void_p]
+    f.tlbm_step.argtypes = [ctypes.c_void_p, ctypes.c_int64]
+    f.tlbm_batch_step.argtypes = [ctypes.c_void_p, ctypes.c_int64]
+    f.tlbm_destroy.restype = f.tlbm_batch_destroy.restype = None
+    f.tlbm_state_bytes.restype = ctypes.c_size_t
+    f.tlbm_set_gamma.argtypes = [ctypes.c_void_p, d, d]
+    f.tlbm_get_state.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t]
+    f.tlbm_adjoint_c3_misfit.argtypes = [ctypes.c_void_p, ctypes.c_int64, ctypes.c_int, dp, dp, dp, dp, dp]
+    f.fake_fail.argtypes = [ctypes.c_char_p, ctypes.c_int]
+    return f
+
+
+def _create(lib, solid=True, precision=1):
+    mask = np.zeros(N[0] * N[1], np.uint8)
+    mask[:N[0]] = 1
+    t = ctypes.c_void_p()
+    rc = lib.tlbm_create(ctypes.byref(t), 9, *N, 1, (ctypes.c_double * 3)(0.01, 0.02, 0.03), 1.0, 1.0, 0.1, 0.1, None,
+                         mask.ctypes.data if solid else None, precision, SIDE)
+    return rc, t
+
+
+@pytest.fixture
+def fake(lib):
+    lib.fake_reset()
+    lib.fake_items(0, 5)
+    yield lib
+    lib.fake_reset()
+
+
+def _steps(lib, t):
+    """What a step saw, run when only the engine's own stream is waited for."""
+    assert lib.tlbm_step(t, 1) == 0
+    out = (ctypes.c_double * 3)()
+    lib.tlbm_step_mass(t, out)
+    return [s for s in lib.fake_log().decode().splitlines() if s.startswith("step")][-1]
+
+
+def test_work_items_are_there_before_the_first_step(fake):
+    rc, t = _create(fake)
+    assert rc == 0
+    assert _steps(fake, t) == "step: 5 items of tile 0"
+    fake.fake_items(2 + 256 * 7, 9)
+    assert fake.tlbm_set_tile(t, 2, 7) == 0
+    assert _steps(fake, t) == f"step: 9 items of tile {2 + 256 * 7}"
+    fake.tlbm_destroy(t)
+    assert fake.fake_allocations() == 0
+
+
+@pytest.mark.parametrize("call", [b"cudaMalloc", b"cudaMemcpy", b"cudaMemcpyAsync", b"cudaStreamSynchronize"])
+def test_a_failed_upload_of_work_items_leaves_one_grid(fake, call):
+    """Every step after it runs on the lattice's one grid; nothing is left allocated."""
+    rc, t = _create(fake)
+    assert rc == 0
+    before = fake.fake_allocations()
+    fake.fake_items(256 * 7, 9)
+    for nth in range(1, 4):
+        fake.fake_fail(call, nth)
+        failed = fake.tlbm_set_tile(t, 0, 7) != 0
+        fake.fake_fail(b"", 0)
+        assert _steps(fake, t) == ("step: one grid" if failed else f"step: 9 items of tile {256 * 7}")
+        assert fake.fake_allocations() <= before
+        assert fake.tlbm_set_tile(t, 0, 0) == 0
+    fake.tlbm_destroy(t)
+    assert fake.fake_allocations() == 0
