@@ -21,7 +21,7 @@ def lib(tmp_path_factory):
     cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_build.nvcc()))), "include")
     if not os.path.exists(os.path.join(cuda, "cuda_runtime.h")):
         cuda = "/usr/local/cuda/include"
-    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", cuda, "-x", "c++",
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", cuda, "-x", "c++",
                     os.path.join(_build.CSRC, "tlbm_api.cu"), os.path.join(HERE, "fake_cuda.cpp"), "-o", out], check=True)
     f = ctypes.CDLL(out)
     f.fake_log.restype = f.tlbm_last_error.restype = f.tlbm_batch_last_error.restype = ctypes.c_char_p
