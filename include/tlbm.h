@@ -126,7 +126,10 @@ tlbm_kernel tlbm_get_kernel(const tlbm *t);
  * others 128 (with solid nodes as well).  D3Q19 and double storage have one tile;
  * the other shapes, and every mode, are accepted and change nothing.
  * chunk = planes marched per block (0 = chosen from the lattice size; blocks near
- * solid nodes march fewer).  Results do not depend on the tile. */
+ * solid nodes march fewer).  Results do not depend on the tile.  With solid nodes, the
+ * first choice of a tile makes its list of work and waits for the engine's stream;
+ * the lists stay until tlbm_destroy (graphs captured of tlbm_step hold them), and a
+ * tile first chosen while the stream is captured is stepped without one. */
 tlbm_status tlbm_set_tile(tlbm *t, int variant, int chunk);
 
 /*

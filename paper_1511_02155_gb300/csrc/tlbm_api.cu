@@ -33,6 +33,13 @@ struct tlbm {
     double kernel_ms;      // accumulated main-kernel time in timing mode
     int64_t kernel_steps;  // steps accumulated in kernel_ms
     std::vector<uint8_t> units;  // solid nodes per 32-node unit (DevState::units)
+    struct Items {
+        int tile;
+        void* at;
+        int n, dirty;
+    };
+    std::vector<Items> items;  // work items of the tiles chosen so far (set_items)
+    int items_late;            // the present tile's are still to be made: it was chosen under a capture
     std::string err;
 };
 
@@ -97,32 +104,54 @@ void mark_units(tlbm* t, const uint8_t* mask) {
     t->d.units = t->units.data();
 }
 
-// work items of the fused step at the current tile (lattices with solid nodes)
+// Work items of the fused step at the current tile (lattices with solid nodes).  A
+// captured graph of steps holds their address, so the items of every tile that was
+// chosen stay until the engine goes, and choosing it again takes them as they are: no
+// call that a capture forbids.  A tile first chosen under a capture, and one whose
+// items would bring the kept ones above kept_items_cap, is stepped on one grid.
+size_t kept_items_cap(const DevState& d) { return (size_t)(d.pop_bytes / 16) + 65536; }
+
 cudaError_t set_items(tlbm* t) {
     DevState& d = t->d;
     if (!d.solid) return cudaSuccess;
-    std::vector<int4> items;
-    const int dirty = t->ops->solid_items(d, items);
-    cudaError_t e = cudaStreamSynchronize(t->st);  // no step in flight reads what is replaced
-    cudaFree(const_cast<void*>(d.items));
     d.items = nullptr;  // where what follows fails: one grid at the new tile
     d.nitems = d.ndirty = 0;
-    if (e != cudaSuccess || items.empty()) return e;
+    t->items_late = 0;
+    const auto use = [&](const tlbm::Items& k) {
+        d.items = k.at;
+        d.nitems = k.n;
+        d.ndirty = k.dirty;
+    };
+    size_t held = 0;
+    for (const tlbm::Items& k : t->items) {
+        if (k.tile == d.tile) return use(k), cudaSuccess;
+        held += sizeof(int4) * (size_t)k.n;
+    }
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(t->st, &cap);
+    if (e != cudaSuccess) return e;
+    if (cap != cudaStreamCaptureStatusNone) {
+        t->items_late = 1;
+        return cudaSuccess;
+    }
+    std::vector<int4> items;
+    const int dirty = t->ops->solid_items(d, items);
+    const size_t bytes = sizeof(int4) * items.size();
+    if (items.empty() || held + bytes > kept_items_cap(d)) return cudaSuccess;
     void* p = nullptr;
-    e = cudaMalloc(&p, sizeof(int4) * items.size());
+    e = cudaMalloc(&p, bytes);
     if (e != cudaSuccess) return e;
     // on the engine's own stream: a copy on the default stream has no order with the
     // steps of a non-blocking one, and a kernel that reads its items too early works
     // on planes that do not exist
-    e = cudaMemcpyAsync(p, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice, t->st);
+    e = cudaMemcpyAsync(p, items.data(), bytes, cudaMemcpyHostToDevice, t->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(t->st);
     if (e != cudaSuccess) {
         cudaFree(p);
         return e;
     }
-    d.items = p;
-    d.nitems = (int)items.size();
-    d.ndirty = dirty;
+    t->items.push_back(tlbm::Items{d.tile, p, (int)items.size(), dirty});
+    use(t->items.back());
     return cudaSuccess;
 }
 
@@ -212,7 +241,7 @@ void tlbm_destroy(tlbm* t) {
     if (t->st) cudaStreamSynchronize(t->st);
     else cudaDeviceSynchronize();
     cudaFree(t->block);  // populations, masks, reductions
-    cudaFree(const_cast<void*>(t->d.items));
+    for (const tlbm::Items& k : t->items) cudaFree(k.at);
     cudaFree(t->d.mom);
     cudaFree(t->d.aux);
     cudaFree(t->staging);
@@ -272,6 +301,7 @@ tlbm_status tlbm_create(tlbm** out, tlbm_lattice lattice, int nx, int ny, int nz
     t->esize = esize; t->tsize = tsize;
     t->staging = nullptr;
     t->block = nullptr;
+    t->items_late = 0;
     t->ev[0] = t->ev[1] = nullptr;
     t->timing = 0;
     t->kernel_ms = 0.0;
@@ -475,6 +505,7 @@ tlbm_status tlbm_step(tlbm* t, int64_t nsteps) {
         tlbm_status s = ensure_mom(t);
         if (s != TLBM_OK) return s;
     }
+    if (t->items_late && nsteps > 0) CK(set_items(t));  // still under the capture: still one grid
     for (int64_t n = 0; n < nsteps; ++n) {
         if (t->timing) {
             CK(t->ops->step(t->d, kind, t->st, t->ev[0], t->ev[1]));

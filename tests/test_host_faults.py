@@ -80,14 +80,54 @@ def test_a_failed_upload_of_work_items_leaves_one_grid(fake, call):
     """Every step after it runs on the lattice's one grid; nothing is left allocated."""
     rc, t = _create(fake)
     assert rc == 0
-    before = fake.fake_allocations()
-    fake.fake_items(256 * 7, 9)
     for nth in range(1, 4):
+        tile = 256 * (6 + nth)
+        fake.fake_items(tile, 9)
+        before = fake.fake_allocations()
         fake.fake_fail(call, nth)
-        failed = fake.tlbm_set_tile(t, 0, 7) != 0
+        failed = fake.tlbm_set_tile(t, 0, 6 + nth) != 0
         fake.fake_fail(b"", 0)
-        assert _steps(fake, t) == ("step: one grid" if failed else f"step: 9 items of tile {256 * 7}")
-        assert fake.fake_allocations() <= before
+        assert _steps(fake, t) == ("step: one grid" if failed else f"step: 9 items of tile {tile}")
+        assert fake.fake_allocations() == before + (0 if failed else 1)
         assert fake.tlbm_set_tile(t, 0, 0) == 0
     fake.tlbm_destroy(t)
     assert fake.fake_allocations() == 0
+
+
+def test_work_items_outlive_a_change_of_tile(fake):
+    """Steps captured at one tile may be replayed at any time later: their items stay,
+    and a tile that was chosen before needs no call that a capture forbids."""
+    rc, t = _create(fake)
+    assert rc == 0
+    tile = 2 + 256 * 7
+    fake.fake_items(tile, 9)
+    assert fake.tlbm_step(t, 1) == 0  # on the stream, not run yet: it holds the items of tile 0
+    late = fake.fake_allocations()
+    assert fake.tlbm_set_tile(t, 2, 7) == 0
+    assert fake.fake_allocations() == late + 1  # and those are still allocated
+    fake.fake_capturing(1)
+    assert fake.tlbm_set_tile(t, 0, 0) == 0 and fake.tlbm_step(t, 1) == 0
+    assert fake.tlbm_set_tile(t, 2, 7) == 0 and fake.tlbm_step(t, 1) == 0
+    fake.fake_items(256 * 3, 4)
+    assert fake.tlbm_set_tile(t, 0, 3) == 0 and fake.tlbm_step(t, 1) == 0
+    fake.fake_capturing(0)
+    assert _steps(fake, t) == f"step: 4 items of tile {256 * 3}"
+    assert fake.fake_log().decode().splitlines() == [
+        "step: 5 items of tile 0", "step: 5 items of tile 0", f"step: 9 items of tile {tile}", "step: one grid",
+        f"step: 4 items of tile {256 * 3}"]
+    fake.tlbm_destroy(t)
+    assert fake.fake_allocations() == 0
+
+
+def test_kept_work_items_are_bounded(fake):
+    rc, t = _create(fake)
+    assert rc == 0
+    cap = fake.tlbm_state_bytes(t) // 16 + 65536
+    seen = set()
+    for chunk in range(1, 41):
+        fake.fake_items(256 * chunk, cap // 16 // 8)
+        assert fake.tlbm_set_tile(t, 0, chunk) == 0
+        seen.add(_steps(fake, t).split(" of ")[0])
+        assert fake.fake_allocations() < 2 + 9
+    assert seen == {f"step: {cap // 16 // 8} items", "step: one grid"}
+    fake.tlbm_destroy(t)
