@@ -766,11 +766,11 @@ void drop_graph(tlbm_batch* b) {
 
 tlbm_status batch_rebuild(tlbm_batch* b) {
     drop_graph(b);
+    b->phys.clear();  // where the build fails, no step before one that succeeds (batch_aligned)
     cudaError_t e = b->ops->batch_build(b->bs, b->st);
     if (e != cudaSuccess)
         return bfail(b, e == cudaErrorInvalidConfiguration ? TLBM_ERR_ARG : TLBM_ERR_CUDA,
                      "batch set-up failed: %s", cudaGetErrorString(e));
-    b->phys.clear();
     for (DevState* d : b->sims) b->phys.push_back(d->phys);
     return TLBM_OK;
 }

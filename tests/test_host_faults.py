@@ -131,3 +131,21 @@ def test_kept_work_items_are_bounded(fake):
         assert fake.fake_allocations() < 2 + 9
     assert seen == {f"step: {cap // 16 // 8} items", "step: one grid"}
     fake.tlbm_destroy(t)
+
+
+def test_no_batched_step_after_a_failed_build(fake):
+    """A build that fails half-way has replaced work items that the descriptors name: the
+    batch builds again before it steps, whatever call had failed."""
+    engines = [_create(fake)[1] for _ in range(2)]
+    b = ctypes.c_void_p()
+    assert fake.tlbm_batch_create(ctypes.byref(b), (ctypes.c_void_p * 2)(*engines), 2) == 0
+    assert fake.tlbm_batch_step(b, 1) == 0
+    fake.fake_build_fails(3)  # set_tile's own, and its return to the tile before; then the next step's
+    assert fake.tlbm_batch_set_tile(b, 0, 7) != 0
+    assert fake.tlbm_batch_step(b, 1) != 0
+    assert fake.tlbm_batch_step(b, 1) == 0
+    assert fake.fake_log().decode().split("\n") == [
+        "batch build", "batch step", "batch build", "batch build", "batch build", "batch build", "batch step", ""]
+    fake.tlbm_batch_destroy(b)
+    for t in engines:
+        fake.tlbm_destroy(t)
