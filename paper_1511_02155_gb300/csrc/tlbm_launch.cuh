@@ -117,12 +117,13 @@ struct FusedCfg {
 // planes per block (0 = pick_chunk).
 // D2Q9 in double: rows of 32 nodes (one warp) where rows of 128 in chunks of four
 // planes leave SMs idle; wider rows recompute fewer halo moments.
-// A given chunk whose blocks' sums do not fit the scratch on narrow rows takes rows of
-// 128.  A batch launches one tile for all members: narrow only if every member is.
+// Where the blocks' sums do not fit the scratch on narrow rows (a short given chunk; a
+// single row of more than 38912 nodes at any chunk) rows of 128 are taken.  A batch
+// launches one tile for all members: narrow only if every member is.
 inline bool narrow_rows(const tlbm_host::DevState& d) {
     if (d.rows != 0) return d.rows == 32;
-    const int mc = d.tile >> 8;
-    return d.N < 512LL * d.sms && (mc == 0 || (long long)((d.nx + 31) / 32) * ((d.ny + mc - 1) / mc) <= d.partials_cap);
+    const int mc = (d.tile >> 8) ? d.tile >> 8 : 64;  // pick_chunk's longest
+    return d.N < 512LL * d.sms && (long long)((d.nx + 31) / 32) * ((d.ny + mc - 1) / mc) <= d.partials_cap;
 }
 
 template <int Q>

@@ -204,3 +204,28 @@ def test_many_steps_in_one_call_equal_single_steps():
             states.append((eng.get_populations(), eng.step_mass()))
             eng.close()
         assert np.array_equal(states[0][0], states[1][0]) and np.array_equal(states[0][1], states[1][1])
+
+
+@pytest.mark.parametrize("nx", [38913, 50000])
+def test_a_single_row_in_double(nx):
+    """Rows of 32 nodes would have more blocks than the scratch has sums, at any chunk."""
+    err, bound = _one_step(9, (nx, 1, 1), "fp64")
+    assert err <= bound
+    states = []
+    for batched in (False, True):
+        engines = []
+        for n in (nx, 40):
+            eng = tl.TernaryLB(9, n, 1, 1, KAPPA, precision="fp64")
+            eng.init_fields(*W.to_aux(*W.spinodal((1, n), seed=n, amp=0.1)))
+            engines.append(eng)
+        if batched:
+            with tl.TernaryBatch(engines) as b:
+                b.step(3)
+        else:
+            for e in engines:
+                e.step(3)
+        states.append([e.get_populations() for e in engines])
+        for e in engines:
+            e.close()
+    for a, b in zip(*states):
+        assert np.abs(a - b).max() <= 3e-13
