@@ -40,7 +40,11 @@
  *   creation (NULL = the legacy default stream).  tlbm_step returns without
  *   waiting; calls that return host data synchronise that stream.
  * Errors: every call returns a tlbm_status; tlbm_last_error() gives a message.
- *   Nothing throws across the ABI and no kernel traps.
+ *   Nothing throws across the ABI and no kernel traps.  If a block of a step gives
+ *   up waiting for its copies into shared memory (after about a second), the state is
+ *   void: every call that returns data of it (tlbm_fields, tlbm_mass, tlbm_step_mass,
+ *   tlbm_get_populations(_box), tlbm_get_state, the adjoint) then writes what it
+ *   found and returns TLBM_ERR_TIMEOUT, until fields, populations or a state are set.
  * Threads: a handle must not be used from two host threads at once.
  */
 #ifndef TLBM_H
@@ -62,7 +66,7 @@ typedef enum {
     TLBM_ERR_CUDA = 3,        /* a CUDA runtime call failed (message has the CUDA error) */
     TLBM_ERR_OOM = 4,         /* device allocation failed */
     TLBM_ERR_NONFINITE = 5,   /* a mass total became NaN or Inf */
-    TLBM_ERR_TIMEOUT = 6,     /* a bounded device wait gave up */
+    TLBM_ERR_TIMEOUT = 6,     /* a bounded device wait gave up (Errors, above) */
     TLBM_ERR_UNSUPPORTED = 7  /* combination not built (e.g. kernel kind for this lattice) */
 } tlbm_status;
 
@@ -175,9 +179,7 @@ tlbm_status tlbm_mass(tlbm *t, double out[3]);
 /*
  * Totals of the state at the start of the most recent step, as accumulated
  * inside that step (NaN before the first step), and the non-finite flag of all
- * steps since the last init.  TLBM_ERR_TIMEOUT if a block of one of these steps
- * gave up waiting for its copies into shared memory (after about a second): the
- * state is void then.  Synchronises the stream.
+ * steps since the last init.  Synchronises the stream.
  */
 tlbm_status tlbm_step_mass(tlbm *t, double out[3]);
 

@@ -155,6 +155,13 @@ cudaError_t set_items(tlbm* t) {
     return cudaSuccess;
 }
 
+// The flag word as read back: bit 1 set where a block of a step gave up waiting for its
+// copies into shared memory, so that the state is void (bit 0: non-finite totals).
+tlbm_status check_arrived(tlbm* t, int flag) {
+    if (flag & 2) return fail(t, TLBM_ERR_TIMEOUT, "a step's copies into shared memory did not arrive: the state is void");
+    return TLBM_OK;
+}
+
 tlbm_status ensure_staging(tlbm* t) {
     if (t->staging) return TLBM_OK;
     CK(cudaMalloc(&t->staging, sizeof(double) * 8 * (size_t)t->d.N));
@@ -562,15 +569,21 @@ tlbm_status tlbm_fields(tlbm* t, double* C1, double* C2, double* C3, double* rho
     if (C3) CK(cudaMemcpyAsync(C3, st + 2 * N, nb, cudaMemcpyDeviceToHost, t->st));
     if (rho) CK(cudaMemcpyAsync(rho, st + 3 * N, nb, cudaMemcpyDeviceToHost, t->st));
     if (u) CK(cudaMemcpyAsync(u, st + 4 * N, 3 * nb, cudaMemcpyDeviceToHost, t->st));
+    int flag = 0;
+    CK(cudaMemcpyAsync(&flag, t->d.flag, sizeof flag, cudaMemcpyDeviceToHost, t->st));
     CK(cudaStreamSynchronize(t->st));
-    return TLBM_OK;
+    return check_arrived(t, flag);
 }
 
 tlbm_status tlbm_mass(tlbm* t, double out[3]) {
     if (!t || !out) return TLBM_ERR_ARG;
     CK(t->ops->mass(t->d, t->d.mass_tmp, t->st));
+    int flag = 0;
     CK(cudaMemcpyAsync(out, t->d.mass_tmp, 3 * sizeof(double), cudaMemcpyDeviceToHost, t->st));
+    CK(cudaMemcpyAsync(&flag, t->d.flag, sizeof flag, cudaMemcpyDeviceToHost, t->st));
     CK(cudaStreamSynchronize(t->st));
+    const tlbm_status s = check_arrived(t, flag);
+    if (s != TLBM_OK) return s;
     for (int c = 0; c < 3; ++c)
         if (!std::isfinite(out[c])) return fail(t, TLBM_ERR_NONFINITE, "mass total %d is not finite", c);
     return TLBM_OK;
@@ -582,7 +595,8 @@ tlbm_status tlbm_step_mass(tlbm* t, double out[3]) {
     CK(cudaMemcpyAsync(out, t->d.step_mass, 3 * sizeof(double), cudaMemcpyDeviceToHost, t->st));
     CK(cudaMemcpyAsync(&flag, t->d.flag, sizeof(int), cudaMemcpyDeviceToHost, t->st));
     CK(cudaStreamSynchronize(t->st));
-    if (flag & 2) return fail(t, TLBM_ERR_TIMEOUT, "a step's copies into shared memory did not arrive");
+    const tlbm_status s = check_arrived(t, flag);
+    if (s != TLBM_OK) return s;
     if (flag) return fail(t, TLBM_ERR_NONFINITE, "a step produced a non-finite mass total");
     return TLBM_OK;
 }
@@ -595,11 +609,13 @@ tlbm_status tlbm_get_populations_box(tlbm* t, int x0, int y0, int z0, int bx, in
     double* dv = nullptr;
     CK(cudaMalloc(&dv, n * sizeof(double)));
     cudaError_t e = t->ops->get_box(t->d, x0, y0, z0, bx, by, bz, dv, t->st);
+    int flag = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(host, dv, n * sizeof(double), cudaMemcpyDeviceToHost, t->st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, t->d.flag, sizeof flag, cudaMemcpyDeviceToHost, t->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(t->st);
     cudaFree(dv);
     if (e != cudaSuccess) return fail(t, TLBM_ERR_CUDA, "get_populations_box: %s", cudaGetErrorString(e));
-    return TLBM_OK;
+    return check_arrived(t, flag);
 }
 
 tlbm_status tlbm_get_populations(tlbm* t, double* host) {
@@ -631,9 +647,11 @@ size_t tlbm_state_bytes(const tlbm* t) {
 tlbm_status tlbm_get_state(tlbm* t, void* host, size_t bytes) {
     if (!t || !host) return TLBM_ERR_ARG;
     if (bytes != tlbm_state_bytes(t)) return fail(t, TLBM_ERR_ARG, "state is %zu bytes", tlbm_state_bytes(t));
+    int flag = 0;
     CK(cudaMemcpyAsync(host, t->d.pop[t->d.cur], bytes, cudaMemcpyDeviceToHost, t->st));
+    CK(cudaMemcpyAsync(&flag, t->d.flag, sizeof flag, cudaMemcpyDeviceToHost, t->st));
     CK(cudaStreamSynchronize(t->st));
-    return TLBM_OK;
+    return check_arrived(t, flag);
 }
 
 tlbm_status tlbm_set_state(tlbm* t, const void* host, size_t bytes) {
@@ -705,6 +723,8 @@ tlbm_status tlbm_adjoint_c3_misfit(tlbm* t, int64_t nsteps, int checkpoint_every
     if (e == cudaSuccess) e = cudaMemcpyAsync(acc, J.acc, sizeof(double) * 8, cudaMemcpyDeviceToHost, t->st);
     if (e == cudaSuccess && dfields)
         e = cudaMemcpyAsync(dfields, J.dfields, sizeof(double) * 3 * N, cudaMemcpyDeviceToHost, t->st);
+    int flag = 0;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, t->d.flag, sizeof flag, cudaMemcpyDeviceToHost, t->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(t->st);
     release();
     if (e != cudaSuccess) return fail(t, TLBM_ERR_CUDA, "adjoint run: %s", cudaGetErrorString(e));
@@ -720,6 +740,8 @@ tlbm_status tlbm_adjoint_c3_misfit(tlbm* t, int64_t nsteps, int checkpoint_every
         dh[m] = dq[m] / (a2 * t->kappa[m]);
         dkappa[m] = acc[1 + m] - dq[m] * q / t->kappa[m];
     }
+    s = check_arrived(t, flag);
+    if (s != TLBM_OK) return s;
     if (!std::isfinite(*loss)) return fail(t, TLBM_ERR_NONFINITE, "non-finite loss");
     return TLBM_OK;
 }

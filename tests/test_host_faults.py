@@ -149,3 +149,46 @@ def test_no_batched_step_after_a_failed_build(fake):
     fake.tlbm_batch_destroy(b)
     for t in engines:
         fake.tlbm_destroy(t)
+
+
+def _reads(fake, t):
+    """Status of every call that returns data of the state."""
+    n = N[0] * N[1]
+    a = np.zeros(3 * 9 * n)
+    p = a.ctypes.data_as(dp)
+    size = fake.tlbm_state_bytes(t)
+    raw = ctypes.create_string_buffer(size)
+    return {"fields": fake.tlbm_fields(t, p, None, None, None, None), "mass": fake.tlbm_mass(t, p),
+            "step_mass": fake.tlbm_step_mass(t, p), "populations": fake.tlbm_get_populations(t, p),
+            "box": fake.tlbm_get_populations_box(t, 0, 0, 0, 1, 1, 1, p), "state": fake.tlbm_get_state(t, raw, size)}
+
+
+def test_every_read_of_a_void_state_says_so(fake):
+    rc, t = _create(fake, solid=False)
+    assert rc == 0
+    one = np.ones(N[0] * N[1]).ctypes.data_as(dp)
+    nothing = (t, one, one, one, None, None, None)
+    assert fake.tlbm_init_fields(*nothing) == 0
+    assert fake.tlbm_step(t, 2) == 0 and set(_reads(fake, t).values()) == {0}
+    fake.fake_flag(2)
+    assert fake.tlbm_step(t, 1) == 0
+    fake.fake_flag(0)
+    assert fake.tlbm_step(t, 1) == 0  # a later step does not make it whole
+    assert set(_reads(fake, t).values()) == {6}  # TLBM_ERR_TIMEOUT
+    assert fake.tlbm_init_fields(*nothing) == 0 and set(_reads(fake, t).values()) == {0}
+    fake.fake_flag(1)  # a non-finite total is step_mass's to report, as before
+    assert fake.tlbm_step(t, 1) == 0
+    assert {k: v for k, v in _reads(fake, t).items() if v} == {"step_mass": 5}
+    fake.tlbm_destroy(t)
+
+
+@pytest.mark.parametrize("flag,status", [(0, 0), (2, 6), (3, 6)])
+def test_a_gradient_from_a_void_state_says_so(fake, flag, status):
+    rc, t = _create(fake, solid=False)
+    assert rc == 0
+    one = np.ones(N[0] * N[1]).ctypes.data_as(dp)
+    assert fake.tlbm_init_fields(t, one, one, one, None, None, None) == 0
+    fake.fake_flag(flag)
+    loss, out = ctypes.c_double(), (ctypes.c_double * 3)()
+    assert fake.tlbm_adjoint_c3_misfit(t, 3, 2, one, ctypes.byref(loss), out, out, None) == status
+    fake.tlbm_destroy(t)
