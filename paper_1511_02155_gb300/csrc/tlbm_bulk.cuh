@@ -159,9 +159,8 @@ __device__ __forceinline__ bool mbar_try(unsigned bar, unsigned parity) {
         : "memory");
     return ok != 0;
 }
-// Waits for the phase with this parity, for at most about a second (a millisecond
-// once a wait of the block has run out): false then.
-__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, bool late) {
+// Waits for the phase with this parity, for at most about a second: false then.
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
     if (mbar_try(bar, parity)) return true;
     unsigned long long t0, t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
@@ -170,9 +169,15 @@ __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, bool la
         for (int n = 0; n < 64; ++n)
             if (mbar_try(bar, parity)) return true;
         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    } while (t - t0 < (late ? 1000000ull : 1000000000ull));
+    } while (t - t0 < 1000000000ull);
     return false;
 }
+// A thread whose wait has run out is late for the rest of its march: it stores nothing
+// more, starts no copy and does not arrive, so that the phases it should arrive at stay
+// open and the block's other threads run out of their next wait in turn.  It gives the
+// copies in flight a second wait before it goes on, so that the block's shared memory
+// is not given up under them.  (Each thread's own word, not a vote at the barrier:
+// __syncthreads_or cost 1 % of a step on 512x256.)
 __device__ __forceinline__ void bulk_load(unsigned dst, const void* src, unsigned bytes, unsigned bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                  "l"(src), "r"(bytes), "r"(bar)
@@ -390,7 +395,10 @@ __device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ 
 
 #pragma unroll 1
     for (int p = 0; p <= last; ++p) {
-        if (!mbar_wait(bar, p & 1, late)) late = true;
+        if (!late && !mbar_wait(bar, p & 1)) {
+            late = true;
+            mbar_wait(bar, p & 1);
+        }
 
         // ---- populations and moments of plane p
         float* const rg = ring + (p & (B::NRING - 1)) * 3 * B::RN;
@@ -437,7 +445,7 @@ __device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ 
             rg[2 * B::RN + cb] = s2;
         }
         __syncthreads();  // the slot is read, the ring written
-        if (p < last) start();
+        if (p < last && !late) start();
 
         // ---- derivatives and collision of plane p - 1
         if (active) {
@@ -459,7 +467,7 @@ __device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ 
                 }
             }
             push(rg, c1);
-            if (p >= 2) {
+            if (p >= 2 && !late) {
                 msum.add(rdc, X[1], X[2]);
                 unsigned char* const out = chk_node<Q, S, CHK>(g, reinterpret_cast<unsigned char*>(dst),
                                                                outb + (long long)(M0 + p - 2) * pstride, 3);
@@ -637,7 +645,11 @@ __device__ __forceinline__ void bulk2_body(const MGeom& g, const S* __restrict__
     bool late = false;
 #pragma unroll 1
     for (int p = 0; p <= last; ++p) {
-        if (!mbar_wait(bar0 + (p & 1) * 8, (p >> 1) & 1, late)) late = true;
+        if (!late && !mbar_wait(bar0 + (p & 1) * 8, (p >> 1) & 1)) {
+            late = true;
+            mbar_wait(bar0 + (p & 1) * 8, (p >> 1) & 1);
+            if (p < last) mbar_wait(bar0 + ((p + 1) & 1) * 8, ((p + 1) >> 1) & 1);
+        }
 
         // ---- populations and moments of plane p
         const unsigned char* const sl = tlbm_smem + (p & 1) * B::SLOT;
@@ -676,7 +688,7 @@ __device__ __forceinline__ void bulk2_body(const MGeom& g, const S* __restrict__
             rg[bset * B::RN + bx] = bset == 0 ? acc + 1.0f : acc;
         }
         __syncthreads();  // the slot is read, the ring written
-        if (p + 2 <= last) start(p + 2);
+        if (p + 2 <= last && !late) start(p + 2);
 
         // ---- derivatives and collision of plane p - 1
         if (active) {
@@ -686,7 +698,7 @@ __device__ __forceinline__ void bulk2_body(const MGeom& g, const S* __restrict__
                     return rg[k * B::RN + (int)chk_index<CHK>(g, tid + i + 1, B::RN, 4) - 1];
                 },
                 c1, X, g12, l6);
-            if (p >= 2) {
+            if (p >= 2 && !late) {
                 msum.add(rdc, X[1], X[2]);
                 unsigned char* const out = chk_node<Q, S, CHK>(g, reinterpret_cast<unsigned char*>(dst),
                                                                outb + (long long)(M0 + p - 2) * g.rowstride, 3);
