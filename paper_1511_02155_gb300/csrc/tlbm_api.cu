@@ -138,6 +138,12 @@ cudaError_t set_items(tlbm* t) {
     const int dirty = t->ops->solid_items(d, items);
     const size_t bytes = sizeof(int4) * items.size();
     if (items.empty() || held + bytes > kept_items_cap(d)) return cudaSuccess;
+    if (d.Q == 19 && !d.joined) {
+        if (!d.side) e = cudaStreamCreateWithFlags(&d.side, cudaStreamNonBlocking);
+        if (e == cudaSuccess && !d.forked) e = cudaEventCreateWithFlags(&d.forked, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&d.joined, cudaEventDisableTiming);
+        if (e != cudaSuccess) return e;
+    }
     void* p = nullptr;
     e = cudaMalloc(&p, bytes);
     if (e != cudaSuccess) return e;
@@ -252,6 +258,9 @@ void tlbm_destroy(tlbm* t) {
     cudaFree(t->d.mom);
     cudaFree(t->d.aux);
     cudaFree(t->staging);
+    if (t->d.side) cudaStreamDestroy(t->d.side);  // its work ended before the stream's (joined)
+    if (t->d.forked) cudaEventDestroy(t->d.forked);
+    if (t->d.joined) cudaEventDestroy(t->d.joined);
     if (t->ev[0]) cudaEventDestroy(t->ev[0]);
     if (t->ev[1]) cudaEventDestroy(t->ev[1]);
     if (prev >= 0) cudaSetDevice(prev);

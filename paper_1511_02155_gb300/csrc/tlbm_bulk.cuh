@@ -349,10 +349,7 @@ __device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ 
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncthreads();
-    // beside the dirty blocks' launch of the same step: that kernel has seen the step
-    // before end, so this one need not wait for it, only end after it (below)
-    if (g.beside) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    else grid_ready();
+    grid_ready();
     start();
 
     // ---- offsets in a slot of the words that a node at lane mu of row r pulls, for
@@ -483,7 +480,6 @@ __device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ 
         jc[2] = jn[2];
         rdc = rdn;
     }
-    if (g.beside) asm volatile("griddepcontrol.wait;" ::: "memory");
     if (late) atomicOr(g.flag, 2);  // a copy did not arrive: the step's results are void
     double mr, mp, ms;
     msum.get(mr, mp, ms);

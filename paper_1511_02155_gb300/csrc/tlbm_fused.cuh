@@ -49,7 +49,6 @@ struct MGeom {
     unsigned long long* check;  // first bounds violation (bounds-checked kernels)
     int* flag;            // raised by a block whose sums are not finite
     const int4* items;    // lattices with solid nodes: the blocks' work (Work), else null
-    int beside;           // second launch of a step, independent of the first (k_bulk)
 };
 
 // Steps are launched with programmatic stream serialisation: a step's blocks may be

@@ -48,6 +48,8 @@ struct DevState {
     const uint8_t* units;  // host: solid nodes per 32-node unit (column_runs), with solids
     const void* items;   // device work items of the fused step (Work), dirty ones first; or null
     int nitems, ndirty;
+    cudaStream_t side;   // D3Q19 with work items: the clean blocks' stream, and the events
+    cudaEvent_t forked, joined;  // between it and the engine's
     void* mom;           // split-step moment arrays [3][Np] (compute type); scratch
     double* partials;    // mass partial sums, 3 per block
     double* step_mass;   // [3] totals accumulated inside the last step

@@ -229,3 +229,31 @@ def test_a_single_row_in_double(nx):
             e.close()
     for a, b in zip(*states):
         assert np.abs(a - b).max() <= 3e-13
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp16"])
+@pytest.mark.parametrize("kind", ["walls", "speck", "porous_floor"])
+def test_solid_d3q19_steps_side_by_side_equal_one_grid(kind, precision):
+    """Clean and dirty blocks in two launches against the solid-aware blocks alone (too few
+    clean columns for two launches at one chunk a column): many steps, the same bits."""
+    shape = (98, 165, 40)
+    if kind == "porous_floor":
+        solid = _mask(19, shape, "walls")
+        solid[2:5][np.random.default_rng(8).random(solid[2:5].shape) < 0.2] = 1
+    else:
+        solid = _mask(19, shape, kind)
+    f = W.to_aux(*W.spinodal(shape[::-1], seed=2, amp=0.1))
+    for a in f:
+        a[solid != 0] = 0.0
+    out = []
+    for chunk, launches in ((0, 3), (4096, 2)):
+        eng = tl.TernaryLB(19, *shape, KAPPA, h=H, solid=solid.reshape(-1), precision=precision)
+        eng.set_tile(0, chunk)
+        assert eng.launches_per_step == launches
+        eng.init_fields(*f)
+        eng.step(41)
+        eng.step(1)
+        eng.step(18)
+        out.append(eng.get_populations())
+        eng.close()
+    assert np.array_equal(out[0], out[1])
