@@ -252,7 +252,7 @@ __device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ 
         }
         const int y = modp(B0 + r - 1 - c.ey, g.NB);
         bsrc = chk_node<Q, S, CHK>(g, srcb, srcb + y * g.rowstride + chunk * F::CHUNK, 1) + c.src;
-        bdst = r * I::BYTES + c.dst;
+        bdst = (unsigned)chk_index<CHK>(g, r * I::BYTES + c.dst, B::SIDE - c.bytes + 1, 4);
         bbytes = c.bytes;
         bez = c.ez;
     }
@@ -298,8 +298,8 @@ __device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ 
             }
             const int x = modp(32 * chunk + mu, g.NA), x2 = modp(x + 1, g.NA), y = modp(B0 + r - 1 - ey, g.NB);
             const int at = (x >> 5) * (int)F::CHUNK + (x & 31) * 4, at2 = (x2 >> 5) * (int)F::CHUNK + (x2 & 31) * 4;
-            isrc[k] = chk_node<Q, S, CHK>(g, srcb, srcb + y * g.rowstride + at, 2) + o0;
-            idst[k] = B::SIDE + d0 + (4 * r + slot) * 4;
+            isrc[k] = chk_node<Q, S, CHK>(g, srcb, srcb + y * g.rowstride + at, 1) + o0;
+            idst[k] = (unsigned)chk_index<CHK>(g, B::SIDE + d0 + (4 * r + slot) * 4, B::SLOT - 4, 4);
             idel[k] = (unsigned)(o1 - o0) << 16 | (unsigned)(d1 - d0);
             // two positions: one 8-byte copy where both lanes are one aligned pair
             idx2[k] = (at2 - at == 4 && (x & 1) == 0) ? 4 : at2 - at + 1;
@@ -312,7 +312,9 @@ __device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ 
     const long long zend = (long long)g.NM * pstride;
     auto start = [&]() {
         if (tid == 0) mbar_expect(bar, rows * I::BYTES);
-        if (bbytes) bulk_load(smem0 + bdst, bsrc + (bez == 0 ? zc : (bez > 0 ? zm : zp)), bbytes, bar);
+        if (bbytes)
+            bulk_load(smem0 + bdst, chk_span<CHK>(g, srcb, bsrc + (bez == 0 ? zc : (bez > 0 ? zm : zp)), bbytes, 1), bbytes,
+                      bar);
 #pragma unroll
         for (int k = 0; k < NI; ++k) {
             if (isrc[k]) {
@@ -320,19 +322,21 @@ __device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ 
                 const int ez = ((iez[k] + 1) & 7) - 1;
                 const unsigned char* s = isrc[k] + (ez == 0 ? zc : (ez > 0 ? zm : zp));
                 const unsigned d = smem0 + idst[k], dd = idel[k] & 0xffffu, ds = idel[k] >> 16;
+                auto c4 = [&](unsigned to, const unsigned char* from) { copy4(to, chk_span<CHK>(g, srcb, from, 4, 1)); };
+                auto c8 = [&](unsigned to, const unsigned char* from) { copy8(to, chk_span<CHK>(g, srcb, from, 8, 1)); };
                 if (two && idx2[k] == 4) {
-                    copy8(d, s);
-                    copy8(d + dd, s + ds);
-                    if (third) copy8(d + 2 * dd, s + 2 * ds);
+                    c8(d, s);
+                    c8(d + dd, s + ds);
+                    if (third) c8(d + 2 * dd, s + 2 * ds);
                 } else {
-                    copy4(d, s);
-                    copy4(d + dd, s + ds);
-                    if (third) copy4(d + 2 * dd, s + 2 * ds);
+                    c4(d, s);
+                    c4(d + dd, s + ds);
+                    if (third) c4(d + 2 * dd, s + 2 * ds);
                     if (two) {
                         const unsigned char* s2 = s + (idx2[k] - 1);
-                        copy4(d + 4, s2);
-                        copy4(d + 4 + dd, s2 + ds);
-                        if (third) copy4(d + 4 + 2 * dd, s2 + 2 * ds);
+                        c4(d + 4, s2);
+                        c4(d + 4 + dd, s2 + ds);
+                        if (third) c4(d + 4 + 2 * dd, s2 + 2 * ds);
                     }
                 }
             }
@@ -355,8 +359,9 @@ __device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ 
     // ---- offsets in a slot of the words that a node at lane mu of row r pulls, for
     // e_x = 0, +1 (from mu - 1), -1 (from mu + 1)
     auto word = [&](int r, int mu) -> int {
-        if (mu >= 0 && mu < W) return r * I::BYTES + mu * 4;
-        return B::SIDE + (4 * r + (mu < 0 ? mu + 2 : min(mu - W, 1) + 2)) * 4;
+        const int at = mu >= 0 && mu < W ? r * I::BYTES + mu * 4
+                                         : B::SIDE + (4 * r + (mu < 0 ? mu + 2 : min(mu - W, 1) + 2)) * 4;
+        return (int)chk_index<CHK>(g, at, B::SIDE + 128, 4);  // its last run ends in the slot
     };
     const int r0 = ty + 1;
     const int own[3] = {r0 * I::BYTES + lane * 4, word(r0, lane - 1), word(r0, lane + 1)};
@@ -549,7 +554,7 @@ __device__ __forceinline__ void bulk2_body(const MGeom& g, const S* __restrict__
                 if (n == k) cp = ck;
             }
             bsrc = chk_node<Q, S, CHK>(g, srcb, srcb + (A0 / 32 + c) * F::CHUNK, 1) + cp.src;
-            bdst = c * I::BYTES + cp.dst;
+            bdst = (unsigned)chk_index<CHK>(g, c * I::BYTES + cp.dst, B::SIDE - cp.bytes + 1, 4);
             bbytes = cp.bytes;
             bey = cp.ey;
         }
@@ -583,8 +588,8 @@ __device__ __forceinline__ void bulk2_body(const MGeom& g, const S* __restrict__
             nm += L::cx(i) < 0;
         }
         const int x = modp(A0 + mu, g.NA);
-        isrc = chk_node<Q, S, CHK>(g, srcb, srcb + (x >> 5) * F::CHUNK + (x & 31) * F::ESZ, 2) + o0;
-        idst = B::SIDE + d0 + slot * 4;
+        isrc = chk_node<Q, S, CHK>(g, srcb, srcb + (x >> 5) * F::CHUNK + (x & 31) * F::ESZ, 1) + o0;
+        idst = (unsigned)chk_index<CHK>(g, B::SIDE + d0 + slot * 4, B::SLOT - 4, 4);
         idel_s = (unsigned)(o1 - o0);
         idel_d = (unsigned)(d1 - d0);
     }
@@ -595,13 +600,15 @@ __device__ __forceinline__ void bulk2_body(const MGeom& g, const S* __restrict__
     auto start = [&](int p) {
         const unsigned sl = smem0 + (p & 1) * B::SLOT, bar = bar0 + (p & 1) * 8;
         if (tid == 32) mbar_expect(bar, nch * I::BYTES);
-        if (bbytes) bulk_load(sl + bdst, bsrc + (bey == 0 ? yc : (bey > 0 ? ym : yp)), bbytes, bar);
+        if (bbytes)
+            bulk_load(sl + bdst, chk_span<CHK>(g, srcb, bsrc + (bey == 0 ? yc : (bey > 0 ? ym : yp)), bbytes, 1), bbytes, bar);
         if (tid < B::ITEMS) {
             const unsigned char* s = isrc + (iey == 0 ? yc : (iey > 0 ? ym : yp));
             const unsigned d = sl + idst;
-            copy4(d, s);
-            copy4(d + idel_d, s + idel_s);
-            if (ithird) copy4(d + 2 * idel_d, s + 2 * idel_s);
+            auto c4 = [&](unsigned to, const unsigned char* from) { copy4(to, chk_span<CHK>(g, srcb, from, 4, 1)); };
+            c4(d, s);
+            c4(d + idel_d, s + idel_s);
+            if (ithird) c4(d + 2 * idel_d, s + 2 * idel_s);
             copy_arrive(bar);
         }
         ym = yc;
@@ -621,8 +628,9 @@ __device__ __forceinline__ void bulk2_body(const MGeom& g, const S* __restrict__
 
     // offset in a slot of the lane word of tile node x (-2 .. W + 1)
     auto word = [&](int x) -> int {
-        if (x >= 0 && x < W) return (x >> 5) * I::BYTES + (x & 31) * 4;
-        return B::SIDE + (x < 0 ? x + 2 : min(x - W, 1) + 2) * 4;
+        const int at = x >= 0 && x < W ? (x >> 5) * I::BYTES + (x & 31) * 4
+                                       : B::SIDE + (x < 0 ? x + 2 : min(x - W, 1) + 2) * 4;
+        return (int)chk_index<CHK>(g, at, B::SIDE + 128, 4);  // its last run ends in the slot
     };
     const int own[3] = {(tid >> 5) * I::BYTES + (tid & 31) * 4, word(tid - 1), word(tid + 1)};
     // the two border nodes: lanes 0, 1, 2 of the last two warps, one set each

@@ -89,7 +89,8 @@ __device__ __forceinline__ void put_block_sums(const MGeom& g, double* __restric
 // Bounds checks of the checked kernel variants (CHK).  A violation is recorded
 // as (code << 56 | offset) in *g.check -- the first one wins -- and the access
 // is redirected to a valid address; nothing traps.  Codes: 1 pull source,
-// 2 bounce-back source, 3 store target, 4 moment-ring index, 5 mask index.
+// 2 bounce-back source, 3 store target, 4 moment-ring index or offset in a slot of
+// bulk copies, 5 mask index.
 __device__ __forceinline__ void chk_record(const MGeom& g, unsigned code, long long v) {
     atomicCAS(g.check, 0ull, ((unsigned long long)code << 56) | ((unsigned long long)v & 0x00ffffffffffffffull));
 }
@@ -99,6 +100,19 @@ __device__ __forceinline__ P* chk_node(const MGeom& g, P* base, P* p, unsigned c
     if constexpr (CHK) {
         const long long off = (const unsigned char*)p - (const unsigned char*)base;
         if (off < 0 || off >= g.bytes || (off % Fmt<Q, S>::CHUNK) >= 32LL * Fmt<Q, S>::ESZ) {
+            chk_record(g, code, off);
+            return base;
+        }
+    }
+    return p;
+}
+// bytes of a population buffer starting at base that one copy reads
+template <bool CHK>
+__device__ __forceinline__ const unsigned char* chk_span(const MGeom& g, const unsigned char* base, const unsigned char* p,
+                                                         unsigned bytes, unsigned code) {
+    if constexpr (CHK) {
+        const long long off = p - base;
+        if (off < 0 || off + bytes > g.bytes) {
             chk_record(g, code, off);
             return base;
         }

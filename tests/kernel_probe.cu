@@ -94,3 +94,28 @@ extern "C" int probe_late(int Q, int* flag, long long* stored, double* seconds) 
     if (b) cudaEventDestroy(b);
     return (int)e;
 }
+
+// The checked step of planes M0 .. M1 - 1 of one tile, told that the populations end
+// `cut` bytes before they do: the word that it records.
+extern "C" int probe_check(int Q, int M0, int M1, long long cut, unsigned long long* word, long long* bytes) {
+    Lattice l;
+    cudaError_t e;
+    if (Q == 19) e = l.make<19>(40, 9, 8, 32, 4);
+    else e = l.make<9>(200, 8, 1, 128, 1);
+    l.g.bytes -= cut;
+    *bytes = l.g.bytes;
+    int4* items = nullptr;
+    const int4 it = make_int4(0, 0, M0, 2 * M1);
+    if (e == cudaSuccess) e = cudaMalloc(&items, sizeof it);
+    l.g.items = items;
+    if (e == cudaSuccess) e = cudaMemcpy(items, &it, sizeof it, cudaMemcpyHostToDevice);
+    const float* src = reinterpret_cast<const float*>(l.src);
+    float* dst = reinterpret_cast<float*>(l.dst);
+    if (e == cudaSuccess) {
+        if (Q == 19) e = launch_bulk<float>(k_bulk<float, true>, 1, nullptr, l.g, src, dst, l.P, l.partials);
+        else e = launch_bulk2<float, 128>(k_bulk2<float, 128, true>, 1, nullptr, l.g, src, dst, l.P, l.partials);
+    }
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) e = cudaMemcpy(word, l.check, sizeof *word, cudaMemcpyDeviceToHost);
+    return (int)e;
+}
