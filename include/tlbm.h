@@ -360,16 +360,16 @@ void tlbm_batch_destroy(tlbm_batch *b);
 /*
  * Bounds-checked step (a debugging aid; the paper has no counterpart).  With
  * on != 0 the fused step of an engine with TLBM_FP32 storage runs checked
- * variants of its default kernels: every population address of a pull, a
- * bounce-back and a store is validated against the population buffer and its
- * 32-node chunk layout, and every index into the on-chip moment ring and the
- * neighbour mask against its extent.  The first violation is recorded in a
- * device word as (code << 56 | offending offset or index), codes 1 pull
- * source, 2 bounce-back source, 3 store target, 4 moment-ring index, 5 mask
- * index; the access is redirected to a valid address and the kernel carries on
- * (no trap, no fault).  The checked kernels use the default tile, the solid-aware
- * one on every block of a lattice with solid nodes, and compute the same results
- * as the unchecked ones.  The checked kernels are those of
+ * variants of its default kernels: every population address of a pull (of a bulk
+ * copy, the first and the last byte), a bounce-back and a store is validated against
+ * the population buffer and its 32-node chunk layout, and every index into the
+ * on-chip moment ring and copy slots and the neighbour mask against its extent.  The
+ * first violation is recorded in a device word as (code << 56 | offending offset or
+ * index), codes 1 pull source, 2 bounce-back source, 3 store target, 4 moment-ring
+ * index or slot offset, 5 mask index; the access is redirected to a valid address and
+ * the kernel carries on (no trap, no fault).  The checked kernels use the default tile
+ * (D2Q9 with solid nodes under a tile of shape 2 or 3: the solid-aware kernel on every
+ * block) and compute the same results as the unchecked ones.  They are those of
  * the pressure-tensor coupling (an engine under TLBM_COUPLING_FORCING runs its
  * unchecked kernels).  TLBM_ERR_UNSUPPORTED for other storage formats.
  * tlbm_bounds_check_word waits for the engine's stream,

@@ -764,20 +764,20 @@ struct Mix {
         return a > solid_smem<Q, S>(TX, 1) ? a : solid_smem<Q, S>(TX, 1);
     }
 };
-template <int Q, typename S, int TX>
+template <int Q, typename S, int TX, bool CHK = false>
 __device__ __forceinline__ void mix_body(const MGeom& g, const S* __restrict__ src, S* __restrict__ dst,
                                          const uint32_t* __restrict__ nbm, const Phys<typename Store<S>::T>& P,
                                          double* __restrict__ partials, const int bid) {
     const Work w = work_of<TX, 1>(g, bid);
-    if (w.dirty) solid_body<Q, S, TX, 1>(g, src, dst, nbm, P, partials, bid, w);
+    if (w.dirty) solid_body<Q, S, TX, 1, CHK>(g, src, dst, nbm, P, partials, bid, w);
     else if constexpr (sizeof(S) == 8) fused_body<Q, S, TX, 1>(g, src, dst, P, partials, bid, w);
-    else bulk2_body<S, TX, false>(g, src, dst, P, partials, bid, w);
+    else bulk2_body<S, TX, CHK>(g, src, dst, P, partials, bid, w);
 }
-template <int Q, typename S, int TX>
+template <int Q, typename S, int TX, bool CHK = false>
 __global__ void __launch_bounds__(TX, blocks_per_sm<S>(TX))
 k_mix(MGeom g, const S* __restrict__ src, S* __restrict__ dst, const uint32_t* __restrict__ nbm,
       Phys<typename Store<S>::T> P, double* __restrict__ partials) {
-    mix_body<Q, S, TX>(g, src, dst, nbm, P, partials, blockIdx.x);
+    mix_body<Q, S, TX, CHK>(g, src, dst, nbm, P, partials, blockIdx.x);
 }
 
 template <int Q, typename S, int TX, int TY>

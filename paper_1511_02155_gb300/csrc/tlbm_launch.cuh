@@ -298,6 +298,14 @@ inline int solid_items(const tlbm_host::DevState& d, std::vector<int4>& out) {
     return dirty;
 }
 
+// Whether a step takes the engine's work items.  A checked step runs on the default
+// tile: it takes them where they are of its row width (a chunk of its own is no matter,
+// the items hold their planes), and else one grid.
+template <int Q>
+inline bool use_items(const tlbm_host::DevState& d) {
+    return d.nitems > 0 && (!d.checked || Q == 19 || ((d.tile & 15) != 2 && (d.tile & 15) != 3));
+}
+
 template <int Q, typename S>
 inline bool fused_supported(const tlbm_host::DevState& d) {
     return d.solid == nullptr || d.nbm != nullptr;
@@ -305,7 +313,7 @@ inline bool fused_supported(const tlbm_host::DevState& d) {
 
 template <int Q, typename S>
 inline int fused_launches(const tlbm_host::DevState& d) {
-    return Q == 19 && d.nitems > 0 && d.ndirty > 0 && !d.checked ? 2 : 1;
+    return Q == 19 && use_items<Q>(d) && d.ndirty > 0 ? 2 : 1;
 }
 
 template <int Q, typename S>
@@ -319,7 +327,7 @@ inline MGeom mgeom(const tlbm_host::DevState& d, const FusedCfg<Q>& c) {
     g.bytes = d.pop_bytes;
     g.check = d.check;
     g.flag = d.flag;
-    g.items = d.checked || d.nitems == 0 ? nullptr : static_cast<const int4*>(d.items);
+    g.items = use_items<Q>(d) ? static_cast<const int4*>(d.items) : nullptr;
     g.tilesA = (g.NA + c.TX - 1) / c.TX;
     g.tilesB = (g.NB + c.TY - 1) / c.TY;
     return g;
@@ -327,7 +335,7 @@ inline MGeom mgeom(const tlbm_host::DevState& d, const FusedCfg<Q>& c) {
 
 template <int Q, typename S>
 inline long long fused_blocks(const tlbm_host::DevState& d) {
-    if (d.nitems > 0 && !d.checked) return d.nitems;
+    if (use_items<Q>(d)) return d.nitems;
     const FusedCfg<Q> c = fused_cfg<Q>(d);
     const MGeom g = mgeom<Q, S>(d, c);
     return (long long)g.tilesA * g.tilesB * g.NC;
@@ -383,6 +391,59 @@ inline cudaError_t launch_bulk(K kern, long long nb, At at, Args... args) {
     return launch_smem(kern, B::SMEM, B::THREADS, B::BPS, nb, at, args...);
 }
 
+// One step of a lattice with solid nodes: work items, or one grid of solid-aware blocks.
+// CHK: the bounds-checked kernels, at the default tile.
+template <int Q, typename S, bool CHK>
+inline cudaError_t solid_step(tlbm_host::DevState& d, const FusedCfg<Q>& c, const MGeom& g, long long nb, const S* src,
+                              S* dst, const Phys<typename Store<S>::T>& P, cudaStream_t st) {
+    if (nb == 0) return cudaSuccess;  // no fluid node
+    cudaError_t e = cudaSuccess;
+    if constexpr (Q == 19) {
+        constexpr int TX = sizeof(S) == 8 ? 16 : 32;
+        const long long nd = use_items<Q>(d) ? d.ndirty : nb;
+        // dirty and clean blocks side by side: the clean ones' launch on a second
+        // stream, between an event behind the step before and one that the next
+        // step waits for.  (Both on one stream, the second launch not waiting for
+        // the first, read the step before without a dependency of their own, and
+        // were no faster: 144x128x80 FP32 210 us a step, 206 with the events.)
+        const bool fork = nd > 0 && nb > nd;
+        if (fork) {
+            e = cudaEventRecord(d.forked, st);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(d.side, d.forked, 0);
+        }
+        if (e == cudaSuccess && nd > 0)
+            e = launch_smem(k_fused_solid<Q, S, TX, 4, CHK>, solid_smem<Q, S>(TX, 4), TX * 4, 512 / (TX * 4), nd, At(st, !fork),
+                            g, src, dst, d.nbm, P, d.partials);
+        if constexpr (sizeof(S) < 8) {
+            if (e == cudaSuccess && nb > nd) {
+                MGeom gc = g;
+                gc.items = g.items + nd;
+                e = launch_bulk<S>(k_bulk<S, CHK>, nb - nd, At(fork ? d.side : st, !fork), gc, src, dst, P,
+                                   d.partials + 3 * nd);
+            }
+        }
+        if (fork) {
+            const cudaError_t e1 = cudaEventRecord(d.joined, d.side), e2 = cudaStreamWaitEvent(st, d.joined, 0);
+            if (e == cudaSuccess) e = e1 != cudaSuccess ? e1 : e2;
+        }
+    } else {
+        auto mix = [&](auto kern, int TX, int dyn) {
+            e = launch_smem(kern, dyn, TX, blocks_per_sm<S>(TX), nb, st, g, src, dst, d.nbm, P, d.partials);
+        };
+        if constexpr (CHK) {
+            mix(k_mix<Q, S, 128, true>, 128, Mix<Q, S>::template smem<128>());
+        } else if constexpr (sizeof(S) == 8) {
+            if (c.TX == 32) mix(k_mix<Q, S, 32>, 32, Mix<Q, S>::template smem<32>());
+            else mix(k_mix<Q, S, 128>, 128, Mix<Q, S>::template smem<128>());
+        } else {
+            if (c.TX == 256) mix(k_mix<Q, S, 256>, 256, Mix<Q, S>::template smem<256>());
+            else if (c.TX == 64) mix(k_mix<Q, S, 64>, 64, Mix<Q, S>::template smem<64>());
+            else mix(k_mix<Q, S, 128>, 128, Mix<Q, S>::template smem<128>());
+        }
+    }
+    return e;
+}
+
 template <int Q, typename S>
 inline cudaError_t fused_step(tlbm_host::DevState& d, const Phys<typename Store<S>::T>& P, cudaStream_t st) {
     const FusedCfg<Q> c = fused_cfg<Q>(d);
@@ -396,73 +457,23 @@ inline cudaError_t fused_step(tlbm_host::DevState& d, const Phys<typename Store<
         k_nbmask<Q><<<grid_of(d.N, d.sms), 256, 0, st>>>(gg, d.solid, d.nbm);
         d.nbm_ready = 1;
     }
+    cudaError_t e = cudaSuccess;
     if (d.checked) {
         // bounds-checked kernels of the default FP32 tiles (recording, never trapping)
         if constexpr (sizeof(S) == 4) {
             if (!d.check) return cudaErrorInvalidValue;
-            if (d.solid) {
-                cudaError_t e;
-                if constexpr (Q == 19) e = launch_smem(k_fused_solid<Q, S, 32, 4, true>, solid_smem<Q, S>(32, 4), 128, 4, nb, st, g, src, dst, d.nbm, P, d.partials);
-                else e = launch_smem(k_fused_solid<Q, S, 128, 1, true>, solid_smem<Q, S>(128, 1), 128, 4, nb, st, g, src, dst, d.nbm, P, d.partials);
-                if (e != cudaSuccess) return e;
-            } else {
-                cudaError_t e;
-                if constexpr (Q == 19) e = launch_bulk<S>(k_bulk<S, true>, nb, st, g, src, dst, P, d.partials);
-                else e = launch_bulk2<S, 128>(k_bulk2<S, 128, true>, nb, st, g, src, dst, P, d.partials);
-                if (e != cudaSuccess) return e;
-            }
-            return cudaGetLastError();
+            if (d.solid) e = solid_step<Q, S, true>(d, c, g, nb, src, dst, P, st);
+            else if constexpr (Q == 19) e = launch_bulk<S>(k_bulk<S, true>, nb, st, g, src, dst, P, d.partials);
+            else e = launch_bulk2<S, 128>(k_bulk2<S, 128, true>, nb, st, g, src, dst, P, d.partials);
+            return e != cudaSuccess ? e : cudaGetLastError();
         } else {
             return cudaErrorNotSupported;
         }
     }
     if (d.solid) {
-        if (nb == 0) return cudaSuccess;  // no fluid node
-        cudaError_t e = cudaSuccess;
-        if constexpr (Q == 19) {
-            constexpr int TX = sizeof(S) == 8 ? 16 : 32;
-            const long long nd = d.nitems > 0 ? d.ndirty : nb;
-            // dirty and clean blocks side by side: the clean ones' launch on a second
-            // stream, between an event behind the step before and one that the next
-            // step waits for.  (Both on one stream, the second launch not waiting for
-            // the first, read the step before without a dependency of their own, and
-            // were no faster: 144x128x80 FP32 210 us a step, 206 with the events.)
-            const bool fork = nd > 0 && nb > nd;
-            if (fork) {
-                e = cudaEventRecord(d.forked, st);
-                if (e == cudaSuccess) e = cudaStreamWaitEvent(d.side, d.forked, 0);
-            }
-            if (e == cudaSuccess && nd > 0)
-                e = launch_smem(k_fused_solid<Q, S, TX, 4>, solid_smem<Q, S>(TX, 4), TX * 4, 512 / (TX * 4), nd, At(st, !fork),
-                                g, src, dst, d.nbm, P, d.partials);
-            if constexpr (sizeof(S) < 8) {
-                if (e == cudaSuccess && nb > nd) {
-                    MGeom gc = g;
-                    gc.items = g.items + nd;
-                    e = launch_bulk<S>(k_bulk<S, false>, nb - nd, At(fork ? d.side : st, !fork), gc, src, dst, P,
-                                       d.partials + 3 * nd);
-                }
-            }
-            if (fork) {
-                const cudaError_t e1 = cudaEventRecord(d.joined, d.side), e2 = cudaStreamWaitEvent(st, d.joined, 0);
-                if (e == cudaSuccess) e = e1 != cudaSuccess ? e1 : e2;
-            }
-        } else {
-            auto mix = [&](auto kern, int TX, int dyn) {
-                e = launch_smem(kern, dyn, TX, blocks_per_sm<S>(TX), nb, st, g, src, dst, d.nbm, P, d.partials);
-            };
-            if constexpr (sizeof(S) == 8) {
-                if (c.TX == 32) mix(k_mix<Q, S, 32>, 32, Mix<Q, S>::template smem<32>());
-                else mix(k_mix<Q, S, 128>, 128, Mix<Q, S>::template smem<128>());
-            } else {
-                if (c.TX == 256) mix(k_mix<Q, S, 256>, 256, Mix<Q, S>::template smem<256>());
-                else if (c.TX == 64) mix(k_mix<Q, S, 64>, 64, Mix<Q, S>::template smem<64>());
-                else mix(k_mix<Q, S, 128>, 128, Mix<Q, S>::template smem<128>());
-            }
-        }
+        e = solid_step<Q, S, false>(d, c, g, nb, src, dst, P, st);
         return e != cudaSuccess ? e : cudaGetLastError();
     }
-    cudaError_t e = cudaSuccess;
     if constexpr (sizeof(S) == 8) {
         // double storage is the parity path: one tile shape per lattice and size
         auto go = [&](auto kern, int threads) {

@@ -257,3 +257,62 @@ def test_solid_d3q19_steps_side_by_side_equal_one_grid(kind, precision):
         out.append(eng.get_populations())
         eng.close()
     assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("Q,shape,kind,tile", [
+    (9, (300, 48, 1), "walls", (0, 0)), (9, (161, 90, 1), "porous", (0, 0)), (9, (300, 48, 1), "block", (0, 7)),
+    (9, (300, 48, 1), "walls", (2, 0)), (9, (161, 90, 1), "block", (3, 5)), (19, (98, 165, 40), "walls", (0, 0)),
+    (19, (98, 165, 40), "speck", (0, 9))])
+def test_checked_steps_take_the_work_items(Q, shape, kind, tile):
+    """Clean and dirty blocks checked: nothing recorded, the unchecked step's bits."""
+    solid = _mask(Q, shape, kind)
+    f = W.to_aux(*W.spinodal(shape[1::-1] if Q == 9 else shape[::-1], seed=6, amp=0.1))
+    for a in f:
+        a[solid != 0] = 0.0
+    out = []
+    for checked in (False, True):
+        eng = tl.TernaryLB(Q, *shape, KAPPA, h=H, solid=solid.reshape(-1), precision="fp32")
+        eng.set_tile(*tile)
+        launches = eng.launches_per_step
+        eng.set_bounds_check(checked)
+        if Q == 19:
+            assert eng.launches_per_step == launches == 3
+        eng.init_fields(*f)
+        eng.step(6)
+        assert eng.bounds_check_word() == 0
+        out.append(eng.get_populations())
+        eng.close()
+    assert np.array_equal(out[0], out[1])
+
+
+def test_captured_steps_replay_with_solid_nodes():
+    """tlbm_step under stream capture, a change of tile between capture and replay, and a
+    capture begun after one."""
+    for Q, shape in ((9, (300, 90, 1)), (19, (98, 165, 40))):
+        solid = _mask(Q, shape, "walls")
+        f = W.to_aux(*W.spinodal(shape[1::-1] if Q == 9 else shape[::-1], seed=6, amp=0.1))
+        for a in f:
+            a[solid != 0] = 0.0
+        side = torch.cuda.Stream()
+        want = tl.TernaryLB(Q, *shape, KAPPA, h=H, solid=solid.reshape(-1), precision="fp32")
+        with torch.cuda.stream(side):
+            eng = tl.TernaryLB(Q, *shape, KAPPA, h=H, solid=solid.reshape(-1), precision="fp32")
+        for e in (want, eng):
+            e.init_fields(*f)
+            e.step(2)
+        graphs = []
+        for tile in ((0, 0), (2, 5)):
+            eng.set_tile(*tile)
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=side):
+                eng.step(2)
+            graphs.append(g)
+        eng.set_tile(3, 9)
+        with torch.cuda.stream(side):
+            for k in (0, 1, 0, 0, 1):
+                graphs[k].replay()
+        side.synchronize()
+        want.step(10)
+        assert np.array_equal(eng.get_populations(), want.get_populations())
+        want.close()
+        eng.close()
