@@ -387,7 +387,7 @@ __device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ 
         reinterpret_cast<unsigned char*>(dst) + (active ? (long long)(B0 + ty) * g.rowstride : 0) +
         (long long)chunk * F::CHUNK + lane * F::ESZ;
 
-    MassSum<float, true> msum;
+    MassSum<float, I::PACKED> msum;
     Roll<Q, float> roll;
     roll.clear();
     NodePops<S> cur, nxt;
@@ -470,7 +470,8 @@ __device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ 
             }
             push(rg, c1);
             if (p >= 2 && !late) {
-                msum.add(rdc, X[1], X[2]);
+                if constexpr (I::PACKED) msum.add(rdc, X[1], X[2]);
+                else msum.add(rho_total<Q, S>(rdc), X[1], X[2]);
                 unsigned char* const out = chk_node<Q, S, CHK>(g, reinterpret_cast<unsigned char*>(dst),
                                                                outb + (long long)(M0 + p - 2) * pstride, 3);
                 float fv[Q], gv[Q], kv[Q];

@@ -149,12 +149,12 @@ __device__ __forceinline__ int wrap1(int v, int n) { return v < 0 ? v + n : (v >
 
 // Mass totals (rho, phi, psi of the step's input state) of the nodes a thread
 // collides, given rd (rho, or rho - 1 where f is stored as f_i - w_i), phi, psi.
-// PAIR false sums in double, as the other kernels do.  PAIR true (float
-// formats) keeps per quantity an error-free pair (hi, lo) updated by Knuth's
-// TwoSum, and rho as the node count plus the summed deviations: no FP64
-// instruction runs per node, and the pairs become doubles once per block.
-// Measured on GB300: the pairs are 1-2 % faster.  The solid-aware FP32 D3Q19 body, at
-// its register limit, spills with them and keeps the double sums.
+// PAIR false sums in double, as the other kernels do.  PAIR true (16-bit formats, and
+// FP32 on D2Q9) keeps per quantity a pair (hi, lo) updated by Knuth's TwoSum, and rho as
+// the node count plus the summed deviations: no FP64 instruction runs per node, and
+// the pairs become doubles once per block; 1-2 % faster.  Its low words round in 24 bits
+// themselves, so sums of values far apart hold fewer bits than a double: FP32 on D3Q19
+// keeps the double sums.
 template <typename T, bool PAIR>
 struct MassSum {
     double r = 0.0, p = 0.0, s = 0.0;

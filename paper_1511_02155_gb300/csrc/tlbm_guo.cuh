@@ -517,7 +517,7 @@ __device__ __forceinline__ void guo_body(const MGeom& g, const S* __restrict__ s
         }
     };
 
-    constexpr bool PAIR = Fmt<Q, S>::OFFSET;
+    constexpr bool PAIR = Fmt<Q, S>::OFFSET && !(Q == 19 && sizeof(S) == 4);
     MassSum<T, PAIR> msum;
 
     grid_ready();

@@ -8,6 +8,8 @@ Bounds, per population:
 - 16-bit storage: 2e-6 plus half a unit in the last place of the stored value,
   |x| 2^-11 (FP16) or |x| 2^-8 (BF16), at the largest moving deviation.
 """
+import math
+
 import numpy as np
 import pytest
 
@@ -316,3 +318,28 @@ def test_captured_steps_replay_with_solid_nodes():
         assert np.array_equal(eng.get_populations(), want.get_populations())
         want.close()
         eng.close()
+
+
+@pytest.mark.parametrize("forcing", [False, True])
+@pytest.mark.parametrize("chunk", [0, 64])
+def test_totals_of_d3q19_fp32_are_double_sums(chunk, forcing):
+    """Values of one column whose sum has 52 bits, and so is exact in double in any order;
+    pairs of floats round it."""
+    shape, rng = (4, 4, 64), np.random.default_rng(9)
+    v = np.concatenate([1 + 2.0 ** -23 * rng.integers(1, 2 ** 22, 32), 2.0 ** -45 * rng.integers(2 ** 19, 2 ** 20, 32)])
+    v = v.astype(np.float32).astype(np.float64)
+    eng = tl.TernaryLB(19, *shape, KAPPA, precision="fp32")
+    if forcing:
+        eng.set_coupling("forcing")
+    eng.set_tile(0, chunk)
+    one, zero = np.ones(eng.N), np.zeros(eng.N)
+    eng.init_fields(one, zero, zero)
+    P = eng.get_populations()
+    P[1:] = 0.0
+    for s, sign in ((1, -1.0), (2, 1.0)):  # rest populations phi and psi of the column at (2, 1)
+        P[s, 0].reshape(64, 4, 4)[:, 1, 2] = sign * v
+    eng.set_populations(P)
+    eng.step(1)
+    m = eng.step_mass()
+    assert m[2] == math.fsum(v) and m[1] == -math.fsum(v)
+    eng.close()
