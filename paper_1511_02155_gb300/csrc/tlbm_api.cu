@@ -58,6 +58,13 @@ tlbm_status fail(tlbm* t, tlbm_status s, const char* fmt, ...) {
     return s;
 }
 
+// Host containers are the one thing here that throws.  What a call catches at the
+// boundary, with its message short enough to need no memory.
+tlbm_status no_memory(std::string& err) {
+    err = "out of memory";
+    return TLBM_ERR_OOM;
+}
+
 #define CK(call)                                                                              \
     do {                                                                                      \
         cudaError_t e_ = (call);                                                              \
@@ -267,10 +274,9 @@ void tlbm_destroy(tlbm* t) {
     delete t;
 }
 
-tlbm_status tlbm_create(tlbm** out, tlbm_lattice lattice, int nx, int ny, int nz, const double kappa[3],
-                        double alpha, double tau_f, double M_phi, double M_psi, const double h[3],
-                        const uint8_t* solid_mask, tlbm_precision precision, void* cuda_stream) {
-    tlbm* t = nullptr;
+static tlbm_status create(tlbm*& t, tlbm** out, tlbm_lattice lattice, int nx, int ny, int nz, const double kappa[3],
+                          double alpha, double tau_f, double M_phi, double M_psi, const double h[3],
+                          const uint8_t* solid_mask, tlbm_precision precision, void* cuda_stream) {
     g_create_err.clear();
     if (!out) return fail(nullptr, TLBM_ERR_ARG, "out is NULL");
     *out = nullptr;
@@ -345,6 +351,7 @@ tlbm_status tlbm_create(tlbm** out, tlbm_lattice lattice, int nx, int ny, int nz
     auto bail = [&](tlbm_status s) {
         g_create_err = t->err;
         tlbm_destroy(t);
+        t = nullptr;
         return s;
     };
     const size_t popbytes = (size_t)d.pop_bytes;
@@ -408,6 +415,18 @@ tlbm_status tlbm_create(tlbm** out, tlbm_lattice lattice, int nx, int ny, int nz
     return TLBM_OK;
 }
 
+tlbm_status tlbm_create(tlbm** out, tlbm_lattice lattice, int nx, int ny, int nz, const double kappa[3],
+                        double alpha, double tau_f, double M_phi, double M_psi, const double h[3],
+                        const uint8_t* solid_mask, tlbm_precision precision, void* cuda_stream) {
+    tlbm* t = nullptr;
+    try {
+        return create(t, out, lattice, nx, ny, nz, kappa, alpha, tau_f, M_phi, M_psi, h, solid_mask, precision, cuda_stream);
+    } catch (...) {
+        tlbm_destroy(t);
+        return no_memory(g_create_err);
+    }
+}
+
 tlbm_status tlbm_set_gamma(tlbm* t, double gamma_phi, double gamma_psi) {
     if (!t) return TLBM_ERR_ARG;
     if (!(gamma_phi > 0) || !(gamma_psi > 0)) return fail(t, TLBM_ERR_PARAM, "Gamma must be > 0");
@@ -433,7 +452,7 @@ tlbm_kernel tlbm_get_kernel(const tlbm* t) {
 }
 
 // Tile choice of the fused step: variant (0 = default) and planes per chunk (0 = auto).
-tlbm_status tlbm_set_tile(tlbm* t, int variant, int chunk) {
+tlbm_status tlbm_set_tile(tlbm* t, int variant, int chunk) try {
     if (!t) return TLBM_ERR_ARG;
     if (variant < 0 || variant > 255 || (variant & 15) > 7 || chunk < 0 || chunk > 4096)
         return fail(t, TLBM_ERR_ARG, "bad tile");
@@ -441,6 +460,8 @@ tlbm_status tlbm_set_tile(tlbm* t, int variant, int chunk) {
     // partial sums must fit: blocks grow as chunks shrink (checked by the step)
     CK(set_items(t));
     return TLBM_OK;
+} catch (...) {
+    return no_memory(t->err);
 }
 
 tlbm_status tlbm_set_coupling(tlbm* t, tlbm_coupling coupling) {
@@ -513,7 +534,7 @@ tlbm_status tlbm_init_fields(tlbm* t, const double* rho, const double* phi, cons
     return TLBM_OK;
 }
 
-tlbm_status tlbm_step(tlbm* t, int64_t nsteps) {
+tlbm_status tlbm_step(tlbm* t, int64_t nsteps) try {
     if (!t) return TLBM_ERR_ARG;
     if (nsteps < 0) return fail(t, TLBM_ERR_ARG, "nsteps must be >= 0");
     const int kind = resolve_kind(t);
@@ -537,6 +558,8 @@ tlbm_status tlbm_step(tlbm* t, int64_t nsteps) {
     }
     if (nsteps > 0) CK(t->ops->totals(t->d, kind, t->st));
     return TLBM_OK;
+} catch (...) {
+    return no_memory(t->err);
 }
 
 int64_t tlbm_steps_done(const tlbm* t) { return t ? t->steps : -1; }
@@ -560,9 +583,11 @@ tlbm_status tlbm_kernel_time(const tlbm* t, double* ms_total, int64_t* steps) {
     return TLBM_OK;
 }
 
-int tlbm_launches_per_step(const tlbm* t) {
+int tlbm_launches_per_step(const tlbm* t) try {
     if (!t) return -1;
     return t->ops->launches(t->d, resolve_kind(t));
+} catch (...) {
+    return -1;
 }
 
 tlbm_status tlbm_fields(tlbm* t, double* C1, double* C2, double* C3, double* rho, double* u) {
@@ -678,7 +703,7 @@ tlbm_status tlbm_set_state(tlbm* t, const void* host, size_t bytes) {
 }
 
 tlbm_status tlbm_adjoint_c3_misfit(tlbm* t, int64_t nsteps, int checkpoint_every, const double* target,
-                                   double* loss, double dkappa[3], double dh[3], double* dfields) {
+                                   double* loss, double dkappa[3], double dh[3], double* dfields) try {
     if (!t) return TLBM_ERR_ARG;
     if (nsteps < 1 || checkpoint_every < 1) return fail(t, TLBM_ERR_ARG, "nsteps and checkpoint_every must be >= 1");
     if (!target || !loss || !dkappa || !dh) return fail(t, TLBM_ERR_ARG, "target, loss, dkappa and dh are required");
@@ -709,15 +734,15 @@ tlbm_status tlbm_adjoint_c3_misfit(tlbm* t, int64_t nsteps, int checkpoint_every
         at[k] = total;
         total += (sizes[k] + 511) / 512 * 512;
     }
-    void* block = nullptr;  // one allocation for the run
-    cudaError_t e = cudaMalloc(&block, total);
-    auto release = [&]() { cudaFree(block); };
-    if (e != cudaSuccess) {
-        release();
+    struct Block {  // one allocation for the run
+        void* at = nullptr;
+        ~Block() { cudaFree(at); }
+    } block;
+    cudaError_t e = cudaMalloc(&block.at, total);
+    if (e != cudaSuccess)
         return fail(t, TLBM_ERR_OOM, "adjoint buffers (%zu MB of checkpoints and segment states): %s",
                     (sizes[0] + sizes[1]) >> 20, cudaGetErrorString(e));
-    }
-    char* const base = static_cast<char*>(block);
+    char* const base = static_cast<char*>(block.at);
     J.ckpt = base + at[0];
     J.seg = base + at[1];
     J.fin = base + at[2];
@@ -739,7 +764,6 @@ tlbm_status tlbm_adjoint_c3_misfit(tlbm* t, int64_t nsteps, int checkpoint_every
     int flag = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, t->d.flag, sizeof flag, cudaMemcpyDeviceToHost, t->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(t->st);
-    release();
     if (e != cudaSuccess) return fail(t, TLBM_ERR_CUDA, "adjoint run: %s", cudaGetErrorString(e));
     t->steps += nsteps;
     t->rest_init = 0;
@@ -757,6 +781,8 @@ tlbm_status tlbm_adjoint_c3_misfit(tlbm* t, int64_t nsteps, int checkpoint_every
     if (s != TLBM_OK) return s;
     if (!std::isfinite(*loss)) return fail(t, TLBM_ERR_NONFINITE, "non-finite loss");
     return TLBM_OK;
+} catch (...) {
+    return no_memory(t->err);
 }
 
 }  // extern "C"
@@ -852,7 +878,7 @@ tlbm_status batch_totals(tlbm_batch* b) {
 
 extern "C" {
 
-tlbm_status tlbm_batch_create(tlbm_batch** out, tlbm* const* members, int count) {
+static tlbm_status create_batch(tlbm_batch*& b, tlbm_batch** out, tlbm* const* members, int count) {
     g_create_err.clear();
     if (!out || !members || count < 1) return bfail(nullptr, TLBM_ERR_ARG, "need at least one member");
     *out = nullptr;
@@ -871,11 +897,11 @@ tlbm_status tlbm_batch_create(tlbm_batch** out, tlbm* const* members, int count)
         for (int j = 0; j < k; ++j)
             if (members[j] == m) return bfail(nullptr, TLBM_ERR_ARG, "member %d appears twice", k);
     }
-    tlbm_batch* b = new tlbm_batch();
+    b = new tlbm_batch();
+    b->st = members[0]->st;
     b->members.assign(members, members + count);
     for (tlbm* m : b->members) b->sims.push_back(&m->d);
     b->ops = members[0]->ops;
-    b->st = members[0]->st;
     b->cap = nullptr;
     b->exec = nullptr;
     b->graph_par = 0;
@@ -892,10 +918,21 @@ tlbm_status tlbm_batch_create(tlbm_batch** out, tlbm* const* members, int count)
     if (s != TLBM_OK) {
         g_create_err = b->err;
         tlbm_batch_destroy(b);
+        b = nullptr;
         return s;
     }
     *out = b;
     return TLBM_OK;
+}
+
+tlbm_status tlbm_batch_create(tlbm_batch** out, tlbm* const* members, int count) {
+    tlbm_batch* b = nullptr;
+    try {
+        return create_batch(b, out, members, count);
+    } catch (...) {
+        tlbm_batch_destroy(b);
+        return no_memory(g_create_err);
+    }
 }
 
 void tlbm_batch_destroy(tlbm_batch* b) {
@@ -915,7 +952,7 @@ const char* tlbm_batch_last_error(const tlbm_batch* b) { return b ? b->err.c_str
 
 int64_t tlbm_batch_blocks(const tlbm_batch* b) { return b ? (int64_t)b->bs.blocks : -1; }
 
-tlbm_status tlbm_batch_set_tile(tlbm_batch* b, int variant, int chunk) {
+tlbm_status tlbm_batch_set_tile(tlbm_batch* b, int variant, int chunk) try {
     if (!b) return TLBM_ERR_ARG;
     if (variant < 0 || variant > 255 || (variant & 15) > 7 || chunk < 0 || chunk > 4096)
         return bfail(b, TLBM_ERR_ARG, "bad tile");
@@ -927,6 +964,8 @@ tlbm_status tlbm_batch_set_tile(tlbm_batch* b, int variant, int chunk) {
         batch_rebuild(b);
     }
     return s;
+} catch (...) {
+    return no_memory(b->err);
 }
 
 tlbm_status tlbm_batch_set_graph(tlbm_batch* b, int on) {
@@ -955,7 +994,7 @@ tlbm_status tlbm_batch_kernel_time(const tlbm_batch* b, double* ms_total, int64_
     return TLBM_OK;
 }
 
-tlbm_status tlbm_batch_step(tlbm_batch* b, int64_t nsteps) {
+tlbm_status tlbm_batch_step(tlbm_batch* b, int64_t nsteps) try {
     if (!b) return TLBM_ERR_ARG;
     if (nsteps < 0) return bfail(b, TLBM_ERR_ARG, "nsteps must be >= 0");
     tlbm_status s = batch_aligned(b);
@@ -979,8 +1018,15 @@ tlbm_status tlbm_batch_step(tlbm_batch* b, int64_t nsteps) {
         if (e == cudaSuccess) e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return bfail(b, TLBM_ERR_CUDA, "graph capture: %s", cudaGetErrorString(e));
         const int par = b->sims[0]->cur;
-        cudaError_t e1 = b->ops->batch_step(b->bs, b->cap, nullptr, nullptr);
-        cudaError_t e2 = b->ops->batch_step(b->bs, b->cap, nullptr, nullptr);  // parity is back to par
+        auto captured = [&]() -> cudaError_t {  // the capture ends whatever happens
+            try {
+                return b->ops->batch_step(b->bs, b->cap, nullptr, nullptr);
+            } catch (...) {
+                return cudaErrorMemoryAllocation;
+            }
+        };
+        cudaError_t e1 = captured();
+        cudaError_t e2 = e1 == cudaSuccess ? captured() : e1;  // parity is back to par
         cudaGraph_t graph = nullptr;
         e = cudaStreamEndCapture(b->cap, &graph);
         if (e == cudaSuccess && e1 == cudaSuccess && e2 == cudaSuccess)
@@ -989,6 +1035,7 @@ tlbm_status tlbm_batch_step(tlbm_batch* b, int64_t nsteps) {
         if (e == cudaSuccess) e = (e1 != cudaSuccess) ? e1 : e2;
         if (e != cudaSuccess) {
             drop_graph(b);
+            for (DevState* d : b->sims) d->cur = par;  // nothing has run
             return bfail(b, TLBM_ERR_CUDA, "graph capture: %s", cudaGetErrorString(e));
         }
         b->graph_par = par;
@@ -1000,9 +1047,11 @@ tlbm_status tlbm_batch_step(tlbm_batch* b, int64_t nsteps) {
     }
     s = batch_plain_steps(b, nsteps & 1);
     return s == TLBM_OK ? batch_totals(b) : s;
+} catch (...) {
+    return no_memory(b->err);
 }
 
-tlbm_status tlbm_batch_autotune(tlbm_batch* b, int trial_steps, int* variant, int* chunk) {
+tlbm_status tlbm_batch_autotune(tlbm_batch* b, int trial_steps, int* variant, int* chunk) try {
     if (!b || trial_steps < 1) return TLBM_ERR_ARG;
     tlbm_status s = batch_aligned(b);
     if (s != TLBM_OK) return s;
@@ -1045,6 +1094,8 @@ tlbm_status tlbm_batch_autotune(tlbm_batch* b, int trial_steps, int* variant, in
     if (variant) *variant = bv;
     if (chunk) *chunk = bc;
     return best < 3.0e38f ? TLBM_OK : bfail(b, TLBM_ERR_CUDA, "no tile candidate ran");
+} catch (...) {
+    return no_memory(b->err);
 }
 
 }  // extern "C"

@@ -13,6 +13,7 @@
 #include <deque>
 #include <functional>
 #include <map>
+#include <new>
 #include <set>
 #include <string>
 #include <vector>
@@ -24,7 +25,7 @@ namespace {
 std::map<cudaStream_t, std::deque<std::function<void()>>> queues;
 std::map<void*, size_t> live;
 std::string text, failing;
-int fail_in = 0, next_flag = 0, capturing = 0, build_fails = 0;
+int fail_in = 0, throws = 0, next_flag = 0, capturing = 0, build_fails = 0;
 std::map<int, std::vector<int4>> items;  // by tile; fake_items
 
 void note(const char* fmt, long long a = 0, long long b = 0, long long c = 0) {
@@ -45,6 +46,9 @@ void drain(cudaStream_t s) {
 void drain_all() {
     for (auto& q : queues) drain(q.first);
 }
+void maybe_throw() {
+    if (throws) throw std::bad_alloc();
+}
 bool alive(const void* p) {
     for (auto& m : live)
         if ((const char*)p >= (char*)m.first && (const char*)p < (char*)m.first + m.second) return true;
@@ -60,7 +64,7 @@ void fake_reset() {
     drain_all();
     text.clear();
     failing.clear();
-    fail_in = next_flag = capturing = build_fails = 0;
+    fail_in = throws = next_flag = capturing = build_fails = 0;
     items.clear();
 }
 const char* fake_log() { return text.c_str(); }
@@ -75,6 +79,7 @@ void fake_items(int tile, int n) {  // the work items of that tile
 void fake_flag(int v) { next_flag = v; }         // raised by the next steps
 void fake_capturing(int on) { capturing = on; }  // every stream
 void fake_build_fails(int n) { build_fails = n; }
+void fake_throws(int on) { throws = on; }  // the kernel tables' host code
 int fake_allocations() { return (int)live.size(); }
 
 // ---- CUDA runtime
@@ -154,6 +159,7 @@ namespace tlbm_host {
 namespace {
 
 cudaError_t step(DevState& d, int, cudaStream_t st, cudaEvent_t, cudaEvent_t) {
+    maybe_throw();
     const int4* it = static_cast<const int4*>(d.items);
     const int n = d.nitems, raise = next_flag;
     int* const flag = d.flag;
@@ -176,24 +182,31 @@ cudaError_t mass(DevState&, double* out, cudaStream_t st) {
 }
 cudaError_t get_box(DevState&, int, int, int, int, int, int, double*, cudaStream_t) { return cudaSuccess; }
 cudaError_t set_pops(DevState&, const double*, cudaStream_t) { return cudaSuccess; }
-int launches(const DevState&, int) { return 2; }
+int launches(const DevState&, int) {
+    maybe_throw();
+    return 2;
+}
 int aux_per_node() { return 8; }
 bool has_fused(const DevState&) { return true; }
 int solid_items(const DevState& d, std::vector<int4>& out) {
+    maybe_throw();
     out = items[d.tile];
     return (int)out.size();
 }
 cudaError_t batch_build(BatchState&, cudaStream_t) {
+    maybe_throw();
     note("batch build");
     return build_fails > 0 && build_fails-- ? cudaErrorInvalidConfiguration : cudaSuccess;
 }
 cudaError_t batch_step(BatchState& b, cudaStream_t, cudaEvent_t, cudaEvent_t) {
+    maybe_throw();
     note("batch step");
     for (int k = 0; k < b.count; ++k) b.sims[k]->cur ^= 1;
     return cudaSuccess;
 }
 cudaError_t batch_totals(BatchState&, cudaStream_t) { return cudaSuccess; }
 cudaError_t adjoint(DevState& d, int, const AdjJob& J, cudaStream_t st) {
+    maybe_throw();
     const int raise = next_flag;
     int* const flag = d.flag;
     double* const acc = J.acc;

@@ -192,3 +192,37 @@ def test_a_gradient_from_a_void_state_says_so(fake, flag, status):
     loss, out = ctypes.c_double(), (ctypes.c_double * 3)()
     assert fake.tlbm_adjoint_c3_misfit(t, 3, 2, one, ctypes.byref(loss), out, out, None) == status
     fake.tlbm_destroy(t)
+
+
+def test_no_exception_leaves_the_c_entries(fake):
+    """Host memory that runs out is TLBM_ERR_OOM, with nothing left behind."""
+    oom = 4
+    rc, t = _create(fake)
+    rc2, t2 = _create(fake)
+    assert rc == rc2 == 0
+    one = np.ones(N[0] * N[1]).ctypes.data_as(dp)
+    assert fake.tlbm_init_fields(t, one, one, one, None, None, None) == 0
+    b = ctypes.c_void_p()
+    assert fake.tlbm_batch_create(ctypes.byref(b), (ctypes.c_void_p * 1)(t2), 1) == 0
+    held = fake.fake_allocations()
+    fake.fake_throws(1)
+    assert _create(fake)[0] == oom and b"memory" in fake.tlbm_last_error(None)
+    none = ctypes.c_void_p()
+    assert fake.tlbm_batch_create(ctypes.byref(none), (ctypes.c_void_p * 1)(t), 1) == oom and not none.value
+    fake.fake_items(256 * 9, 3)
+    loss, out = ctypes.c_double(), (ctypes.c_double * 3)()
+    assert fake.tlbm_adjoint_c3_misfit(t, 3, 2, one, ctypes.byref(loss), out, out, None) == oom
+    assert fake.tlbm_set_tile(t, 0, 9) == oom
+    assert fake.tlbm_step(t, 1) == oom and b"memory" in fake.tlbm_last_error(t)
+    assert fake.tlbm_launches_per_step(t) == -1
+    assert fake.tlbm_batch_step(b, 1) == oom and b"memory" in fake.tlbm_batch_last_error(b)
+    assert fake.tlbm_batch_set_tile(b, 0, 9) == oom
+    assert fake.tlbm_batch_autotune(b, 1, None, None) == oom
+    fake.fake_throws(0)
+    assert fake.fake_allocations() == held
+    assert fake.tlbm_batch_step(b, 1) == 0  # builds again first
+    assert _steps(fake, t) == "step: one grid"
+    fake.tlbm_batch_destroy(b)
+    fake.tlbm_destroy(t)
+    fake.tlbm_destroy(t2)
+    assert fake.fake_allocations() == 0
