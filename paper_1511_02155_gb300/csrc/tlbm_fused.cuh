@@ -211,7 +211,7 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
     using T = typename Store<S>::T;
     using A = Axes<Q>;
     extern __shared__ __align__(16) unsigned char tlbm_smem[];
-    constexpr bool CHK = false;  // the checked kernels are those of FP32 storage
+    static_assert(sizeof(S) == 8, "the other storages take their populations by bulk copies");
     constexpr int D = Lat<Q>::D;
     constexpr int HY = (D == 3) ? 1 : 0;  // halo rows along b
     constexpr int HW = TX + 2;
@@ -257,7 +257,7 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
         }
 #pragma unroll
         for (int n = 0; n < 2; ++n) {
-            h[n] = (int)chk_index<CHK>(g, hy[n] * HW + hx[n], HN, 4);
+            h[n] = hy[n] * HW + hx[n];
             const int aa = modp(A0 + hx[n] - 1, g.NA);
             const int bb = (D == 3) ? modp(B0 + hy[n] - HY, g.NB) : 0;
             const int xs[3] = {wrap1(aa - 1, g.NA), aa, wrap1(aa + 1, g.NA)};
@@ -277,11 +277,11 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
     constexpr int BN = NT >= 64 ? 1 : 2;
     const int lane = tid & 31;
     const bool bwarp = D == 2 && (NT < 64 || tid < 64);
-    int boff[BN], bslot[BN], bval_off = 0, bcm = 0, bdir = 0;  // byte offset in a row, ring slot; of the lane's population
+    int boff[BN], bslot[BN], bval_off = 0, bcm = 0;  // byte offset in a row, ring slot; of the lane's population
     if constexpr (D == 2) {
         const int l = lane < 3 * Q ? lane : 3 * Q - 1, bs = l / Q;
         int bca = 0;
-        bdir = l % Q;
+        const int bdir = l % Q;
 #pragma unroll
         for (int i = 0; i < Q; ++i)
 #pragma unroll
@@ -301,17 +301,15 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
     }
 
     const unsigned char* srcb = reinterpret_cast<const unsigned char*>(src);
-    // stored value (x - bias) of (s, i) at node pointer p
     auto ldp = [&](const unsigned char* p, int s, int i) -> T { return Fmt<Q, S>::ld_delta(p, s, i); };
     // pull source of direction (ca, cb, cm) for node n at plane rows zr
     auto src_of = [&](int n, const int (&zr)[3], int ca, int cb, int cm) -> const unsigned char* {
         const long long row = (long long)zr[1 - cm] * g.NB + yb[n][1 - cb];
-        return chk_node<Q, S, CHK>(g, srcb, srcb + row * g.rowstride + xc[n][1 - ca], 1);
+        return srcb + row * g.rowstride + xc[n][1 - ca];
     };
 
     // Phase M: moments of plane m for this thread's nodes into ring slot `slot`;
-    // node 0's momentum density is returned in j and its summed f deviations
-    // (rho - 1 in the 16-bit formats, rho otherwise) in rd.
+    // node 0's momentum density is returned in j and its rho in rd.
     auto moments_plane = [&](int m, int slot, T (&j)[3], T& rd) {
         const int mm = wrap1(m, g.NM);
         const int zr[3] = {wrap1(mm - 1, g.NM), mm, wrap1(mm + 1, g.NM)};
@@ -323,21 +321,14 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
             if (bwarp) {
                 const int row = bcm == 0 ? zr[1] : (bcm > 0 ? zr[0] : zr[2]);
 #pragma unroll
-                for (int n = 0; n < BN; ++n) {
-                    const unsigned char* p =
-                        chk_node<Q, S, CHK>(g, srcb, srcb + (long long)row * g.rowstride + boff[n], 1) + bval_off;
-                    if (Fmt<Q, S>::PACKED && bdir == 0) bval[n] = *reinterpret_cast<const T*>(p);
-                    else bval[n] = Store<S>::get(*reinterpret_cast<const S*>(p));
-                }
+                for (int n = 0; n < BN; ++n)
+                    bval[n] = *reinterpret_cast<const T*>(srcb + (long long)row * g.rowstride + boff[n] + bval_off);
             }
         }
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             const unsigned char* p0 = src_of(0, zr, A::ca(i), A::cb(i), A::cm(i));
-            T f, gg;
-            if (Fmt<Q, S>::PAIRED && i > 0) Fmt<Q, S>::ld_fg(p0, i, f, gg);  // one lane word
-            else f = ldp(p0, 0, i), gg = ldp(p0, 1, i);
-            const T kk = ldp(p0, 2, i);
+            const T f = ldp(p0, 0, i), gg = ldp(p0, 1, i), kk = ldp(p0, 2, i);
             rho0 += f;
             if (A::ca(i)) ja += T(A::ca(i)) * f;
             if (A::cb(i)) jb += T(A::cb(i)) * f;
@@ -349,23 +340,12 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
                 const unsigned char* p1 = src_of(1, zr, A::ca(i), A::cb(i), A::cm(i));
-                if (Fmt<Q, S>::PAIRED && i > 0) {
-                    T a, b;
-                    Fmt<Q, S>::ld_fg(p1, i, a, b);
-                    rho1 += a;
-                    phi1 += b;
-                } else {
-                    rho1 += ldp(p1, 0, i);
-                    phi1 += ldp(p1, 1, i);
-                }
+                rho1 += ldp(p1, 0, i);
+                phi1 += ldp(p1, 1, i);
                 psi1 += ldp(p1, 2, i);
             }
         }
         rd = rho0;
-        if (Fmt<Q, S>::OFFSET) {  // sums of f deviations: rho - 1
-            rho0 += T(1);
-            rho1 += T(1);
-        }
         sm[slot][0][h[0]] = rho0;
         sm[slot][1][h[0]] = phi0;
         sm[slot][2][h[0]] = psi0;
@@ -376,9 +356,7 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
                     T acc = T(0);
 #pragma unroll
                     for (int i = 0; i < Q; ++i) acc += __shfl_sync(0xffffffffu, bval[n], (lane % 3) * Q + i);
-                    if (lane < 3)
-                        sm[slot][lane][(int)chk_index<CHK>(g, bslot[n], HN, 4)] =
-                            Fmt<Q, S>::OFFSET && lane == 0 ? acc + T(1) : acc;
+                    if (lane < 3) sm[slot][lane][bslot[n]] = acc;
                 }
             }
         }
@@ -392,8 +370,7 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
         j[2] = jm;
     };
 
-    constexpr bool PAIR = Fmt<Q, S>::OFFSET;
-    MassSum<T, PAIR> msum;
+    MassSum<T, false> msum;
     T jc[3], jn[3], rdc, rdn;
 
     grid_ready();
@@ -410,11 +387,7 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
     auto push_plane = [&](int m, T (&X)[3], T (&gr)[3][3], T (&la)[3]) {
         const int slot = m & 3;
         const T c1[3] = {sm[slot][0][h[0]], sm[slot][1][h[0]], sm[slot][2][h[0]]};
-        roll.push(
-            [&](int k, int i, int jj) -> T {
-                return sm[slot][k][(int)chk_index<CHK>(g, h[0] + jj * HW + i, HN, 4)];
-            },
-            c1, X, gr, la);
+        roll.push([&](int k, int i, int jj) -> T { return sm[slot][k][h[0] + jj * HW + i]; }, c1, X, gr, la);
     };
     if (KEEP) {
         __syncthreads();
@@ -432,8 +405,7 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
         }
         push_plane(m + 1, X0, g12, l6);
         if (active) {
-            // stored values (deviations x - bias) of the node's pulled populations: phase M
-            // read them one iteration ago
+            // the node's pulled populations: phase M read them one iteration ago
             const int zr[3] = {wrap1(m - 1, g.NM), m, wrap1(m + 1, g.NM)};
             T fv[Q], gv[Q], kv[Q];
 #pragma unroll
@@ -444,11 +416,9 @@ __device__ __forceinline__ void fused_body(const MGeom& g, const S* __restrict__
                 kv[i] = ldp(pi, 2, i);
             }
             const T jl[3] = {jc[0], D == 3 ? jc[1] : jc[2], D == 3 ? jc[2] : T(0)};  // lattice axes
-            if constexpr (PAIR) msum.add(rdc, X0[1], X0[2]);
-            else msum.add(rho_total<Q, S>(rdc), X0[1], X0[2]);
-            unsigned char* out = chk_node<Q, S, CHK>(
-                g, reinterpret_cast<unsigned char*>(dst),
-                reinterpret_cast<unsigned char*>(dst) + ((long long)m * g.NB + yb[0][1]) * g.rowstride + xc[0][1], 3);
+            msum.add(rho_total<Q, S>(rdc), X0[1], X0[2]);
+            unsigned char* out =
+                reinterpret_cast<unsigned char*>(dst) + ((long long)m * g.NB + yb[0][1]) * g.rowstride + xc[0][1];
             collide_node<Q, S, false>(out, fv, gv, kv, rdc, X0, jl, g12, l6, P);
         }
         jc[0] = jn[0];

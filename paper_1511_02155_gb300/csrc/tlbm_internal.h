@@ -77,7 +77,6 @@ struct BatchState {
     int auto_tile;       // the same with the chunk resolved for the whole grid
     int narrow;          // every member takes one-warp rows (D2Q9 in double)
     long long blocks;    // blocks of one batched step
-    int built;           // descriptors are current
 };
 
 // Buffers of one adjoint run (all device memory, allocated by the caller).

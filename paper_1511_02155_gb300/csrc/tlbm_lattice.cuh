@@ -276,25 +276,10 @@ struct Fmt {
             return *reinterpret_cast<const S*>(n + off(s, i));
         }
     }
-    // value from its stored deviation and back (no add where the bias is zero:
-    // x + 0 is not x for x = -0, so the compiler would keep it)
-    static __device__ __forceinline__ T unbias(int s, int i, T d) {
-        const double b = bias(s, i);
-        return b == 0.0 ? d : d + T(b);
-    }
-    static __device__ __forceinline__ T dev(int s, int i, T v) {
-        const double b = bias(s, i);
-        return b == 0.0 ? v : v - T(b);
-    }
     // population (s, i) at node pointer n
     static __device__ __forceinline__ T ld(const unsigned char* n, int s, int i) {
         const double b = bias(s, i);
         return b == 0.0 ? ld_delta(n, s, i) : ld_delta(n, s, i) + T(b);
-    }
-    // the same, marking the line evict-first (its last use in this kernel)
-    static __device__ __forceinline__ T ld_last(const unsigned char* n, int s, int i) {
-        const double b = bias(s, i);
-        return b == 0.0 ? ld_last_delta(n, s, i) : ld_last_delta(n, s, i) + T(b);
     }
     // stored value of (s, i), marking the line evict-first (its last use)
     static __device__ __forceinline__ T ld_last_delta(const unsigned char* n, int s, int i) {
@@ -332,11 +317,6 @@ struct Fmt {
             if (i > 0) return Store<S>::get(Store<S>::put(d));
         }
         return d;
-    }
-    // store with an evict-first hint (streamed out, read only by the next step)
-    static __device__ __forceinline__ void st_stream(unsigned char* n, int s, int i, T v) {
-        const double b = bias(s, i);
-        st_stream_delta(n, s, i, b == 0.0 ? v : v - T(b));
     }
     // store the deviation d = x - bias of (s, i)
     static __device__ __forceinline__ void st_delta(unsigned char* n, int s, int i, T d) {

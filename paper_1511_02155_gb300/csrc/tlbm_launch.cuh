@@ -29,11 +29,13 @@ inline int grid_of(long long n, int sms) {
 // moments with the halo), and below that by the latency of a warp's own chain (3.5
 // us for either): 64x64 takes one plane a block, walled 256x128 two (seven, the
 // choice by operations alone, left 1.7 warps on an SM).
-// Against the measured times of 14 lattices (64^2 .. 1000x701, 40^3 .. 160^2x96)
-// over chunks of 1 .. 64 planes the cheapest chunk of this model is within 8 % of
-// the fastest measured; halving 64 or 16 until 4 blocks per SM are reached, the
-// earlier rule, lost up to 27 % (FP32, one step: 64x64 15.4 us against 11.3,
-// 96^3 117.4 against 102.9, walled 144x128x80 299 against 267).
+// The constants of FP32 and 16 bits were fitted to kernels with plain loads; against the
+// present ones, over 57 lattices (64^2 .. 2048x1024, 40^3 .. 160^2x96, periodic and
+// between walls, all storages) and 15 chunks of 1 .. 64 planes, the chosen chunk is the
+// fastest to 1 % for 41, within 6 % for 48, and 7 to 15 % off for D3Q19 between walls
+// and 256x128 between walls; 40^3, periodic, takes six planes where three are 26 %
+// faster (FP32; 16 bits 19 %).  Halving 64 or 16 until 4 blocks per SM are reached, the
+// earlier rule, had lost up to 27 % with the kernels it was made for.
 inline double march_cost(double nb, int mc, int halo, int res, int threads, int sms, bool dbl) {
     const double full = (double)res * sms;
     if (dbl) {
@@ -619,7 +621,6 @@ inline cudaError_t batch_build(tlbm_host::BatchState& b, cudaStream_t st) {
     if (!b.desc) e = cudaMalloc(&b.desc, sizeof(SimDesc<T>) * 2 * (size_t)n);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b.desc, h.data(), sizeof(SimDesc<T>) * 2 * (size_t)n, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e == cudaSuccess) b.built = 1;
     return e;
 }
 
