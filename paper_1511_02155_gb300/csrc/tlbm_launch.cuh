@@ -36,7 +36,11 @@ inline int grid_of(long long n, int sms) {
 // and 256x128 between walls; 40^3, periodic, takes six planes where three are 26 %
 // faster (FP32; 16 bits 19 %).  Halving 64 or 16 until 4 blocks per SM are reached, the
 // earlier rule, had lost up to 27 % with the kernels it was made for.
-inline double march_cost(double nb, int mc, int halo, int res, int threads, int sms, bool dbl) {
+// Solid-aware blocks (`solid`) wait for one another's loads less: a plane takes 0.62 +
+// 0.095 b' of a full SM's (porous lattices, 5 % solid, FP32 517x391: 2.3, 2.6, 3.1, 3.2 us
+// a plane at 1 to 4 blocks; 300x20x20 5.7, 6.3, 8.7 at 1, 2, 4).  By the other curve
+// 300x20x20 took seven planes a block, 62.3 us a step; at two it is 52.2.
+inline double march_cost(double nb, int mc, int halo, int res, int threads, int sms, bool dbl, bool solid) {
     const double full = (double)res * sms;
     if (dbl) {
         const double per = nb / sms, b = per > 8.0 ? per : (double)(long long)(per + 0.9999);
@@ -44,7 +48,8 @@ inline double march_cost(double nb, int mc, int halo, int res, int threads, int 
         const double chain = 3.5 * (2 * mc + halo), units = b * warps * (2.8 * mc + 0.75 * (mc + halo));
         return chain > units ? chain : units;
     }
-    auto plane = [&](double b) { return 0.25 + 0.19 * 4.0 * b / res; };
+    const double alone = solid ? 0.62 : 0.25, more = solid ? 0.095 : 0.19;
+    auto plane = [&](double b) { return alone + more * 4.0 * b / res; };
     const double rounds = nb / full;
     if (rounds >= 4.0) return (mc + halo) * plane(res) * rounds;
     const double whole = (double)(long long)rounds;
@@ -72,7 +77,7 @@ inline int dirty_chunk(int mc) { return mc <= 4 ? mc : (mc / 2 - 2 > 4 ? mc / 2 
 // planes 0.692 of HBM, 24..128 planes 0.66..0.69: blocks that start together share
 // their halo rows in L2).
 inline int pick_chunk(const std::vector<Run>& runs, const std::vector<long long>& caps, int halo, int res, int threads,
-                      int sms, bool three_d, bool dbl) {
+                      int sms, bool three_d, bool dbl, bool solid) {
     double best = 0.0;
     int bmc = 0;
     std::vector<long long> nbs(caps.size());
@@ -82,16 +87,17 @@ inline int pick_chunk(const std::vector<Run>& runs, const std::vector<long long>
         for (long long& v : nbs) v = 0;
         for (const Run& r : runs) {
             const int ch = r.dirty ? dirty_chunk(mc) : mc;
-            const int nc = (r.nm + ch - 1) / ch, per = r.dirty ? 0 : (r.nm + nc - 1) / nc;
+            const int nc = (r.nm + ch - 1) / ch, per = (r.nm + nc - 1) / nc;
             nb += (double)r.cols * nc;
             nbs[(size_t)r.member] += r.cols * nc;
-            used = per > used ? per : used;
+            // the longest block, in planes of the body that most planes need
+            const int as = r.dirty && !solid && per == ch ? mc : per;
+            used = as > used ? as : used;
         }
         bool fits = true;
-        if (used == 0) used = mc;
         for (size_t k = 0; k < caps.size(); ++k) fits = fits && nbs[k] <= caps[k];
         if (!fits) continue;
-        const double c = march_cost(nb, used, halo, res, threads, sms, dbl);
+        const double c = march_cost(nb, used, halo, res, threads, sms, dbl, solid);
         if (three_d && used > 16 && nb >= 8.0 * res * sms) continue;
         if (bmc == 0 || c < best) {
             best = c;
@@ -168,7 +174,8 @@ inline FusedCfg<Q> fused_cfg(const tlbm_host::DevState& d) {
     }
     if (mc <= 0) {
         const long long cols = (long long)((NA + c.TX - 1) / c.TX) * ((NB + c.TY - 1) / c.TY);
-        mc = pick_chunk({Run{cols, NM, 0, false}}, {d.partials_cap}, c.halo(d), c.res(d), c.TX * c.TY, d.sms, Q == 19, dbl);
+        mc = pick_chunk({Run{cols, NM, 0, false}}, {d.partials_cap}, c.halo(d), c.res(d), c.TX * c.TY, d.sms, Q == 19, dbl,
+                        d.solid != nullptr);
     }
     c.MC = mc < 1 ? 1 : (mc > NM ? NM : mc);
     return c;
@@ -289,7 +296,8 @@ inline int solid_items(const tlbm_host::DevState& d, std::vector<int4>& out) {
     if (mc == 0) {
         std::vector<Run> all;
         add_runs(runs, 0, all);
-        mc = pick_chunk(all, {d.partials_cap}, runs_halo(runs), c.res(d), c.TX * c.TY, d.sms, Q == 19, d.prec == 0);
+        const int halo = runs_halo(runs);
+        mc = pick_chunk(all, {d.partials_cap}, halo, c.res(d), c.TX * c.TY, d.sms, Q == 19, d.prec == 0, halo == 4);
     }
     int dirty = make_items(runs, mc, out);
     const long long clean = (long long)out.size() - dirty;
@@ -556,8 +564,9 @@ inline cudaError_t batch_build(tlbm_host::BatchState& b, cudaStream_t st) {
             caps.push_back(dd.partials_cap);
         }
         if (own >= 2LL * c.res(d0) * d0.sms) {
-            const int mc = pick_chunk(runs, caps, (halo + n / 2) / n, c.res(d0), c.TX * c.TY, d0.sms, Q == 19,
-                                      d0.prec == 0);
+            halo = (halo + n / 2) / n;
+            const int mc = pick_chunk(runs, caps, halo, c.res(d0), c.TX * c.TY, d0.sms, Q == 19, d0.prec == 0,
+                                      solid && halo == 4);
             b.auto_tile = (b.tile & 255) | mc << 8;
         }
     }
