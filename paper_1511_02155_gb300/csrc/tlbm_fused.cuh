@@ -722,8 +722,12 @@ __device__ __forceinline__ void solid_body(const MGeom& g, const S* __restrict__
     if (tid == 0) put_block_sums(g, partials, bid, mr, mp, ms);
 }
 
-template <int Q, typename S, int TX, int TY, bool CHK = false>
-__global__ void __launch_bounds__(TX * TY, blocks_per_sm<S>(TX * TY))
+// BPS, blocks per SM: D3Q19 in FP32 and 16 bits spills at 128 registers (FP32 296 bytes
+// a thread).  Alone on the lattice three blocks with 168 are faster (5 % solid nodes,
+// FP32: 128^3 468 us a step with four, 416 with three; 40^3 47.5 and 36.8); beside the
+// clean blocks' launch four are (144x128x80, drop on a wall: 50 steps 10.99 and 11.53 ms).
+template <int Q, typename S, int TX, int TY, bool CHK = false, int BPS = blocks_per_sm<S>(TX * TY)>
+__global__ void __launch_bounds__(TX * TY, BPS)
 k_fused_solid(MGeom g, const S* __restrict__ src, S* __restrict__ dst, const uint32_t* __restrict__ nbm,
               Phys<typename Store<S>::T> P, double* __restrict__ partials) {
     solid_body<Q, S, TX, TY, CHK>(g, src, dst, nbm, P, partials, blockIdx.x, work_of<TX, TY>(g, blockIdx.x));

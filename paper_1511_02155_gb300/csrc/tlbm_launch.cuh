@@ -91,7 +91,7 @@ inline int pick_chunk(const std::vector<Run>& runs, const std::vector<long long>
             nb += (double)r.cols * nc;
             nbs[(size_t)r.member] += r.cols * nc;
             // the longest block, in planes of the body that most planes need
-            const int as = r.dirty && !solid && per == ch ? mc : per;
+            const int as = r.dirty && (dbl || !solid) && per == ch ? mc : per;
             used = as > used ? as : used;
         }
         bool fits = true;
@@ -110,10 +110,12 @@ inline int pick_chunk(const std::vector<Run>& runs, const std::vector<long long>
 template <int Q>
 struct FusedCfg {
     int TX, TY, MC;
-    // prologue planes a block recomputes, and blocks per SM (blocks_per_sm)
+    // prologue planes a block recomputes, and blocks per SM of the kernel that has the
+    // lattice to itself (mixed: of work items)
     int halo(const tlbm_host::DevState& d) const { return d.solid || d.coupling ? 4 : 2; }
-    int res(const tlbm_host::DevState& d) const {
+    int res(const tlbm_host::DevState& d, bool mixed = false) const {
         if (Q == 19 && d.prec != 0 && !d.solid && !d.coupling) return d.prec == 1 ? BulkShape<float>::BPS : BulkShape<__half>::BPS;  // k_bulk
+        if (Q == 19 && d.prec != 0 && d.solid && !mixed) return 3;  // k_fused_solid
         return d.prec == 0 && TX == 32 ? 8 : 512 / (TX * TY);
     }
 };
@@ -297,7 +299,7 @@ inline int solid_items(const tlbm_host::DevState& d, std::vector<int4>& out) {
         std::vector<Run> all;
         add_runs(runs, 0, all);
         const int halo = runs_halo(runs);
-        mc = pick_chunk(all, {d.partials_cap}, halo, c.res(d), c.TX * c.TY, d.sms, Q == 19, d.prec == 0, halo == 4);
+        mc = pick_chunk(all, {d.partials_cap}, halo, c.res(d, true), c.TX * c.TY, d.sms, Q == 19, d.prec == 0, halo == 4);
     }
     int dirty = make_items(runs, mc, out);
     const long long clean = (long long)out.size() - dirty;
@@ -421,9 +423,14 @@ inline cudaError_t solid_step(tlbm_host::DevState& d, const FusedCfg<Q>& c, cons
             e = cudaEventRecord(d.forked, st);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(d.side, d.forked, 0);
         }
-        if (e == cudaSuccess && nd > 0)
-            e = launch_smem(k_fused_solid<Q, S, TX, 4, CHK>, solid_smem<Q, S>(TX, 4), TX * 4, 512 / (TX * 4), nd, At(st, !fork),
-                            g, src, dst, d.nbm, P, d.partials);
+        auto dirty = [&](auto kern, int bps) {
+            return launch_smem(kern, solid_smem<Q, S>(TX, 4), TX * 4, bps, nd, At(st, !fork), g, src, dst, d.nbm, P, d.partials);
+        };
+        if (e == cudaSuccess && nd > 0) {
+            if constexpr (sizeof(S) < 8 && !CHK)
+                e = fork ? dirty(k_fused_solid<Q, S, TX, 4>, 4) : dirty(k_fused_solid<Q, S, TX, 4, false, 3>, 3);
+            else e = dirty(k_fused_solid<Q, S, TX, 4, CHK>, 512 / (TX * 4));
+        }
         if constexpr (sizeof(S) < 8) {
             if (e == cudaSuccess && nb > nd) {
                 MGeom gc = g;
@@ -538,10 +545,10 @@ inline cudaError_t batch_build(tlbm_host::BatchState& b, cudaStream_t st) {
         return fused_blocks<Q, S>(dd);
     };
     if ((b.tile >> 8) == 0) {
-        // members whose own chunks do not fill the device twice keep them; beyond
-        // that the halo planes of short chunks are what costs, and one chunk is
-        // chosen for the whole grid (24 wells of 128x64 .. 768x384, FP32: 343 us a
-        // step with chunks of 4 to 8 planes)
+        // members whose own chunks fit the device at once keep them; beyond that a few
+        // blocks of a second round, and then the halo planes of short chunks, are what
+        // costs, and one chunk is chosen for the whole grid (24 wells of 128x64 ..
+        // 768x384, FP32: 343 us a step with chunks of 4 to 8 planes)
         std::vector<Run> runs;
         std::vector<long long> caps;
         long long own = 0;
@@ -563,9 +570,9 @@ inline cudaError_t batch_build(tlbm_host::BatchState& b, cudaStream_t st) {
             }
             caps.push_back(dd.partials_cap);
         }
-        if (own >= 2LL * c.res(d0) * d0.sms) {
+        if (own > (long long)c.res(d0, true) * d0.sms) {
             halo = (halo + n / 2) / n;
-            const int mc = pick_chunk(runs, caps, halo, c.res(d0), c.TX * c.TY, d0.sms, Q == 19, d0.prec == 0,
+            const int mc = pick_chunk(runs, caps, halo, c.res(d0, true), c.TX * c.TY, d0.sms, Q == 19, d0.prec == 0,
                                       solid && halo == 4);
             b.auto_tile = (b.tile & 255) | mc << 8;
         }

@@ -37,3 +37,28 @@ extern "C" long long rule_blocks(int Q, int prec, int nx, int ny, int nz, int so
     if (Q == 9) return prec == 0 ? blocks<9, double>(d) : blocks<9, float>(d);
     return prec == 0 ? blocks<19, double>(d) : blocks<19, float>(d);
 }
+
+// longest block of planes near solid nodes on a D2Q9 FP32 lattice that has them
+// everywhere but in `clean` planes of its last 32-node column
+extern "C" int rule_longest_dirty(int nx, int ny, int clean, int sms) {
+    tlbm_host::DevState d{};
+    static const uint8_t some = 1;
+    d.Q = 9;
+    d.prec = 1;
+    d.nx = nx;
+    d.ny = ny;
+    d.nz = 1;
+    d.N = (long long)nx * ny;
+    d.ncx = (nx + 31) / 32;
+    d.solid = &some;
+    d.sms = sms;
+    d.partials_cap = std::max(d.N / 64 + 1, (long long)tlbm_host::kMassBlocks);
+    std::vector<uint8_t> units((size_t)ny * d.ncx, (uint8_t)1);
+    for (int m = 0; m < clean; ++m) units[(size_t)(ny / 2 + m) * d.ncx + d.ncx - 1] = 0;
+    d.units = units.data();
+    std::vector<int4> items;
+    const int dirty = tlbm_dev::solid_items<9, float>(d, items);
+    int most = 0;
+    for (int k = 0; k < dirty; ++k) most = std::max(most, (items[k].w >> 1) - items[k].z);
+    return most;
+}

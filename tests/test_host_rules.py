@@ -18,9 +18,9 @@ def rules(tmp_path_factory):
     out = str(tmp_path_factory.mktemp("rules") / "librules.so")
     subprocess.run([_build.nvcc(), *_build.ARCH, "-std=c++17", "--expt-relaxed-constexpr", "-O1", "-shared", "-Xcompiler",
                     "-fPIC", os.path.join(HERE, "host_rules.cu"), "-o", out, "-cudart", "static"], check=True)
-    f = ctypes.CDLL(out).rule_blocks
-    f.restype = ctypes.c_longlong
-    return f
+    lib = ctypes.CDLL(out)
+    lib.rule_blocks.restype = ctypes.c_longlong
+    return lib
 
 
 def _plain_fits(Q, prec, shape, solid, coupling, chunk):
@@ -51,5 +51,13 @@ def test_every_lattice_that_plain_tiles_take_is_taken(rules, Q, prec, coupling, 
     sizes = [(x, y, 1) for x, y in itertools.product(ROWS, ROWS)] if Q == 9 else \
         [(x, y, z) for x, y, z in itertools.product(ROWS[::3], ROWS[::4], ROWS[1::4])]
     lost = [s for s in sizes if s[0] * s[1] * s[2] < 4e7 and _plain_fits(Q, prec, s, solid, coupling, chunk)
-            and rules(Q, prec, *s, solid, coupling, 256 * chunk, SMS) < 0]
+            and rules.rule_blocks(Q, prec, *s, solid, coupling, 256 * chunk, SMS) < 0]
     assert not lost, lost[:10]
+
+
+@pytest.mark.parametrize("nx,ny", [(517, 391), (389, 500), (1000, 701)])
+def test_a_short_clean_run_does_not_set_the_chunk_of_all_blocks(rules, nx, ny):
+    """Planes near solid nodes march as far as they would without one gap among them."""
+    alone = rules.rule_longest_dirty(nx, ny, 0, SMS)
+    for clean in (9, 12):  # five and eight planes that are two nodes from the others
+        assert abs(rules.rule_longest_dirty(nx, ny, clean, SMS) - alone) <= 1
