@@ -176,8 +176,8 @@ __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
 // more, starts no copy and does not arrive, so that the phases it should arrive at stay
 // open and the block's other threads run out of their next wait in turn.  It gives the
 // copies in flight a second wait before it goes on, so that the block's shared memory
-// is not given up under them.  (Each thread's own word, not a vote at the barrier:
-// __syncthreads_or cost 1 % of a step on 512x256.)
+// is not given up under them.  (Each thread's own words, not a vote at the barrier:
+// __syncthreads_or cost 1 % of a step on 517x391 in 16 bits.)
 __device__ __forceinline__ void bulk_load(unsigned dst, const void* src, unsigned bytes, unsigned bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                  "l"(src), "r"(bytes), "r"(bar)
@@ -233,7 +233,7 @@ __device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ 
     const int W = min(32, g.NA - 32 * chunk);  // nodes of this chunk
     const int H = min(TY, g.NB - B0);          // rows of this tile
     const int rows = H + 2;
-    const bool active = lane < W && ty < H;
+    bool active = lane < W && ty < H;
     const unsigned char* const srcb = reinterpret_cast<const unsigned char*>(src);
     const long long pstride = (long long)g.NB * g.rowstride;
     const int last = M1 - M0 + 1;  // planes 0 .. last of the march: M0 - 1 .. M1
@@ -393,12 +393,13 @@ __device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ 
     NodePops<S> cur, nxt;
     cur.clear();
     float jc[3] = {0.0f, 0.0f, 0.0f}, rdc = 0.0f;
-    bool late = false;
+    int upto = last;  // copies of the planes up to here; below 0: late
 
 #pragma unroll 1
     for (int p = 0; p <= last; ++p) {
-        if (!late && !mbar_wait(bar, p & 1)) {
-            late = true;
+        if (upto >= 0 && !mbar_wait(bar, p & 1)) {
+            upto = -1;
+            active = false;
             mbar_wait(bar, p & 1);
         }
 
@@ -447,7 +448,7 @@ __device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ 
             rg[2 * B::RN + cb] = s2;
         }
         __syncthreads();  // the slot is read, the ring written
-        if (p < last && !late) start();
+        if (p < upto) start();
 
         // ---- derivatives and collision of plane p - 1
         if (active) {
@@ -469,7 +470,7 @@ __device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ 
                 }
             }
             push(rg, c1);
-            if (p >= 2 && !late) {
+            if (p >= 2) {
                 if constexpr (I::PACKED) msum.add(rdc, X[1], X[2]);
                 else msum.add(rho_total<Q, S>(rdc), X[1], X[2]);
                 unsigned char* const out = chk_node<Q, S, CHK>(g, reinterpret_cast<unsigned char*>(dst),
@@ -486,7 +487,7 @@ __device__ __forceinline__ void bulk_body(const MGeom& g, const S* __restrict__ 
         jc[2] = jn[2];
         rdc = rdn;
     }
-    if (late) atomicOr(g.flag, 2);  // a copy did not arrive: the step's results are void
+    if (upto < 0) atomicOr(g.flag, 2);  // a copy did not arrive: the step's results are void
     double mr, mp, ms;
     msum.get(mr, mp, ms);
     block_sum3(mr, mp, ms);
@@ -535,7 +536,7 @@ __device__ __forceinline__ void bulk2_body(const MGeom& g, const S* __restrict__
     const int tid = threadIdx.x;
     const int A0 = wk.A0, M0 = wk.M0, M1 = wk.M1;
     const int W = min(TX, g.NA - A0);  // nodes of this tile
-    const bool active = tid < W;
+    bool active = tid < W;
     const unsigned char* const srcb = reinterpret_cast<const unsigned char*>(src);
     const int last = M1 - M0 + 1;
 
@@ -647,11 +648,12 @@ __device__ __forceinline__ void bulk2_body(const MGeom& g, const S* __restrict__
     NodePops<S, Q> cur, nxt;
     cur.clear();
     float jc[3] = {0.0f, 0.0f, 0.0f}, rdc = 0.0f;
-    bool late = false;
+    int upto = last;  // as in bulk_body
 #pragma unroll 1
     for (int p = 0; p <= last; ++p) {
-        if (!late && !mbar_wait(bar0 + (p & 1) * 8, (p >> 1) & 1)) {
-            late = true;
+        if (upto >= 0 && !mbar_wait(bar0 + (p & 1) * 8, (p >> 1) & 1)) {
+            upto = -1;
+            active = false;
             mbar_wait(bar0 + (p & 1) * 8, (p >> 1) & 1);
             if (p < last) mbar_wait(bar0 + ((p + 1) & 1) * 8, ((p + 1) >> 1) & 1);
         }
@@ -693,7 +695,7 @@ __device__ __forceinline__ void bulk2_body(const MGeom& g, const S* __restrict__
             rg[bset * B::RN + bx] = bset == 0 ? acc + 1.0f : acc;
         }
         __syncthreads();  // the slot is read, the ring written
-        if (p + 2 <= last && !late) start(p + 2);
+        if (p + 2 <= upto) start(p + 2);
 
         // ---- derivatives and collision of plane p - 1
         if (active) {
@@ -703,7 +705,7 @@ __device__ __forceinline__ void bulk2_body(const MGeom& g, const S* __restrict__
                     return rg[k * B::RN + (int)chk_index<CHK>(g, tid + i + 1, B::RN, 4) - 1];
                 },
                 c1, X, g12, l6);
-            if (p >= 2 && !late) {
+            if (p >= 2) {
                 msum.add(rdc, X[1], X[2]);
                 unsigned char* const out = chk_node<Q, S, CHK>(g, reinterpret_cast<unsigned char*>(dst),
                                                                outb + (long long)(M0 + p - 2) * g.rowstride, 3);
@@ -718,7 +720,7 @@ __device__ __forceinline__ void bulk2_body(const MGeom& g, const S* __restrict__
         jc[1] = jn[1];
         rdc = rdn;
     }
-    if (late) atomicOr(g.flag, 2);  // a copy did not arrive: the step's results are void
+    if (upto < 0) atomicOr(g.flag, 2);  // a copy did not arrive: the step's results are void
     double mr, mp, ms;
     msum.get(mr, mp, ms);
     block_sum3(mr, mp, ms);
