@@ -136,7 +136,12 @@ cudaError_t set_items(tlbm* t) {
     }
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(t->st, &cap);
-    if (e != cudaSuccess) return e;
+    if (e == cudaErrorStreamCaptureImplicit) {  // the default stream, while another one is captured
+        cudaGetLastError();
+        cap = cudaStreamCaptureStatusActive;
+    } else if (e != cudaSuccess) {
+        return e;
+    }
     if (cap != cudaStreamCaptureStatusNone) {
         t->items_late = 1;
         return cudaSuccess;

@@ -77,7 +77,7 @@ void fake_items(int tile, int n) {  // the work items of that tile
     for (int k = 0; k < n; ++k) items[tile].push_back(make_int4(tile, k, 0, 3));
 }
 void fake_flag(int v) { next_flag = v; }         // raised by the next steps
-void fake_capturing(int on) { capturing = on; }  // every stream
+void fake_capturing(int on) { capturing = on; }  // every stream; 2: another than the engine's, the default one
 void fake_build_fails(int n) { build_fails = n; }
 void fake_throws(int on) { throws = on; }  // the kernel tables' host code
 int fake_allocations() { return (int)live.size(); }
@@ -125,6 +125,7 @@ cudaError_t cudaStreamSynchronize(cudaStream_t st) {
     return cudaSuccess;
 }
 cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* s) {
+    if (capturing == 2) return cudaErrorStreamCaptureImplicit;
     *s = capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
     return cudaSuccess;
 }

@@ -94,7 +94,8 @@ def test_a_failed_upload_of_work_items_leaves_one_grid(fake, call):
     assert fake.fake_allocations() == 0
 
 
-def test_work_items_outlive_a_change_of_tile(fake):
+@pytest.mark.parametrize("capture", [1, 2])
+def test_work_items_outlive_a_change_of_tile(fake, capture):
     """Steps captured at one tile may be replayed at any time later: their items stay,
     and a tile that was chosen before needs no call that a capture forbids."""
     rc, t = _create(fake)
@@ -105,7 +106,7 @@ def test_work_items_outlive_a_change_of_tile(fake):
     late = fake.fake_allocations()
     assert fake.tlbm_set_tile(t, 2, 7) == 0
     assert fake.fake_allocations() == late + 1  # and those are still allocated
-    fake.fake_capturing(1)
+    fake.fake_capturing(capture)
     assert fake.tlbm_set_tile(t, 0, 0) == 0 and fake.tlbm_step(t, 1) == 0
     assert fake.tlbm_set_tile(t, 2, 7) == 0 and fake.tlbm_step(t, 1) == 0
     fake.fake_items(256 * 3, 4)
