@@ -205,7 +205,9 @@ size_t tlbm_state_bytes(const tlbm *t);
  * A state saved by tlbm_get_state resumes bitwise identically.  The bytes are
  * the device layout of this library build (chunked lane words per storage
  * format and lattice), not an interchange format: use tlbm_get_populations /
- * tlbm_set_populations to move a state between builds.  Synchronises. */
+ * tlbm_set_populations to move a state between builds.  Only the size is checked:
+ * another build's state of the same size is read in this build's order.
+ * Synchronises. */
 tlbm_status tlbm_get_state(tlbm *t, void *host, size_t bytes);
 tlbm_status tlbm_set_state(tlbm *t, const void *host, size_t bytes);
 
