@@ -25,7 +25,8 @@
 //   derivatives of p - 1 (Roll), collision of p - 1 from registers, store
 // One slot: the copies run while the plane before is collided, the larger part of
 // the work, and the other blocks of the SM fill what wait is left.  A second slot
-// measured slower (FP32 1.96 against 1.55 ms at 256^3, FP16 1.38 against 1.00): it
+// measured slower (side by side, with 4-byte words at the ends: FP32 1.96 against 1.55
+// ms at 256^3, FP16 1.38 against 1.00; the present kernel takes 1.46 to 1.54 and 1.04): it
 // takes the L1 that the words of x neighbours need on their way, a 128-byte line
 // for each.  One barrier a plane, since the ring holds two planes or more.
 #pragma once
