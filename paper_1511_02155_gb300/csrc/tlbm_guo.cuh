@@ -385,7 +385,8 @@ k_guo_velocity(Geom g, const T* __restrict__ mom, const T* __restrict__ aux, dou
 // What it costs is the halo: with 32x4 tiles on D3Q19 the moments of 288 nodes and Pi
 // of 204 for 128 of the tile.  Tiles of 32x8 (432 and 340 for 256), mu kept from P
 // instead of a second set of derivatives in C, and link pairs in the collision:
-// 128^3 FP32 351 us a step before, 337 after.
+// 128^3 FP32 351 us a step before, 345 after (338 with totals in pairs of floats, which
+// hold fewer bits).
 template <int Q, typename S>
 constexpr int guo_smem(int TX, int TY) {
     const int b = Q == 19 ? 1 : 0, hn = (TX + 4) * (TY + 4 * b), pn = (TX + 2) * (TY + 2 * b);
